@@ -24,6 +24,13 @@ constexpr int kBlocksPerSM = 4;     // forward apply: 256-thread CTAs resident p
 constexpr int kBwdBlocksPerSM = 3;  // backward apply pass (85 registers per thread)
 constexpr int kReduceBlocksPerSM = 2;  // backward reduce pass: four rows' loads in flight per thread
 constexpr int kReduceUnroll = 4;
+// Forward apply of tensors above this size: last row first.  The convolution before it wrote y from
+// row 0 on, so the end of y is still in L2 when the pass starts, and the pass leaves the first rows of
+// out there for the next convolution, which starts at row 0.  Two convolutions and their passes
+// (a residual block) against row order: 206 MB and 103 MB tensors 401 -> 394 and 217 -> 210 us, 103 MB
+// at 128 channels 267 -> 260 us; at 51 MB, where everything between two passes fits in L2 anyway,
+// 143.1 -> 145.5 us and 116.6 -> 118.9 us, so those stay in row order.
+constexpr int64_t kReverseAboveBytes = 64ll << 20;
 
 __device__ __forceinline__ void unpack8(const uint4& v, float (&f)[8])
 {
@@ -129,7 +136,7 @@ __global__ void __launch_bounds__(dbl::dev::kPartialsThreads) bn_fwd_finalize_pa
 // channel's scale and shift stay in registers.
 __global__ void __launch_bounds__(kThreads, kBlocksPerSM)
     bn_apply_kernel(const act_t* __restrict__ y, const act_t* __restrict__ res,
-                    act_t* __restrict__ out, int count, int C, int relu, const float* __restrict__ gamma,
+                    act_t* __restrict__ out, int count, int C, int relu, int reverse, const float* __restrict__ gamma,
                     const float* __restrict__ beta, const float* __restrict__ mean, const float* __restrict__ invstd)
 {
     dbl::dev::grid_dependency_trigger();  // a convolution launched next may start its set-up
@@ -156,19 +163,20 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM)
     };
     const uint4 zero = make_uint4(0, 0, 0, 0);  // bf16 +0 in every lane
     int r = blockIdx.x * rstep + threadIdx.x / groups;
+    const int base = reverse ? count - 1 : 0, dir = reverse ? -1 : 1;
     for (; r + (kUnroll - 1) * step < count; r += kUnroll * step) {
         uint4 yv[kUnroll], rv[kUnroll];
 #pragma unroll
         for (int u = 0; u < kUnroll; ++u) {
-            const int v = (r + u * step) * groups + g;
+            const int v = (base + dir * (r + u * step)) * groups + g;
             yv[u] = __ldcs(reinterpret_cast<const uint4*>(y) + v);
             rv[u] = res ? __ldcs(reinterpret_cast<const uint4*>(res) + v) : zero;
         }
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) emit(yv[u], rv[u], (r + u * step) * groups + g);
+        for (int u = 0; u < kUnroll; ++u) emit(yv[u], rv[u], (base + dir * (r + u * step)) * groups + g);
     }
     for (; r < count; r += step) {
-        const int v = r * groups + g;
+        const int v = (base + dir * r) * groups + g;
         emit(__ldcs(reinterpret_cast<const uint4*>(y) + v), res ? __ldcs(reinterpret_cast<const uint4*>(res) + v) : zero,
              v);
     }
@@ -187,14 +195,23 @@ struct Vec8 {
     uint4 d, d2, o, y;
 };
 
-template <int MASK>
+// One 16-byte vector.  KEEP: the apply pass reads the tensor again, so its lines stay in L2; otherwise
+// they leave it first.
+template <bool KEEP>
+__device__ __forceinline__ uint4 load_vec(const act_t* p, int v)
+{
+    const uint4* q = reinterpret_cast<const uint4*>(p) + v;
+    return KEEP ? __ldg(q) : __ldcs(q);
+}
+
+template <int MASK, bool KEEP_G, bool KEEP_Y>
 __device__ __forceinline__ void load_g_raw(const act_t* dout, const act_t* dout2,
                                            const act_t* out, const act_t* y, int v, Vec8& g, Vec8& yv)
 {
-    g.d = __ldcs(reinterpret_cast<const uint4*>(dout) + v);
-    g.d2 = dout2 ? __ldcs(reinterpret_cast<const uint4*>(dout2) + v) : make_uint4(0, 0, 0, 0);
-    g.o = MASK == kMaskOut ? __ldcs(reinterpret_cast<const uint4*>(out) + v) : make_uint4(0, 0, 0, 0);
-    yv.y = __ldcs(reinterpret_cast<const uint4*>(y) + v);
+    g.d = load_vec<KEEP_G>(dout, v);
+    g.d2 = dout2 ? load_vec<KEEP_G>(dout2, v) : make_uint4(0, 0, 0, 0);
+    g.o = MASK == kMaskOut ? load_vec<KEEP_G>(out, v) : make_uint4(0, 0, 0, 0);
+    yv.y = load_vec<KEEP_Y>(y, v);
 }
 
 template <int MASK>
@@ -247,7 +264,7 @@ __device__ __forceinline__ void accumulate_g(const Vec8& graw, const Vec8& yraw,
     float gg[8], yy[8];
     unpack8(yraw.y, yy);
     combine_g(graw, yy, two, relu, gg);
-    if constexpr (WRITE_G) __stcs(reinterpret_cast<uint4*>(g_out) + v, pack8(gg));
+    if constexpr (WRITE_G) reinterpret_cast<uint4*>(g_out)[v] = pack8(gg);
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
         sg[k] += gg[k];
@@ -261,6 +278,12 @@ __device__ __forceinline__ void accumulate_g(const Vec8& graw, const Vec8& yraw,
 // b + gridDim.x, ....  Interleaved chunks keep all CTAs streaming through the same
 // region of the tensors, and each partial adds its rows in a fixed order, so the
 // result does not depend on the grid.
+// The rows are visited last to first: the data gradient before this pass wrote dout from
+// row 0 on, so its end is still in L2, and the apply pass after it, which goes from row 0
+// on, finds the rows visited last here.  What the apply pass reads again (y, and g or
+// dout) is loaded and stored with the default cache policy, the rest evict-first.  Both
+// passes at HBM rate before and after: a residual block's backward at 128 channels, batch 185,
+// 28 x 28 (37 MB tensors) 320 -> 306 us, at 64 channels, batch 512, 56 x 56 (206 MB) 883 -> 865 us.
 template <int MASK, bool WRITE_G>
 __global__ void __launch_bounds__(kThreads, kReduceBlocksPerSM)
     bn_bwd_reduce_kernel(const act_t* __restrict__ dout, const act_t* __restrict__ dout2,
@@ -283,19 +306,21 @@ __global__ void __launch_bounds__(kThreads, kReduceBlocksPerSM)
     for (int blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
     float sg[8] = {}, sgx[8] = {};
     int r = blk * rstep + threadIdx.x / groups;
+    const int last = count - 1;
     for (; r + (U - 1) * cstep < count; r += U * cstep) {
         Vec8 gg[U], yy[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) load_g_raw<MASK>(dout, dout2, out, y, (r + u * cstep) * groups + g, gg[u], yy[u]);
+        for (int u = 0; u < U; ++u)
+            load_g_raw<MASK, !WRITE_G, true>(dout, dout2, out, y, (last - (r + u * cstep)) * groups + g, gg[u], yy[u]);
 #pragma unroll
         for (int u = 0; u < U; ++u)
             accumulate_g<MASK, WRITE_G>(gg[u], yy[u], dout2 != nullptr, rm, mu, sg, sgx, g_out,
-                                        (r + u * cstep) * groups + g);
+                                        (last - (r + u * cstep)) * groups + g);
     }
     for (; r < count; r += cstep) {
         Vec8 gg, yy;
-        load_g_raw<MASK>(dout, dout2, out, y, r * groups + g, gg, yy);
-        accumulate_g<MASK, WRITE_G>(gg, yy, dout2 != nullptr, rm, mu, sg, sgx, g_out, r * groups + g);
+        load_g_raw<MASK, !WRITE_G, true>(dout, dout2, out, y, (last - r) * groups + g, gg, yy);
+        accumulate_g<MASK, WRITE_G>(gg, yy, dout2 != nullptr, rm, mu, sg, sgx, g_out, (last - r) * groups + g);
     }
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
@@ -373,20 +398,20 @@ __global__ void __launch_bounds__(kThreads, kBwdBlocksPerSM)
         combine_g(graw, yy, dout2 != nullptr, rm, gg);
 #pragma unroll
         for (int k = 0; k < 8; ++k) d[k] = fmaf(ca[k], gg[k], fmaf(cb[k], yy[k], cc[k]));
-        __stcs(reinterpret_cast<uint4*>(dy) + v, pack8(d));
+        reinterpret_cast<uint4*>(dy)[v] = pack8(d);
         if (dres) __stcs(reinterpret_cast<uint4*>(dres) + v, pack8(gg));
     };
     int r = blockIdx.x * rstep + threadIdx.x / groups;
     for (; r + (kUnroll - 1) * step < count; r += kUnroll * step) {
         Vec8 gg[kUnroll], yy[kUnroll];
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) load_g_raw<MASK>(dout, dout2, out, y, (r + u * step) * groups + g, gg[u], yy[u]);
+        for (int u = 0; u < kUnroll; ++u) load_g_raw<MASK, false, false>(dout, dout2, out, y, (r + u * step) * groups + g, gg[u], yy[u]);
 #pragma unroll
         for (int u = 0; u < kUnroll; ++u) emit(gg[u], yy[u], (r + u * step) * groups + g);
     }
     for (; r < count; r += step) {
         Vec8 gg, yy;
-        load_g_raw<MASK>(dout, dout2, out, y, r * groups + g, gg, yy);
+        load_g_raw<MASK, false, false>(dout, dout2, out, y, r * groups + g, gg, yy);
         emit(gg, yy, r * groups + g);
     }
 }
@@ -407,6 +432,8 @@ int reduce_grid(int64_t nblk)
     const int64_t per_cta = (nblk + cap - 1) / cap;
     return (int)((nblk + per_cta - 1) / per_cta);
 }
+
+int apply_reversed(const dbl_bn_shape* s) { return s->count * s->c * (int64_t)sizeof(act_t) > kReverseAboveBytes; }
 
 int check_shape(const dbl_bn_shape* s, const char* who)
 {
@@ -538,7 +565,8 @@ int dbl_bn_relu_fused(const dbl_bn_shape* s, const void* y, const float* ch_sum,
     if ((rc = bn_fwd_finalize(s->count, s->c, s->eps, ch_sum, ch_sumsq, save_mean, save_invstd, st))) return rc;
     bn_apply_kernel<<<bn_grid(s->count * s->c / 8), kThreads, 0, st>>>(
         static_cast<const act_t*>(y), static_cast<const act_t*>(residual),
-        static_cast<act_t*>(out), (int)s->count, s->c, s->relu, gamma, beta, save_mean, save_invstd);
+        static_cast<act_t*>(out), (int)s->count, s->c, s->relu, apply_reversed(s), gamma, beta,
+        save_mean, save_invstd);
     return launch_check("bn_relu_fused launch");
 }
 
@@ -562,7 +590,8 @@ int dbl_bn_relu_fused_parts(const dbl_bn_shape* s, const void* y, const float* p
     if ((rc = launch_check("bn_fwd_finalize_parts launch"))) return rc;
     bn_apply_kernel<<<bn_grid(s->count * s->c / 8), kThreads, 0, st>>>(
         static_cast<const act_t*>(y), static_cast<const act_t*>(residual),
-        static_cast<act_t*>(out), (int)s->count, s->c, s->relu, gamma, beta, save_mean, save_invstd);
+        static_cast<act_t*>(out), (int)s->count, s->c, s->relu, apply_reversed(s), gamma, beta,
+        save_mean, save_invstd);
     return launch_check("bn_relu_fused_parts launch");
 }
 
