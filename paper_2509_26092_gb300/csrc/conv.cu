@@ -82,7 +82,10 @@ struct ConvParams {
     int win_srows;            // padded rows loaded per strip (weight gradient: x strip)
     int win_dyrows;           // weight gradient: padded rows of the dy strip
     int win_strip_bytes;      // bytes of one strip buffer, or of one x + dy stage (a multiple of 1024)
-    int win_margin;           // CTA pairs: bytes before and after each strip buffer (0 for single CTAs)
+    int win_margin;           // CTA pairs: bytes before and after each strip buffer (0 for single CTAs);
+                              // row-block weight gradient: offset of the dy strip in a stage
+    int win_stages;           // row-block weight gradient: x + dy stages
+    int win_bpi;              // row-block weight gradient: K-blocks per image
     int test_stall;           // dbl_conv_test_stall_next: block 0 never loads its first K-block
 };
 
@@ -1261,6 +1264,189 @@ __global__ void __launch_bounds__(kWinThreads, 1)
     }
 }
 
+// ----------------------------------------------------------------------------- row-block weight gradient
+// dW[k][r][s][c] of a 3x3 stride-1 layer with 64 input and 64 output channels.  A K-block is R whole
+// output rows of one image at a row pitch of `win_Wp` >= W + 2*pw positions (R * pitch a multiple of
+// 16): one x strip of R + 2 padded rows from column -pw, and one dy strip of R rows from column -2, so
+// that strip position h*pitch + w + n holds dy at column w + n - 2 (zeros outside the output).  Then
+//     dW[r][s] = sum over L of x[L + r*pitch] * dy[L + 2 - s]
+// and a column tap is a shift of dy, a row tap a shift of x.  Both are 128-byte rows of one strip
+// apart, so MN-major operand atoms that overlap in shared memory (a leading-dimension step of one or
+// two rows, or of one pitch) put two row taps on M and three column taps on N:
+//     accumulator 0, 128 x 192: A = x rows {L, L + pitch}, B = dy rows {L, L + 1, L + 2}: taps (0..1, 2..0)
+//     accumulator 1, 128 x 128: A = x rows {L + 2*pitch, + 1}, B = dy rows {L, L + 2}: taps (2, 2), (2, 0)
+//                               in the first half, (2, 1) and an unused product in the second
+// Two MMAs of 320 columns (160 tensor cycles) per 16 positions.  One tap pair per N = 64 MMA, five of
+// them per 16 positions, is bound by their operand reads (6 KB of shared memory per 32 cycles of tensor
+// time): 56x56, batch 512 and 128: 114.8 -> 94.9 us and 43.6 -> 38.0 us with the reduce; 72x72, batch
+// 185 75.5 -> 59.9; 24x24, batch 512 36.3 -> 28.7; 32x32, batch 64 19.2 -> 17.4.
+// Position shifts reach two rows past the dy strip and one past the x strip: those 128-byte rows
+// are the next row's columns -2, -1 and -pw, which are zeros in any strip and are written here once.
+constexpr int kWgRowMaxStages = 4;
+
+__global__ void __launch_bounds__(kWinThreads, 1)
+    conv_wgrow_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmDY,
+                      const ConvParams p)
+{
+    dbl::dev::grid_dependency_trigger();  // a convolution launched next may start its set-up
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t full_bar[kWgRowMaxStages], empty_bar[kWgRowMaxStages], accf_bar, drain_bar;
+    __shared__ uint32_t tmem_slot;
+    __shared__ volatile int abort_flag;
+
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    uint8_t* sgen = smem_raw + (sbase - smem_u32(smem_raw));
+    const int pitch = p.win_Wp, rows = p.win_dyrows;
+    const int xbytes = p.win_srows * pitch * 128, ybytes = rows * pitch * 128;
+    const int xalign = p.win_margin;  // dy strip offset in a stage
+    const int stage_bytes = p.win_strip_bytes, stages = p.win_stages;
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < stages; ++i) {
+            mbar_init(&full_bar[i], 2);  // one expect_tx arrival per producer warp
+            mbar_init(&empty_bar[i], 1);
+        }
+        mbar_init(&accf_bar, 1);
+        mbar_init(&drain_bar, 1);
+        abort_flag = 0;
+        fence_mbar_init();
+    }
+    // the zero rows behind each strip (8 16-byte words per row), before any MMA reads them
+    for (int i = threadIdx.x; i < stages * 24; i += blockDim.x) {
+        const int s = i / 24, w = i % 24;
+        uint8_t* dst = sgen + s * stage_bytes + (w < 8 ? xbytes + 16 * w : xalign + ybytes + 16 * (w - 8));
+        *reinterpret_cast<uint4*>(dst) = make_uint4(0, 0, 0, 0);
+    }
+    fence_async_shared();
+    if ((warp == 4 || warp == 5) && lane == 0) tma_prefetch_desc(warp == 4 ? &tmX : &tmDY);
+    if (warp == 6) {
+        tmem_alloc(&tmem_slot, 512);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    grid_dependency_wait();  // the set-up above may overlap the previous kernel; memory only after it
+    const uint32_t tmem = tmem_slot;
+    // this CTA's K-blocks (grid = slices: at least one K-block each)
+    const int z = blockIdx.x;
+    const int kb0 = z * p.kb_per_split, kb1 = min(p.num_kb, kb0 + p.kb_per_split);
+
+    if (warp == 4 || warp == 5) {
+        // ------------------------------------------------------------------ producers: x strips (4), dy strips (5)
+        const bool is_x = warp == 4;
+        const int bpi = p.win_bpi;  // K-blocks per image
+        int s = 0, it = 0;
+        uint32_t phase = 1;
+        bool failed = false;
+        for (int kb = kb0; kb < kb1; ++kb, ++it) {
+            const uint32_t ok = mbar_wait_warp(&empty_bar[s], phase, &abort_flag);
+            if (__any_sync(0xffffffffu, ok == 0u)) {
+                failed = true;
+                break;
+            }
+            uint8_t* dst = sgen + s * stage_bytes + (is_x ? 0 : xalign);
+            const int n = kb / bpi, h0 = (kb - n * bpi) * rows;
+            mbar_arrive_expect_tx_elect(&full_bar[s], (uint32_t)(is_x ? xbytes : ybytes));
+            if (is_x)
+                tma_load_4d_elect(dst, &tmX, &full_bar[s], 0, -p.win_pw, h0 - p.win_ph, n);
+            else
+                tma_load_4d_elect(dst, &tmDY, &full_bar[s], 0, -2, h0, n);
+            if (++s == stages) {
+                s = 0;
+                phase ^= 1;
+            }
+        }
+        if (failed) {
+            if (lane == 0) report_timeout(&abort_flag);
+            for (int i = it - 1; i >= 0 && i >= it - stages; --i)
+                (void)mbar_drain_warp(&full_bar[i % stages], (i / stages) & 1);
+        }
+    } else if (warp == 6) {
+        // ------------------------------------------------------------------ MMA issuer
+        const uint32_t idesc0 = idesc_act(BM, 192, 1u, 1u), idesc1 = idesc_act(BM, 128, 1u, 1u);
+        const uint64_t dA0 = smem_desc(0, (uint32_t)(pitch * 128), 1024, kSwizzle128B);
+        const uint64_t dA1 = smem_desc(0, 128, 1024, kSwizzle128B);
+        const uint64_t dB0 = smem_desc(0, 128, 1024, kSwizzle128B);
+        const uint64_t dB1 = smem_desc(0, 256, 1024, kSwizzle128B);
+        const uint32_t row2 = (uint32_t)(2 * pitch * 8);  // two rows, in 16-byte units
+        const int ksteps = p.win_tile / 16;
+        bool failed = false;
+        int s = 0;
+        uint32_t phase = 0;
+        const uint32_t ok = mbar_wait_warp(&full_bar[0], 0, &abort_flag);
+        failed = __any_sync(0xffffffffu, ok == 0u);
+        for (int kb = kb0; kb < kb1 && !failed; ++kb) {
+            tc_fence_after();
+            const uint32_t xa = (sbase + (uint32_t)(s * stage_bytes)) >> 4, ya = xa + ((uint32_t)xalign >> 4);
+            auto step = [&](int j, uint32_t acc) {
+                const uint32_t xj = xa + (uint32_t)(j * 128), yj = ya + (uint32_t)(j * 128);  // 16 rows of 128 bytes
+                mma_act_elect(tmem, dA0 + xj, dB0 + yj, idesc0, acc);
+                mma_act_elect(tmem + 192, dA1 + (xj + row2), dB1 + yj, idesc1, acc);
+            };
+            step(0, kb > kb0 ? 1u : 0u);
+#pragma unroll 4
+            for (int j = 1; j < ksteps - 1; ++j) step(j, 1u);
+            const int sc = s;
+            if (++s == stages) {
+                s = 0;
+                phase ^= 1;
+            }
+            // the next stage's wait while the tensor pipe still has work queued
+            if (kb + 1 < kb1) {
+                const uint32_t okn = mbar_wait_warp(&full_bar[s], phase, &abort_flag);
+                failed = __any_sync(0xffffffffu, okn == 0u);
+            }
+            if (ksteps > 1) step(ksteps - 1, 1u);
+            mma_commit_elect(&empty_bar[sc]);
+        }
+        mma_commit_elect(&accf_bar);  // arrives when this slice's MMAs have completed
+        if (failed && lane == 0) report_timeout(&abort_flag);
+        mma_commit_elect(&drain_bar);
+        (void)mbar_drain_warp(&drain_bar, 0);
+    } else {
+        // ------------------------------------------------------------------ epilogue (warps 0-3)
+        const int i = warp * 32 + lane;  // TMEM lane = accumulator row
+        const int half = i >> 6, c = i & 63;
+        const uint32_t ok = mbar_wait_warp(&accf_bar, 0, &abort_flag);
+        if (__any_sync(0xffffffffu, ok == 0u)) {
+            if (lane == 0) report_timeout(&abort_flag);
+        } else {
+            tc_fence_after();
+#pragma unroll 1
+            for (int b = 0; b < 5; ++b) {  // 64-column blocks: one tap per half
+                const int tap = b < 3 ? half * 3 + 2 - b : half == 0 ? 6 + (b == 3 ? 2 : 0) : b == 4 ? 7 : -1;
+                const int m = tap * 64 + c;  // row of dW viewed as [k][(r, s, c)]
+#pragma unroll 1
+                for (int ch = 0; ch < 2; ++ch) {
+                    uint32_t v[32];
+                    tmem_ld_32x32b_x32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(b * 64 + ch * 32), v);
+                    tmem_ld_wait();
+                    if (tap >= 0) {
+                        // [slice][k][m]: consecutive lanes hold consecutive m, one 128-byte line per store
+                        float* o = static_cast<float*>(p.out) + ((int64_t)z * 64 + ch * 32) * p.M + m;
+                        if (p.zdim == 1 && p.wg_accumulate) {
+#pragma unroll
+                            for (int k = 0; k < 32; ++k) o[(int64_t)k * p.M] += __uint_as_float(v[k]);
+                        } else {
+#pragma unroll
+                            for (int k = 0; k < 32; ++k) o[(int64_t)k * p.M] = __uint_as_float(v[k]);
+                        }
+                    }
+                }
+            }
+            tc_fence_before();
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 6) {
+        tc_fence_after();
+        tmem_dealloc(tmem, 512);
+    }
+}
+
 // ----------------------------------------------------------------------------- reductions
 // Per-output-channel sums of the conv epilogue's per-CTA partials part[nparts][2][K]
 // (partials_colsum, fixed order).
@@ -1350,6 +1536,7 @@ struct Plan {
     size_t ws_main = 0;  // bytes: fwd channel-sum partials, or wgrad split-K slices
     bool win = false;    // conv_win_kernel (3x3 stride-1 correlation over padded strips)
     bool res = false;    // window kernel with all weights resident in shared memory
+    bool wgrow = false;  // conv_wgrow_kernel (3x3 stride-1 weight gradient, 64 channels)
     size_t smem = 0;     // window kernel dynamic shared memory
 };
 
@@ -1520,16 +1707,74 @@ bool win_setup(const dbl_conv_shape* s, int red_c, int out_c, bool dgrad, Plan& 
     return true;
 }
 
+// Row-block weight-gradient eligibility and geometry (see conv_wgrow_kernel): 3x3 filters at stride 1,
+// 64 input and 64 output channels.  The row pitch and the rows per K-block minimise the modelled time
+// of the busiest CTA: per K-block the longer of its MMAs (160 cycles per 16 positions) and its loads
+// (the real columns of R + 2 x rows and R dy rows at 40 bytes per cycle), and ~100 cycles of hand-over.
+bool wgrow_setup(const dbl_conv_shape* s, Plan& pl)
+{
+    const Geom g = geom(s);
+    if (g.sh != 1 || g.sw != 1 || s->r != 3 || s->s != 3 || s->c != 64 || s->k != 64) return false;
+    const int Wp = s->w + 2 * g.pw, P = s->h + 2 * g.ph - 2, Q = Wp - 2;
+    if (Wp < 10 || P <= 0 || Q <= 0) return false;
+    const int sms = 152;  // a fixed count: the split must not depend on the device
+    int64_t best = INT64_MAX;
+    ConvParams& p = pl.p;
+    for (int pitch = Wp; pitch < Wp + 16 && pitch <= 256; ++pitch)
+        for (int R = 1; R <= 16; ++R) {
+            if ((R * pitch) % 16) continue;
+            const int xalign = ((R + 2) * pitch * 128 + 128 + 1023) / 1024 * 1024;
+            const int stage = xalign + (R * pitch * 128 + 256 + 1023) / 1024 * 1024;
+            const int stages = std::min<int>(kWgRowMaxStages, (int)((kWinSmemMax - 1024) / stage));
+            if (stages < 2) continue;
+            const int64_t blocks = (int64_t)s->n * ((P + R - 1) / R);
+            if (blocks > INT32_MAX / 4) continue;
+            const int64_t mma = (int64_t)R * pitch * 10, load = (int64_t)(2 * R + 2) * s->w * 128 / 40;
+            const int64_t cost = (blocks + sms - 1) / sms * (std::max(mma, load) + 100);
+            if (cost >= best) continue;
+            best = cost;
+            p.win_Wp = pitch;
+            p.win_dyrows = R;
+            p.win_srows = R + 2;
+            p.win_tile = R * pitch;
+            p.win_margin = xalign;
+            p.win_strip_bytes = stage;
+            p.win_stages = stages;
+            p.win_bpi = (P + R - 1) / R;
+            p.num_kb = (int)blocks;
+            pl.smem = (size_t)stages * stage + 1024;
+        }
+    if (best == INT64_MAX) return false;
+    pl.win = pl.wgrow = true;
+    pl.BN = 64;
+    pl.mode = p.mode = kWgrad;
+    p.win_R = p.win_S = 3;
+    p.win_ph = g.ph;
+    p.win_pw = g.pw;
+    p.win_P = P;
+    p.win_Q = Q;
+    p.M = 9 * 64;
+    p.Ncols = 64;
+    p.m_tiles = p.n_tiles = 1;
+    p.gN = s->n;
+    // one contiguous range of K-blocks per CTA
+    const int splits = grid_size(p.num_kb);
+    p.kb_per_split = (p.num_kb + splits - 1) / splits;
+    p.zdim = (p.num_kb + p.kb_per_split - 1) / p.kb_per_split;
+    pl.ws_main = p.zdim > 1 ? (size_t)p.zdim * p.M * 64 * sizeof(float) : 0;
+    return true;
+}
+
 // Window weight-gradient eligibility and geometry (see conv_wgwin_kernel):
-// stride 1, 64 input and 64 output channels, at most 10 taps, padded rows of
-// 10..256 positions.
+// stride 1, 64 input and 64 output channels, three or four taps (the stems), padded
+// rows of 10..256 positions.
 bool wgwin_setup(const dbl_conv_shape* s, Plan& pl)
 {
     const Geom g = geom(s);
     if (g.sh != 1 || g.sw != 1) return false;
     if (s->c != 64 || s->k != 64) return false;
     const int ntaps = s->r * s->s;
-    if ((ntaps + 1) / 2 != 2 && (ntaps + 1) / 2 != 5) return false;  // the instantiated accumulator counts
+    if ((ntaps + 1) / 2 != 2) return false;  // the instantiated accumulator count
     const int Wp = s->w + 2 * g.pw, Hp = s->h + 2 * g.ph;
     if (Wp < 10 || Wp > 256) return false;
     const int P = Hp - s->r + 1, Q = Wp - s->s + 1;
@@ -1627,8 +1872,8 @@ int make_plan(const dbl_conv_shape* s, int pass, Plan& pl)
         pl.ws_main = (size_t)kMaxGrid * 2 * s->k * sizeof(float);
     } else if (pass == DBL_PASS_DGRAD && s->c % 64 == 0 && win_setup(s, s->k, s->c, true, pl)) {
         pl.mode = p.mode = kDgrad;
-    } else if (pass == DBL_PASS_WGRAD && wgwin_setup(s, pl)) {
-        // conv_wgwin_kernel: tiles are the split-K ranges
+    } else if (pass == DBL_PASS_WGRAD && (wgrow_setup(s, pl) || wgwin_setup(s, pl))) {
+        // conv_wgrow_kernel, conv_wgwin_kernel: tiles are the split-K ranges
     } else if (pass == DBL_PASS_FWD) {
         pl.mode = p.mode = c8 ? kFwdC8 : kFwd;
         if (c8 && p.ntaps > 56) return set_error(DBL_ERR_UNSUPPORTED, "conv_fwd: stem filter too large");
@@ -2044,15 +2289,15 @@ int launch_win(const Plan& pl, const CUtensorMap& a, const CUtensorMap& b, int g
               : launch_win_cfg<64, false, false, 1>(pl, a, b, grid, st);
 }
 
-template <int NACC>
+// KERNEL: conv_wgwin_kernel<NACC> or conv_wgrow_kernel (one CTA per split-K range).
+template <auto KERNEL>
 int launch_wgwin(const Plan& pl, const CUtensorMap& a, const CUtensorMap& b, cudaStream_t st)
 {
     static bool attr_set[64] = {false};
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev >= 0 && dev < 64 && !attr_set[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(conv_wgwin_kernel<NACC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)kWinSmemMax);
+        cudaError_t e = cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWinSmemMax);
         if (e != cudaSuccess) return dbl::cuda_check(e, "conv: set smem attribute");
         attr_set[dev] = true;
     }
@@ -2064,7 +2309,7 @@ int launch_wgwin(const Plan& pl, const CUtensorMap& a, const CUtensorMap& b, cud
     cfg.stream = st;
     cfg.attrs = at;
     cfg.numAttrs = conv_attrs(1, at);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, conv_wgwin_kernel<NACC>, a, b, pl.p);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, KERNEL, a, b, pl.p);
     if (e != cudaSuccess) {
         dbl::count_launch();
         return dbl::cuda_check(e, "conv_wgwin launch");
@@ -2073,12 +2318,12 @@ int launch_wgwin(const Plan& pl, const CUtensorMap& a, const CUtensorMap& b, cud
 }
 
 // Tensor map of the window kernel's strip operand: one padded row (Wp pixels
-// x 64 channels, starting at w = -1) of an NHWC tensor per copy.
-int enc_win_rows(CUtensorMap* m, const void* base, int N, int H, int W, int C, int Wp)
+// x 64 channels, starting at w = -1) of an NHWC tensor per copy, or `rows` of them.
+int enc_win_rows(CUtensorMap* m, const void* base, int N, int H, int W, int C, int Wp, int rows = 1)
 {
     cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)N};
     cuuint64_t str[3] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2, (cuuint64_t)H * W * C * 2};
-    cuuint32_t box[4] = {64, (cuuint32_t)Wp, 1, 1};
+    cuuint32_t box[4] = {64, (cuuint32_t)Wp, (cuuint32_t)rows, 1};
     return enc_tiled(m, base, 4, dims, str, box, true);
 }
 
@@ -2293,12 +2538,14 @@ int dbl_conv_wgrad(const dbl_conv_shape* s, const void* x, const void* dy, float
     cudaStream_t st = as_stream(stream);
     const bool sliced = pl.p.zdim > 1;
     if (pl.win) {
-        if ((rc = enc_win_rows(&ta, x, s->n, s->h, s->w, s->c, pl.p.win_Wp))) return rc;
-        if ((rc = enc_win_rows(&tb, dy, s->n, P, Q, s->k, pl.p.win_Wp))) return rc;
+        const int xr = pl.wgrow ? pl.p.win_srows : 1, yr = pl.wgrow ? pl.p.win_dyrows : 1;  // rows per copy
+        if ((rc = enc_win_rows(&ta, x, s->n, s->h, s->w, s->c, pl.p.win_Wp, xr))) return rc;
+        if ((rc = enc_win_rows(&tb, dy, s->n, P, Q, s->k, pl.p.win_Wp, yr))) return rc;
         pl.p.out = sliced ? ws : static_cast<void*>(dw);
         pl.p.wg_accumulate = accumulate;
-        const int nacc = (pl.p.win_R * pl.p.win_S + 1) / 2;
-        if ((rc = nacc == 5 ? launch_wgwin<5>(pl, ta, tb, st) : launch_wgwin<2>(pl, ta, tb, st))) return rc;
+        if ((rc = pl.wgrow ? launch_wgwin<conv_wgrow_kernel>(pl, ta, tb, st)
+                           : launch_wgwin<conv_wgwin_kernel<2>>(pl, ta, tb, st)))
+            return rc;
     } else {
     const bool c8 = pl.mode == kWgradC8;
     if ((rc = enc_im2col(&ta, x, s->n, s->h, s->w, s->c, -g.ph, g.ph - (s->r - 1), -g.pw, g.pw - (s->s - 1), g.sh, g.sw,

@@ -384,6 +384,9 @@ __device__ __forceinline__ void tma_load_4d_elect(void* dst, const void* tmap, u
         : "memory");
 }
 
+// Shared-memory writes of this thread, visible to the asynchronous proxy (TMA, tcgen05.mma).
+__device__ __forceinline__ void fence_async_shared() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
 // ---------------------------------------------------------------------------- CTA pairs (clusters of 2)
 // A kernel whose MMAs span a CTA pair (tcgen05 .cta_group::2) uses these forms
 // throughout: PTX forbids mixing .cta_group::1 and ::2 tcgen05 instructions in
