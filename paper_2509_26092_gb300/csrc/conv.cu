@@ -698,6 +698,253 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, CG>::THREADS, 1)
     }
 }
 
+// ----------------------------------------------------------------------------- split-K forward / data gradient
+// The 256-column pair tiles of the forward pass and the data gradient when there are too few of them
+// for the GPU (the layers of a few thousand pixels): a cluster of SK CTA pairs shares one tile, pair j
+// reducing K-blocks j*nkb/SK .. (j+1)*nkb/SK - 1.  When every pair's MMAs are done (cluster barrier;
+// the operand rings are free), pair j owns columns j*256/SK ..: each CTA sends the other pairs'
+// columns of its accumulator rows into the ring of the CTA of the same rank in those pairs
+// (distributed shared memory, 16 bytes per thread and store, lanes contiguous), and after a second
+// barrier adds what it received to its own columns in the pairs' order and runs the epilogue on them.
+// The other pair's partial sums are fp32 as they leave TMEM, so the result is that of a different
+// order of fp32 additions.
+// Why: with one pair per tile a 4x4 or 3x3 map of 512 channels runs 72 K-blocks (36.9 k tensor cycles)
+// on 6 to 36 of 76 pairs.  128-column tiles instead would need 1.5 times the operand bytes per MMA.
+// Channel sums: the CTAs of a row block write disjoint columns of one partial row (2 * m_tiles rows).
+template <int SK>
+struct SplitCfg {
+    using C = Cfg<256, kFamFwd, 2>;
+    static constexpr int W = 256 / SK;              // columns a CTA finishes
+    static constexpr int SLOT = 128 * W * 4;        // one received part: [W / 4][128 rows] float4
+    static constexpr int EPI_TILE = 4 * 32 * 33 * 4;
+    static constexpr int EPI_SUM = 4 * 2 * W * 4;   // per-warp channel sums
+    static constexpr int SMEM = C::RING + EPI_TILE + EPI_SUM + 1024;
+    static_assert((SK - 1) * SLOT <= C::RING, "received parts fit in the ring");
+};
+
+template <int SK>
+__global__ void __launch_bounds__(Cfg<256, kFamFwd, 2>::THREADS, 1)
+    conv_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                       const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2,
+                       const ConvParams p)
+{
+    dbl::dev::grid_dependency_trigger();  // a convolution launched next may start its set-up
+    using S = SplitCfg<SK>;
+    using C = typename S::C;
+    constexpr int BN = 256, STAGES = C::STAGES, W = S::W;
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t full_bar[STAGES], empty_bar[STAGES], accf_bar, drain_bar;
+    __shared__ uint32_t tmem_slot;
+    __shared__ volatile int abort_flag;
+
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    uint8_t* sgen = smem_raw + (sbase - smem_u32(smem_raw));
+    const int crank = (int)cluster_ctarank(), rank = crank & 1, split = crank >> 1;
+    const uint32_t leader = (uint32_t)(crank & ~1);  // the CTA of this pair that issues its MMAs
+    const int t = blockIdx.x / (2 * SK);
+    const TileCoord tc = decode_tile(p, t, gridDim.x);
+    int kb0 = 0, nkb_all = 0;
+    kb_range(p, tc.z, kb0, nkb_all);
+    const int k0 = nkb_all * split / SK, nkb = nkb_all * (split + 1) / SK - k0;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; ++s) {
+            mbar_init(&full_bar[s], 1);
+            mbar_init(&empty_bar[s], 1);
+        }
+        mbar_init(&accf_bar, 1);
+        mbar_init(&drain_bar, 1);
+        abort_flag = 0;
+        fence_mbar_init();
+    }
+    if (warp >= 4 && warp < 4 + kProducers && lane == 0) {
+        tma_prefetch_desc(&tmA);
+        tma_prefetch_desc(&tmB);
+        if (p.proj_kb) {
+            tma_prefetch_desc(&tmA2);
+            tma_prefetch_desc(&tmB2);
+        }
+    }
+    if (warp == C::MMA_WARP) {
+        tmem_alloc_cg<2>(&tmem_slot, BN);
+        tmem_relinquish_cg<2>();
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();  // every CTA's barriers initialised, TMEM allocated
+    tc_fence_after();
+    grid_dependency_wait();  // the set-up above may overlap the previous kernel; memory only after it
+    const uint32_t tmem = tmem_slot;
+    const int64_t gPQ = (int64_t)p.gP * p.gQ;
+
+    if (warp >= 4 && warp < 4 + kProducers) {
+        // ------------------------------------------------------------------ TMA producers
+        const int prod = warp - 4;
+        const int64_t m0 = ((int64_t)tc.m_tile * 2 + rank) * 128;
+        const int tn = (int)(m0 / gPQ);
+        const int64_t rem = m0 - (int64_t)tn * gPQ;
+        const int tp = (int)(rem / p.gQ), tq = (int)(rem - (int64_t)tp * p.gQ);
+        bool failed = false;
+        int last_it = -1;
+        for (int k = prod; k < nkb; k += kProducers) {
+            const int s = k % STAGES;
+            const uint32_t ok = mbar_wait_warp(&empty_bar[s], ((k / STAGES) & 1) ^ 1, &abort_flag);
+            if (__any_sync(0xffffffffu, ok == 0u)) {
+                failed = true;
+                break;
+            }
+            uint8_t* sa = sgen + s * C::STAGE_BYTES;
+            if (rank == 0) mbar_arrive_expect_tx_elect(&full_bar[s], (uint32_t)(2 * C::STAGE_BYTES));
+            load_kblock<BN, kFamFwd, 2>(p, &tmA, &tmB, &tmA2, &tmB2, sa, sa + C::A_BYTES,
+                                        mapa_shared(smem_u32(&full_bar[s]), leader), tc, k0 + k, tn, tp, tq, rank);
+            last_it = k;
+        }
+        if (failed) {
+            if (lane == 0) report_timeout(&abort_flag);
+            if (rank == 0) {
+                // let copies this producer issued land before the shared memory is used for anything else
+                for (int i = last_it; i >= 0 && i > last_it - STAGES * kProducers; i -= kProducers)
+                    (void)mbar_drain_warp(&full_bar[i % STAGES], (i / STAGES) & 1);
+            } else {
+                // rank 1's copies complete on rank 0's barriers: give them a fixed time instead
+                const uint64_t t0 = globaltimer();
+                while (globaltimer() - t0 < 1000000ull) {
+                }
+            }
+        }
+    } else if (warp == C::MMA_WARP) {
+        // ------------------------------------------------------------------ MMA issuer (rank 0 of each pair)
+        if (rank == 0) {
+            const bool fwd = p.mode == kFwd;
+            const uint32_t idesc = idesc_act(BM * 2, BN, 0u, fwd ? 0u : 1u);
+            const uint16_t both = (uint16_t)(3u << leader);
+            const uint64_t dA = smem_desc(0, 16, 1024, kSwizzle128B);
+            const uint64_t dB = fwd ? smem_desc(0, 16, 1024, kSwizzle128B) : smem_desc(0, 8192, 1024, kSwizzle128B);
+            const int b_step16 = fwd ? 2 : 2048 / 16;
+            bool failed = false;
+            if (nkb > 0) {
+                const uint32_t ok = mbar_wait_warp(&full_bar[0], 0, &abort_flag);
+                failed = __any_sync(0xffffffffu, ok == 0u);
+            }
+            for (int k = 0; k < nkb && !failed; ++k) {
+                tc_fence_after();
+                const int s = k % STAGES;
+                const uint32_t sa = sbase + s * C::STAGE_BYTES, sb = sa + C::A_BYTES;
+                const uint64_t ad0 = dA | (uint64_t)((sa >> 4) & 0x3FFFu), bd0 = dB | (uint64_t)((sb >> 4) & 0x3FFFu);
+#pragma unroll
+                for (int j = 0; j < C::KSTEPS; ++j) {
+                    if (j == C::KSTEPS - 1 && k + 1 < nkb) {  // the next stage's wait while MMAs are queued
+                        const uint32_t ok =
+                            mbar_wait_warp(&full_bar[(k + 1) % STAGES], ((k + 1) / STAGES) & 1, &abort_flag);
+                        failed = __any_sync(0xffffffffu, ok == 0u);
+                    }
+                    mma_act_elect_cg<2>(tmem, ad0 + (uint64_t)(j * 2), bd0 + (uint64_t)(j * b_step16), idesc,
+                                        (k > 0 || j > 0) ? 1u : 0u);
+                }
+                mma_commit_elect_cg<2>(&empty_bar[s], both);
+            }
+            mma_commit_elect_cg<2>(&accf_bar, both);  // arrives when this pair's MMAs have completed
+            if (failed && lane == 0) report_timeout(&abort_flag);
+            mma_commit_elect_cg<2>(&drain_bar, (uint16_t)(1u << leader));
+            (void)mbar_drain_warp(&drain_bar, 0);
+        }
+    } else {
+        const uint32_t ok = mbar_wait_warp(&accf_bar, 0, &abort_flag);
+        if (__any_sync(0xffffffffu, ok == 0u) && lane == 0) report_timeout(&abort_flag);
+        tc_fence_after();
+    }
+    __syncwarp();
+    cluster_sync_all();  // every pair's MMAs are done: the rings may be overwritten
+
+    const int row = warp * 32 + lane;  // TMEM lane = row within the 128-row accumulator (warps 0-3)
+    const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16);
+    if (warp < 4) {
+#pragma unroll 1
+        for (int d = 1; d < SK; ++d) {
+            const int to = (split + d) % SK;                  // pair that finishes these columns
+            const int slot = split < to ? split : split - 1;  // its parts are kept in the pairs' order
+            const uint32_t dst = mapa_shared(sbase, (uint32_t)(2 * to + rank)) + (uint32_t)(slot * S::SLOT + row * 16);
+#pragma unroll 1
+            for (int ch = 0; ch < W / 32; ++ch) {
+                uint32_t v[32];
+                if (nkb > 0) {
+                    tmem_ld_32x32b_x32(taddr + (uint32_t)(to * W + ch * 32), v);
+                    tmem_ld_wait();
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 32; ++k) v[k] = 0u;
+                }
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    st_cluster_v4(dst + (uint32_t)((ch * 8 + k) * 2048), v[4 * k], v[4 * k + 1], v[4 * k + 2],
+                                  v[4 * k + 3]);
+            }
+        }
+    }
+    __syncwarp();
+    cluster_sync_all();  // the parts have arrived
+
+    if (warp < 4) {
+        // ------------------------------------------------------------------ epilogue of this CTA's columns
+        float* st_tile = reinterpret_cast<float*>(sgen + C::RING) + warp * 32 * 33;
+        float* sums = reinterpret_cast<float*>(sgen + C::RING + S::EPI_TILE);
+        const bool want_stats = p.mode == kFwd && p.stats != nullptr;
+        const int64_t m = ((int64_t)tc.m_tile * 2 + rank) * 128 + row;
+        const bool valid = m < p.M;
+        int64_t out_row = m;
+        if (p.mode == kDgrad && p.phase_div == 2) {
+            const int64_t n = m / gPQ, rem = m - n * gPQ;
+            const int i = (int)(rem / p.gQ), j = (int)(rem - (int64_t)(rem / p.gQ) * p.gQ);
+            out_row = (n * p.out_h + 2 * i + (tc.z >> 1)) * p.out_w + 2 * j + (tc.z & 1);
+        }
+        RowStats<W> rs;
+        rs.zero();
+#pragma unroll
+        for (int ch = 0; ch < W / 32; ++ch) {
+            uint32_t v[32];
+            if (nkb > 0) {
+                tmem_ld_32x32b_x32(taddr + (uint32_t)(split * W + ch * 32), v);
+                tmem_ld_wait();
+            } else {
+#pragma unroll
+                for (int k = 0; k < 32; ++k) v[k] = 0u;
+            }
+            const float4* src = reinterpret_cast<const float4*>(sgen + ch * 8 * 2048 + row * 16);
+#pragma unroll
+            for (int q = 0; q < SK - 1; ++q)
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const float4 f = src[q * (S::SLOT / 16) + k * 128];
+                    v[4 * k] = __float_as_uint(__uint_as_float(v[4 * k]) + f.x);
+                    v[4 * k + 1] = __float_as_uint(__uint_as_float(v[4 * k + 1]) + f.y);
+                    v[4 * k + 2] = __float_as_uint(__uint_as_float(v[4 * k + 2]) + f.z);
+                    v[4 * k + 3] = __float_as_uint(__uint_as_float(v[4 * k + 3]) + f.w);
+                }
+            float back[32];
+            store_row_chunk_act(p, v, valid, out_row, tc.n_tile * BN + split * W + ch * 32, back);
+            if (want_stats) rs.add(ch, back, lane);
+        }
+        if (want_stats) {
+            float* wsum = sums + warp * 2 * W;
+            for (int c = lane; c < 2 * W; c += 32) wsum[c] = 0.f;
+            __syncwarp();
+            rs.flush(st_tile, wsum, W, 0, lane);
+            asm volatile("bar.sync 1, 128;" ::: "memory");
+            float* dst = p.stats + (int64_t)(tc.m_tile * 2 + rank) * 2 * p.Ncols + tc.n_tile * BN + split * W;
+            for (int c = threadIdx.x; c < 2 * W; c += 128)
+                dst[(c / W) * p.Ncols + c % W] = (sums[c] + sums[2 * W + c]) + (sums[4 * W + c] + sums[6 * W + c]);
+        }
+        tc_fence_before();
+    }
+    __syncthreads();
+    cluster_sync_all();  // neither CTA of a pair frees its TMEM while the other may still use it
+    if (warp == C::MMA_WARP) {
+        tc_fence_after();
+        tmem_dealloc_cg<2>(tmem, BN);
+    }
+}
+
 // ----------------------------------------------------------------------------- window kernel
 // 3x3, stride-1, pad-1 correlation (the forward pass, and the data gradient
 // with the taps flipped) without im2col.  Position (h, w) of image n of the
@@ -1532,6 +1779,7 @@ struct Plan {
     int mode;
     int BN;
     int cg = 1;          // conv_igemm_kernel CTAs per tile (2: CTA pairs with M = 256 MMAs)
+    int sk = 1;          // conv_splitk_kernel CTA pairs per tile (forward and data gradient)
     ConvParams p;
     size_t ws_main = 0;  // bytes: fwd channel-sum partials, or wgrad split-K slices
     bool win = false;    // conv_win_kernel (3x3 stride-1 correlation over padded strips)
@@ -1852,6 +2100,35 @@ bool pair_tiles(int BN, bool wgrad)
 // turns them off with the others.
 bool win_pairs() { return cta_pair_level() != 0; }
 
+// CTA pairs per tile of the forward pass and the data gradient (conv_splitk_kernel), 256-column pair
+// tiles: the count with the least modelled time, in K-blocks (~0.22 us each) of the longest phase.
+// One pair per tile runs on the persistent grid, whose epilogues overlap the next tile; split tiles
+// pay kTileCost (set-up, first loads, epilogue) every round of the clusters that GB300's 152 SMs hold
+// at one time.  A fixed function of the shape: the order of the sums must not depend on the device.
+// Measured with 1 / 2 / 4 / 8 pairs (us, data gradient): 36 tiles of 72 K-blocks (3x3x512, batch 512)
+// 27.1 / 19.1 / - / -, 16 of 36 (8x8x256, batch 64) 16.7 / 13.3 / 20.8 (two rounds) / -, 10 of 72
+// (3x3x512, batch 128) 26.3 / - / 13.8 / -, 6 of 72 (batch 64) 26.2 / - / 13.2 / 12.1.
+constexpr int kTileCost = 20;
+
+int fwd_splits(int tiles, int num_kb)
+{
+    static const int counts[4] = {1, 2, 4, 8}, resident[4] = {76, 36, 15, 7};
+    int best = 1;
+    int64_t best_cost = INT64_MAX;
+    for (int i = 0; i < 4; ++i) {
+        const int sk = counts[i];
+        if (sk > 1 && (tiles * 2 * sk > kMaxGrid || num_kb < 2 * sk)) continue;
+        const int64_t rounds = (tiles + resident[i] - 1) / resident[i];
+        const int64_t kb = (num_kb + sk - 1) / sk;
+        const int64_t cost = sk == 1 ? rounds * kb + kTileCost : rounds * (kb + kTileCost);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = sk;
+        }
+    }
+    return best;
+}
+
 int make_plan(const dbl_conv_shape* s, int pass, Plan& pl)
 {
     using dbl::set_error;
@@ -1988,6 +2265,13 @@ int make_plan(const dbl_conv_shape* s, int pass, Plan& pl)
         pl.ws_main = splits > 1 ? (size_t)splits * p.M * s->k * sizeof(float) : 0;
     }
     p.total_tiles = p.m_tiles * p.n_tiles * p.zdim;
+    if (!pl.win && pl.BN == 256 && pl.cg == 2 && (pl.mode == kFwd || pl.mode == kDgrad)) {
+        int kb = p.num_kb;  // data gradient: the longest phase
+        if (pl.mode == kDgrad)
+            for (int z = 0; z < p.zdim; ++z)
+                kb = std::max(kb, (p.phase_off[z + 1] - p.phase_off[z]) * p.cblocks);
+        pl.sk = fwd_splits(p.total_tiles, kb);
+    }
     return DBL_OK;
 }
 
@@ -2089,6 +2373,7 @@ int win_grid(const Plan& pl);
 int plan_grid(const Plan& pl)
 {
     if (pl.win) return win_grid(pl);
+    if (pl.sk > 1) return 2 * pl.sk * pl.p.total_tiles;
     if (pl.cg == 1) return grid_size(pl.p.total_tiles);
     const bool wg = pl.mode == kWgrad || pl.mode == kWgradC8;
     int pairs = pl.BN == 256 ? (wg ? resident_pairs<256, kFamWgrad>() : resident_pairs<256, kFamFwd>())
@@ -2097,7 +2382,7 @@ int plan_grid(const Plan& pl)
     return 2 * std::max(pairs, 1);
 }
 
-// Launch attributes of a convolution kernel: a cluster of two for CTA pairs, and, with
+// Launch attributes of a convolution kernel: a cluster of two (or 2 * SK) for CTA pairs, and, with
 // DBL_CONV_PDL=1 in the environment (read once per process), programmatic stream
 // serialization, so that the kernel's set-up (barriers, TMEM, descriptor prefetch) overlaps the
 // end of the kernel before it (its memory accesses wait in grid_dependency_wait).  Measured on
@@ -2117,12 +2402,12 @@ bool conv_pdl()
     return o < 0 ? env_on : o != 0;
 }
 
-int conv_attrs(int cg, cudaLaunchAttribute (&at)[2])
+int conv_attrs(int cluster, cudaLaunchAttribute (&at)[2])
 {
     int n = 0;
-    if (cg == 2) {
+    if (cluster > 1) {
         at[n].id = cudaLaunchAttributeClusterDimension;
-        at[n].val.clusterDim.x = 2;
+        at[n].val.clusterDim.x = cluster;
         at[n].val.clusterDim.y = 1;
         at[n].val.clusterDim.z = 1;
         ++n;
@@ -2160,11 +2445,46 @@ int launch_cfg(const Plan& pl, const CUtensorMap& a, const CUtensorMap& b, const
     return dbl::launch_check("conv_igemm launch");
 }
 
+template <int SK>
+int launch_splitk(const Plan& pl, const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& a2,
+                  const CUtensorMap& b2, int grid, cudaStream_t st)
+{
+    static bool attr_set[64] = {false};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev >= 0 && dev < 64 && !attr_set[dev]) {
+        cudaError_t e = cudaFuncSetAttribute(conv_splitk_kernel<SK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             SplitCfg<SK>::SMEM);
+        // a cluster of sixteen CTAs is above the portable size of eight
+        if (e == cudaSuccess && 2 * SK > 8)
+            e = cudaFuncSetAttribute(conv_splitk_kernel<SK>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) return dbl::cuda_check(e, "conv: set smem attribute");
+        attr_set[dev] = true;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[2];
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(Cfg<256, kFamFwd, 2>::THREADS);
+    cfg.dynamicSmemBytes = SplitCfg<SK>::SMEM;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = conv_attrs(2 * SK, at);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, conv_splitk_kernel<SK>, a, b, a2, b2, pl.p);
+    if (e != cudaSuccess) {
+        dbl::count_launch();
+        return dbl::cuda_check(e, "conv_splitk launch");
+    }
+    return dbl::launch_check("conv_splitk launch");
+}
+
 // a2, b2: the projection operands of a fused data gradient (unused otherwise).
 int launch(const Plan& pl, const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& a2, const CUtensorMap& b2,
            int grid, cudaStream_t st)
 {
     const bool wg = pl.mode == kWgrad || pl.mode == kWgradC8;
+    if (pl.sk == 2) return launch_splitk<2>(pl, a, b, a2, b2, grid, st);
+    if (pl.sk == 4) return launch_splitk<4>(pl, a, b, a2, b2, grid, st);
+    if (pl.sk == 8) return launch_splitk<8>(pl, a, b, a2, b2, grid, st);
     if (pl.cg == 2) {
         if (pl.BN == 256) return wg ? launch_cfg<256, kFamWgrad, 2>(pl, a, b, a2, b2, grid, st)
                                     : launch_cfg<256, kFamFwd, 2>(pl, a, b, a2, b2, grid, st);
@@ -2379,12 +2699,13 @@ int conv_fwd_impl(const dbl_conv_shape* s, const void* x, const void* w, void* y
     pl.p.st32 = (reinterpret_cast<uintptr_t>(y) % 32 == 0) && (pl.p.ldo * (int64_t)sizeof(act_t)) % 32 == 0;
     pl.p.stats = stats ? static_cast<float*>(ws) : nullptr;
     const int grid = plan_grid(pl);
+    const int parts = pl.sk > 1 ? 2 * pl.p.m_tiles : grid;  // rows of channel-sum partials
     cudaStream_t st = as_stream(stream);
     if ((rc = pl.win ? launch_win(pl, ta, tb, grid, st) : launch(pl, ta, tb, ta, tb, grid, st))) return rc;
     if (nparts) {
-        *nparts = grid;
+        *nparts = parts;
     } else if (stats) {
-        stats_reduce_kernel<<<(s->k + kPartialsChannels - 1) / kPartialsChannels, kPartialsThreads, 0, st>>>(pl.p.stats, grid, s->k, ch_sum, ch_sumsq);
+        stats_reduce_kernel<<<(s->k + kPartialsChannels - 1) / kPartialsChannels, kPartialsThreads, 0, st>>>(pl.p.stats, parts, s->k, ch_sum, ch_sumsq);
         if ((rc = launch_check("conv stats reduce"))) return rc;
     }
     return DBL_OK;

@@ -419,6 +419,13 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr)
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 
+// 16-byte store to a shared::cluster address (the shared memory of a CTA of this cluster).
+__device__ __forceinline__ void st_cluster_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d)
+                 : "memory");
+}
+
 // TMA loads whose completion is signalled on the mbarrier at shared::cluster
 // address bar.  CG = 2 (.cta_group::2): bar may be in the peer CTA of the pair,
 // which is how both CTAs' operand halves complete on the MMA-issuing CTA's barrier.

@@ -1,5 +1,5 @@
 """Edges of the convolution kernels chosen by shape: row-block weight gradients (3x3 stride 1, 64
-channels), against the fp64 oracle."""
+channels) and tiles split over clusters of CTA pairs, against the fp64 oracle."""
 import numpy as np
 import pytest
 import torch
@@ -45,4 +45,47 @@ def test_row_block_wgrad_matches_oracle(D, n, h, w, pad):
     assert max_norm_rel(host(dw), ref) <= WGRAD_TOL
     D.dbl_conv_wgrad(shape, xd, dyd, dw, True, work, wsb)
     assert max_norm_rel(host(dw), 2 * ref) <= WGRAD_TOL
+    check_status(D)
+
+
+# 16-bit outputs: one rounding of the result, 2^-9 of its size (bf16), far above the fp32 sums' error
+CONV_TOL = 4e-3
+
+
+def _conv_case(D, n, h, c, k, r, stride, pad, seed):
+    g = rng(seed)
+    x = bf16_values(g.standard_normal((n, h, h, c)))
+    wt = bf16_values(g.standard_normal((k, r, r, c)) * np.sqrt(2.0 / (r * r * c)))
+    p = (h + 2 * pad - r) // stride + 1
+    return D.conv_shape(n, h, h, c, k, r, stride, pad), x, wt, p
+
+
+@pytest.mark.parametrize("n,h,c,k,r,stride,pad", [
+    (1, 3, 512, 512, 3, 1, 1),     # 9 rows in a 256-row tile: eight pairs per tile
+    (29, 3, 512, 512, 3, 1, 1),    # 261 rows: a second tile with five rows, all of rank 1's beyond the batch
+    (100, 3, 512, 512, 3, 1, 1),   # 8 tiles: four pairs per tile
+    (65, 8, 256, 512, 3, 2, 1),    # ragged batch, two column tiles
+    (500, 3, 512, 512, 3, 1, 1),   # 36 tiles: two pairs per tile
+    (32, 6, 256, 256, 1, 2, 0),    # a short reduction (4 K-blocks): not split
+])
+def test_split_conv_matches_oracle(D, n, h, c, k, r, stride, pad):
+    """Forward (with its channel sums) and data gradient of layers with few 256-column tiles."""
+    shape, x, wt, p = _conv_case(D, n, h, c, k, r, stride, pad, n + h)
+    xd, wd = to_bf16_dev(x), to_bf16_dev(wt)
+    y = torch.full((n, p, p, k), float("nan"), dtype=torch.bfloat16, device="cuda")
+    s1, s2 = torch.empty(k, device="cuda"), torch.empty(k, device="cuda")
+    wsb = D.dbl_conv_workspace_bytes(shape, D.DBL_PASS_FWD)
+    D.dbl_conv_fwd(shape, xd, wd, y, s1, s2, ws(wsb), wsb)
+    ref = orc.conv2d_fwd(x, wt, stride, pad)
+    assert np.all(np.isfinite(host(y)))
+    assert max_norm_rel(host(y), ref) <= CONV_TOL
+    rows = host(y).reshape(-1, k)  # the statistics are those of the stored values, summed in fp32
+    assert max_norm_rel(host(s1), rows.sum(0)) <= 1e-4
+    assert max_norm_rel(host(s2), (rows * rows).sum(0)) <= 1e-5
+    if r == 3:
+        dy = bf16_values(rng(n).standard_normal((n, p, p, k)))
+        dx = torch.full((n, h, h, c), float("nan"), dtype=torch.bfloat16, device="cuda")
+        D.dbl_conv_dgrad(shape, to_bf16_dev(dy), wd, dx)
+        assert np.all(np.isfinite(host(dx)))
+        assert max_norm_rel(host(dx), orc.conv2d_dgrad(dy, wt, x.shape, stride, pad)) <= CONV_TOL
     check_status(D)
