@@ -27,6 +27,7 @@
 // records DBL_ERR_TIMEOUT in the device status word and the CTA winds down.
 #include <algorithm>
 #include <cstdlib>
+#include <type_traits>
 
 #include <atomic>
 
@@ -287,16 +288,16 @@ __device__ __forceinline__ void store_row_chunk_act(const ConvParams& p, const u
 // in registers across the tiles of a CTA instead of being reduced across the
 // warp for every tile (which costs shared-memory bandwidth that the mainloop
 // needs).  Thread (warp, lane) adds the values of its own accumulator row.
-// For BN > 64 the rows are first folded pairwise across lanes (LEVELS
-// shuffle steps), so that every thread holds 128 sums: after the folding,
-// value k of chunk ch belongs to column ch*32 + (lane & (32 - V)) + k.
+// For 128 columns the rows are first folded pairwise across lanes (one shuffle
+// step), so that every thread holds 128 sums: after the folding, value k of chunk
+// ch belongs to column ch*32 + (lane & (32 - V)) + k.
 // flush() reduces over the lanes through the warp's 32x33 scratch and adds the
-// column totals to the warp's channel sums (once per CTA, and whenever the
-// CTA moves to another column tile).
+// column totals to the warp's channel sums (once per CTA).
 template <int BN>
 struct RowStats {
     static constexpr int NCH = BN / 32;
-    static constexpr int LEVELS = BN <= 64 ? 0 : (BN <= 128 ? 1 : 2);
+    static constexpr int LEVELS = BN <= 64 ? 0 : 1;
+    static_assert(BN <= 128, "ColStats holds wider tiles");
     static constexpr int V = 32 >> LEVELS;
     float s[NCH][V], q[NCH][V];
 
@@ -338,8 +339,7 @@ struct RowStats {
                 a[k] = x[k];
                 b[k] = x[k] * x[k];
             }
-            if constexpr (LEVELS >= 1) fold<32, 16>(a, b, lane);
-            if constexpr (LEVELS >= 2) fold<16, 8>(a, b, lane);
+            fold<32, 16>(a, b, lane);
 #pragma unroll
             for (int k = 0; k < V; ++k) {
                 s[ch][k] += a[k];
@@ -369,6 +369,84 @@ struct RowStats {
         zero();
     }
 };
+
+// The same sums for tiles of 128 and 256 columns, without shuffles per tile: the accumulator is read a
+// second time in the 16x256b layout (tmem_ld_16x256b_x4), in which a thread holds 4 of the warp's 32
+// rows at 8 of each 32 columns, and rounds them to the storage format as the store does.  flush()
+// adds the eight lanes that share columns (seven shuffles per array of eight), once per CTA.  RowStats
+// at these widths spends about 300 instructions, 32 to 48 of them shuffles, per 32 x 32 chunk against
+// about 130 here, which one-tile CTAs cannot hide: forward at 28x28x128, batch 512 87.0 -> 80.4 us,
+// 7x7x512, batch 128 32.2 -> 30.1, a 20x20 1x1 projection 128 -> 256, batch 128 12.3 -> 10.9 (without
+// channel sums 74.1, 27.2 and 8.1).
+template <int BN>
+struct ColStats {
+    static constexpr int NCH = BN / 32;
+    float s[NCH][8], q[NCH][8];  // [chunk][2 * group + e]: column 8*group + 2*(lane%4) + e
+
+    __device__ __forceinline__ void zero()
+    {
+#pragma unroll
+        for (int c = 0; c < NCH; ++c)
+#pragma unroll
+            for (int k = 0; k < 8; ++k) s[c][k] = q[c][k] = 0.f;
+    }
+
+    // lo, hi: rows 0-15 and 16-31 of chunk ch; valid: bit i = row i is an output.
+    __device__ __forceinline__ void add(int ch, const uint32_t (&lo)[16], const uint32_t (&hi)[16], uint32_t valid,
+                                        int lane)
+    {
+        const uint32_t v = valid >> (lane / 4);
+        const bool ok[4] = {(v & 1u) != 0, (v & 0x100u) != 0, (v & 0x10000u) != 0, (v & 0x1000000u) != 0};
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            float2 f[4];  // rows lane/4, +8, +16, +24
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                const uint32_t a = h < 2 ? lo[4 * g + 2 * h] : hi[4 * g + 2 * (h - 2)];
+                const uint32_t b = h < 2 ? lo[4 * g + 2 * h + 1] : hi[4 * g + 2 * (h - 2) + 1];
+                f[h] = dbl::act::unpack2_u32(ok[h] ? dbl::act::pack2_u32(__uint_as_float(a), __uint_as_float(b)) : 0u);
+            }
+            s[ch][2 * g] += (f[0].x + f[1].x) + (f[2].x + f[3].x);
+            s[ch][2 * g + 1] += (f[0].y + f[1].y) + (f[2].y + f[3].y);
+            q[ch][2 * g] += fmaf(f[0].x, f[0].x, f[1].x * f[1].x) + fmaf(f[2].x, f[2].x, f[3].x * f[3].x);
+            q[ch][2 * g + 1] += fmaf(f[0].y, f[0].y, f[1].y * f[1].y) + fmaf(f[2].y, f[2].y, f[3].y * f[3].y);
+        }
+    }
+
+    // One step of the sum over lanes: lanes with bit O keep the upper half of the N values.
+    template <int N, int O>
+    __device__ __forceinline__ static void fold(float (&a)[8], int lane)
+    {
+        const bool up = (lane & O) != 0;
+#pragma unroll
+        for (int k = 0; k < N / 2; ++k) {
+            const float send = up ? a[k] : a[k + N / 2], keep = up ? a[k + N / 2] : a[k];
+            a[k] = keep + __shfl_xor_sync(0xffffffffu, send, O);
+        }
+    }
+
+    __device__ __forceinline__ void flush(float* wsum, int ncols, int col_base, int lane)
+    {
+        const int k = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);  // the value this lane keeps
+        float* dst = wsum + col_base + 8 * (k >> 1) + 2 * (lane & 3) + (k & 1);
+#pragma unroll
+        for (int c = 0; c < NCH; ++c) {
+            fold<8, 16>(s[c], lane);
+            fold<4, 8>(s[c], lane);
+            fold<2, 4>(s[c], lane);
+            fold<8, 16>(q[c], lane);
+            fold<4, 8>(q[c], lane);
+            fold<2, 4>(q[c], lane);
+            dst[c * 32] += s[c][0];
+            dst[ncols + c * 32] += q[c][0];
+        }
+        __syncwarp();
+        zero();
+    }
+};
+
+template <int BN>
+using TileStats = std::conditional_t<(BN > 64), ColStats<BN>, RowStats<BN>>;
 
 // Persistent kernel: CTA b processes tiles b, b + gridDim.x, ...  The ring of
 // STAGES shared-memory stages runs continuously across tiles; two producer
@@ -596,8 +674,14 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, CG>::THREADS, 1)
         // ------------------------------------------------------------------ epilogue (warps 0-3)
         float* st_tile = epi_tile + warp * 32 * 33;
         float* wsum = epi_sum + warp * 2 * p.Ncols;
-        RowStats<BN> rs;
+        TileStats<BN> rs;
         rs.zero();
+        auto flush = [&](int ntile) {
+            if constexpr (BN > 64)
+                rs.flush(wsum, p.Ncols, ntile * BN, lane);
+            else
+                rs.flush(st_tile, wsum, p.Ncols, ntile * BN, lane);
+        };
         int stats_ntile = -1;  // column tile the register sums belong to
         int lt = 0;
         for (int t = unit0; t < p.total_tiles; t += nunits, ++lt) {
@@ -614,7 +698,7 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, CG>::THREADS, 1)
             const int row = warp * 32 + lane;  // TMEM lane = row within a 128-row accumulator
             const bool have_acc = nkb > 0;
             if (want_stats && stats_ntile != tc.n_tile) {
-                if (stats_ntile >= 0) rs.flush(st_tile, wsum, p.Ncols, stats_ntile * BN, lane);
+                if (stats_ntile >= 0) flush(stats_ntile);
                 stats_ntile = tc.n_tile;
             }
 #pragma unroll 1
@@ -655,19 +739,37 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, CG>::THREADS, 1)
                         const int pa = tc.z >> 1, pb = tc.z & 1;
                         out_row = (n * p.out_h + 2 * i + pa) * p.out_w + 2 * j + pb;
                     }
+                    const uint32_t rows_ok = __ballot_sync(0xffffffffu, valid);
 #pragma unroll
                     for (int ch = 0; ch < BN / 32; ++ch) {
                         uint32_t v[32];
+                        [[maybe_unused]] uint32_t lo[16], hi[16];
                         if (have_acc) {
                             tmem_ld_32x32b_x32(taddr + ch * 32, v);
-                            tmem_ld_wait();
+                            if constexpr (BN > 64) {
+                                if (want_stats) {
+                                    tmem_ld_16x256b_x4(taddr + ch * 32, lo);
+                                    tmem_ld_16x256b_x4(taddr + (16u << 16) + ch * 32, hi);
+                                }
+                            }
+                            tmem_ld_wait_regs(v);
+                            if constexpr (BN > 64) {
+                                if (want_stats) {
+                                    tmem_ld_wait_regs(lo);
+                                    tmem_ld_wait_regs(hi);
+                                }
+                            }
                         } else {
 #pragma unroll
                             for (int k = 0; k < 32; ++k) v[k] = 0u;
                         }
                         float back[32];
                         store_row_chunk_act(p, v, valid, out_row, tc.n_tile * BN + ch * 32, back);
-                        if (want_stats) rs.add(ch, back, lane);
+                        if constexpr (BN > 64) {  // want_stats: the forward pass, whose tiles all have K-blocks
+                            if (want_stats) rs.add(ch, lo, hi, rows_ok, lane);
+                        } else {
+                            if (want_stats) rs.add(ch, back, lane);
+                        }
                     }
                 }
             }
@@ -680,7 +782,7 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, CG>::THREADS, 1)
                     mbar_arrive(&acce_bar[buf]);
             }
         }
-        if (want_stats && stats_ntile >= 0) rs.flush(st_tile, wsum, p.Ncols, stats_ntile * BN, lane);
+        if (want_stats && stats_ntile >= 0) flush(stats_ntile);
         if (want_stats) {
             asm volatile("bar.sync 1, 128;" ::: "memory");
             float* dst = p.stats + (int64_t)blockIdx.x * 2 * p.Ncols;
@@ -870,7 +972,7 @@ __global__ void __launch_bounds__(Cfg<256, kFamFwd, 2>::THREADS, 1)
                 uint32_t v[32];
                 if (nkb > 0) {
                     tmem_ld_32x32b_x32(taddr + (uint32_t)(to * W + ch * 32), v);
-                    tmem_ld_wait();
+                    tmem_ld_wait_regs(v);
                 } else {
 #pragma unroll
                     for (int k = 0; k < 32; ++k) v[k] = 0u;
@@ -905,7 +1007,7 @@ __global__ void __launch_bounds__(Cfg<256, kFamFwd, 2>::THREADS, 1)
             uint32_t v[32];
             if (nkb > 0) {
                 tmem_ld_32x32b_x32(taddr + (uint32_t)(split * W + ch * 32), v);
-                tmem_ld_wait();
+                tmem_ld_wait_regs(v);
             } else {
 #pragma unroll
                 for (int k = 0; k < 32; ++k) v[k] = 0u;
@@ -1241,7 +1343,7 @@ __global__ void __launch_bounds__(WinCfg<BN>::THREADS, 1)
         const int quarter = warp & 3, col0 = (warp >> 2) * CW;  // TMEM lanes 32*quarter.., columns col0..
         float* st_tile = epi_tile + warp * 32 * 33;
         float* wsum = epi_sum + warp * 2 * p.Ncols;
-        RowStats<CW> rs;
+        TileStats<CW> rs;
         rs.zero();
         const int img = p.win_Hp * Wp;
         int lt = 0;
@@ -1282,8 +1384,24 @@ __global__ void __launch_bounds__(WinCfg<BN>::THREADS, 1)
                 if (c + 1 < NC)
                     tmem_ld_32x32b_x32(taddr + (uint32_t)(((c + 1) / NCH) * BN + ((c + 1) % NCH) * 32), nxt);
                 float back[32];
-                store_row_chunk_act(p, cur, valid[a], out_row[a], col0 + ch * 32, back);
-                if (want_stats) rs.add(ch, back, lane);
+                if constexpr (CW > 64) {
+                    uint32_t lo[16], hi[16];
+                    if (want_stats) {
+                        const uint32_t ta = taddr + (uint32_t)(a * BN + ch * 32);
+                        tmem_ld_16x256b_x4(ta, lo);
+                        tmem_ld_16x256b_x4(ta + (16u << 16), hi);
+                    }
+                    store_row_chunk_act(p, cur, valid[a], out_row[a], col0 + ch * 32, back);
+                    if (want_stats) {
+                        const uint32_t rows_ok = __ballot_sync(0xffffffffu, valid[a]);
+                        tmem_ld_wait_regs(lo);
+                        tmem_ld_wait_regs(hi);
+                        rs.add(ch, lo, hi, rows_ok, lane);
+                    }
+                } else {
+                    store_row_chunk_act(p, cur, valid[a], out_row[a], col0 + ch * 32, back);
+                    if (want_stats) rs.add(ch, back, lane);
+                }
             }
             tc_fence_before();
             __syncwarp();
@@ -1295,7 +1413,10 @@ __global__ void __launch_bounds__(WinCfg<BN>::THREADS, 1)
             }
         }
         if (want_stats) {
-            rs.flush(st_tile, wsum, p.Ncols, col0, lane);  // the window kernel has one column tile
+            if constexpr (CW > 64)
+                rs.flush(wsum, p.Ncols, col0, lane);  // the window kernel has one column tile
+            else
+                rs.flush(st_tile, wsum, p.Ncols, col0, lane);
             asm volatile("bar.sync 1, %0;" ::"r"(C::EPI * 32) : "memory");
             float* dst = p.stats + (int64_t)blockIdx.x * 2 * p.Ncols;
             const int nc = 2 * p.Ncols;
