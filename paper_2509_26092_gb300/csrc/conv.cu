@@ -328,9 +328,14 @@ struct RowStats {
     {
         if constexpr (LEVELS == 0) {  // no folding: sum of squares by fused multiply-add
 #pragma unroll
-            for (int k = 0; k < 32; ++k) {
-                s[ch][k] += x[k];
-                q[ch][k] = fmaf(x[k], x[k], q[ch][k]);
+            for (int k = 0; k < 32; k += 2) {
+                const float2 v = make_float2(x[k], x[k + 1]);
+                const float2 a = add2(make_float2(s[ch][k], s[ch][k + 1]), v);
+                const float2 b = fma2(v, v, make_float2(q[ch][k], q[ch][k + 1]));
+                s[ch][k] = a.x;
+                s[ch][k + 1] = a.y;
+                q[ch][k] = b.x;
+                q[ch][k + 1] = b.y;
             }
         } else {
             float a[32], b[32];
@@ -381,14 +386,14 @@ struct RowStats {
 template <int BN>
 struct ColStats {
     static constexpr int NCH = BN / 32;
-    float s[NCH][8], q[NCH][8];  // [chunk][2 * group + e]: column 8*group + 2*(lane%4) + e
+    float2 s[NCH][4], q[NCH][4];  // [chunk][group]: columns 8*group + 2*(lane%4), + 1
 
     __device__ __forceinline__ void zero()
     {
 #pragma unroll
         for (int c = 0; c < NCH; ++c)
 #pragma unroll
-            for (int k = 0; k < 8; ++k) s[c][k] = q[c][k] = 0.f;
+            for (int g = 0; g < 4; ++g) s[c][g] = q[c][g] = make_float2(0.f, 0.f);
     }
 
     // lo, hi: rows 0-15 and 16-31 of chunk ch; valid: bit i = row i is an output.
@@ -406,23 +411,27 @@ struct ColStats {
                 const uint32_t b = h < 2 ? lo[4 * g + 2 * h + 1] : hi[4 * g + 2 * (h - 2) + 1];
                 f[h] = dbl::act::unpack2_u32(ok[h] ? dbl::act::pack2_u32(__uint_as_float(a), __uint_as_float(b)) : 0u);
             }
-            s[ch][2 * g] += (f[0].x + f[1].x) + (f[2].x + f[3].x);
-            s[ch][2 * g + 1] += (f[0].y + f[1].y) + (f[2].y + f[3].y);
-            q[ch][2 * g] += fmaf(f[0].x, f[0].x, f[1].x * f[1].x) + fmaf(f[2].x, f[2].x, f[3].x * f[3].x);
-            q[ch][2 * g + 1] += fmaf(f[0].y, f[0].y, f[1].y * f[1].y) + fmaf(f[2].y, f[2].y, f[3].y * f[3].y);
+            s[ch][g] = add2(s[ch][g], add2(add2(f[0], f[1]), add2(f[2], f[3])));
+            q[ch][g] = add2(q[ch][g], add2(fma2(f[0], f[0], mul2(f[1], f[1])), fma2(f[2], f[2], mul2(f[3], f[3]))));
         }
     }
 
-    // One step of the sum over lanes: lanes with bit O keep the upper half of the N values.
-    template <int N, int O>
-    __device__ __forceinline__ static void fold(float (&a)[8], int lane)
+    // Sum over the eight lanes that share columns: three steps that halve the values a lane keeps;
+    // returns value k (see flush) of 2*group + e.
+    __device__ __forceinline__ static float fold(const float2 (&f)[4], int lane)
     {
-        const bool up = (lane & O) != 0;
+        const bool b16 = (lane & 16) != 0, b8 = (lane & 8) != 0, b4 = (lane & 4) != 0;
+        float2 h[2];
 #pragma unroll
-        for (int k = 0; k < N / 2; ++k) {
-            const float send = up ? a[k] : a[k + N / 2], keep = up ? a[k + N / 2] : a[k];
-            a[k] = keep + __shfl_xor_sync(0xffffffffu, send, O);
+        for (int g = 0; g < 2; ++g) {
+            const float2 send = b16 ? f[g] : f[g + 2], keep = b16 ? f[g + 2] : f[g];
+            h[g].x = keep.x + __shfl_xor_sync(0xffffffffu, send.x, 16);
+            h[g].y = keep.y + __shfl_xor_sync(0xffffffffu, send.y, 16);
         }
+        const float2 send = b8 ? h[0] : h[1], keep = b8 ? h[1] : h[0];
+        const float x = keep.x + __shfl_xor_sync(0xffffffffu, send.x, 8);
+        const float y = keep.y + __shfl_xor_sync(0xffffffffu, send.y, 8);
+        return (b4 ? y : x) + __shfl_xor_sync(0xffffffffu, b4 ? x : y, 4);
     }
 
     __device__ __forceinline__ void flush(float* wsum, int ncols, int col_base, int lane)
@@ -431,14 +440,8 @@ struct ColStats {
         float* dst = wsum + col_base + 8 * (k >> 1) + 2 * (lane & 3) + (k & 1);
 #pragma unroll
         for (int c = 0; c < NCH; ++c) {
-            fold<8, 16>(s[c], lane);
-            fold<4, 8>(s[c], lane);
-            fold<2, 4>(s[c], lane);
-            fold<8, 16>(q[c], lane);
-            fold<4, 8>(q[c], lane);
-            fold<2, 4>(q[c], lane);
-            dst[c * 32] += s[c][0];
-            dst[ncols + c * 32] += q[c][0];
+            dst[c * 32] += fold(s[c], lane);
+            dst[ncols + c * 32] += fold(q[c], lane);
         }
         __syncwarp();
         zero();
