@@ -286,6 +286,27 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
 }
 
 // ---------------------------------------------------------------------------- per-block partial sums
+// An unevaluated sum of two fp32 values, |lo| <= ulp(hi) / 2: 48 bits, at the rate of fp32 (this GPU
+// runs an fp64 instruction of a warp in about 16 cycles).
+struct PairF {
+    float hi, lo;
+};
+
+// a + b exactly, for |a| >= |b| or a = 0 (Dekker).
+__device__ __forceinline__ PairF pair_from(float a, float b)
+{
+    const float s = __fadd_rn(a, b);
+    return {s, __fsub_rn(b, __fsub_rn(s, a))};
+}
+
+// Sum of two pairs: the high parts exactly (Knuth's two-sum), the low parts rounded to fp32.
+__device__ __forceinline__ PairF pair_add(PairF a, PairF b)
+{
+    const float s = __fadd_rn(a.hi, b.hi), v = __fsub_rn(s, a.hi);
+    const float e = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, v)), __fsub_rn(b.hi, v));
+    return pair_from(s, __fadd_rn(e, __fadd_rn(a.lo, b.lo)));
+}
+
 // sum += v with Kahan compensation (comp carries the lost low-order part)
 __device__ __forceinline__ void kahan_add(float& sum, float& comp, float v)
 {
@@ -303,7 +324,7 @@ __device__ __forceinline__ void kahan_add(float& sum, float& comp, float v)
 // s = t / 8 of 32, and stream s adds the partials s, s+32, ... in fp32 with Kahan
 // compensation (sixteen loads in flight).  A warp's load then reads four partial
 // rows of eight adjacent channels, four whole 32-byte sectors.  The 32 stream sums
-// are added in fp64 by a fixed binary tree over the stream index, lowest bit first
+// are added as pairs of fp32 by a fixed binary tree over the stream index, lowest bit first
 // (shuffles across lanes 8 and 16 apart, then pairs of warps through shared
 // memory).  The order depends only on nparts, so the result is the same on every
 // launch and GPU.  Returns the channel (for threads t < 8 whose channel is below
@@ -315,7 +336,7 @@ static_assert(kPartialsThreads == 32 * kPartialsChannels, "32 streams of 8 chann
 __device__ __forceinline__ int partials_colsum(const float* __restrict__ part, int nparts, int K, double& sum0,
                                                double& sum1)
 {
-    __shared__ double red[2][kPartialsThreads / 32][kPartialsChannels];
+    __shared__ PairF red[2][kPartialsThreads / 32][kPartialsChannels];
     const int cl = threadIdx.x % kPartialsChannels, stream = threadIdx.x / kPartialsChannels;
     const int c = blockIdx.x * kPartialsChannels + cl;
     float s = 0.f, sc = 0.f, q = 0.f, qc = 0.f;
@@ -337,12 +358,15 @@ __device__ __forceinline__ int partials_colsum(const float* __restrict__ part, i
                 }
         }
     }
-    double ds = (double)s - (double)sc, dq = (double)q - (double)qc;
+    PairF ds = pair_from(s, -sc), dq = pair_from(q, -qc);
     // stream bits 0 and 1 are lane bits 3 and 4
 #pragma unroll
     for (int o = 8; o < 32; o <<= 1) {
-        ds += __shfl_xor_sync(0xffffffffu, ds, o);
-        dq += __shfl_xor_sync(0xffffffffu, dq, o);
+        const PairF os{__shfl_xor_sync(0xffffffffu, ds.hi, o), __shfl_xor_sync(0xffffffffu, ds.lo, o)};
+        const PairF oq{__shfl_xor_sync(0xffffffffu, dq.hi, o), __shfl_xor_sync(0xffffffffu, dq.lo, o)};
+        // lower stream first on both sides, so that every lane holds the same bits
+        ds = (threadIdx.x & o) ? pair_add(os, ds) : pair_add(ds, os);
+        dq = (threadIdx.x & o) ? pair_add(oq, dq) : pair_add(dq, oq);
     }
     const int w = threadIdx.x / 32;
     if ((threadIdx.x & 31) < kPartialsChannels) {
@@ -352,14 +376,17 @@ __device__ __forceinline__ int partials_colsum(const float* __restrict__ part, i
     __syncthreads();
     if (threadIdx.x < kPartialsChannels) {
         // stream bits 2, 3 and 4 are warp bits 0, 1 and 2
-        const double(&a)[8][kPartialsChannels] = red[0];
-        const double(&b)[8][kPartialsChannels] = red[1];
-        ds = ((a[0][cl] + a[1][cl]) + (a[2][cl] + a[3][cl])) + ((a[4][cl] + a[5][cl]) + (a[6][cl] + a[7][cl]));
-        dq = ((b[0][cl] + b[1][cl]) + (b[2][cl] + b[3][cl])) + ((b[4][cl] + b[5][cl]) + (b[6][cl] + b[7][cl]));
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+            const PairF(&a)[8][kPartialsChannels] = red[x];
+            const PairF t = pair_add(pair_add(pair_add(a[0][cl], a[1][cl]), pair_add(a[2][cl], a[3][cl])),
+                                     pair_add(pair_add(a[4][cl], a[5][cl]), pair_add(a[6][cl], a[7][cl])));
+            (x ? dq : ds) = t;
+        }
     }
     __syncthreads();
-    sum0 = ds;
-    sum1 = dq;
+    sum0 = (double)ds.hi + (double)ds.lo;
+    sum1 = (double)dq.hi + (double)dq.lo;
     return (threadIdx.x < kPartialsChannels && c < K) ? c : -1;
 }
 

@@ -48,7 +48,7 @@ def test_row_block_wgrad_matches_oracle(D, n, h, w, pad):
     check_status(D)
 
 
-# 16-bit outputs: one rounding of the result, 2^-9 of its size (bf16), far above the fp32 sums' error
+# 16-bit outputs: one rounding of the result, at most 2^-8 of its size (bf16), and the fp32 sums' error
 CONV_TOL = 4e-3
 
 
