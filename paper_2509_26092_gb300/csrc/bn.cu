@@ -452,6 +452,155 @@ __global__ void __launch_bounds__(kThreads, kBwdBlocksPerSM)
     }
 }
 
+// ----------------------------------------------------------------------------- small tensors
+// Backward of small tensors in one launch instead of three: a cluster of CL CTAs owns 32 channels, each
+// CTA an equal run of the rows.  Both passes over the rows read global memory (the second finds its
+// CTA's rows in L1 and L2); between them the CTAs add up their channel sums through distributed shared
+// memory, in rank order, and each forms the three coefficients of the apply pass for itself.  Bound
+// by latency: three launches of the general path cost about 3 us each before they move a byte.
+// General path -> here, bwd without / with a second gradient and g stored (us): 576 rows of 512 channels
+// 11.4 -> 6.2 / 11.0 -> 6.5; 4608 of 512 14.7 -> 12.6 / 15.6 -> 16.3 (stays); 4608 of 256 12.4 -> 8.7 /
+// 12.7 -> 11.5; 12,800 of 256 16.2 -> 15.5 / 17.8 -> 20.9 (stays); 16,384 of 128 12.9 -> 14.0 (stays).
+constexpr int kSliceC = 32;                    // channels of a slice: 64 bytes of a row
+constexpr int kSliceVec = kSliceC / 8;         // 16-byte vectors of a slice row
+constexpr int kSliceRows = kThreads / kSliceVec;  // rows a CTA covers in one step
+
+template <int MASK, bool WRITE_G>
+__global__ void __launch_bounds__(kThreads, 2)
+    bn_bwd_cluster_kernel(const act_t* __restrict__ dout, const act_t* __restrict__ dout2,
+                          const act_t* __restrict__ out, const act_t* __restrict__ y, int count, int C,
+                          double inv_n, const float* __restrict__ gamma, const float* __restrict__ beta,
+                          const float* __restrict__ mean, const float* __restrict__ invstd,
+                          float* __restrict__ dgamma, float* __restrict__ dbeta, act_t* __restrict__ dy,
+                          act_t* dres, int CL)
+{
+    dbl::dev::grid_dependency_trigger();  // a convolution launched next may start its set-up
+    __shared__ float red[kThreads / 32][2][kSliceC];
+    __shared__ float tot[2][kSliceC];   // this CTA's sums, read by the whole cluster
+    __shared__ __align__(16) float coef[3][kSliceC];
+    const int rank = (int)dbl::dev::cluster_ctarank(), slice = blockIdx.x / CL;
+    const int c0 = slice * kSliceC, vl = threadIdx.x % kSliceVec, g = c0 / 8 + vl, groups = C / 8;
+    const int per = (count + CL - 1) / CL, r0 = rank * per, r1 = min(count, r0 + per);
+    const bool two = dout2 != nullptr;
+    __shared__ __align__(16) float chan[3 * kSliceC];  // mean (, scale, shift)
+    if (threadIdx.x < kSliceC) chan[threadIdx.x] = mean[c0 + threadIdx.x];
+    stage_relu<MASK>(gamma, beta, mean, invstd, c0, kSliceC, chan + kSliceC);
+    __syncthreads();
+    ReluMask<MASK> rm;
+    rm.init(chan + kSliceC, kSliceC, 8 * vl);
+    float mu[8];
+    load8(chan + 8 * vl, mu);
+    constexpr int U = 4;  // rows whose loads are in flight together
+    float sg[8] = {}, sgx[8] = {};
+    for (int r = r0 + threadIdx.x / kSliceVec; r < r1; r += U * kSliceRows) {
+        Vec8 gg[U], yy[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (r + u * kSliceRows < r1)
+                load_g_raw<MASK, true, true>(dout, dout2, out, y, (r + u * kSliceRows) * groups + g, gg[u], yy[u]);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (r + u * kSliceRows < r1)
+                accumulate_g<MASK, WRITE_G>(gg[u], yy[u], two, rm, mu, sg, sgx, dres,
+                                            (r + u * kSliceRows) * groups + g);
+    }
+    // lanes that share a vector, then the warps in order
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+#pragma unroll
+        for (int o = kSliceVec; o < 32; o <<= 1) {
+            sg[k] += __shfl_xor_sync(0xffffffffu, sg[k], o);
+            sgx[k] += __shfl_xor_sync(0xffffffffu, sgx[k], o);
+        }
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    if (lane < kSliceVec)
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            red[warp][0][8 * vl + k] = sg[k];
+            red[warp][1][8 * vl + k] = sgx[k];
+        }
+    __syncthreads();
+    if (threadIdx.x < 2 * kSliceC) {
+        const int st = threadIdx.x / kSliceC, c = threadIdx.x % kSliceC;
+        float t = 0.f;
+#pragma unroll
+        for (int w = 0; w < kThreads / 32; ++w) t += red[w][st][c];
+        tot[st][c] = st ? t * invstd[c0 + c] : t;  // sum g*(y-mean) -> sum g*xhat
+    }
+    __syncwarp();
+    dbl::dev::cluster_sync_all();
+    if (threadIdx.x < kSliceC) {
+        const int c = threadIdx.x;
+        float v[2][16];
+#pragma unroll
+        for (int r = 0; r < 16; ++r)
+#pragma unroll
+            for (int st = 0; st < 2; ++st)
+                v[st][r] = r < CL ? dbl::dev::ld_cluster_f32(dbl::dev::mapa_shared(dbl::dev::smem_u32(&tot[st][c]), r))
+                                  : 0.f;
+        double sums[2];
+#pragma unroll
+        for (int st = 0; st < 2; ++st) {
+            dbl::dev::PairF t{0.f, 0.f};
+#pragma unroll
+            for (int r = 0; r < 16; ++r)
+                if (r < CL) t = dbl::dev::pair_add(t, {v[st][r], 0.f});
+            sums[st] = (double)t.hi + (double)t.lo;
+        }
+        if (rank == 0) {
+            dbeta[c0 + c] = (float)sums[0];
+            dgamma[c0 + c] = (float)sums[1];
+        }
+        bwd_coefficients(sums[0], sums[1], inv_n, gamma[c0 + c], invstd[c0 + c], mean[c0 + c], coef[0][c], coef[1][c],
+                         coef[2][c]);
+    }
+    __syncthreads();
+    float ca[8], cb[8], cc[8];
+    load8(&coef[0][8 * vl], ca);
+    load8(&coef[1][8 * vl], cb);
+    load8(&coef[2][8 * vl], cc);
+    for (int r = r0 + threadIdx.x / kSliceVec; r < r1; r += 2 * kSliceRows) {
+        Vec8 gg[2], yy[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+            if (r + u * kSliceRows < r1) {
+                const int v = (r + u * kSliceRows) * groups + g;
+                if constexpr (WRITE_G) {  // the g this thread stored, as the general path reads it back
+                    gg[u].d = __ldcg(reinterpret_cast<const uint4*>(dres) + v);
+                    yy[u].y = load_vec<true>(y, v);
+                } else {
+                    load_g_raw<MASK, true, true>(dout, dout2, out, y, v, gg[u], yy[u]);
+                }
+            }
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+            if (r + u * kSliceRows < r1) {
+                float f[8], x[8], d[8];
+                unpack8(yy[u].y, x);
+                if constexpr (WRITE_G)
+                    unpack8(gg[u].d, f);
+                else
+                    combine_g(gg[u], x, two, rm, f);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) d[k] = fmaf(ca[k], f[k], fmaf(cb[k], x[k], cc[k]));
+                reinterpret_cast<uint4*>(dy)[(r + u * kSliceRows) * groups + g] = pack8(d);
+            }
+    }
+    dbl::dev::cluster_sync_all();  // no CTA leaves while another may still read its sums
+}
+
+// CTAs per cluster of the one-launch backward, or 0 for the general path: the channels must come in
+// whole slices, and a CTA's rows (kClusterRows, with g to store kClusterRowsG) stay few enough that its
+// two passes cost less than the two launches saved.
+constexpr int kClusterRows = 800, kClusterRowsG = 512;
+
+int bwd_cluster(int64_t count, int C, bool with_g)
+{
+    if (C % kSliceC) return 0;
+    const int cl = C >= 512 ? 8 : 16;  // at least 64 CTAs; sixteen is above the portable cluster size
+    return count <= (int64_t)cl * (with_g ? kClusterRowsG : kClusterRows) ? cl : 0;
+}
+
 int bn_grid(int64_t nvec, int per_sm = kBlocksPerSM)
 {
     int64_t b = (nvec + kThreads - 1) / kThreads;
@@ -513,6 +662,29 @@ int bwd_launch_mask(const dbl_bn_shape* s, const void* dout, const void* dout2, 
     // When the caller wants g (the residual branch's gradient), the reduce pass stores it and the
     // apply pass reads it back instead of re-reading dout, dout2 and out.
     act_t* g_store = static_cast<act_t*>(dresidual);
+    if (const int cl = bwd_cluster(s->count, C, g_store != nullptr)) {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = cl;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3(C / kSliceC * cl);
+        cfg.blockDim = dim3(kThreads);
+        cfg.stream = st;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        auto k = g_store ? bn_bwd_cluster_kernel<MASK, true> : bn_bwd_cluster_kernel<MASK, false>;
+        cudaError_t e = cl > 8 ? cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : cudaSuccess;
+        if (e == cudaSuccess)
+            e = cudaLaunchKernelEx(&cfg, k, bd(dout), bd(dout2), bd(out), bd(y), (int)s->count, C,
+                                   1.0 / (double)s->count, gamma, beta, mean, invstd, dgamma, dbeta,
+                                   static_cast<act_t*>(dy), g_store, cl);
+        if (e != cudaSuccess) {
+            count_launch();
+            return cuda_check(e, "bn_bwd_cluster launch");
+        }
+        return launch_check("bn_bwd_cluster launch");
+    }
     const size_t smem_r = (MASK == kMaskY ? 3 : 1) * C * sizeof(float);
     if (g_store)
         bn_bwd_reduce_kernel<MASK, true><<<reduce_grid(nblk), kThreads, smem_r, st>>>(

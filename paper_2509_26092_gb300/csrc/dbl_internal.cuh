@@ -484,6 +484,14 @@ __device__ __forceinline__ void st_cluster_v4(uint32_t addr, uint32_t a, uint32_
                  : "memory");
 }
 
+// The float at a shared::cluster address.
+__device__ __forceinline__ float ld_cluster_f32(uint32_t addr)
+{
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+    return v;
+}
+
 // TMA loads whose completion is signalled on the mbarrier at shared::cluster
 // address bar.  CG = 2 (.cta_group::2): bar may be in the peer CTA of the pair,
 // which is how both CTAs' operand halves complete on the MMA-issuing CTA's barrier.

@@ -1,0 +1,61 @@
+"""Edges of the one-launch BatchNorm backward of small tensors (a cluster of CTAs per 32 channels)
+against the fp64 oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as orc
+from conftest import max_norm_rel
+from gpu_common import bf16_values, check_status, host, load_dbl, rng, to_bf16_dev, to_f32_dev, ws
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def D():
+    return load_dbl()
+
+
+@pytest.mark.parametrize("count,C", [
+    (1, 512),      # one row: seven CTAs of a cluster have none
+    (9, 64),       # fewer rows than CTAs
+    (577, 256),    # a last CTA with fewer rows
+    (4096, 512),   # the largest with g stored
+    (6400, 512),   # the largest without
+    (6401, 512),   # the general path
+])
+@pytest.mark.parametrize("mask", ["out", "y", "none"])
+def test_small_bn_backward_matches_oracle(D, count, C, mask):
+    """mask "out": with a second gradient and the masked gradient stored over it; "y": the mask from y."""
+    g = rng(count + C)
+    y = bf16_values(g.standard_normal((count, C)) * 2.0 + 0.5)
+    gamma = (1.0 + 0.2 * g.standard_normal(C)).astype(np.float32)
+    beta = (0.1 * g.standard_normal(C)).astype(np.float32)
+    mean, istd = y.mean(0).astype(np.float32), (1.0 / np.sqrt(y.var(0) + 1e-5)).astype(np.float32)
+    dout, dout2 = (bf16_values(g.standard_normal((count, C))) for _ in range(2))
+    sc = gamma * istd  # the forward pass's fp32 operations
+    pre = y.astype(np.float32) * sc + (beta - mean * sc)
+    out = bf16_values(np.maximum(pre, 0.0)) if mask != "none" else bf16_values(pre)
+    sure = np.abs(pre) > 1e-5  # elements whose mask a fused multiply-add cannot decide otherwise
+    dout, dout2 = dout * sure, dout2 * sure
+    two = mask == "out"
+    shape = D.bn_shape(count, C, 1e-5, mask != "none")
+    dy = torch.full((count, C), float("nan"), dtype=torch.bfloat16, device="cuda")
+    dg, db = torch.full((C,), float("nan"), device="cuda"), torch.full((C,), float("nan"), device="cuda")
+    d2 = to_bf16_dev(dout2) if two else None
+    wsb = D.dbl_bn_workspace_bytes(shape)
+    D.dbl_bn_relu_fused_bwd(shape, to_bf16_dev(dout), d2, to_bf16_dev(y), to_bf16_dev(out) if two else None,
+                            to_f32_dev(gamma), to_f32_dev(mean), to_f32_dev(istd), dy, d2, dg, db, ws(wsb), wsb,
+                            beta=to_f32_dev(beta))
+    rdy, rdg, rdb, rres = orc.bn_bwd(dout, out, y, gamma, mean.astype(np.float64), istd.astype(np.float64),
+                                     relu=mask != "none", dout2=dout2 if two else None, want_dres=True)
+    # dy = A*(g - ...), A = gamma/std: g rounded to bf16 where it is stored (bf16 has 8 significant bits:
+    # half a unit is at most 2^-8 of the value) and dy once more, 2^-7 together; of a single row the exact
+    # dy is 0 and A is 316
+    scale = max(np.abs(rdy).max(), np.abs(gamma * istd).max() * np.abs(rres).max())
+    assert np.abs(host(dy) - rdy).max() <= 2.0 ** -7 * scale
+    for got, ref in ((dg, rdg), (db, rdb)):
+        assert np.abs(host(got) - ref).max() <= 1e-5 * (np.abs(rres).sum(0).max() * 4)
+    if two:
+        assert max_norm_rel(host(d2), rres) <= 4e-3
+    check_status(D)
