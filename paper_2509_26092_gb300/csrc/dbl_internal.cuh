@@ -492,6 +492,16 @@ __device__ __forceinline__ float ld_cluster_f32(uint32_t addr)
     return v;
 }
 
+__device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t addr)
+{
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(addr)
+                 : "memory");
+    return v;
+}
+
 // TMA loads whose completion is signalled on the mbarrier at shared::cluster
 // address bar.  CG = 2 (.cta_group::2): bar may be in the peer CTA of the pair,
 // which is how both CTAs' operand halves complete on the MMA-issuing CTA's barrier.

@@ -5,7 +5,7 @@
 //
 // These are a few percent of a step's time: the max pool is a bandwidth
 // pass over the stem output, the head works on [n, 512] features.  The FC
-// products are done by a small tiled fp32 GEMM on the CUDA cores.
+// products are done by a tiled fp32 GEMM on the CUDA cores.
 #include <float.h>
 
 #include <algorithm>
@@ -32,6 +32,14 @@ __device__ __forceinline__ uint4 pack8(const float (&f)[8])
 #pragma unroll
     for (int k = 0; k < 4; ++k) h[k] = dbl::act::pack2(f[2 * k], f[2 * k + 1]);
     return v;
+}
+
+// Eight floats at a 16-byte aligned address.
+__device__ __forceinline__ void load8(const float* p, float (&f)[8])
+{
+    const float4 a = __ldg(reinterpret_cast<const float4*>(p)), b = __ldg(reinterpret_cast<const float4*>(p) + 1);
+    f[0] = a.x, f[1] = a.y, f[2] = a.z, f[3] = a.w;
+    f[4] = b.x, f[5] = b.y, f[6] = b.z, f[7] = b.w;
 }
 
 int grid_for(int64_t items, int threads, int per_sm = 8)
@@ -418,195 +426,295 @@ __global__ void __launch_bounds__(256) avgpool_kernel(const act_t* __restrict__ 
     }
 }
 
-// out[m, n] = sum_k A(m,k) * B(n,k) (+ bias[n]); A(m,k) = A[m*sam + k*sak], B(n,k) = B[n*sbn + k*sbk].
-// fp32 on the CUDA cores (the head is fp32 end to end): 64 x 64 output tiles, 16-deep K tiles
-// stored K-major in shared memory (double-buffered: the next tile is fetched into registers
-// while the current one is multiplied), 4 x 4 outputs per thread from float4 reads.  The
-// reduction is cut into gridDim.z fixed chunks of kchunk (a function of the shape only), each a
-// sequential fmaf over its k; with more than one chunk the partial sums go to part[z][M][N] and
-// gemm_chunk_reduce_kernel adds them in chunk order.  Tile loads are coalesced along whichever
-// index of an operand has unit stride.
-constexpr int GBM = 64, GBN = 64, GBK = 16;
-constexpr int kGemmThreads = 256;
-constexpr int kGemmTargetCTAs = 304;  // two 64 x 64 tiles per SM of a 152-SM GPU
+// out[m, n] = sum_k A(m,k) * B(n,k) (+ bias[n]); A(m,k) = A[m*sam + k*sak], B(n,k) = B[n*sbn + k*sbk],
+// one of the two strides of each operand being 1.  fp32 on the CUDA cores (the head is fp32 end to
+// end): 64 x 128 output tiles, 16-deep K tiles stored K-major in shared memory (double-buffered: the
+// next tile is fetched into registers while the current one is multiplied), 8 x 8 outputs per thread,
+// two per instruction (fma.rn.f32x2).  The reduction is cut into chunks of kchunk, each a sequential
+// fmaf over its k; the chunks of a tile are the CTAs of a cluster (along z), which add their partial
+// sums in chunk order through distributed shared memory.  Two products, and the loss and bias-gradient
+// sums that need the same input, share a launch.
+// Bound by fp32 issue: 512 x 1000 x 512 is 7 us of the GPU's fp32 rate.  With 4 x 4 outputs per thread
+// (half the FMAs per shared-memory byte), the partial sums through global memory and a launch of their
+// own, the head of 512 images and 1000 classes took 128.9 us in ten launches; @head@
+constexpr int GBM = 64, GBN = 128, GBK = 16;
+constexpr int GLA = GBM + 4, GLB = GBN + 4;  // row pitches of the K-major tiles
+constexpr int kGemmThreads = 128;
+constexpr int kGemmMaxCTAs = 608;  // four CTAs per SM of a 152-SM GPU
+constexpr int kGemmMaxChunks = 8;  // a cluster
 
-struct GemmTileRegs {
-    float v[GBM * GBK / kGemmThreads];
+struct GemmJob {
+    const float *A, *B, *bias;
+    float* out;
+    int64_t sam, sak, sbn, sbk, ldo;
+    int M, N, K, kchunk, tiles;
+    int vec;  // bits: A, B and out may be accessed 16 bytes at a time
 };
 
-// Thread's share of the K tile [k0, k0 + GBK) of rows [row0, row0 + GBM): element e = tid + 256 q.
-__device__ __forceinline__ void gemm_fetch(const float* __restrict__ X, int64_t s_row, int64_t s_k, int row0, int rows,
-                                           int k0, int kend, GemmTileRegs& t)
+// Thread's share of the K tile [k0, k0 + GBK) of rows [row0, row0 + R): float4 number e = tid + 128 q,
+// along k or along the rows, whichever is contiguous.
+template <int R>
+__device__ __forceinline__ void gemm_fetch(const float* __restrict__ X, int64_t s_row, int64_t s_k, bool vec, int row0,
+                                           int rows, int k0, int kend, float4 (&t)[R / 32])
 {
 #pragma unroll
-    for (int q = 0; q < GBM * GBK / kGemmThreads; ++q) {
+    for (int q = 0; q < R / 32; ++q) {
         const int e = threadIdx.x + kGemmThreads * q;
-        const int r = s_k == 1 ? e / GBK : e % GBM, k = s_k == 1 ? e % GBK : e / GBM;
-        const int row = row0 + r, kk = k0 + k;
-        t.v[q] = (row < rows && kk < kend) ? __ldg(X + (int64_t)row * s_row + (int64_t)kk * s_k) : 0.f;
-    }
-}
-
-__device__ __forceinline__ void gemm_stash(int64_t s_k, const GemmTileRegs& t, float (*dst)[GBM + 4])
-{
-#pragma unroll
-    for (int q = 0; q < GBM * GBK / kGemmThreads; ++q) {
-        const int e = threadIdx.x + kGemmThreads * q;
-        const int r = s_k == 1 ? e / GBK : e % GBM, k = s_k == 1 ? e % GBK : e / GBM;
-        dst[k][r] = t.v[q];
-    }
-}
-
-__global__ void __launch_bounds__(kGemmThreads) gemm_f32_kernel(const float* __restrict__ A, int64_t sam, int64_t sak,
-                                                                const float* __restrict__ B, int64_t sbn, int64_t sbk,
-                                                                const float* __restrict__ bias, float* __restrict__ out,
-                                                                int64_t ldo, int M, int N, int K, int kchunk,
-                                                                float* __restrict__ part)
-{
-    __shared__ __align__(16) float As[2][GBK][GBM + 4], Bs[2][GBK][GBN + 4];
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;  // thread owns rows 4ty.., columns 4tx..
-    const int m0 = blockIdx.y * GBM, n0 = blockIdx.x * GBN;
-    const int kb = blockIdx.z * kchunk, ke = min(K, kb + kchunk);
-    float acc[4][4] = {};
-    GemmTileRegs ra, rb;
-    gemm_fetch(A, sam, sak, m0, M, kb, ke, ra);
-    gemm_fetch(B, sbn, sbk, n0, N, kb, ke, rb);
-    int buf = 0;
-    for (int k0 = kb; k0 < ke; k0 += GBK, buf ^= 1) {
-        gemm_stash(sak, ra, As[buf]);
-        gemm_stash(sbk, rb, Bs[buf]);
-        __syncthreads();
-        if (k0 + GBK < ke) {  // next tile in flight during the multiply
-            gemm_fetch(A, sam, sak, m0, M, k0 + GBK, ke, ra);
-            gemm_fetch(B, sbn, sbk, n0, N, k0 + GBK, ke, rb);
-        }
-#pragma unroll
-        for (int k = 0; k < GBK; ++k) {
-            const float4 a = *reinterpret_cast<const float4*>(&As[buf][k][4 * ty]);
-            const float4 b = *reinterpret_cast<const float4*>(&Bs[buf][k][4 * tx]);
-            const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+        const bool along_k = s_k == 1;
+        const int row = row0 + (along_k ? e / 4 : e % (R / 4) * 4), k = k0 + (along_k ? e % 4 * 4 : e / (R / 4));
+        const float* p = X + (int64_t)row * s_row + (int64_t)k * s_k;
+        float f[4];
+        if (vec && row + (along_k ? 0 : 3) < rows && k + (along_k ? 3 : 0) < kend) {
+            t[q] = __ldg(reinterpret_cast<const float4*>(p));
+        } else {
 #pragma unroll
             for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
+                f[i] = (row + (along_k ? 0 : i) < rows && k + (along_k ? i : 0) < kend) ? __ldg(p + i) : 0.f;
+            t[q] = make_float4(f[0], f[1], f[2], f[3]);
         }
     }
-    float* dst = part ? part + (int64_t)blockIdx.z * M * N : out;
-    const int64_t ld = part ? N : ldo;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int m = m0 + 4 * ty + i, n = n0 + 4 * tx + j;
-            if (m < M && n < N) dst[(int64_t)m * ld + n] = part ? acc[i][j] : acc[i][j] + (bias ? bias[n] : 0.f);
-        }
 }
 
-// out[m, n] = sum over chunks z = 0..nz-1 in order of part[z][m][n] (+ bias[n]).
-__global__ void __launch_bounds__(256) gemm_chunk_reduce_kernel(const float* __restrict__ part, int nz, int M, int N,
-                                                                const float* __restrict__ bias, float* __restrict__ out,
-                                                                int64_t ldo)
+template <int R>
+__device__ __forceinline__ void gemm_stash(bool along_k, const float4 (&t)[R / 32], float* dst)
 {
-    const int64_t total = (int64_t)M * N;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        float v = part[i];
-        for (int z = 1; z < nz; ++z) v += part[z * total + i];
-        const int m = (int)(i / N), n = (int)(i % N);
-        out[(int64_t)m * ldo + n] = v + (bias ? bias[n] : 0.f);
+#pragma unroll
+    for (int q = 0; q < R / 32; ++q) {
+        const int e = threadIdx.x + kGemmThreads * q;
+        if (along_k) {
+            float* d = dst + e % 4 * 4 * (R + 4) + e / 4;
+            d[0] = t[q].x;
+            d[R + 4] = t[q].y;
+            d[2 * (R + 4)] = t[q].z;
+            d[3 * (R + 4)] = t[q].w;
+        } else {
+            *reinterpret_cast<float4*>(dst + e / (R / 4) * (R + 4) + e % (R / 4) * 4) = t[q];
+        }
     }
 }
 
-// K-chunking of an M x N x K head GEMM: enough chunks for ~kGemmTargetCTAs CTAs, at least
-// four K tiles per chunk.  Returns the chunk length; *nz receives the chunk count.
-int gemm_chunking(int M, int N, int K, int* nz)
+// What the launch that has dlogits as input also computes (J = 0: nothing): loss = mean(row_loss)
+// and db[j] = sum_n dl[n, j].
+struct HeadSums {
+    const float *row_loss, *dl;
+    float *loss, *db;
+    int n, J;
+};
+
+constexpr int kHeadRedCols = 32;
+
+// Block 0: the loss (256 strided sums, two per thread, then a tree); blocks 1..: 32 columns of db each,
+// eight sums of rows w, w + 8, ... in order (two per warp), added in that order.
+__device__ __forceinline__ void head_sums(const HeadSums& h, int block, float* red)
 {
-    const int tiles = ((M + GBM - 1) / GBM) * ((N + GBN - 1) / GBN);
-    int z = (kGemmTargetCTAs + tiles - 1) / tiles;
-    const int zmax = std::max(1, (K + 4 * GBK - 1) / (4 * GBK));
-    z = std::min(std::max(z, 1), zmax);
-    int kchunk = (K + z - 1) / z;
-    kchunk = (kchunk + GBK - 1) / GBK * GBK;
-    *nz = (K + kchunk - 1) / kchunk;
-    return kchunk;
+    const int t = threadIdx.x;
+    if (block == 0) {
+        float s[2] = {0.f, 0.f};
+        for (int i = t; i < h.n; i += 256) {
+            s[0] += h.row_loss[i];
+            if (i + 128 < h.n) s[1] += h.row_loss[i + 128];
+        }
+        red[t] = s[0];
+        red[t + 128] = s[1];
+        __syncthreads();
+        for (int w = 128; w; w >>= 1) {
+            if (t < w) red[t] += red[t + w];
+            __syncthreads();
+        }
+        if (t == 0) *h.loss = red[0] / (float)h.n;
+        return;
+    }
+    const int lane = t % 32, w = t / 32, j = (block - 1) * kHeadRedCols + lane;
+    float s[2] = {0.f, 0.f};
+    if (j < h.J) {
+#pragma unroll 8
+        for (int i = w; i < h.n; i += 8) {
+            s[0] += h.dl[(int64_t)i * h.J + j];
+            if (i + 4 < h.n) s[1] += h.dl[(int64_t)(i + 4) * h.J + j];
+        }
+    }
+    red[t] = s[0];
+    red[t + 128] = s[1];
+    __syncthreads();
+    if (w == 0 && j < h.J) {
+        float v = red[lane];
+#pragma unroll
+        for (int k = 1; k < 8; ++k) v += red[k * 32 + lane];
+        h.db[j] = v;
+    }
 }
 
-size_t gemm_part_floats(int M, int N, int K)
+__global__ void __launch_bounds__(kGemmThreads, 4) head_gemm_kernel(const __grid_constant__ GemmJob j0,
+                                                                    const __grid_constant__ GemmJob j1,
+                                                                    const __grid_constant__ HeadSums hs)
 {
-    int nz;
-    gemm_chunking(M, N, K, &nz);
-    return nz > 1 ? (size_t)nz * M * N : 0;
+    using namespace dbl::dev;
+    __shared__ __align__(16) float sm[GBM * GBN];  // K tiles, then the partial sums of this CTA
+    static_assert(2 * GBK * (GLA + GLB) <= GBM * GBN, "K tiles");
+    const int nz = gridDim.z, z = blockIdx.z;  // the cluster: one CTA per chunk
+    int tile = blockIdx.x;
+    if (tile >= j0.tiles + j1.tiles) {
+        const int b = (tile - j0.tiles - j1.tiles) * nz + z;
+        if (b <= (hs.J + kHeadRedCols - 1) / kHeadRedCols) head_sums(hs, b, sm);
+        return;
+    }
+    const GemmJob& j = tile < j0.tiles ? j0 : j1;
+    if (tile >= j0.tiles) tile -= j0.tiles;
+    const int tn = (j.N + GBN - 1) / GBN;
+    const int m0 = tile / tn * GBM, n0 = tile % tn * GBN;
+    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;  // rows 4ty.., 32 + 4ty..; columns 4tx.., 64 + 4tx..
+    const int kb = z * j.kchunk, ke = min(j.K, kb + j.kchunk);
+    float2 acc[8][4];
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[r][c] = make_float2(0.f, 0.f);
+    float4 ra[GBM / 32], rb[GBN / 32];
+    gemm_fetch<GBM>(j.A, j.sam, j.sak, j.vec & 1, m0, j.M, kb, ke, ra);
+    gemm_fetch<GBN>(j.B, j.sbn, j.sbk, j.vec & 2, n0, j.N, kb, ke, rb);
+    float* buf = sm;
+    for (int k0 = kb; k0 < ke; k0 += GBK) {
+        gemm_stash<GBM>(j.sak == 1, ra, buf);
+        gemm_stash<GBN>(j.sbk == 1, rb, buf + GBK * GLA);
+        __syncthreads();
+        if (k0 + GBK < ke) {  // next tile in flight during the multiply
+            gemm_fetch<GBM>(j.A, j.sam, j.sak, j.vec & 1, m0, j.M, k0 + GBK, ke, ra);
+            gemm_fetch<GBN>(j.B, j.sbn, j.sbk, j.vec & 2, n0, j.N, k0 + GBK, ke, rb);
+        }
+        const float *as = buf + 4 * ty, *bs = buf + GBK * GLA + 4 * tx;
+#pragma unroll
+        for (int k = 0; k < GBK; ++k) {
+            const float4 a0 = *reinterpret_cast<const float4*>(as + k * GLA);
+            const float4 a1 = *reinterpret_cast<const float4*>(as + k * GLA + 32);
+            const float4 b0 = *reinterpret_cast<const float4*>(bs + k * GLB);
+            const float4 b1 = *reinterpret_cast<const float4*>(bs + k * GLB + 64);
+            const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+            const float2 bv[4] = {{b0.x, b0.y}, {b0.z, b0.w}, {b1.x, b1.y}, {b1.z, b1.w}};
+#pragma unroll
+            for (int r = 0; r < 8; ++r)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) acc[r][c] = fma2(make_float2(av[r], av[r]), bv[c], acc[r][c]);
+        }
+        buf = buf == sm ? sm + GBK * (GLA + GLB) : sm;
+    }
+    __syncthreads();  // the last tile has been read: sm takes the partial sums
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+        float* d = sm + (r / 4 * 32 + 4 * ty + r % 4) * GBN + 4 * tx;
+        *reinterpret_cast<float4*>(d) = make_float4(acc[r][0].x, acc[r][0].y, acc[r][1].x, acc[r][1].y);
+        *reinterpret_cast<float4*>(d + 64) = make_float4(acc[r][2].x, acc[r][2].y, acc[r][3].x, acc[r][3].y);
+    }
+    __syncthreads();
+    cluster_sync_all();
+    // CTA z finishes rows z, z + nz, ... groups of four: 32 threads per row
+    const int c = threadIdx.x % 32 * 4, n = n0 + c;
+    float bias[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) bias[i] = j.bias && n + i < j.N ? j.bias[n + i] : 0.f;
+    for (int r = z * 4 + threadIdx.x / 32; r < GBM; r += 4 * nz) {
+        const uint32_t a = smem_u32(sm + r * GBN + c);
+        float4 v[kGemmMaxChunks];
+#pragma unroll
+        for (int q = 0; q < kGemmMaxChunks; ++q)
+            if (q < nz) v[q] = ld_cluster_f32x4(mapa_shared(a, (uint32_t)q));
+        float4 s = v[0];
+#pragma unroll
+        for (int q = 1; q < kGemmMaxChunks; ++q)
+            if (q < nz) {
+                s.x += v[q].x;
+                s.y += v[q].y;
+                s.z += v[q].z;
+                s.w += v[q].w;
+            }
+        const float o[4] = {s.x + bias[0], s.y + bias[1], s.z + bias[2], s.w + bias[3]};
+        const int m = m0 + r;
+        if (m < j.M) {
+            float* d = j.out + (int64_t)m * j.ldo + n;
+            if ((j.vec & 4) && n + 3 < j.N) {
+                *reinterpret_cast<float4*>(d) = make_float4(o[0], o[1], o[2], o[3]);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (n + i < j.N) d[i] = o[i];
+            }
+        }
+    }
+    cluster_sync_all();  // no CTA leaves while another may still read its partial sums
 }
 
-int gemm_f32(const float* A, int64_t sam, int64_t sak, const float* B, int64_t sbn, int64_t sbk, const float* bias,
-             float* out, int64_t ldo, int M, int N, int K, float* part, cudaStream_t s, const char* what)
+GemmJob gemm_job(const float* A, int64_t sam, int64_t sak, const float* B, int64_t sbn, int64_t sbk, const float* bias,
+                 float* out, int64_t ldo, int M, int N, int K)
 {
-    int nz;
-    const int kchunk = gemm_chunking(M, N, K, &nz);
-    dim3 g((N + GBN - 1) / GBN, (M + GBM - 1) / GBM, nz);
-    gemm_f32_kernel<<<g, kGemmThreads, 0, s>>>(A, sam, sak, B, sbn, sbk, bias, out, ldo, M, N, K, kchunk,
-                                                nz > 1 ? part : nullptr);
-    int rc = dbl::launch_check(what);
-    if (rc || nz == 1) return rc;
-    const int64_t total = (int64_t)M * N;
-    const int blocks = (int)std::min<int64_t>((total + 255) / 256, (int64_t)dbl::sm_count() * 8);
-    gemm_chunk_reduce_kernel<<<blocks, 256, 0, s>>>(part, nz, M, N, bias, out, ldo);
+    GemmJob j{A, B, bias, out, sam, sak, sbn, sbk, ldo, M, N, K, 0, 0, 0};
+    j.tiles = ((M + GBM - 1) / GBM) * ((N + GBN - 1) / GBN);
+    auto vec = [](const float* p, int64_t ld) { return dbl::aligned16(p) && ld % 4 == 0; };
+    j.vec = (vec(A, sak == 1 ? sam : sak) ? 1 : 0) | (vec(B, sbk == 1 ? sbn : sbk) ? 2 : 0) | (vec(out, ldo) ? 4 : 0);
+    return j;
+}
+
+// One or two products (j1 may have no tiles) and the sums of hs.  The number of K chunks is a function of the
+// shapes only: the most, of 1, 2, 4 and 8, that leaves the longer reduction two K tiles per chunk and
+// the grid within the CTAs that are resident at one time.
+int head_gemm(GemmJob j0, GemmJob j1, const HeadSums& hs, cudaStream_t s, const char* what)
+{
+    const int K = std::max(j0.K, j1.tiles ? j1.K : 0), tiles = j0.tiles + j1.tiles;
+    int nz = 1;
+    while (nz < kGemmMaxChunks && tiles * nz * 2 <= kGemmMaxCTAs && K >= 2 * nz * 2 * GBK) nz *= 2;
+    for (GemmJob* j : {&j0, &j1}) j->kchunk = ((j->K + nz - 1) / nz + GBK - 1) / GBK * GBK;
+    const int sums = hs.J ? 1 + (hs.J + kHeadRedCols - 1) / kHeadRedCols : 0;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = nz;
+    cfg.gridDim = dim3(tiles + (sums + nz - 1) / nz, 1, nz);
+    cfg.blockDim = dim3(kGemmThreads);
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, head_gemm_kernel, j0, j1, hs);
+    if (e != cudaSuccess) {
+        dbl::count_launch();
+        return dbl::cuda_check(e, what);
+    }
     return dbl::launch_check(what);
 }
 
-// One warp per row: loss_n = logsumexp(l) - l[label]; dl = (softmax - onehot) * S/n (in place), S the
-// loss scale (1 without loss scaling).
-__global__ void softmax_ce_kernel(float* __restrict__ logits, const int32_t* __restrict__ labels, int n, int J,
-                                  float* __restrict__ row_loss, const float* __restrict__ loss_scale)
+// One CTA per row: loss_n = logsumexp(l) - l[label]; dl = (softmax - onehot) * S/n (in place), S the
+// loss scale (1 without loss scaling).  (One warp per row, eight rows per CTA, left 88 SMs idle at
+// 512 rows and walked 1000 classes in 32 dependent steps per pass.)
+constexpr int kSoftmaxThreads = 128;
+__global__ void __launch_bounds__(kSoftmaxThreads) softmax_ce_kernel(float* __restrict__ logits,
+                                                                     const int32_t* __restrict__ labels, int n, int J,
+                                                                     float* __restrict__ row_loss,
+                                                                     const float* __restrict__ loss_scale)
 {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) / 32, lane = threadIdx.x % 32;
-    if (warp >= n) return;
-    float* l = logits + (int64_t)warp * J;
-    float mx = -FLT_MAX;
-    for (int j = lane; j < J; j += 32) mx = fmaxf(mx, l[j]);
-    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    float z = 0.f;
-    for (int j = lane; j < J; j += 32) z += expf(l[j] - mx);
-    for (int o = 16; o; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-    const float lse = mx + logf(z);
-    const int lab = labels[warp];
-    if (lane == 0) row_loss[warp] = lse - l[lab];
+    __shared__ float red[2][kSoftmaxThreads / 32];
+    const int row = blockIdx.x, t = threadIdx.x, w = t / 32;
+    float* l = logits + (int64_t)row * J;
+    const int lab = labels[row];
     const float invn = (loss_scale ? *loss_scale : 1.0f) / (float)n;
-    for (int j = lane; j < J; j += 32) l[j] = (expf(l[j] - lse) - (j == lab ? 1.f : 0.f)) * invn;
-}
-
-// loss = mean(row_loss) (block 0, fixed order); db[j] = sum_n dl[n, j] (blocks 1..: 32 columns each,
-// warp w adding rows w, w + 8, ... in order, then the eight warp sums added in warp order).  Each
-// column's rows are spread over eight warps instead of one thread's chain of n dependent adds.
-constexpr int kHeadRedCols = 32;
-__global__ void __launch_bounds__(256) head_reduce_kernel(const float* __restrict__ row_loss, const float* __restrict__ dl,
-                                                          int n, int J, float* __restrict__ loss, float* __restrict__ db)
-{
-    __shared__ float red[256];
-    if (blockIdx.x == 0) {
-        float s = 0.f;
-        for (int i = threadIdx.x; i < n; i += blockDim.x) s += row_loss[i];
-        red[threadIdx.x] = s;
-        __syncthreads();
-        for (int w = blockDim.x / 2; w; w >>= 1) {
-            if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) *loss = red[0] / (float)n;
-        return;
-    }
-    const int lane = threadIdx.x % 32, w = threadIdx.x / 32;
-    const int j = (blockIdx.x - 1) * kHeadRedCols + lane;
-    float s = 0.f;
-    if (j < J)
-        for (int i = w; i < n; i += 8) s += dl[(int64_t)i * J + j];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    if (w == 0 && j < J) {
-        float t = red[lane];
+    float mx = -FLT_MAX;
+#pragma unroll 8
+    for (int j = t; j < J; j += kSoftmaxThreads) mx = fmaxf(mx, l[j]);
 #pragma unroll
-        for (int k = 1; k < 8; ++k) t += red[k * 32 + lane];
-        db[j] = t;
-    }
+    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (t % 32 == 0) red[0][w] = mx;
+    __syncthreads();
+    mx = fmaxf(fmaxf(red[0][0], red[0][1]), fmaxf(red[0][2], red[0][3]));
+    float z = 0.f;
+#pragma unroll 8
+    for (int j = t; j < J; j += kSoftmaxThreads) z += expf(l[j] - mx);
+#pragma unroll
+    for (int o = 16; o; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+    if (t % 32 == 0) red[1][w] = z;
+    __syncthreads();
+    z = (red[1][0] + red[1][1]) + (red[1][2] + red[1][3]);
+    const float lse = mx + logf(z);
+    if (t == 0) row_loss[row] = lse - l[lab];
+    __syncthreads();  // l[lab] has been read
+#pragma unroll 8
+    for (int j = t; j < J; j += kSoftmaxThreads) l[j] = (expf(l[j] - lse) - (j == lab ? 1.f : 0.f)) * invn;
 }
 
 // The same two passes with one CTA per image, blockDim = S slices x (C/8) channel groups: thread
@@ -667,11 +775,15 @@ __global__ void __launch_bounds__(1024) avgpool_bwd_img_kernel(const float* __re
     const int b = blockIdx.x;
     const float inv = 1.0f / (float)hw;
     float f[8];
+    load8(df + (int64_t)b * C + 8 * g, f);
+    if (mult) {
+        float m[8];
+        load8(mult + (int64_t)b * C + 8 * g, m);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        const int64_t e = (int64_t)b * C + 8 * g + k;
-        f[k] = (mult ? df[e] * mult[e] : df[e]) * inv;
+        for (int k = 0; k < 8; ++k) f[k] *= m[k];
     }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) f[k] *= inv;
     const uint4 v = pack8(f);
     uint4* row = reinterpret_cast<uint4*>(dx + (int64_t)b * hw * C) + g;
     for (int i = sl; i < hw; i += S) row[(int64_t)i * groups] = v;
@@ -775,12 +887,9 @@ int dbl_maxpool_bwd(int32_t n, int32_t h, int32_t w, int32_t c, const void* dy, 
 size_t dbl_head_workspace_bytes(int32_t n, int32_t c, int32_t classes)
 {
     if (n <= 0 || c <= 0 || classes <= 0) return 0;
-    // feat [n,c], logits/dlogits [n,classes], df [n,c], row_loss [n], dropout multipliers [n,c],
-    // then the K-chunk partial sums of the largest of the three GEMMs
+    // feat, df and the dropout multipliers [n,c], logits/dlogits [n,classes], row_loss [n]
     const size_t f = (size_t)n * c * 3 + (size_t)n * classes + (size_t)n;
-    const size_t part = std::max({gemm_part_floats(n, classes, c), gemm_part_floats(classes, c, n),
-                                  gemm_part_floats(n, c, classes)});
-    return (((f + 3) / 4 * 4 + part) * sizeof(float) + 255) / 256 * 256;
+    return (f * sizeof(float) + 16 + 255) / 256 * 256;  // 16: alignment of the caller's pointer
 }
 
 }  // extern "C"
@@ -804,12 +913,12 @@ int head_fwd_bwd(int32_t n, int32_t hw, int32_t c, int32_t classes, const void* 
         return set_error(DBL_ERR_INVALID, "%s: dropout needs an 8-byte aligned device step counter", name);
     const size_t need = dbl_head_workspace_bytes(n, c, classes);
     if (!ws || ws_bytes < need) return set_error(DBL_ERR_WORKSPACE, "%s: workspace %zu < %zu", name, ws_bytes, need);
-    float* feat = static_cast<float*>(ws);
-    float* logits = feat + (size_t)n * c;
-    float* df = logits + (size_t)n * classes;
-    float* row_loss = df + (size_t)n * c;
-    float* mult = row_loss + (size_t)n;
-    float* part = feat + ((size_t)n * c * 3 + (size_t)n * classes + (size_t)n + 3) / 4 * 4;
+    // c is a multiple of 8, so feat, df, mult and logits are all 16-byte aligned
+    float* feat = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(ws) + 15) / 16 * 16);
+    float* df = feat + (size_t)n * c;
+    float* mult = df + (size_t)n * c;
+    float* logits = mult + (size_t)n * c;
+    float* row_loss = logits + (size_t)n * classes;
     Dropout dp{0u, 1.f, seed, step, mult};
     if (drop_rate > 0.f) {
         dp.thr = (uint32_t)floor((double)drop_rate * 4294967296.0);
@@ -828,18 +937,15 @@ int head_fwd_bwd(int32_t n, int32_t hw, int32_t c, int32_t classes, const void* 
                                                                            c, dp);
     if ((rc = launch_check("avgpool launch"))) return rc;
     // logits = feat * W^T + b
-    if ((rc = gemm_f32(feat, c, 1, fc_w, c, 1, fc_b, logits, classes, n, classes, c, part, s, "fc fwd launch")))
+    if ((rc = head_gemm(gemm_job(feat, c, 1, fc_w, c, 1, fc_b, logits, classes, n, classes, c), GemmJob{}, HeadSums{}, s,
+                        "fc fwd launch")))
         return rc;
-    softmax_ce_kernel<<<(n * 32 + 255) / 256, 256, 0, s>>>(logits, labels, n, classes, row_loss, loss_scale);
+    softmax_ce_kernel<<<n, kSoftmaxThreads, 0, s>>>(logits, labels, n, classes, row_loss, loss_scale);
     if ((rc = launch_check("softmax_ce launch"))) return rc;
-    head_reduce_kernel<<<1 + (classes + kHeadRedCols - 1) / kHeadRedCols, 256, 0, s>>>(row_loss, logits, n, classes,
-                                                                                        loss, dfc_b);
-    if ((rc = launch_check("head reduce launch"))) return rc;
-    // dW[j, c] = sum_n dl[n, j] feat[n, c]
-    if ((rc = gemm_f32(logits, 1, classes, feat, 1, c, nullptr, dfc_w, c, classes, c, n, part, s, "fc dW launch")))
-        return rc;
-    // df[n, c] = sum_j dl[n, j] W[j, c]
-    if ((rc = gemm_f32(logits, classes, 1, fc_w, 1, c, nullptr, df, c, n, c, classes, part, s, "fc dX launch")))
+    // df[n, c] = sum_j dl[n, j] W[j, c]; dW[j, c] = sum_n dl[n, j] feat[n, c]; the loss and db
+    if ((rc = head_gemm(gemm_job(logits, classes, 1, fc_w, 1, c, nullptr, df, c, n, c, classes),
+                        gemm_job(logits, 1, classes, feat, 1, c, nullptr, dfc_w, c, classes, c, n),
+                        HeadSums{row_loss, logits, loss, dfc_b, n, classes}, s, "fc bwd launch")))
         return rc;
     // with dropout, the pool's backward also advances the step counter (the next call draws a fresh mask)
     uint64_t* adv = dp.thr ? step : nullptr;
