@@ -119,13 +119,19 @@ struct Cfg {
     static constexpr int MAX_STAGES = CG == 2 ? 6 : 4;
     static constexpr int STAGES = (196608 / STAGE_BYTES) < MAX_STAGES ? (196608 / STAGE_BYTES) : MAX_STAGES;
     static constexpr int RING = STAGES * STAGE_BYTES;
-    static constexpr int EPI_TILE = 4 * 32 * 33 * 4;           // per-warp 32x32 transpose scratch
-    static constexpr int EPI_SUM = 4 * 2 * kMaxNcols * 4;      // per-warp channel sums (fwd)
+    // Epilogue warps: two per TMEM lane quarter for the wider tiles, each draining half of the columns
+    // (the last tile's epilogue is not hidden behind MMAs; with four warps it takes 750 cycles per 32
+    // columns with channel sums): forward at 10x10x256, batch 128 20.4 -> 18.5 us, 7x7x512, batch 128
+    // 30.1 -> 28.2, its data gradient 27.5 -> 27.2; a 14x14 1x1 projection 256 -> 512 11.5 -> 9.8
+    static constexpr int EPI = BN > 64 ? 8 : 4;
+    static constexpr int CW = BN * 4 / EPI;                    // columns one epilogue warp drains
+    static constexpr int EPI_TILE = BN > 64 ? 0 : 4 * 32 * 33 * 4;  // per-warp 32x32 transpose scratch (RowStats)
+    static constexpr int EPI_SUM = 4 * 2 * kMaxNcols * 4;      // channel sums per lane quarter (fwd)
     static constexpr int SMEM = RING + EPI_TILE + EPI_SUM + 1024;  // + 1 KB alignment slack
     static constexpr int NB = ACC * BN <= 128 ? 4 : 2;          // tiles in flight (TMEM accumulator buffers)
     static constexpr uint32_t TMEM_COLS = NB * ACC * BN;
-    static constexpr int THREADS = 32 * (4 + kProducers + 1);   // epilogue, producers, MMA
-    static constexpr int MMA_WARP = 4 + kProducers;
+    static constexpr int THREADS = 32 * (EPI + kProducers + 1);  // epilogue, producers, MMA
+    static constexpr int MMA_WARP = EPI + kProducers;
     static_assert(STAGES >= 2, "ring too shallow");
     static_assert(TMEM_COLS <= 512, "TMEM holds 512 columns");
     static_assert(SMEM <= 232448 - 1024, "shared memory per CTA");
@@ -288,85 +294,50 @@ __device__ __forceinline__ void store_row_chunk_act(const ConvParams& p, const u
 // in registers across the tiles of a CTA instead of being reduced across the
 // warp for every tile (which costs shared-memory bandwidth that the mainloop
 // needs).  Thread (warp, lane) adds the values of its own accumulator row.
-// For 128 columns the rows are first folded pairwise across lanes (one shuffle
-// step), so that every thread holds 128 sums: after the folding, value k of chunk
-// ch belongs to column ch*32 + (lane & (32 - V)) + k.
 // flush() reduces over the lanes through the warp's 32x33 scratch and adds the
 // column totals to the warp's channel sums (once per CTA).
 template <int BN>
 struct RowStats {
     static constexpr int NCH = BN / 32;
-    static constexpr int LEVELS = BN <= 64 ? 0 : 1;
-    static_assert(BN <= 128, "ColStats holds wider tiles");
-    static constexpr int V = 32 >> LEVELS;
-    float s[NCH][V], q[NCH][V];
+    float s[NCH][32], q[NCH][32];
 
     __device__ __forceinline__ void zero()
     {
 #pragma unroll
         for (int c = 0; c < NCH; ++c)
 #pragma unroll
-            for (int k = 0; k < V; ++k) s[c][k] = q[c][k] = 0.f;
-    }
-
-    template <int N, int O>
-    __device__ __forceinline__ static void fold(float (&a)[32], float (&b)[32], int lane)
-    {
-        const bool up = (lane & O) != 0;
-#pragma unroll
-        for (int k = 0; k < N / 2; ++k) {
-            const float sa = up ? a[k] : a[k + N / 2], ka = up ? a[k + N / 2] : a[k];
-            const float sb = up ? b[k] : b[k + N / 2], kb = up ? b[k + N / 2] : b[k];
-            a[k] = ka + __shfl_xor_sync(0xffffffffu, sa, O);
-            b[k] = kb + __shfl_xor_sync(0xffffffffu, sb, O);
-        }
+            for (int k = 0; k < 32; ++k) s[c][k] = q[c][k] = 0.f;
     }
 
     // x: the stored values of chunk ch of this thread's row (call with ch a compile-time
-    // constant after unrolling).  Every lane of the warp must call it.
-    __device__ __forceinline__ void add(int ch, const float (&x)[32], int lane)
+    // constant after unrolling); the sum of squares by fused multiply-add.
+    __device__ __forceinline__ void add(int ch, const float (&x)[32])
     {
-        if constexpr (LEVELS == 0) {  // no folding: sum of squares by fused multiply-add
 #pragma unroll
-            for (int k = 0; k < 32; k += 2) {
-                const float2 v = make_float2(x[k], x[k + 1]);
-                const float2 a = add2(make_float2(s[ch][k], s[ch][k + 1]), v);
-                const float2 b = fma2(v, v, make_float2(q[ch][k], q[ch][k + 1]));
-                s[ch][k] = a.x;
-                s[ch][k + 1] = a.y;
-                q[ch][k] = b.x;
-                q[ch][k + 1] = b.y;
-            }
-        } else {
-            float a[32], b[32];
-#pragma unroll
-            for (int k = 0; k < 32; ++k) {
-                a[k] = x[k];
-                b[k] = x[k] * x[k];
-            }
-            fold<32, 16>(a, b, lane);
-#pragma unroll
-            for (int k = 0; k < V; ++k) {
-                s[ch][k] += a[k];
-                q[ch][k] += b[k];
-            }
+        for (int k = 0; k < 32; k += 2) {
+            const float2 v = make_float2(x[k], x[k + 1]);
+            const float2 a = add2(make_float2(s[ch][k], s[ch][k + 1]), v);
+            const float2 b = fma2(v, v, make_float2(q[ch][k], q[ch][k + 1]));
+            s[ch][k] = a.x;
+            s[ch][k + 1] = a.y;
+            q[ch][k] = b.x;
+            q[ch][k + 1] = b.y;
         }
     }
 
-    // wsum: this warp's [2][Ncols] channel sums; col_base: first column of the tile.
+    // wsum: [2][ncols] channel sums; col_base: the warp's first column.
     __device__ __forceinline__ void flush(float* st_tile, float* wsum, int ncols, int col_base, int lane)
     {
-        const int hb = lane & (32 - V), kk = lane & (V - 1);
 #pragma unroll
         for (int c = 0; c < NCH; ++c) {
 #pragma unroll
             for (int w = 0; w < 2; ++w) {
 #pragma unroll
-                for (int k = 0; k < V; ++k) st_tile[lane * 33 + k] = w ? q[c][k] : s[c][k];
+                for (int k = 0; k < 32; ++k) st_tile[lane * 33 + k] = w ? q[c][k] : s[c][k];
                 __syncwarp();
                 float tot = 0.f;
 #pragma unroll
-                for (int u = 0; u < V; ++u) tot += st_tile[(hb + u) * 33 + kk];
+                for (int u = 0; u < 32; ++u) tot += st_tile[u * 33 + lane];
                 __syncwarp();
                 wsum[w * ncols + col_base + c * 32 + lane] += tot;
             }
@@ -448,8 +419,9 @@ struct ColStats {
     }
 };
 
+// The statistics of an epilogue warp of a BN-column tile: ColStats over half of the columns, or RowStats.
 template <int BN>
-using TileStats = std::conditional_t<(BN > 64), ColStats<BN>, RowStats<BN>>;
+using TileStats = std::conditional_t<(BN > 64), ColStats<BN / 2>, RowStats<BN>>;
 
 // Persistent kernel: CTA b processes tiles b, b + gridDim.x, ...  The ring of
 // STAGES shared-memory stages runs continuously across tiles; two producer
@@ -494,7 +466,7 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, CG>::THREADS, 1)
         }
         for (int b = 0; b < C::NB; ++b) {
             mbar_init(&accf_bar[b], 1);
-            mbar_init(&acce_bar[b], 4 * CG);  // one arrival per epilogue warp of the pair
+            mbar_init(&acce_bar[b], C::EPI * CG);  // one arrival per epilogue warp of the pair
         }
         mbar_init(&drain_bar, 1);
         abort_flag = 0;
@@ -503,7 +475,7 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, CG>::THREADS, 1)
     const bool want_stats = FAM == kFamFwd && (p.mode == kFwd || p.mode == kFwdC8) && p.stats != nullptr;
     if (want_stats)
         for (int i = threadIdx.x; i < 4 * 2 * p.Ncols; i += blockDim.x) epi_sum[i] = 0.f;
-    if (warp >= 4 && warp < 4 + kProducers && lane == 0) {
+    if (warp >= C::EPI && warp < C::MMA_WARP && lane == 0) {
         tma_prefetch_desc(&tmA);
         tma_prefetch_desc(&tmB);
         if (p.proj_kb) {
@@ -523,9 +495,9 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, CG>::THREADS, 1)
     const uint32_t tmem = tmem_slot;
     const int64_t gPQ = (int64_t)p.gP * p.gQ;
 
-    if (warp >= 4 && warp < 4 + kProducers) {
+    if (warp >= C::EPI && warp < C::MMA_WARP) {
         // ------------------------------------------------------------------ TMA producers (whole warp, one lane issues)
-        const int prod = warp - 4;
+        const int prod = warp - C::EPI;
         int it = 0, last_it = -1;
         bool failed = false;
         for (int t = unit0; t < p.total_tiles; t += nunits) {
@@ -674,14 +646,16 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, CG>::THREADS, 1)
             (void)mbar_drain_warp(&drain_bar, 0);
         }
     } else {
-        // ------------------------------------------------------------------ epilogue (warps 0-3)
-        float* st_tile = epi_tile + warp * 32 * 33;
-        float* wsum = epi_sum + warp * 2 * p.Ncols;
+        // ------------------------------------------------------------------ epilogue (warps 0 .. EPI-1)
+        constexpr int CW = C::CW, NCH = CW / 32;
+        const int quarter = warp & 3, cw0 = (warp >> 2) * CW;  // TMEM lanes 32*quarter.., tile columns cw0..
+        [[maybe_unused]] float* st_tile = epi_tile + warp * 32 * 33;
+        float* wsum = epi_sum + quarter * 2 * p.Ncols;
         TileStats<BN> rs;
         rs.zero();
         auto flush = [&](int ntile) {
             if constexpr (BN > 64)
-                rs.flush(wsum, p.Ncols, ntile * BN, lane);
+                rs.flush(wsum, p.Ncols, ntile * BN + cw0, lane);
             else
                 rs.flush(st_tile, wsum, p.Ncols, ntile * BN, lane);
         };
@@ -698,7 +672,7 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, CG>::THREADS, 1)
                 break;
             }
             tc_fence_after();
-            const int row = warp * 32 + lane;  // TMEM lane = row within a 128-row accumulator
+            const int row = quarter * 32 + lane;  // TMEM lane = row within a 128-row accumulator
             const bool have_acc = nkb > 0;
             if (want_stats && stats_ntile != tc.n_tile) {
                 if (stats_ntile >= 0) flush(stats_ntile);
@@ -708,10 +682,11 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, CG>::THREADS, 1)
             for (int a = 0; a < C::ACC; ++a) {
                 const int64_t m = ((int64_t)tc.m_tile * CG + rank) * C::BMT + a * 128 + row;
                 const bool valid = m < p.M;
-                const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)((buf * C::ACC + a) * BN);
+                const uint32_t taddr =
+                    tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)((buf * C::ACC + a) * BN + cw0);
                 if constexpr (FAM == kFamWgrad) {
 #pragma unroll 1
-                    for (int ch = 0; ch < BN / 32; ++ch) {
+                    for (int ch = 0; ch < NCH; ++ch) {
                         uint32_t v[32];
                         if (have_acc) {
                             tmem_ld_32x32b_x32(taddr + ch * 32, v);
@@ -720,7 +695,7 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, CG>::THREADS, 1)
 #pragma unroll
                             for (int k = 0; k < 32; ++k) v[k] = 0u;
                         }
-                        const int col0 = tc.n_tile * BN + ch * 32;
+                        const int col0 = tc.n_tile * BN + cw0 + ch * 32;
                         // D row m = (tap, c), column = output channel k; stored as [slice][k][m]:
                         // consecutive lanes hold consecutive m, so each store is one 128-byte line
                         if (valid) {
@@ -744,7 +719,7 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, CG>::THREADS, 1)
                     }
                     const uint32_t rows_ok = __ballot_sync(0xffffffffu, valid);
 #pragma unroll
-                    for (int ch = 0; ch < BN / 32; ++ch) {
+                    for (int ch = 0; ch < NCH; ++ch) {
                         uint32_t v[32];
                         [[maybe_unused]] uint32_t lo[16], hi[16];
                         if (have_acc) {
@@ -767,11 +742,11 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, CG>::THREADS, 1)
                             for (int k = 0; k < 32; ++k) v[k] = 0u;
                         }
                         float back[32];
-                        store_row_chunk_act(p, v, valid, out_row, tc.n_tile * BN + ch * 32, back);
+                        store_row_chunk_act(p, v, valid, out_row, tc.n_tile * BN + cw0 + ch * 32, back);
                         if constexpr (BN > 64) {  // want_stats: the forward pass, whose tiles all have K-blocks
                             if (want_stats) rs.add(ch, lo, hi, rows_ok, lane);
                         } else {
-                            if (want_stats) rs.add(ch, back, lane);
+                            if (want_stats) rs.add(ch, back);
                         }
                     }
                 }
@@ -787,9 +762,9 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, CG>::THREADS, 1)
         }
         if (want_stats && stats_ntile >= 0) flush(stats_ntile);
         if (want_stats) {
-            asm volatile("bar.sync 1, 128;" ::: "memory");
+            asm volatile("bar.sync 1, %0;" ::"r"(C::EPI * 32) : "memory");
             float* dst = p.stats + (int64_t)blockIdx.x * 2 * p.Ncols;
-            for (int c = threadIdx.x; c < 2 * p.Ncols; c += 128)
+            for (int c = threadIdx.x; c < 2 * p.Ncols; c += C::EPI * 32)
                 dst[c] = (epi_sum[c] + epi_sum[2 * p.Ncols + c]) + (epi_sum[4 * p.Ncols + c] + epi_sum[6 * p.Ncols + c]);
         }
     }
@@ -821,10 +796,11 @@ struct SplitCfg {
     using C = Cfg<256, kFamFwd, 2>;
     static constexpr int W = 256 / SK;              // columns a CTA finishes
     static constexpr int SLOT = 128 * W * 4;        // one received part: [W / 4][128 rows] float4
-    static constexpr int EPI_TILE = 4 * 32 * 33 * 4;
-    static constexpr int EPI_SUM = 4 * 2 * W * 4;   // per-warp channel sums
-    static constexpr int SMEM = C::RING + EPI_TILE + EPI_SUM + 1024;
-    static_assert((SK - 1) * SLOT <= C::RING, "received parts fit in the ring");
+    static constexpr int CW = W > 32 ? W / 2 : 32;  // columns an epilogue warp finishes (of W = 32: one warp per quarter)
+    static constexpr int EPI_TILE = 8 * 32 * 33 * 4;
+    static constexpr int EPI_SUM = 4 * 2 * W * 4;   // channel sums per lane quarter
+    static constexpr int SMEM = C::RING + EPI_SUM + 1024;
+    static_assert((SK - 1) * SLOT + EPI_TILE <= C::RING, "received parts and transposes fit in the ring");
 };
 
 template <int SK>
@@ -863,7 +839,7 @@ __global__ void __launch_bounds__(Cfg<256, kFamFwd, 2>::THREADS, 1)
         abort_flag = 0;
         fence_mbar_init();
     }
-    if (warp >= 4 && warp < 4 + kProducers && lane == 0) {
+    if (warp >= C::EPI && warp < C::MMA_WARP && lane == 0) {
         tma_prefetch_desc(&tmA);
         tma_prefetch_desc(&tmB);
         if (p.proj_kb) {
@@ -883,9 +859,9 @@ __global__ void __launch_bounds__(Cfg<256, kFamFwd, 2>::THREADS, 1)
     const uint32_t tmem = tmem_slot;
     const int64_t gPQ = (int64_t)p.gP * p.gQ;
 
-    if (warp >= 4 && warp < 4 + kProducers) {
+    if (warp >= C::EPI && warp < C::MMA_WARP) {
         // ------------------------------------------------------------------ TMA producers
-        const int prod = warp - 4;
+        const int prod = warp - C::EPI;
         const int64_t m0 = ((int64_t)tc.m_tile * 2 + rank) * 128;
         const int tn = (int)(m0 / gPQ);
         const int64_t rem = m0 - (int64_t)tn * gPQ;
@@ -962,38 +938,55 @@ __global__ void __launch_bounds__(Cfg<256, kFamFwd, 2>::THREADS, 1)
     __syncwarp();
     cluster_sync_all();  // every pair's MMAs are done: the rings may be overwritten
 
-    const int row = warp * 32 + lane;  // TMEM lane = row within the 128-row accumulator (warps 0-3)
-    const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16);
-    if (warp < 4) {
+    const int quarter = warp & 3, half = warp >> 2;  // epilogue warps (0-7): TMEM lanes 32*quarter..
+    const int row = quarter * 32 + lane;             // row within the 128-row accumulator
+    const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16);
+    constexpr int CW = S::CW, NCH = CW / 32;
+    const bool finishes = warp < C::EPI && half * CW < W;
+    uint32_t own[NCH][32];  // this warp's part of the CTA's own columns
+    if (warp < C::EPI) {
+        // the other pairs' chunks of 32 columns, the two warps of a quarter taking alternate ones
 #pragma unroll 1
-        for (int d = 1; d < SK; ++d) {
-            const int to = (split + d) % SK;                  // pair that finishes these columns
+        for (int e = half; e < (SK - 1) * (W / 32); e += 2) {
+            const int to = (split + 1 + e / (W / 32)) % SK;   // pair that finishes these columns
+            const int ch = e % (W / 32);
             const int slot = split < to ? split : split - 1;  // its parts are kept in the pairs' order
             const uint32_t dst = mapa_shared(sbase, (uint32_t)(2 * to + rank)) + (uint32_t)(slot * S::SLOT + row * 16);
-#pragma unroll 1
-            for (int ch = 0; ch < W / 32; ++ch) {
-                uint32_t v[32];
-                if (nkb > 0) {
-                    tmem_ld_32x32b_x32(taddr + (uint32_t)(to * W + ch * 32), v);
-                    tmem_ld_wait_regs(v);
-                } else {
+            uint32_t v[32];
+            if (nkb > 0) {
+                tmem_ld_32x32b_x32(taddr + (uint32_t)(to * W + ch * 32), v);
+                tmem_ld_wait_regs(v);
+            } else {
 #pragma unroll
-                    for (int k = 0; k < 32; ++k) v[k] = 0u;
-                }
+                for (int k = 0; k < 32; ++k) v[k] = 0u;
+            }
 #pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    st_cluster_v4(dst + (uint32_t)((ch * 8 + k) * 2048), v[4 * k], v[4 * k + 1], v[4 * k + 2],
-                                  v[4 * k + 3]);
+            for (int k = 0; k < 8; ++k)
+                st_cluster_v4(dst + (uint32_t)((ch * 8 + k) * 2048), v[4 * k], v[4 * k + 1], v[4 * k + 2],
+                              v[4 * k + 3]);
+        }
+#pragma unroll
+        for (int ch = 0; ch < NCH; ++ch) {
+            if (nkb > 0 && finishes) {
+                tmem_ld_32x32b_x32(taddr + (uint32_t)(split * W + half * CW + ch * 32), own[ch]);
+                tmem_ld_wait_regs(own[ch]);
+            } else {
+#pragma unroll
+                for (int k = 0; k < 32; ++k) own[ch][k] = 0u;
             }
         }
+        tc_fence_before();
     }
     __syncwarp();
-    cluster_sync_all();  // the parts have arrived
+    cluster_sync_all();  // the parts have arrived, and every accumulator has been read
+    if (warp == C::MMA_WARP) {
+        tc_fence_after();
+        tmem_dealloc_cg<2>(tmem, BN);
+    }
 
-    if (warp < 4) {
+    if (warp < C::EPI) {
         // ------------------------------------------------------------------ epilogue of this CTA's columns
-        float* st_tile = reinterpret_cast<float*>(sgen + C::RING) + warp * 32 * 33;
-        float* sums = reinterpret_cast<float*>(sgen + C::RING + S::EPI_TILE);
+        float* sums = reinterpret_cast<float*>(sgen + C::RING);
         const bool want_stats = p.mode == kFwd && p.stats != nullptr;
         const int64_t m = ((int64_t)tc.m_tile * 2 + rank) * 128 + row;
         const bool valid = m < p.M;
@@ -1003,50 +996,41 @@ __global__ void __launch_bounds__(Cfg<256, kFamFwd, 2>::THREADS, 1)
             const int i = (int)(rem / p.gQ), j = (int)(rem - (int64_t)(rem / p.gQ) * p.gQ);
             out_row = (n * p.out_h + 2 * i + (tc.z >> 1)) * p.out_w + 2 * j + (tc.z & 1);
         }
-        RowStats<W> rs;
-        rs.zero();
+        if (finishes) {
+            RowStats<CW> rs;
+            rs.zero();
 #pragma unroll
-        for (int ch = 0; ch < W / 32; ++ch) {
-            uint32_t v[32];
-            if (nkb > 0) {
-                tmem_ld_32x32b_x32(taddr + (uint32_t)(split * W + ch * 32), v);
-                tmem_ld_wait_regs(v);
-            } else {
+            for (int ch = 0; ch < NCH; ++ch) {
+                uint32_t(&v)[32] = own[ch];
+                const float4* src = reinterpret_cast<const float4*>(sgen + (half * NCH + ch) * 8 * 2048 + row * 16);
 #pragma unroll
-                for (int k = 0; k < 32; ++k) v[k] = 0u;
+                for (int q = 0; q < SK - 1; ++q)
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const float4 f = src[q * (S::SLOT / 16) + k * 128];
+                        v[4 * k] = __float_as_uint(__uint_as_float(v[4 * k]) + f.x);
+                        v[4 * k + 1] = __float_as_uint(__uint_as_float(v[4 * k + 1]) + f.y);
+                        v[4 * k + 2] = __float_as_uint(__uint_as_float(v[4 * k + 2]) + f.z);
+                        v[4 * k + 3] = __float_as_uint(__uint_as_float(v[4 * k + 3]) + f.w);
+                    }
+                float back[32];
+                store_row_chunk_act(p, v, valid, out_row, tc.n_tile * BN + split * W + half * CW + ch * 32, back);
+                if (want_stats) rs.add(ch, back);
             }
-            const float4* src = reinterpret_cast<const float4*>(sgen + ch * 8 * 2048 + row * 16);
-#pragma unroll
-            for (int q = 0; q < SK - 1; ++q)
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const float4 f = src[q * (S::SLOT / 16) + k * 128];
-                    v[4 * k] = __float_as_uint(__uint_as_float(v[4 * k]) + f.x);
-                    v[4 * k + 1] = __float_as_uint(__uint_as_float(v[4 * k + 1]) + f.y);
-                    v[4 * k + 2] = __float_as_uint(__uint_as_float(v[4 * k + 2]) + f.z);
-                    v[4 * k + 3] = __float_as_uint(__uint_as_float(v[4 * k + 3]) + f.w);
-                }
-            float back[32];
-            store_row_chunk_act(p, v, valid, out_row, tc.n_tile * BN + split * W + ch * 32, back);
-            if (want_stats) rs.add(ch, back, lane);
+            if (want_stats) {
+                float* st_tile = reinterpret_cast<float*>(sgen + (SK - 1) * S::SLOT) + warp * 32 * 33;
+                float* wsum = sums + quarter * 2 * W;
+                for (int c = lane; c < 2 * CW; c += 32) wsum[(c / CW) * W + half * CW + c % CW] = 0.f;
+                __syncwarp();
+                rs.flush(st_tile, wsum, W, half * CW, lane);
+            }
         }
         if (want_stats) {
-            float* wsum = sums + warp * 2 * W;
-            for (int c = lane; c < 2 * W; c += 32) wsum[c] = 0.f;
-            __syncwarp();
-            rs.flush(st_tile, wsum, W, 0, lane);
-            asm volatile("bar.sync 1, 128;" ::: "memory");
+            asm volatile("bar.sync 1, 256;" ::: "memory");
             float* dst = p.stats + (int64_t)(tc.m_tile * 2 + rank) * 2 * p.Ncols + tc.n_tile * BN + split * W;
-            for (int c = threadIdx.x; c < 2 * W; c += 128)
+            for (int c = threadIdx.x; c < 2 * W; c += 256)
                 dst[(c / W) * p.Ncols + c % W] = (sums[c] + sums[2 * W + c]) + (sums[4 * W + c] + sums[6 * W + c]);
         }
-        tc_fence_before();
-    }
-    __syncthreads();
-    cluster_sync_all();  // neither CTA of a pair frees its TMEM while the other may still use it
-    if (warp == C::MMA_WARP) {
-        tc_fence_after();
-        tmem_dealloc_cg<2>(tmem, BN);
     }
 }
 
@@ -1081,7 +1065,7 @@ struct WinCfg {
     static constexpr int B_TILE = BN * 64 * 2;  // one tap x one 64-channel block of weights
     static constexpr int NB = BN == 64 ? 4 : 2;  // accumulator buffers (tiles in flight)
     static constexpr uint32_t TMEM_COLS = NB * kWinACC * BN;
-    static constexpr int EPI = 4;                // epilogue warps
+    static constexpr int EPI = BN == 128 ? 8 : 4;  // epilogue warps
     static constexpr int CW = BN * 4 / EPI;      // columns one epilogue warp drains
     static constexpr int W_STRIP = EPI, W_WEIGHT = EPI + 1, W_MMA = EPI + 2;
     static constexpr int THREADS = 32 * (EPI + 3);
@@ -1193,7 +1177,7 @@ __global__ void __launch_bounds__(WinCfg<BN>::THREADS, 1)
         for (int t = unit0; t < total_units; t += nunits) {
             const int m_tile = t * CG + rank;
             const int L0 = m_tile * p.win_tile;
-            const int g0 = L0 / Wp;
+            const int g0 = L0 / Wp, n0 = g0 / p.win_Hp, hp0 = g0 - n0 * p.win_Hp;
             // rank 1: rows between its strip and rank 0's, so that both tiles sit at rank 0's offsets
             const int shift = (CG == 2 && rank == 1) ? ((L0 - p.win_tile) % Wp) - (L0 % Wp) : 0;
             for (int cb = 0; cb < CB; ++cb, ++it) {
@@ -1207,12 +1191,15 @@ __global__ void __launch_bounds__(WinCfg<BN>::THREADS, 1)
                 uint32_t fb = smem_u32(&sfull[s]);
                 if (CG == 1 || rank == 0) mbar_arrive_expect_tx_elect(&sfull[s], (uint32_t)CG * strip_tx);
                 if (CG == 2) fb = mapa_shared(fb, 0);
+                int n = n0, hp = hp0;
                 for (int r = 0; r < p.win_srows; ++r) {
-                    const int g = g0 + r;
-                    const int n = g / p.win_Hp, hp = g - n * p.win_Hp;
                     // padded row hp of image n = input row hp - ph from column -pw (padding rows and
                     // columns, and images past the batch, are outside the tensor and arrive as zeros)
                     tma_load_4d_cg<CG>(dst + r * Wp * 128, &tmA, fb, cb * 64, -p.win_pw, hp - p.win_ph, n);
+                    if (++hp == p.win_Hp) {
+                        hp = 0;
+                        ++n;
+                    }
                 }
             }
             if (failed) break;
@@ -1346,7 +1333,7 @@ __global__ void __launch_bounds__(WinCfg<BN>::THREADS, 1)
         const int quarter = warp & 3, col0 = (warp >> 2) * CW;  // TMEM lanes 32*quarter.., columns col0..
         float* st_tile = epi_tile + warp * 32 * 33;
         float* wsum = epi_sum + warp * 2 * p.Ncols;
-        TileStats<CW> rs;
+        TileStats<BN> rs;
         rs.zero();
         const int img = p.win_Hp * Wp;
         int lt = 0;
@@ -1387,7 +1374,7 @@ __global__ void __launch_bounds__(WinCfg<BN>::THREADS, 1)
                 if (c + 1 < NC)
                     tmem_ld_32x32b_x32(taddr + (uint32_t)(((c + 1) / NCH) * BN + ((c + 1) % NCH) * 32), nxt);
                 float back[32];
-                if constexpr (CW > 64) {
+                if constexpr (BN > 64) {
                     uint32_t lo[16], hi[16];
                     if (want_stats) {
                         const uint32_t ta = taddr + (uint32_t)(a * BN + ch * 32);
@@ -1403,7 +1390,7 @@ __global__ void __launch_bounds__(WinCfg<BN>::THREADS, 1)
                     }
                 } else {
                     store_row_chunk_act(p, cur, valid[a], out_row[a], col0 + ch * 32, back);
-                    if (want_stats) rs.add(ch, back, lane);
+                    if (want_stats) rs.add(ch, back);
                 }
             }
             tc_fence_before();
@@ -1416,7 +1403,7 @@ __global__ void __launch_bounds__(WinCfg<BN>::THREADS, 1)
             }
         }
         if (want_stats) {
-            if constexpr (CW > 64)
+            if constexpr (BN > 64)
                 rs.flush(wsum, p.Ncols, col0, lane);  // the window kernel has one column tile
             else
                 rs.flush(st_tile, wsum, p.Ncols, col0, lane);
