@@ -86,7 +86,9 @@ struct ConvParams {
     int win_margin;           // CTA pairs: bytes before and after each strip buffer (0 for single CTAs);
                               // row-block weight gradient: offset of the dy strip in a stage
     int win_stages;           // row-block weight gradient: x + dy stages
-    int win_bpi;              // row-block weight gradient: K-blocks per image
+    int win_bpi;              // row-block and filter-row weight gradient: K-blocks per image
+    int win_ni;               // filter-row weight gradient: images per K-block
+    int win_cl;               // filter-row weight gradient: CTAs per cluster, which add their sums on chip
     int test_stall;           // dbl_conv_test_stall_next: block 0 never loads its first K-block
 };
 
@@ -1737,7 +1739,7 @@ __global__ void __launch_bounds__(kWinThreads, 1)
         failed = __any_sync(0xffffffffu, ok == 0u);
         for (int kb = kb0; kb < kb1 && !failed; ++kb) {
             tc_fence_after();
-            const uint32_t xa = (sbase + (uint32_t)(s * stage_bytes)) >> 4, ya = xa + ((uint32_t)xalign >> 4);
+            const uint32_t xa = ((sbase + (uint32_t)(s * stage_bytes)) >> 4) & 0x3FFFu, ya = xa + ((uint32_t)xalign >> 4);
             auto step = [&](int j, uint32_t acc) {
                 const uint32_t xj = xa + (uint32_t)(j * 128), yj = ya + (uint32_t)(j * 128);  // 16 rows of 128 bytes
                 mma_act_elect(tmem, dA0 + xj, dB0 + yj, idesc0, acc);
@@ -1800,6 +1802,227 @@ __global__ void __launch_bounds__(kWinThreads, 1)
     tc_fence_before();
     __syncthreads();
     if (warp == 6) {
+        tc_fence_after();
+        tmem_dealloc(tmem, 512);
+    }
+}
+
+// ----------------------------------------------------------------------------- filter-row weight gradient
+// dW[k][r][s][c] of a 3x3 stride-1 layer whose channels come in 128s.  A CTA owns one filter row r,
+// 128 input channels and 128 output channels (384 accumulator columns of 128 rows), and one range of
+// K-blocks.  A K-block is R whole output rows of one image, or all rows of several small images, at
+// a pitch of Wp = W + 2*pw positions: the x rows that filter row r reads (from column -pw) and the dy
+// rows from column -2, each as two 64-channel strips.  As in conv_wgrow_kernel a column tap is a shift
+// of dy by one 128-byte row, so that one MN-major B operand of three overlapping atoms holds the three
+// column taps:
+//     accumulator h, 128 x 192: A = x rows L (two 64-channel strips), B = dy strip h, rows {L, L + 1, L + 2}: s = 2..0
+// Two N = 192 MMAs per 16 positions (192 tensor cycles) read 16 x 512 bytes that TMA loaded once, 43
+// bytes per cycle, where the implicit GEMM loads x once per tap (96 bytes per cycle at 128 columns).
+// The positions of a block are rounded up to 16: the rows behind the strips are zeros written once.
+// Every CTA ends with 196 KB of partial sums.  A cluster of CL CTAs (win_cl; the same outputs, CL
+// consecutive K ranges) adds them before they leave the SMs: when all MMAs of the cluster are done, each
+// CTA sends the 32-column chunks it does not own into the strip buffers of their owner (distributed
+// shared memory, as in conv_splitk_kernel), and adds what it received in rank order.
+constexpr int kWgTapMaxStages = 4;
+constexpr int kWgTapThreads = 32 * 11;  // 8 epilogue warps, 2 producers, MMA
+
+__global__ void __launch_bounds__(kWgTapThreads, 1)
+    conv_wgtap_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmDY,
+                      const ConvParams p)
+{
+    dbl::dev::grid_dependency_trigger();  // a convolution launched next may start its set-up
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t full_bar[kWgTapMaxStages], empty_bar[kWgTapMaxStages], accf_bar, drain_bar;
+    __shared__ uint32_t tmem_slot;
+    __shared__ volatile int abort_flag;
+
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    uint8_t* sgen = smem_raw + (sbase - smem_u32(smem_raw));
+    const int strip = p.win_strip_bytes;  // one 64-channel strip; a stage holds x0, x1, dy0, dy1
+    const int loaded = p.win_dyrows * 128;  // bytes TMA writes of it
+    const int stages = p.win_stages;
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < stages; ++i) {
+            mbar_init(&full_bar[i], 2);  // one expect_tx arrival per producer warp
+            mbar_init(&empty_bar[i], 1);
+        }
+        mbar_init(&accf_bar, 1);
+        mbar_init(&drain_bar, 1);
+        abort_flag = 0;
+        fence_mbar_init();
+    }
+    // the zero rows behind each strip, before any MMA reads them
+    const int tail = (strip - loaded) / 16;
+    for (int i = threadIdx.x; i < stages * 4 * tail; i += blockDim.x)
+        *reinterpret_cast<uint4*>(sgen + (i / tail) * strip + loaded + i % tail * 16) = make_uint4(0, 0, 0, 0);
+    fence_async_shared();
+    if ((warp == 8 || warp == 9) && lane == 0) tma_prefetch_desc(warp == 8 ? &tmX : &tmDY);
+    if (warp == 10) {
+        tmem_alloc(&tmem_slot, 512);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    grid_dependency_wait();  // the set-up above may overlap the previous kernel; memory only after it
+    const uint32_t tmem = tmem_slot;
+    // this CTA's outputs and K-blocks (possibly none): the clusters of one slice are adjacent
+    const int groups = p.m_tiles * p.n_tiles;  // 3 filter rows x 128-channel blocks of x, 128-channel blocks of dy
+    const int CL = p.win_cl, rank = CL > 1 ? (int)cluster_ctarank() : 0;
+    const int cluster = blockIdx.x / CL, slice = cluster / groups, gi = cluster - slice * groups;
+    const int z = slice * CL + rank;
+    const int r = gi % 3, c0 = gi / 3 % (p.m_tiles / 3) * 128, n0 = gi / p.m_tiles * 128;
+    const int kb0 = z * p.kb_per_split, kb1 = min(p.num_kb, kb0 + p.kb_per_split);
+
+    if (warp == 8 || warp == 9) {
+        // ------------------------------------------------------------------ producers: x strips (8), dy strips (9)
+        const bool is_x = warp == 8;
+        int s = 0, it = 0;
+        uint32_t phase = 1;
+        bool failed = false;
+        for (int kb = kb0; kb < kb1; ++kb, ++it) {
+            const uint32_t ok = mbar_wait_warp(&empty_bar[s], phase, &abort_flag);
+            if (__any_sync(0xffffffffu, ok == 0u)) {
+                failed = true;
+                break;
+            }
+            uint8_t* dst = sgen + (4 * s + (is_x ? 0 : 2)) * strip;
+            const int i = kb / p.win_bpi, h0 = (kb - i * p.win_bpi) * p.win_srows, img = i * p.win_ni;
+            mbar_arrive_expect_tx_elect(&full_bar[s], (uint32_t)(2 * loaded));
+            for (int h = 0; h < 2; ++h) {
+                if (is_x)
+                    tma_load_4d_elect(dst + h * strip, &tmX, &full_bar[s], c0 + 64 * h, -p.win_pw, h0 + r - p.win_ph, img);
+                else
+                    tma_load_4d_elect(dst + h * strip, &tmDY, &full_bar[s], n0 + 64 * h, -2, h0, img);
+            }
+            if (++s == stages) {
+                s = 0;
+                phase ^= 1;
+            }
+        }
+        if (failed) {
+            if (lane == 0) report_timeout(&abort_flag);
+            for (int i = it - 1; i >= 0 && i >= it - stages; --i)
+                (void)mbar_drain_warp(&full_bar[i % stages], (i / stages) & 1);
+        }
+    } else if (warp == 10) {
+        // ------------------------------------------------------------------ MMA issuer
+        const uint32_t idesc = idesc_act(BM, 192, 1u, 1u);
+        const uint64_t dA = smem_desc(0, (uint32_t)strip, 1024, kSwizzle128B);
+        const uint64_t dB = smem_desc(0, 128, 1024, kSwizzle128B);
+        const uint32_t strip16 = (uint32_t)strip >> 4;
+        const int ksteps = p.win_tile / 16;
+        int s = 0;
+        uint32_t phase = 0;
+        bool failed = false;
+        if (kb0 < kb1) {
+            const uint32_t ok = mbar_wait_warp(&full_bar[0], 0, &abort_flag);
+            failed = __any_sync(0xffffffffu, ok == 0u);
+        }
+        for (int kb = kb0; kb < kb1 && !failed; ++kb) {
+            tc_fence_after();
+            // descriptor addresses are 14 bits: in a cluster the upper bits of sbase hold the CTA's rank
+            const uint32_t xa = ((sbase + (uint32_t)(4 * s * strip)) >> 4) & 0x3FFFu, ya = xa + 2 * strip16;
+            auto step = [&](int j, uint32_t acc) {
+                const uint32_t xj = xa + (uint32_t)(j * 128), yj = ya + (uint32_t)(j * 128);  // 16 rows of 128 bytes
+                mma_act_elect(tmem, dA + xj, dB + yj, idesc, acc);
+                mma_act_elect(tmem + 192, dA + xj, dB + (yj + strip16), idesc, acc);
+            };
+            if (ksteps > 1) step(0, kb > kb0 ? 1u : 0u);
+#pragma unroll 4
+            for (int j = 1; j < ksteps - 1; ++j) step(j, 1u);
+            const int sc = s;
+            if (++s == stages) {
+                s = 0;
+                phase ^= 1;
+            }
+            // the next stage's wait while the tensor pipe still has work queued
+            if (kb + 1 < kb1) {
+                const uint32_t okn = mbar_wait_warp(&full_bar[s], phase, &abort_flag);
+                failed = __any_sync(0xffffffffu, okn == 0u);
+            }
+            step(ksteps - 1, (kb > kb0 || ksteps > 1) ? 1u : 0u);
+            mma_commit_elect(&empty_bar[sc]);
+        }
+        mma_commit_elect(&accf_bar);  // arrives when this slice's MMAs have completed
+        if (failed && lane == 0) report_timeout(&abort_flag);
+        mma_commit_elect(&drain_bar);
+        (void)mbar_drain_warp(&drain_bar, 0);
+    } else {
+        const uint32_t ok = mbar_wait_warp(&accf_bar, 0, &abort_flag);
+        if (__any_sync(0xffffffffu, ok == 0u) && lane == 0) report_timeout(&abort_flag);
+        tc_fence_after();
+    }
+    // ---------------------------------------------------------------------- epilogue (warps 0-7)
+    // chunk e of 32 accumulator columns: accumulator e / 6, atom e % 6 / 2 (column tap 2 - e % 6 / 2);
+    // rank q of the cluster owns chunks q * 12 / CL .., warps of one lane quarter take alternate chunks
+    const int quarter = warp & 3, half = warp >> 2, own = 12 / CL;
+    const int row = quarter * 32 + lane;
+    const bool have_acc = kb0 < kb1;
+    auto load_chunk = [&](int e, uint32_t(&v)[32]) {
+        if (have_acc) {
+            tmem_ld_32x32b_x32(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(e * 32), v);
+            tmem_ld_wait_regs(v);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 32; ++k) v[k] = 0u;
+        }
+    };
+    const int part = own * 128 * 32 * 4;  // bytes one CTA sends to another: [chunk][8 x float4][128 rows]
+    if (CL > 1) {
+        __syncwarp();
+        cluster_sync_all();  // every CTA's MMAs are done: the strips may be overwritten
+        if (warp < 8) {
+#pragma unroll 1
+            for (int i = half; i < 12 - own; i += 2) {
+                const int e = (rank * own + own + i) % 12, to = e / own;
+                const int slot = rank < to ? rank : rank - 1;
+                const uint32_t dst = mapa_shared(sbase, (uint32_t)to) + (uint32_t)(slot * part + (e - to * own) * 16384 + row * 16);
+                uint32_t v[32];
+                load_chunk(e, v);
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    st_cluster_v4(dst + (uint32_t)(k * 2048), v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+            }
+        }
+        __syncwarp();
+        cluster_sync_all();  // the parts have arrived
+    }
+    if (warp < 8) {
+        float* out = static_cast<float*>(p.out) + (int64_t)slice * p.Ncols * p.M;
+#pragma unroll 1
+        for (int i = half; i < own; i += 2) {
+            const int e = rank * own + i;
+            uint32_t v[32];
+            load_chunk(e, v);
+            const float4* src = reinterpret_cast<const float4*>(sgen + i * 16384 + row * 16);
+            for (int q = 0; q < CL - 1; ++q)
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const float4 f = src[q * (part / 16) + k * 128];
+                    v[4 * k] = __float_as_uint(__uint_as_float(v[4 * k]) + f.x);
+                    v[4 * k + 1] = __float_as_uint(__uint_as_float(v[4 * k + 1]) + f.y);
+                    v[4 * k + 2] = __float_as_uint(__uint_as_float(v[4 * k + 2]) + f.z);
+                    v[4 * k + 3] = __float_as_uint(__uint_as_float(v[4 * k + 3]) + f.w);
+                }
+            // [slice][k][m]: consecutive lanes hold consecutive m, one 128-byte line per store
+            const int m = (r * 3 + 2 - e % 6 / 2) * p.Cin + c0 + row;
+            float* o = out + (int64_t)(n0 + e / 6 * 64 + e % 2 * 32) * p.M + m;
+            if (p.zdim == 1 && p.wg_accumulate) {
+#pragma unroll
+                for (int k = 0; k < 32; ++k) o[(int64_t)k * p.M] += __uint_as_float(v[k]);
+            } else {
+#pragma unroll
+                for (int k = 0; k < 32; ++k) o[(int64_t)k * p.M] = __uint_as_float(v[k]);
+            }
+        }
+        tc_fence_before();
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 10) {
         tc_fence_after();
         tmem_dealloc(tmem, 512);
     }
@@ -1896,6 +2119,7 @@ struct Plan {
     bool win = false;    // conv_win_kernel (3x3 stride-1 correlation over padded strips)
     bool res = false;    // window kernel with all weights resident in shared memory
     bool wgrow = false;  // conv_wgrow_kernel (3x3 stride-1 weight gradient, 64 channels)
+    bool wgtap = false;  // conv_wgtap_kernel (3x3 stride-1 weight gradient, multiples of 128 channels)
     size_t smem = 0;     // window kernel dynamic shared memory
 };
 
@@ -2124,6 +2348,88 @@ bool wgrow_setup(const dbl_conv_shape* s, Plan& pl)
     return true;
 }
 
+// Filter-row weight-gradient eligibility and geometry (see conv_wgtap_kernel): 3x3 filters at stride 1,
+// input and output channels in 128s.  The K-block (rows of an image, or whole images) and the number of
+// K ranges, and the CTAs per cluster, minimise the modelled time of the busiest CTA on a 152-SM GPU, in
+// tensor cycles: 192 per 16 positions and ~150 of hand-over per K-block, ~4000 of set-up and ~3000 of
+// stores per CTA, ~9000 for sending all partial sums to other SMs (22 bytes per cycle), and the launch
+// and the traffic of the fixed-order reduce of the slices.
+bool wgtap_setup(const dbl_conv_shape* s, Plan& pl)
+{
+    const Geom g = geom(s);
+    if (g.sh != 1 || g.sw != 1 || s->r != 3 || s->s != 3 || s->c % 128 || s->k % 128) return false;
+    const int Wp = s->w + 2 * g.pw, P = s->h + 2 * g.ph - 2;
+    if (P <= 0 || Wp <= 2 || Wp > 256) return false;
+    // CTAs that 152 SMs hold in clusters of 1..4: fixed counts, the split must not depend on the device
+    static const int resident[5] = {0, 152, 152, 108, 144};
+    constexpr double kExchange = 9000.0, kReduce = 4000.0, kReduceSlice = 0.0030;
+    constexpr int kMaxPos = 208;
+    const int groups = 3 * (s->c / 128) * (s->k / 128);
+    const int64_t elems = (int64_t)9 * s->c * s->k;
+    double best = 1e300;
+    ConvParams& p = pl.p;
+    for (int u = 1; u <= kMaxPos; ++u) {  // u rows of an image, then u - P + 1 images
+        const int R = std::min(u, P), ni = std::max(1, u - P + 1);
+        const int pos = ni * R * Wp;
+        if (pos > kMaxPos || ni > 256) break;
+        const int ksteps = (pos + 15) / 16;
+        const int strip = ((ksteps * 16 + 2) * 128 + 1023) / 1024 * 1024;
+        const int stages = std::min<int>(kWgTapMaxStages, (int)((kWinSmemMax - 1024) / (4 * strip)));
+        if (stages < 2) break;
+        const int64_t blocks = ni > 1 ? (s->n + ni - 1) / ni : (int64_t)s->n * ((P + R - 1) / R);
+        if (blocks > INT32_MAX / 4) continue;
+        for (int cl = 1; cl <= 4; ++cl)
+            for (int slices = 1; slices == 1 || groups * slices * cl <= resident[cl]; ++slices) {
+                const int sp = slices * cl;
+                const int64_t kbs = (blocks + sp - 1) / sp;
+                if ((slices - 1) * cl * kbs >= blocks) break;  // a cluster without a K-block
+                if (cl > 1 && (size_t)stages * 4 * strip < (size_t)(cl - 1) * (12 / cl) * 16384) break;
+                const int rounds = (groups * sp + resident[cl] - 1) / resident[cl];
+                const double cost = rounds * (kbs * (ksteps * 192.0 + 150.0) + 4000.0 + 3000.0 / cl +
+                                              (cl > 1 ? 2000.0 + kExchange * (cl - 1) / cl : 0.0)) +
+                                    (slices > 1 ? kReduce + kReduceSlice * elems * slices : 0.0);
+                if (cost >= best) continue;
+                best = cost;
+                p.win_Wp = Wp;
+                p.win_srows = R;
+                p.win_ni = ni;
+                p.win_bpi = ni > 1 ? 1 : (P + R - 1) / R;
+                p.win_dyrows = pos;
+                p.win_tile = ksteps * 16;
+                p.win_strip_bytes = strip;
+                p.win_stages = stages;
+                p.win_cl = cl;
+                p.num_kb = (int)blocks;
+                p.kb_per_split = (int)kbs;
+                p.zdim = slices;
+                pl.smem = (size_t)stages * 4 * strip + 1024;
+            }
+    }
+    if (best == 1e300) return false;
+    // Against the implicit GEMM (kernel and reduce, us): 28x28x128, batch 512 120 -> 81 and 128 39.0 -> 33.4;
+    // 14x14x256, batch 512 91.3 -> 77.0 and 128 30.9 -> 30.4; 12x12x128, batch 512 32.0 -> 30.9.  It stays
+    // the better one where the padding of a block's positions costs more than a fifth of them (10x10x256,
+    // batch 128 21.4 -> 23.6), where a CTA's K range is shorter than ~22,000 tensor cycles (12x12x128, batch
+    // 128 16.7 -> 18.0) and for 512 x 512 channels, whose 48 tiles leave three ranges (7x7, batch 512, three
+    // slices without clusters 91.6 -> 94.6).
+    const double used = (double)s->n * P * (Wp - 2) / ((double)p.num_kb * p.win_tile);
+    if (groups > 12 || used < 0.8 || (double)p.kb_per_split * p.win_tile * 12 < 22000.0) return false;
+    pl.win = pl.wgtap = true;
+    pl.BN = 128;
+    pl.mode = p.mode = kWgrad;
+    p.win_R = p.win_S = 3;
+    p.win_ph = g.ph;
+    p.win_pw = g.pw;
+    p.M = 9 * s->c;
+    p.Ncols = s->k;
+    p.Cin = s->c;
+    p.m_tiles = 3 * (s->c / 128);
+    p.n_tiles = s->k / 128;
+    p.gN = s->n;
+    pl.ws_main = p.zdim > 1 ? (size_t)p.zdim * p.M * s->k * sizeof(float) : 0;
+    return true;
+}
+
 // Window weight-gradient eligibility and geometry (see conv_wgwin_kernel):
 // stride 1, 64 input and 64 output channels, three or four taps (the stems), padded
 // rows of 10..256 positions.
@@ -2260,8 +2566,8 @@ int make_plan(const dbl_conv_shape* s, int pass, Plan& pl)
         pl.ws_main = (size_t)kMaxGrid * 2 * s->k * sizeof(float);
     } else if (pass == DBL_PASS_DGRAD && s->c % 64 == 0 && win_setup(s, s->k, s->c, true, pl)) {
         pl.mode = p.mode = kDgrad;
-    } else if (pass == DBL_PASS_WGRAD && (wgrow_setup(s, pl) || wgwin_setup(s, pl))) {
-        // conv_wgrow_kernel, conv_wgwin_kernel: tiles are the split-K ranges
+    } else if (pass == DBL_PASS_WGRAD && (wgrow_setup(s, pl) || wgtap_setup(s, pl) || wgwin_setup(s, pl))) {
+        // conv_wgrow_kernel, conv_wgtap_kernel, conv_wgwin_kernel
     } else if (pass == DBL_PASS_FWD) {
         pl.mode = p.mode = c8 ? kFwdC8 : kFwd;
         if (c8 && p.ntaps > 56) return set_error(DBL_ERR_UNSUPPORTED, "conv_fwd: stem filter too large");
@@ -2720,9 +3026,15 @@ int launch_win(const Plan& pl, const CUtensorMap& a, const CUtensorMap& b, int g
               : launch_win_cfg<64, false, false, 1>(pl, a, b, grid, st);
 }
 
-// KERNEL: conv_wgwin_kernel<NACC> or conv_wgrow_kernel (one CTA per split-K range).
+int wgwin_grid(const Plan& pl)
+{
+    return pl.wgtap ? pl.p.m_tiles * pl.p.n_tiles * pl.p.zdim * pl.p.win_cl : grid_size(pl.p.zdim);
+}
+
+// KERNEL: conv_wgwin_kernel<NACC> or conv_wgrow_kernel (one CTA per split-K range), or
+// conv_wgtap_kernel (a CTA per split-K range of each of its tiles).
 template <auto KERNEL>
-int launch_wgwin(const Plan& pl, const CUtensorMap& a, const CUtensorMap& b, cudaStream_t st)
+int launch_wgwin(const Plan& pl, const CUtensorMap& a, const CUtensorMap& b, int threads, cudaStream_t st)
 {
     static bool attr_set[64] = {false};
     int dev = 0;
@@ -2734,12 +3046,12 @@ int launch_wgwin(const Plan& pl, const CUtensorMap& a, const CUtensorMap& b, cud
     }
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[2];
-    cfg.gridDim = dim3(grid_size(pl.p.zdim));
-    cfg.blockDim = dim3(kWinThreads);
+    cfg.gridDim = dim3(wgwin_grid(pl));
+    cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = pl.smem;
     cfg.stream = st;
     cfg.attrs = at;
-    cfg.numAttrs = conv_attrs(1, at);
+    cfg.numAttrs = conv_attrs(pl.wgtap ? pl.p.win_cl : 1, at);
     cudaError_t e = cudaLaunchKernelEx(&cfg, KERNEL, a, b, pl.p);
     if (e != cudaSuccess) {
         dbl::count_launch();
@@ -2749,12 +3061,12 @@ int launch_wgwin(const Plan& pl, const CUtensorMap& a, const CUtensorMap& b, cud
 }
 
 // Tensor map of the window kernel's strip operand: one padded row (Wp pixels
-// x 64 channels, starting at w = -1) of an NHWC tensor per copy, or `rows` of them.
-int enc_win_rows(CUtensorMap* m, const void* base, int N, int H, int W, int C, int Wp, int rows = 1)
+// x 64 channels, starting at w = -1) of an NHWC tensor per copy, or `rows` of them of each of `images`.
+int enc_win_rows(CUtensorMap* m, const void* base, int N, int H, int W, int C, int Wp, int rows = 1, int images = 1)
 {
     cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)N};
     cuuint64_t str[3] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2, (cuuint64_t)H * W * C * 2};
-    cuuint32_t box[4] = {64, (cuuint32_t)Wp, (cuuint32_t)rows, 1};
+    cuuint32_t box[4] = {64, (cuuint32_t)Wp, (cuuint32_t)rows, (cuuint32_t)images};
     return enc_tiled(m, base, 4, dims, str, box, true);
 }
 
@@ -2898,11 +3210,11 @@ int dbl_conv_plan(const dbl_conv_shape* s, int pass, dbl_conv_plan_info* info)
     if (rc) return rc;
     const bool wgwin = pl.win && pass == DBL_PASS_WGRAD;
     info->kernel = wgwin ? DBL_KERNEL_WINDOW_WGRAD : pl.win ? DBL_KERNEL_WINDOW : DBL_KERNEL_IGEMM;
-    info->tile_cols = wgwin ? s->k : pl.BN;
+    info->tile_cols = wgwin && !pl.wgtap ? s->k : pl.BN;
     info->ctas_per_mma = pl.cg;
     info->tiles = pl.p.total_tiles;
     info->zdim = pl.p.zdim;
-    info->grid = wgwin ? grid_size(pl.p.zdim) : plan_grid(pl);
+    info->grid = wgwin ? wgwin_grid(pl) : plan_grid(pl);
     info->smem_bytes = pl.win ? (int64_t)pl.smem : 0;
     return DBL_OK;
 }
@@ -2970,13 +3282,16 @@ int dbl_conv_wgrad(const dbl_conv_shape* s, const void* x, const void* dy, float
     cudaStream_t st = as_stream(stream);
     const bool sliced = pl.p.zdim > 1;
     if (pl.win) {
-        const int xr = pl.wgrow ? pl.p.win_srows : 1, yr = pl.wgrow ? pl.p.win_dyrows : 1;  // rows per copy
-        if ((rc = enc_win_rows(&ta, x, s->n, s->h, s->w, s->c, pl.p.win_Wp, xr))) return rc;
-        if ((rc = enc_win_rows(&tb, dy, s->n, P, Q, s->k, pl.p.win_Wp, yr))) return rc;
+        // rows (and images) per copy
+        const int xr = pl.wgrow || pl.wgtap ? pl.p.win_srows : 1;
+        const int yr = pl.wgrow ? pl.p.win_dyrows : xr, ni = pl.wgtap ? pl.p.win_ni : 1;
+        if ((rc = enc_win_rows(&ta, x, s->n, s->h, s->w, s->c, pl.p.win_Wp, xr, ni))) return rc;
+        if ((rc = enc_win_rows(&tb, dy, s->n, P, Q, s->k, pl.p.win_Wp, yr, ni))) return rc;
         pl.p.out = sliced ? ws : static_cast<void*>(dw);
         pl.p.wg_accumulate = accumulate;
-        if ((rc = pl.wgrow ? launch_wgwin<conv_wgrow_kernel>(pl, ta, tb, st)
-                           : launch_wgwin<conv_wgwin_kernel<2>>(pl, ta, tb, st)))
+        if ((rc = pl.wgrow   ? launch_wgwin<conv_wgrow_kernel>(pl, ta, tb, kWinThreads, st)
+                  : pl.wgtap ? launch_wgwin<conv_wgtap_kernel>(pl, ta, tb, kWgTapThreads, st)
+                             : launch_wgwin<conv_wgwin_kernel<2>>(pl, ta, tb, kWinThreads, st)))
             return rc;
     } else {
     const bool c8 = pl.mode == kWgradC8;

@@ -89,3 +89,38 @@ def test_split_conv_matches_oracle(D, n, h, c, k, r, stride, pad):
         assert np.all(np.isfinite(host(dx)))
         assert max_norm_rel(host(dx), orc.conv2d_dgrad(dy, wt, x.shape, stride, pad)) <= CONV_TOL
     check_status(D)
+
+
+@pytest.mark.parametrize("n,h,w,c,k,pad", [
+    (220, 23, 26, 128, 128, 1),  # a ragged last block of every image
+    (700, 12, 12, 128, 128, 1),  # the twelve rows of one image per block
+    (1500, 8, 14, 128, 128, 0),  # whole small images per block, no padding, the last block past the batch
+    (40, 30, 62, 128, 128, 2),   # padding of two
+    (160, 14, 30, 256, 128, 1),  # two input-channel blocks
+    (160, 14, 30, 128, 256, 1),  # two output-channel blocks
+    (64, 20, 102, 128, 128, 1),  # one wide row per block
+])
+def test_filter_row_wgrad_matches_oracle(D, n, h, w, c, k, pad):
+    g = rng(1000 * n + w)
+    p, q = h + 2 * pad - 2, w + 2 * pad - 2
+    # the oracle's loops are too slow for these sizes: gradients at 24 outputs, the tensor's corners among
+    # them, of which x and dy are nonzero everywhere
+    x = bf16_values(g.standard_normal((n, h, w, c), dtype=np.float32))
+    dy = bf16_values(g.standard_normal((n, p, q, k), dtype=np.float32))
+    at = [(0, 0, 0, 0), (k - 1, 2, 2, c - 1), (0, 2, 0, c - 1), (k - 1, 0, 2, 0)]
+    at += [tuple(int(g.integers(0, m)) for m in (k, 3, 3, c)) for _ in range(20)]
+    ref = np.array([orc.conv2d_wgrad_at(x, dy, (k, 3, 3, c), 1, pad, *i) for i in at])
+    shape = D.conv_shape(n, h, w, c, k, 3, 1, pad)
+    assert D.dbl_conv_plan(shape, D.DBL_PASS_WGRAD).kernel == D.DBL_KERNEL_WINDOW_WGRAD
+    wsb = D.dbl_conv_workspace_bytes(shape, D.DBL_PASS_WGRAD)
+    dw = torch.full((k, 3, 3, c), float("nan"), device="cuda")
+    work, xd, dyd = ws(wsb), to_bf16_dev(x), to_bf16_dev(dy)
+    D.dbl_conv_wgrad(shape, xd, dyd, dw, False, work, wsb)
+    got = host(dw)
+    assert np.all(np.isfinite(got))
+    # each of a CTA's accumulation steps (16 positions; at most ~250 here) may lose 2^-24 of its partial sum
+    # by rounding towards zero, all of them the same way
+    assert np.abs(np.array([got[i] for i in at]) - ref).max() <= 250 * 2.0 ** -24 * np.abs(ref).max()
+    D.dbl_conv_wgrad(shape, xd, dyd, dw, True, work, wsb)
+    assert np.abs(host(dw) - 2 * got).max() <= 2.0 ** -22 * np.abs(got).max()
+    check_status(D)
