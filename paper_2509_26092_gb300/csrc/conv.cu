@@ -2365,6 +2365,7 @@ bool wgtap_setup(const dbl_conv_shape* s, Plan& pl)
     constexpr double kExchange = 9000.0, kReduce = 4000.0, kReduceSlice = 0.0030;
     constexpr int kMaxPos = 208;
     const int groups = 3 * (s->c / 128) * (s->k / 128);
+    if (groups > 12) return false;  // see below
     const int64_t elems = (int64_t)9 * s->c * s->k;
     double best = 1e300;
     ConvParams& p = pl.p;
@@ -2379,10 +2380,13 @@ bool wgtap_setup(const dbl_conv_shape* s, Plan& pl)
         const int64_t blocks = ni > 1 ? (s->n + ni - 1) / ni : (int64_t)s->n * ((P + R - 1) / R);
         if (blocks > INT32_MAX / 4) continue;
         for (int cl = 1; cl <= 4; ++cl)
-            for (int slices = 1; slices == 1 || groups * slices * cl <= resident[cl]; ++slices) {
+            for (int sixth = 6, last = 0; sixth >= 1; --sixth) {  // all the slices that fit, or fewer
+                int slices = std::max(1, resident[cl] / (groups * cl) * sixth / 6);
+                const int64_t kbs = (blocks + slices * cl - 1) / (slices * cl);
+                slices = (int)((blocks + cl * kbs - 1) / (cl * kbs));  // no cluster without a K-block
+                if (slices == last) continue;
+                last = slices;
                 const int sp = slices * cl;
-                const int64_t kbs = (blocks + sp - 1) / sp;
-                if ((slices - 1) * cl * kbs >= blocks) break;  // a cluster without a K-block
                 if (cl > 1 && (size_t)stages * 4 * strip < (size_t)(cl - 1) * (12 / cl) * 16384) break;
                 const int rounds = (groups * sp + resident[cl] - 1) / resident[cl];
                 const double cost = rounds * (kbs * (ksteps * 192.0 + 150.0) + 4000.0 + 3000.0 / cl +
@@ -2413,7 +2417,7 @@ bool wgtap_setup(const dbl_conv_shape* s, Plan& pl)
     // 128 16.7 -> 18.0) and for 512 x 512 channels, whose 48 tiles leave three ranges (7x7, batch 512, three
     // slices without clusters 91.6 -> 94.6).
     const double used = (double)s->n * P * (Wp - 2) / ((double)p.num_kb * p.win_tile);
-    if (groups > 12 || used < 0.8 || (double)p.kb_per_split * p.win_tile * 12 < 22000.0) return false;
+    if (used < 0.8 || (double)p.kb_per_split * p.win_tile * 12 < 22000.0) return false;
     pl.win = pl.wgtap = true;
     pl.BN = 128;
     pl.mode = p.mode = kWgrad;

@@ -188,6 +188,14 @@ class ResNet18Spec:
         e = self.by_name[name]
         return flat[e.offset:e.offset + e.numel].view(e.shape)
 
+    def addresses(self, flat):
+        """name -> device address in a flat buffer: what a call that only needs the pointer takes, without
+        two tensor views per parameter (5 us of host time each; a step passes 172 of them)."""
+        if not flat.is_contiguous() or flat.numel() < self.n_flat:
+            raise ValueError(f"a flat buffer has {self.n_flat} contiguous elements")
+        base, size, table = flat.data_ptr(), flat.element_size(), self.by_name
+        return lambda name: base + table[name].offset * size
+
     def pack(self, tensors, device="cuda", dtype=torch.float32):
         """Flat buffer from {name: array of the logical shape} (stem padding zero)."""
         flat = torch.zeros(self.n_flat, dtype=dtype, device=device)
@@ -421,17 +429,7 @@ class Worker:
         spec, B, eps = self.spec, self.batch, self.eps
         s = stream.cuda_stream if hasattr(stream, "cuda_stream") else stream
         ws, wsb = self.ws, self.ws.numel()
-        W16, W, G = server.w16, server.w, self.grad
-
-        def wv(name):
-            return spec.view(W16, name)
-
-        def pv(name):
-            return spec.view(W, name)
-
-        def gv(name):
-            return spec.view(G, name)
-
+        wv, pv, gv = spec.addresses(server.w16), spec.addresses(server.w), spec.addresses(self.grad)
         st = spec.stem
         self.stem_prepare(images, native_res, s)
         # ---- forward
@@ -529,7 +527,7 @@ class Worker:
         else:
             D.dbl_bn_relu_fused_bwd(bns, dout, dout2, self.stem_y, None, pv("bn1.g"), s_mean, s_istd,
                                     self.stem_dy, None, gv("bn1.g"), gv("bn1.b"), ws, wsb, s, beta=pv("bn1.b"))
-        self.stem_wgrad(self.stem_dy, gv("conv1.w"), ws, wsb, s)
+        self.stem_wgrad(self.stem_dy, spec.view(self.grad, "conv1.w"), ws, wsb, s)
 
 
 def collect_pushes(done, deadline_s, wait, clock=time.monotonic):
