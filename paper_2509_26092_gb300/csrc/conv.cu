@@ -1431,6 +1431,263 @@ __global__ void __launch_bounds__(WinCfg<BN>::THREADS, 1)
     }
 }
 
+// ----------------------------------------------------------------------------- window kernel, pixel pairs
+// 3x3 stride-1 pad-1 correlation of 64 to 64 channels (forward, or the data gradient with the taps
+// flipped) with an even row width.  An accumulator row is a pair of neighbouring pixels (2j, 2j + 1) and
+// its 128 columns are both pixels' 64 outputs, which are contiguous in memory.  The strip holds the
+// even and the odd pixels of a padded row apart (E, O: 64-channel strips of W/2 + 1 entries, the first a
+// zero that also pads the row before), so that the four input pixels a pair's filter row reads are
+//     O[j-1]: w0 to the even output          (N = 64)
+//     E[j]:   w1 to the even, w0 to the odd  (N = 128)
+//     O[j]:   w2 to the even, w1 to the odd  (N = 128)
+//     E[j+1]: w2 to the odd                  (N = 64)
+// With the resident weight tiles of a filter row stored in the order w2, w1, w0 every B operand is one run
+// of them, and in this order every output adds its taps as conv_win_kernel does (the same bits).  256 pixels take 24 MMAs of 64 columns and 24 of 128 instead of 72 of 64, which are bound by
+// their operand reads and issue (54 against ~70 cycles each): forward at 56x56, batch 512 112 -> 91 us,
+// data gradient 110 -> 89; 72x72, batch 185 79 -> 57 and 77 -> 55; 24x24, batch 512 27.9 -> 23.2 and 26.5 -> 21.5;
+// 32x32, batch 64 11.2 -> 10.1 and 10.3 -> 8.8.
+// CG = 2 (forward only, selected by DBL_CONV_CTA_PAIRS=2): two CTAs, each with its own tile, as M = 256 MMAs;
+// each holds half of every B operand, one pixel's tap for N = 128 and 32 outputs for N = 64, and rank 1
+// shifts its strips as in conv_win_kernel.
+// Warp roles as in conv_win_kernel: warps 0-3 drain TMEM, 4 loads strips, 5 the weights, 6 issues MMAs.
+constexpr int kPairNB = 4;  // accumulator buffers of 128 columns
+
+template <bool DG, int CG>
+__global__ void __launch_bounds__(kWinThreads, 1)
+    conv_winpair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                        const __grid_constant__ CUtensorMap tmB32, const ConvParams p)
+{
+    dbl::dev::grid_dependency_trigger();  // a convolution launched next may start its set-up
+    static_assert(CG == 1 || !DG, "a 32-column half of an MN-major operand has no layout");
+    constexpr int BT = 64 * 64 * 2;  // one tap of weights
+    // Resident weights.  CG = 1: tap (r, s) at slot 3r + 2 - s.  CG = 2, per filter row r: this rank's tap of
+    // the two N = 128 operands, then its 32 outputs of w0 and of w2; behind them 32 outputs of (0, w1).
+    constexpr int kWeights = CG == 1 ? 9 * BT : 9 * BT + BT / 2;
+    constexpr uint16_t kAll = CG == 2 ? 3 : 1;
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t sfull[2], sempty[2], wfull, accf_bar[kPairNB], acce_bar[kPairNB], drain_bar;
+    __shared__ uint32_t tmem_slot;
+    __shared__ volatile int abort_flag;
+
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    uint8_t* sgen = smem_raw + (sbase - smem_u32(smem_raw));
+    const int rank = CG == 2 ? (int)cluster_ctarank() : 0;
+    const int unit0 = blockIdx.x / CG, nunits = gridDim.x / CG, total_units = (p.total_tiles + CG - 1) / CG;
+    const int pitch = p.win_Wp, half_bytes = p.win_strip_bytes;  // one parity's strip, with rank 1's shift
+    uint8_t* strip = sgen + (CG == 1 ? kWeights : (kWeights + 1023) / 1024 * 1024);  // stage s, parity e: + (2s + e) * half_bytes
+    float* epi_tile = reinterpret_cast<float*>(strip);  // once the last tile's MMAs are done
+    float* epi_sum = reinterpret_cast<float*>(strip + 4 * half_bytes);
+    // entry of a strip buffer at which rank 0's strip starts: room for rank 1's shift of -(128 % pitch)
+    const int first = CG == 2 ? p.win_margin : 0;
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&sfull[i], 1);
+            mbar_init(&sempty[i], 1);
+        }
+        mbar_init(&wfull, 1);
+        for (int i = 0; i < kPairNB; ++i) {
+            mbar_init(&accf_bar[i], 1);
+            mbar_init(&acce_bar[i], 4 * CG);  // one arrival per epilogue warp
+        }
+        mbar_init(&drain_bar, 1);
+        abort_flag = 0;
+        fence_mbar_init();
+    }
+    const bool want_stats = !DG && p.stats != nullptr;
+    if (want_stats)
+        for (int i = threadIdx.x; i < 4 * 2 * 64; i += blockDim.x) epi_sum[i] = 0.f;
+    if ((warp == 4 || warp == 5) && lane == 0) tma_prefetch_desc(warp == 4 ? &tmA : &tmB);
+    if (warp == 6) {
+        tmem_alloc_cg<CG>(&tmem_slot, kPairNB * 128);
+        tmem_relinquish_cg<CG>();
+    }
+    tc_fence_before();
+    __syncthreads();
+    if constexpr (CG == 2) cluster_sync_all();  // both CTAs' barriers initialised, TMEM allocated
+    tc_fence_after();
+    grid_dependency_wait();  // the set-up above may overlap the previous kernel; memory only after it
+    const uint32_t tmem = tmem_slot;
+
+    if (warp == 4) {
+        // ------------------------------------------------------------------ strip producer
+        int it = 0;
+        bool failed = false;
+        const uint32_t tx = (uint32_t)(2 * p.win_srows * pitch * 128);
+        for (int t = unit0; t < total_units; t += nunits, ++it) {
+            const int s = it & 1;
+            const uint32_t ok = mbar_wait_warp(&sempty[s], ((it >> 1) & 1) ^ 1, &abort_flag);
+            if (__any_sync(0xffffffffu, ok == 0u)) {
+                failed = true;
+                break;
+            }
+            const int L0 = (t * CG + rank) * 128, g0 = L0 / pitch;
+            int n = g0 / p.win_Hp, hp = g0 - n * p.win_Hp;
+            // rank 1: entries between its strip and rank 0's, so that both tiles sit at rank 0's offset
+            const int shift = (CG == 2 && rank == 1) ? (L0 - 128) % pitch - L0 % pitch : 0;
+            uint8_t* dst = strip + 2 * s * half_bytes + (first + shift) * 128;
+            uint32_t fb = smem_u32(&sfull[s]);
+            if (rank == 0) mbar_arrive_expect_tx_elect(&sfull[s], CG * tx);
+            if (CG == 2) fb = mapa_shared(fb, 0);
+            for (int r = 0; r < p.win_srows; ++r) {
+                // padded row hp of image n = row hp - 1 from pair -1 (padding rows, pair -1 and images past the
+                // batch are outside the tensor and arrive as zeros)
+                tma_load_5d_cg<CG>(dst + r * pitch * 128, &tmA, fb, 0, 0, -1, hp - 1, n);
+                tma_load_5d_cg<CG>(dst + half_bytes + r * pitch * 128, &tmA, fb, 0, 1, -1, hp - 1, n);
+                if (++hp == p.win_Hp) {
+                    hp = 0;
+                    ++n;
+                }
+            }
+        }
+        if (failed) {
+            if (lane == 0) report_timeout(&abort_flag);
+            if (rank == 0) {
+                for (int i = it - 1; i >= 0 && i >= it - 2; --i) (void)mbar_drain_warp(&sfull[i & 1], (i >> 1) & 1);
+            } else {
+                // rank 1's copies complete on rank 0's barriers: give them a fixed time instead
+                const uint64_t t0 = globaltimer();
+                while (globaltimer() - t0 < 1000000ull) {
+                }
+            }
+        }
+    } else if (warp == 5) {
+        // ------------------------------------------------------------------ weights
+        uint32_t fb = smem_u32(&wfull);
+        if (rank == 0) mbar_arrive_expect_tx_elect(&wfull, (uint32_t)(CG * kWeights));
+        if (CG == 2) fb = mapa_shared(fb, 0);
+        if constexpr (CG == 1) {
+            for (int tap = 0; tap < 9; ++tap)
+                win_load_wtile<64, DG, 1>(p, &tmB, sgen + (tap / 3 * 3 + 2 - tap % 3) * BT, fb, tap, 0, 0, 0);
+        } else {
+            for (int r = 0; r < 3; ++r) {
+                uint8_t* w = sgen + 3 * r * BT;
+                tma_load_2d_cg<2>(w, &tmB, fb, (3 * r + 1 - rank) * 64, 0);
+                tma_load_2d_cg<2>(w + BT, &tmB, fb, (3 * r + 2 - rank) * 64, 0);
+                tma_load_2d_cg<2>(w + 2 * BT, &tmB32, fb, 3 * r * 64, 32 * rank);
+                tma_load_2d_cg<2>(w + 2 * BT + BT / 2, &tmB32, fb, (3 * r + 2) * 64, 32 * rank);
+            }
+            tma_load_2d_cg<2>(sgen + 9 * BT, &tmB32, fb, 64, 32 * rank);
+        }
+        if (rank == 0) (void)mbar_drain_warp(&wfull, 0);
+    } else if (warp == 6) {
+        // ------------------------------------------------------------------ MMA issuer (rank 0 of a pair)
+        const uint32_t id64 = idesc_act(BM * CG, 64, 0u, DG ? 1u : 0u), id128 = idesc_act(BM * CG, 128, 0u, DG ? 1u : 0u);
+        const uint64_t dB = DG ? smem_desc(sbase, 8192, 1024, kSwizzle128B) : smem_desc(sbase, 16, 1024, kSwizzle128B);
+        constexpr uint64_t kB = DG ? (2048 >> 4) : (32 >> 4);  // a K-step of B
+        // B operands of filter row r: E[j] and O[j] (N = 128), O[j-1] and E[j+1] (N = 64); of the first
+        // K-step of E[j] its two halves
+        constexpr uint64_t kTap = BT >> 4;
+        constexpr uint64_t kE = CG == 1 ? kTap : 0, kO = CG == 1 ? 0 : kTap, kO1 = 2 * kTap,
+                           kE1 = CG == 1 ? 0 : 2 * kTap + kTap / 2, kW1 = CG == 1 ? kTap : 9 * kTap;
+        int it = 0;
+        bool failed = false;
+        if (rank == 0) {
+            const uint32_t ok = mbar_wait_warp(&wfull, 0, &abort_flag);
+            failed = __any_sync(0xffffffffu, ok == 0u);
+        }
+        for (int t = unit0; t < total_units && rank == 0 && !failed; t += nunits, ++it) {
+            const int buf = it % kPairNB, s = it & 1;
+            const uint32_t ok = mbar_wait_warp(&acce_bar[buf], ((it / kPairNB) & 1) ^ 1, &abort_flag);
+            const uint32_t oks = mbar_wait_warp(&sfull[s], (it >> 1) & 1, &abort_flag);
+            if (__any_sync(0xffffffffu, ok == 0u || oks == 0u)) {
+                failed = true;
+                break;
+            }
+            tc_fence_after();
+            const int L0 = t * CG * 128, off = L0 - (L0 / pitch) * pitch;  // the tile's start within the strip's first row
+            const uint32_t d = tmem + (uint32_t)(buf * 128);
+            const uint32_t sa = smem_u32(strip + 2 * s * half_bytes) + (uint32_t)((first + off) * 128);
+            const uint64_t e0 = smem_desc(sa, 16, 1024, kSwizzle128B);
+            const uint64_t o0 = smem_desc(sa + (uint32_t)half_bytes, 16, 1024, kSwizzle128B);
+#pragma unroll
+            for (int r = 0; r < 3; ++r) {
+                const uint64_t row = (uint64_t)(r * pitch * 8);  // 128-byte entries in 16-byte units
+                const uint64_t w = dB + 3 * r * kTap;
+                mma_act_x4_elect_cg<CG>(d, o0 + row, 2, w + kO1, kB, id64, r > 0 ? 1u : 0u);
+                if (r == 0) {  // the odd pixel's first K-step does not accumulate, the even one's does
+                    mma_act_elect_cg<CG>(d, e0 + 8, w + kW1, id64, 1u);
+                    mma_act_elect_cg<CG>(d + 64, e0 + 8, w + kO1, id64, 0u);
+#pragma unroll
+                    for (int k = 1; k < 4; ++k)
+                        mma_act_elect_cg<CG>(d, e0 + (uint64_t)(8 + 2 * k), w + kE + k * kB, id128, 1u);
+                } else {
+                    mma_act_x4_elect_cg<CG>(d, e0 + row + 8, 2, w + kE, kB, id128, 1u);
+                }
+                mma_act_x4_elect_cg<CG>(d, o0 + row + 8, 2, w + kO, kB, id128, 1u);
+                mma_act_x4_elect_cg<CG>(d + 64, e0 + row + 16, 2, w + kE1, kB, id64, 1u);
+            }
+            mma_commit_elect_cg<CG>(&sempty[s], kAll);
+            mma_commit_elect_cg<CG>(&accf_bar[buf], kAll);  // arrives when this unit's MMAs have completed
+        }
+        if (rank == 0) {
+            if (failed && lane == 0) report_timeout(&abort_flag);
+            mma_commit_elect_cg<CG>(&drain_bar, 1);
+            (void)mbar_drain_warp(&drain_bar, 0);
+        }
+    } else {
+        // ------------------------------------------------------------------ epilogue (warps 0-3)
+        float* st_tile = epi_tile + warp * 32 * 33;
+        float* wsum = epi_sum + warp * 2 * 64;
+        RowStats<64> rs;
+        rs.zero();
+        const int img = p.win_Hp * pitch;
+        int it = 0;
+        for (int t = unit0; t < total_units; t += nunits, ++it) {
+            const int buf = it % kPairNB, tile = t * CG + rank;
+            const uint32_t ok = mbar_wait_warp(&accf_bar[buf], (it / kPairNB) & 1, &abort_flag);
+            if (__any_sync(0xffffffffu, ok == 0u)) {
+                if (lane == 0) report_timeout(&abort_flag);
+                break;
+            }
+            tc_fence_after();
+            const int L = tile * 128 + warp * 32 + lane;
+            const int n = L / img, rem = L - n * img;
+            const int hp = rem / pitch, j = rem - hp * pitch;
+            const bool valid = tile < p.total_tiles && n < p.gN && hp < p.win_P && j < pitch - 1;
+            const int64_t out_row = ((int64_t)n * p.win_P + hp) * (pitch - 1) + j;
+            const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(buf * 128);
+            // the next chunk's TMEM load in flight while this one is converted and stored
+            uint32_t va[32], vb[32];
+            tmem_ld_32x32b_x32(taddr, va);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {  // pixel c / 2, channels 32 * (c % 2) ..
+                uint32_t(&cur)[32] = (c & 1) ? vb : va;
+                uint32_t(&nxt)[32] = (c & 1) ? va : vb;
+                tmem_ld_wait_regs(cur);
+                if (c < 3) tmem_ld_32x32b_x32(taddr + (uint32_t)((c + 1) * 32), nxt);
+                float back[32];
+                store_row_chunk_act(p, cur, valid, out_row, c * 32, back);
+                if (want_stats) rs.add(c % 2, back);
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) {
+                if constexpr (CG == 2)
+                    mbar_arrive_cluster(mapa_shared(smem_u32(&acce_bar[buf]), 0));
+                else
+                    mbar_arrive(&acce_bar[buf]);
+            }
+        }
+        if (want_stats) {
+            rs.flush(st_tile, wsum, 64, 0, lane);
+            asm volatile("bar.sync 1, 128;" ::: "memory");
+            float* dst = p.stats + (int64_t)blockIdx.x * 128;
+            const int c = threadIdx.x;
+            dst[c] = (epi_sum[c] + epi_sum[128 + c]) + (epi_sum[256 + c] + epi_sum[384 + c]);
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    // neither CTA of a pair leaves while the other may still signal its barriers or read its TMEM
+    if constexpr (CG == 2) cluster_sync_all();
+    if (warp == 6) {
+        tc_fence_after();
+        tmem_dealloc_cg<CG>(tmem, kPairNB * 128);
+    }
+}
+
 // ----------------------------------------------------------------------------- window weight gradient
 // dW[k][r][s][c] = sum over positions L of dy[L][k] * x_pad[L + r*Wp + s][c] for stride-1
 // layers with 64 input and 64 output channels and at most 10 taps, in the padded position space
@@ -2118,6 +2375,7 @@ struct Plan {
     size_t ws_main = 0;  // bytes: fwd channel-sum partials, or wgrad split-K slices
     bool win = false;    // conv_win_kernel (3x3 stride-1 correlation over padded strips)
     bool res = false;    // window kernel with all weights resident in shared memory
+    bool winpair = false;  // conv_winpair_kernel (64 to 64 channels, even rows)
     bool wgrow = false;  // conv_wgrow_kernel (3x3 stride-1 weight gradient, 64 channels)
     bool wgtap = false;  // conv_wgtap_kernel (3x3 stride-1 weight gradient, multiples of 128 channels)
     size_t smem = 0;     // window kernel dynamic shared memory
@@ -2213,13 +2471,61 @@ constexpr size_t kWinSmemMax = 232448 - 2048;
 // strip row for a misaligned start).
 int win_tile_positions(int Wp) { return Wp >= 64 ? (kWinBMT / Wp) * Wp : kWinBMT; }
 
+bool win_pairs();
+int cta_pair_level();
+
+// Pixel-pair window kernel (conv_winpair_kernel): 3x3, stride 1, pad 1, 64 to 64 channels, even rows whose
+// two stages fit in shared memory beside the weights (W <= 98).  CTA pairs for the forward pass only
+// with DBL_CONV_CTA_PAIRS=2 (56x56, batch 512 114 us against 91: the two CTAs' loads and epilogues wait for each
+// other).
+bool winpair_setup(const dbl_conv_shape* s, bool dgrad, Plan& pl)
+{
+    const Geom g = geom(s);
+    if (g.sh != 1 || g.sw != 1 || s->r != 3 || s->s != 3 || g.ph != 1 || g.pw != 1) return false;
+    if (s->c != 64 || s->k != 64 || (s->w & 1) || s->w < 8) return false;
+    const int pitch = s->w / 2 + 1, Hp = s->h + 2;
+    const int64_t L = (int64_t)s->n * Hp * pitch;
+    if (pitch > 256 || L > INT32_MAX / 8) return false;
+    // entries one tile's 128 accumulator rows read: start offset within a row, plus 127, plus the last tap's
+    const int rows = (pitch - 1 + 127 + 2 * pitch + 2) / pitch + 1;
+    int cg = !dgrad && cta_pair_level() == 2 ? 2 : 1, half = 0;
+    size_t smem = 0;
+    for (;; cg = 1) {
+        half = ((rows + (cg == 2)) * pitch * 128 + 1023) / 1024 * 1024;  // pairs: rank 1's shift, one row in all
+        smem = (cg == 2 ? 77 * 1024 : 72 * 1024) + 4 * (size_t)half + 4 * 2 * 64 * 4 + 1024;
+        if (smem <= kWinSmemMax && 4 * (size_t)half >= 4 * 32 * 33 * 4) break;
+        if (cg == 1) return false;
+    }
+    ConvParams& p = pl.p;
+    pl.win = pl.winpair = pl.res = true;
+    pl.BN = 64;
+    pl.cg = cg;
+    pl.smem = smem;
+    p.win_margin = 128 % pitch;
+    p.win_R = p.win_S = 3;
+    p.win_ph = p.win_pw = 1;
+    p.win_P = s->h;
+    p.win_Q = s->w;
+    p.win_Hp = Hp;
+    p.win_Wp = pitch;
+    p.win_tile = 128;
+    p.win_srows = rows;
+    p.win_strip_bytes = half;
+    p.M = s->n * s->h * s->w;
+    p.m_tiles = (int)((L + 127) / 128);
+    p.n_tiles = 1;
+    p.cblocks = 1;
+    p.gN = s->n;
+    p.Ncols = 64;
+    p.ldo = 128;  // a row of the output is a pair of pixels
+    p.Cin = 64;
+    return true;
+}
+
 // Window-kernel eligibility and geometry (see conv_win_kernel): stride 1 on both
 // axes, 64-channel blocks of the reduced operand (red_c), 64 or 128 output
 // channels, padded rows of 10..256 positions; the data gradient (dgrad) for
 // 3x3 filters with pad 1 only (its taps are the forward taps flipped).
-bool win_pairs();
-int cta_pair_level();
-
 bool win_setup(const dbl_conv_shape* s, int red_c, int out_c, bool dgrad, Plan& pl)
 {
     const Geom g = geom(s);
@@ -2565,10 +2871,10 @@ int make_plan(const dbl_conv_shape* s, int pass, Plan& pl)
     p.S = s->s;
     p.Cin = s->c;
     p.zdim = 1;
-    if (pass == DBL_PASS_FWD && !c8 && win_setup(s, s->c, s->k, false, pl)) {
+    if (pass == DBL_PASS_FWD && !c8 && (winpair_setup(s, false, pl) || win_setup(s, s->c, s->k, false, pl))) {
         pl.mode = p.mode = kFwd;
         pl.ws_main = (size_t)kMaxGrid * 2 * s->k * sizeof(float);
-    } else if (pass == DBL_PASS_DGRAD && s->c % 64 == 0 && win_setup(s, s->k, s->c, true, pl)) {
+    } else if (pass == DBL_PASS_DGRAD && s->c % 64 == 0 && (winpair_setup(s, true, pl) || win_setup(s, s->k, s->c, true, pl))) {
         pl.mode = p.mode = kDgrad;
     } else if (pass == DBL_PASS_WGRAD && (wgrow_setup(s, pl) || wgtap_setup(s, pl) || wgwin_setup(s, pl))) {
         // conv_wgrow_kernel, conv_wgtap_kernel, conv_wgwin_kernel
@@ -3013,9 +3319,44 @@ int launch_win_cfg(const Plan& pl, const CUtensorMap& a, const CUtensorMap& b, i
     return dbl::launch_check("conv_win launch");
 }
 
-int launch_win(const Plan& pl, const CUtensorMap& a, const CUtensorMap& b, int grid, cudaStream_t st)
+template <bool DG, int CG>
+int launch_winpair(const Plan& pl, const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& b32, int grid,
+                   cudaStream_t st)
+{
+    static bool attr_set[64] = {false};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev >= 0 && dev < 64 && !attr_set[dev]) {
+        cudaError_t e = cudaFuncSetAttribute(conv_winpair_kernel<DG, CG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)kWinSmemMax);
+        if (e != cudaSuccess) return dbl::cuda_check(e, "conv: set smem attribute");
+        attr_set[dev] = true;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[2];
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kWinThreads);
+    cfg.dynamicSmemBytes = pl.smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = conv_attrs(CG, at);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, conv_winpair_kernel<DG, CG>, a, b, b32, pl.p);
+    if (e != cudaSuccess) {
+        dbl::count_launch();
+        return dbl::cuda_check(e, "conv_winpair launch");
+    }
+    return dbl::launch_check("conv_winpair launch");
+}
+
+// b32: 32-row boxes of the weights (the pixel-pair kernel's CTA pairs).
+int launch_win(const Plan& pl, const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& b32, int grid,
+               cudaStream_t st)
 {
     const bool dg = pl.mode == kDgrad;
+    if (pl.winpair)
+        return dg           ? launch_winpair<true, 1>(pl, a, b, b32, grid, st)
+               : pl.cg == 2 ? launch_winpair<false, 2>(pl, a, b, b32, grid, st)
+                            : launch_winpair<false, 1>(pl, a, b, b32, grid, st);
     if (pl.cg == 2) {
         if (pl.BN == 128) return dg ? launch_win_cfg<128, true, false, 2>(pl, a, b, grid, st)
                                     : launch_win_cfg<128, false, false, 2>(pl, a, b, grid, st);
@@ -3074,6 +3415,16 @@ int enc_win_rows(CUtensorMap* m, const void* base, int N, int H, int W, int C, i
     return enc_tiled(m, base, 4, dims, str, box, true);
 }
 
+// Tensor map of conv_winpair_kernel's strips: one padded row of one parity per copy, over an NHWC tensor of 64
+// channels viewed as [N][H][W/2][2][64].
+int enc_winpair_rows(CUtensorMap* m, const void* base, int N, int H, int W, int pitch)
+{
+    cuuint64_t dims[5] = {64, 2, (cuuint64_t)W / 2, (cuuint64_t)H, (cuuint64_t)N};
+    cuuint64_t str[4] = {128, 256, (cuuint64_t)W * 128, (cuuint64_t)H * W * 128};
+    cuuint32_t box[5] = {64, 1, (cuuint32_t)pitch, 1, 1};
+    return enc_tiled(m, base, 5, dims, str, box, true);
+}
+
 // Rows of one tile of the forward family (see Cfg).
 int fwd_tile_rows(int BN) { return BN <= 128 ? 256 : 128; }
 
@@ -3094,15 +3445,20 @@ int conv_fwd_impl(const dbl_conv_shape* s, const void* x, const void* w, void* y
     const bool stats = ch_sum != nullptr || nparts != nullptr;
     if (stats && (!ws || ws_bytes < plan_ws(pl)))
         return set_error(DBL_ERR_WORKSPACE, "%s: workspace %zu < %zu bytes", who, ws_bytes, plan_ws(pl));
-    CUtensorMap ta, tb;
+    CUtensorMap ta, tb, tb32;
     const Geom g = geom(s);
     if (pl.win) {
-        if ((rc = enc_win_rows(&ta, x, s->n, s->h, s->w, s->c, pl.p.win_Wp))) return rc;
+        if ((rc = pl.winpair ? enc_winpair_rows(&ta, x, s->n, s->h, s->w, pl.p.win_Wp)
+                             : enc_win_rows(&ta, x, s->n, s->h, s->w, s->c, pl.p.win_Wp)))
+            return rc;
         const int64_t rsc = (int64_t)s->r * s->s * s->c;
         cuuint64_t dims[2] = {(cuuint64_t)rsc, (cuuint64_t)s->k};
         cuuint64_t str[1] = {(cuuint64_t)rsc * 2};
-        cuuint32_t box[2] = {64, (cuuint32_t)(pl.BN / pl.cg)};  // a CTA pair stages half the columns each
+        // a CTA pair stages half the columns each (the pixel-pair kernel: whole taps and half taps)
+        cuuint32_t box[2] = {64, (cuuint32_t)(pl.winpair ? 64 : pl.BN / pl.cg)}, box32[2] = {64, 32};
         if ((rc = enc_tiled(&tb, w, 2, dims, str, box, true))) return rc;
+        tb32 = tb;
+        if (pl.winpair && pl.cg == 2 && (rc = enc_tiled(&tb32, w, 2, dims, str, box32, true))) return rc;
     } else if (pl.mode == kFwdC8) {
         if ((rc = enc_im2col(&ta, x, s->n, s->h, s->w, 8, -g.ph, g.ph - (s->r - 1), -g.pw, g.pw - (s->s - 1), g.sh,
                              g.sw, 8, fwd_tile_rows(pl.BN), false)))
@@ -3128,7 +3484,7 @@ int conv_fwd_impl(const dbl_conv_shape* s, const void* x, const void* w, void* y
     const int grid = plan_grid(pl);
     const int parts = pl.sk > 1 ? 2 * pl.p.m_tiles : grid;  // rows of channel-sum partials
     cudaStream_t st = as_stream(stream);
-    if ((rc = pl.win ? launch_win(pl, ta, tb, grid, st) : launch(pl, ta, tb, ta, tb, grid, st))) return rc;
+    if ((rc = pl.win ? launch_win(pl, ta, tb, tb32, grid, st) : launch(pl, ta, tb, ta, tb, grid, st))) return rc;
     if (nparts) {
         *nparts = parts;
     } else if (stats) {
@@ -3154,7 +3510,9 @@ int conv_dgrad_impl(const dbl_conv_shape* s, const void* dy, const void* w, int 
     const int P = out_dim(s->h, s->r, s->stride, s->pad), Q = out_dim(s->w, s->s, s->stride, s->pad);
     CUtensorMap ta, tb, ta2, tb2;
     if (pl.win) {
-        if ((rc = enc_win_rows(&ta, dy, s->n, P, Q, s->k, pl.p.win_Wp))) return rc;
+        if ((rc = pl.winpair ? enc_winpair_rows(&ta, dy, s->n, P, Q, pl.p.win_Wp)
+                             : enc_win_rows(&ta, dy, s->n, P, Q, s->k, pl.p.win_Wp)))
+            return rc;
     } else {
         // im2col over dy [n, P, Q, k]: origins cover the dx grid (stride 1) or one phase grid (stride 2)
         int lower = 0, upper = 0;
@@ -3190,7 +3548,7 @@ int conv_dgrad_impl(const dbl_conv_shape* s, const void* dy, const void* w, int 
     pl.p.out = dx;
     pl.p.st32 = (reinterpret_cast<uintptr_t>(dx) % 32 == 0) && (pl.p.ldo * (int64_t)sizeof(act_t)) % 32 == 0;
     const int grid = plan_grid(pl);
-    return pl.win ? launch_win(pl, ta, tb, grid, as_stream(stream))
+    return pl.win ? launch_win(pl, ta, tb, tb, grid, as_stream(stream))
                   : launch(pl, ta, tb, ta2, tb2, grid, as_stream(stream));
 }
 

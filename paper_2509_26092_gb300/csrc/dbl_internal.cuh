@@ -571,6 +571,28 @@ __device__ __forceinline__ void tma_load_4d_cg(void* dst, const void* tmap, uint
 }
 
 template <int CG>
+__device__ __forceinline__ void tma_load_5d_cg(void* dst, const void* tmap, uint32_t bar, int32_t c0, int32_t c1,
+                                               int32_t c2, int32_t c3, int32_t c4)
+{
+    if constexpr (CG == 2)
+        asm volatile(
+            "{\n\t.reg .pred E;\n\t.reg .b32 l;\n\t"
+            "elect.sync l|E, 0xffffffff;\n\t"
+            "@E cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+            " [%0], [%1, {%3, %4, %5, %6, %7}], [%2];\n\t}" ::"r"(smem_u32(dst)),
+            "l"(reinterpret_cast<uint64_t>(tmap)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4)
+            : "memory");
+    else
+        asm volatile(
+            "{\n\t.reg .pred E;\n\t.reg .b32 l;\n\t"
+            "elect.sync l|E, 0xffffffff;\n\t"
+            "@E cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+            " [%0], [%1, {%3, %4, %5, %6, %7}], [%2];\n\t}" ::"r"(smem_u32(dst)),
+            "l"(reinterpret_cast<uint64_t>(tmap)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4)
+            : "memory");
+}
+
+template <int CG>
 __device__ __forceinline__ void tma_load_im2col_4d_cg(void* dst, const void* tmap, uint32_t bar, int32_t c, int32_t w,
                                                       int32_t h, int32_t n, uint16_t off_w, uint16_t off_h)
 {
@@ -712,6 +734,44 @@ __device__ __forceinline__ void mma_act_x8_elect_cg(uint32_t d0, uint32_t d1, ui
             : "memory");
     else
         mma_act_x8_elect(d0, d1, a0, a1_off, a_step, b0, b_step, idesc, acc0);
+}
+
+// Four K-steps of one accumulator: A and B descriptors stepped by a_step and b_step; acc0: whether the
+// first accumulates (CG-CTA MMAs as in mma_act_x8_elect_cg).
+template <int CG>
+__device__ __forceinline__ void mma_act_x4_elect_cg(uint32_t d, uint64_t a0, uint64_t a_step, uint64_t b0,
+                                                     uint64_t b_step, uint32_t idesc, uint32_t acc0)
+{
+    if constexpr (CG == 2)
+        asm volatile(
+            "{\n\t.reg .pred E, P, T;\n\t.reg .b32 l;\n\t.reg .b64 a, b;\n\t"
+            "elect.sync l|E, 0xffffffff;\n\t"
+            "setp.ne.b32 P, %6, 0;\n\t"
+            "setp.eq.b32 T, 0, 0;\n\t"
+            "@E tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %3, %5, P;\n\t"
+            "add.s64 a, %1, %2;\n\tadd.s64 b, %3, %4;\n\t"
+            "@E tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %5, T;\n\t"
+            "add.s64 a, a, %2;\n\tadd.s64 b, b, %4;\n\t"
+            "@E tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %5, T;\n\t"
+            "add.s64 a, a, %2;\n\tadd.s64 b, b, %4;\n\t"
+            "@E tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %5, T;\n\t}" ::"r"(d),
+            "l"(a0), "l"(a_step), "l"(b0), "l"(b_step), "r"(idesc), "r"(acc0)
+            : "memory");
+    else
+        asm volatile(
+            "{\n\t.reg .pred E, P, T;\n\t.reg .b32 l;\n\t.reg .b64 a, b;\n\t"
+            "elect.sync l|E, 0xffffffff;\n\t"
+            "setp.ne.b32 P, %6, 0;\n\t"
+            "setp.eq.b32 T, 0, 0;\n\t"
+            "@E tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %3, %5, P;\n\t"
+            "add.s64 a, %1, %2;\n\tadd.s64 b, %3, %4;\n\t"
+            "@E tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, T;\n\t"
+            "add.s64 a, a, %2;\n\tadd.s64 b, b, %4;\n\t"
+            "@E tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, T;\n\t"
+            "add.s64 a, a, %2;\n\tadd.s64 b, b, %4;\n\t"
+            "@E tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, T;\n\t}" ::"r"(d),
+            "l"(a0), "l"(a_step), "l"(b0), "l"(b_step), "r"(idesc), "r"(acc0)
+            : "memory");
 }
 
 // Elected-lane commit: arrive once on the mbarrier at shared::cta offset bar

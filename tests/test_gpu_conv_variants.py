@@ -124,3 +124,34 @@ def test_filter_row_wgrad_matches_oracle(D, n, h, w, c, k, pad):
     D.dbl_conv_wgrad(shape, xd, dyd, dw, True, work, wsb)
     assert np.abs(host(dw) - 2 * got).max() <= 2.0 ** -22 * np.abs(got).max()
     check_status(D)
+
+
+@pytest.mark.parametrize("n,h,w", [
+    (1, 1, 8),       # the narrowest rows
+    (3, 5, 10),      # tiles spanning small images
+    (2, 9, 98),      # the widest rows
+    (2, 7, 100),     # wider: the window kernel without pixel pairs
+    (5, 13, 22),     # a ragged last tile
+])
+def test_pixel_pair_conv_matches_oracle(D, n, h, w):
+    """64 to 64 channels, 3x3 stride 1: forward with its channel sums, and the data gradient."""
+    g = rng(n * h + w)
+    x = bf16_values(g.standard_normal((n, h, w, 64)))
+    wt = bf16_values(g.standard_normal((64, 3, 3, 64)) * np.sqrt(2.0 / 576))
+    shape = D.conv_shape(n, h, w, 64, 64, 3, 1, 1)
+    xd, wd = to_bf16_dev(x), to_bf16_dev(wt)
+    y = torch.full((n, h, w, 64), float("nan"), dtype=torch.bfloat16, device="cuda")
+    s1, s2 = torch.empty(64, device="cuda"), torch.empty(64, device="cuda")
+    wsb = D.dbl_conv_workspace_bytes(shape, D.DBL_PASS_FWD)
+    D.dbl_conv_fwd(shape, xd, wd, y, s1, s2, ws(wsb), wsb)
+    assert np.all(np.isfinite(host(y)))
+    assert max_norm_rel(host(y), orc.conv2d_fwd(x, wt, 1, 1)) <= CONV_TOL
+    rows = host(y).reshape(-1, 64)
+    assert np.abs(host(s1) - rows.sum(0)).max() <= 1e-5 * np.abs(rows).sum(0).max()
+    assert max_norm_rel(host(s2), (rows * rows).sum(0)) <= 1e-5
+    dy = bf16_values(rng(n).standard_normal((n, h, w, 64)))
+    dx = torch.full((n, h, w, 64), float("nan"), dtype=torch.bfloat16, device="cuda")
+    D.dbl_conv_dgrad(shape, to_bf16_dev(dy), wd, dx)
+    assert np.all(np.isfinite(host(dx)))
+    assert max_norm_rel(host(dx), orc.conv2d_dgrad(dy, wt, x.shape, 1, 1)) <= CONV_TOL
+    check_status(D)
