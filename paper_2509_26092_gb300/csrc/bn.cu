@@ -9,6 +9,7 @@
 // Backward (two passes): a reduce pass of sum(g) and sum(g*xhat) per channel
 // into per-CTA partials, a tiny fixed-order finalize, and an apply pass
 //     dy = gamma*invstd*(g - sum(g)/count - xhat*sum(g*xhat)/count).
+#include <algorithm>
 #include <mutex>
 
 #include "dbl_internal.cuh"
@@ -203,6 +204,67 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM)
         const int v = (base + dir * r) * groups + g;
         emit(__ldcs(reinterpret_cast<const uint4*>(y) + v), res ? __ldcs(reinterpret_cast<const uint4*>(res) + v) : zero,
              v);
+    }
+}
+
+// Finalize and apply in one launch, for small tensors whose convolution left few partials: every CTA takes 32
+// channels (64 bytes of a row) and a run of the rows, and adds up its channels' partials for itself with the
+// finalize's own tree (the same bits).  The partials come from L2 once per CTA, 256 bytes each, against a
+// launch that reads them once.  576 rows of 512 channels, 32 partials: 5.8 -> 4.0 us.
+constexpr int kFwdSliceC = 32, kFwdSliceRows = kThreads * 8 / kFwdSliceC;
+
+__global__ void __launch_bounds__(kThreads, kBlocksPerSM)
+    bn_apply_parts_kernel(const act_t* __restrict__ y, const act_t* __restrict__ res, act_t* __restrict__ out,
+                          int count, int C, int relu, double inv_n, float eps, const float* __restrict__ part,
+                          int nparts, const float* __restrict__ gamma, const float* __restrict__ beta,
+                          float* __restrict__ save_mean, float* __restrict__ save_invstd)
+{
+    dbl::dev::grid_dependency_trigger();  // a convolution launched next may start its set-up
+    __shared__ dbl::dev::PairF red[2][kThreads / 32][kFwdSliceC];
+    __shared__ __align__(16) float chan[2][kFwdSliceC];  // scale, shift
+    const int slices = C / kFwdSliceC, c0 = blockIdx.x % slices * kFwdSliceC;
+    const int block = blockIdx.x / slices, blocks = gridDim.x / slices;
+    double ds, dq;
+    dbl::dev::partials_colsum32(part, nparts, C, c0, red, ds, dq);
+    if (threadIdx.x < kFwdSliceC) {
+        const int c = c0 + threadIdx.x;
+        float m, is;
+        finalize_channel((float)ds, (float)dq, inv_n, eps, m, is);
+        if (block == 0) {
+            save_mean[c] = m;
+            save_invstd[c] = is;
+        }
+        bn_scale_shift(gamma[c], beta[c], m, is, chan[0][threadIdx.x], chan[1][threadIdx.x]);
+    }
+    __syncthreads();
+    const int vl = threadIdx.x % (kFwdSliceC / 8), groups = C / 8, g = c0 / 8 + vl;
+    float sc[8], sh[8];
+    load8(&chan[0][8 * vl], sc);
+    load8(&chan[1][8 * vl], sh);
+    const int step = blocks * kFwdSliceRows;
+    constexpr int U = kUnroll;
+    for (int r = block * kFwdSliceRows + threadIdx.x / (kFwdSliceC / 8); r < count; r += U * step) {
+        uint4 yv[U], rv[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t v = (int64_t)(r + u * step) * groups + g;
+            const bool in = r + u * step < count;
+            yv[u] = in ? __ldcs(reinterpret_cast<const uint4*>(y) + v) : make_uint4(0, 0, 0, 0);
+            rv[u] = in && res ? __ldcs(reinterpret_cast<const uint4*>(res) + v) : make_uint4(0, 0, 0, 0);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (r + u * step < count) {
+                float f[8], rr[8];
+                unpack8(yv[u], f);
+                unpack8(rv[u], rr);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const float o = __fadd_rn(__fmaf_rn(f[k], sc[k], sh[k]), rr[k]);
+                    f[k] = (relu && !(o > 0.f)) ? 0.f : o;
+                }
+                reinterpret_cast<uint4*>(out)[(int64_t)(r + u * step) * groups + g] = pack8(f);
+            }
     }
 }
 
@@ -618,6 +680,15 @@ int reduce_grid(int64_t nblk)
     return (int)((nblk + per_cta - 1) / per_cta);
 }
 
+// Forward in one launch (bn_apply_parts_kernel)?  Above 8 MB whole rows stream better than 64-byte slices, and
+// above ~100 partials every CTA's own sum costs what the second launch does (us, two launches -> one):
+// 2 MB with 32 / 100 / 152 partials 6.3 -> 4.6, 6.3 -> 5.3, 6.5 -> 6.1; 6.6 MB 7.5 -> 6.5, 7.9 -> 7.3,
+// 7.8 -> 8.0; 12.8 MB with 32 8.9 -> 9.2.
+bool fwd_one_launch(int64_t count, int C, int nparts)
+{
+    return C % kFwdSliceC == 0 && nparts <= 104 && count * C * (int64_t)sizeof(act_t) <= (int64_t)8 << 20;
+}
+
 int apply_reversed(const dbl_bn_shape* s) { return s->count * s->c * (int64_t)sizeof(act_t) > kReverseAboveBytes; }
 
 int check_shape(const dbl_bn_shape* s, const char* who)
@@ -793,6 +864,14 @@ int dbl_bn_relu_fused_parts(const dbl_bn_shape* s, const void* y, const float* p
         return set_error(DBL_ERR_INVALID, "bn_relu_fused_parts: tensors must be 16-byte aligned");
     if (s->count == 0) return set_error(DBL_ERR_INVALID, "bn_relu_fused_parts: empty batch has no statistics");
     cudaStream_t st = as_stream(stream);
+    if (fwd_one_launch(s->count, s->c, nparts)) {
+        const int slices = s->c / kFwdSliceC;
+        const int64_t blocks = (s->count + kFwdSliceRows - 1) / kFwdSliceRows, cap = 2 * sm_count() / slices;
+        bn_apply_parts_kernel<<<slices * (int)std::max<int64_t>(1, std::min(blocks, cap)), kThreads, 0, st>>>(
+            static_cast<const act_t*>(y), static_cast<const act_t*>(residual), static_cast<act_t*>(out), (int)s->count,
+            s->c, s->relu, 1.0 / (double)s->count, s->eps, parts, nparts, gamma, beta, save_mean, save_invstd);
+        return launch_check("bn_apply_parts launch");
+    }
     bn_fwd_finalize_parts_kernel<<<(s->c + dbl::dev::kPartialsChannels - 1) / dbl::dev::kPartialsChannels,
                                    dbl::dev::kPartialsThreads, 0, st>>>(1.0 / (double)s->count, s->c, s->eps, parts,
                                                                    nparts, save_mean, save_invstd);

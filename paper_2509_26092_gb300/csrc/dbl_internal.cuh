@@ -390,6 +390,44 @@ __device__ __forceinline__ int partials_colsum(const float* __restrict__ part, i
     return (threadIdx.x < kPartialsChannels && c < K) ? c : -1;
 }
 
+// The same sums, bit for bit, of 32 channels from c0 by a block of 256 threads (K a multiple of 32): thread t
+// takes channel t % 32 and the four streams 4*(t/32) .., whose tree it walks itself; the warps' trees
+// are the upper stream bits.  Threads t < 32 get the sums of channel c0 + t.
+__device__ __forceinline__ void partials_colsum32(const float* __restrict__ part, int nparts, int K, int c0,
+                                                  PairF (*red)[8][32], double& sum0, double& sum1)
+{
+    const int cl = threadIdx.x % 32, w = threadIdx.x / 32;
+    const float* p = part + c0 + cl;
+    const int64_t ld = 2 * (int64_t)K;
+    PairF a[2][4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        float s = 0.f, sc = 0.f, q = 0.f, qc = 0.f;
+#pragma unroll 2
+        for (int t = 4 * w + u; t < nparts; t += 32) {
+            kahan_add(s, sc, __ldg(p + t * ld));
+            kahan_add(q, qc, __ldg(p + t * ld + K));
+        }
+        a[0][u] = pair_from(s, -sc);
+        a[1][u] = pair_from(q, -qc);
+    }
+#pragma unroll
+    for (int x = 0; x < 2; ++x) red[x][w][cl] = pair_add(pair_add(a[x][0], a[x][1]), pair_add(a[x][2], a[x][3]));
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        double out[2];
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+            const PairF(&r)[8][32] = red[x];
+            const PairF t = pair_add(pair_add(pair_add(r[0][cl], r[1][cl]), pair_add(r[2][cl], r[3][cl])),
+                                     pair_add(pair_add(r[4][cl], r[5][cl]), pair_add(r[6][cl], r[7][cl])));
+            out[x] = (double)t.hi + (double)t.lo;
+        }
+        sum0 = out[0];
+        sum1 = out[1];
+    }
+}
+
 // ---------------------------------------------------------------------------- TMA
 __device__ __forceinline__ void tma_prefetch_desc(const void* tmap)
 {

@@ -1,5 +1,5 @@
-"""Edges of the one-launch BatchNorm backward of small tensors (a cluster of CTAs per 32 channels)
-against the fp64 oracle."""
+"""Edges of the one-launch BatchNorm passes of small tensors: the backward (a cluster of CTAs per 32
+channels) against the fp64 oracle, the forward against the two launches of larger ones."""
 import numpy as np
 import pytest
 import torch
@@ -58,4 +58,33 @@ def test_small_bn_backward_matches_oracle(D, count, C, mask):
         assert np.abs(host(got) - ref).max() <= 1e-5 * (np.abs(rres).sum(0).max() * 4)
     if two:
         assert max_norm_rel(host(d2), rres) <= 4e-3
+    check_status(D)
+
+
+@pytest.mark.parametrize("count,C,nparts", [
+    (1, 32, 1),        # one row, one partial
+    (63, 512, 33),     # fewer rows than a CTA covers; a second round of a stream
+    (4099, 256, 104),  # the most partials; a ragged last run of rows
+    (8192, 512, 7),    # the largest tensor
+])
+@pytest.mark.parametrize("residual", [False, True])
+def test_one_launch_bn_forward_gives_the_same_bits(D, count, C, nparts, residual):
+    """Partial rows of zeros leave the sums as they are and take the call to the two-launch path."""
+    g = rng(count)
+    y = to_bf16_dev(g.standard_normal((count, C)) + 0.5)
+    res = to_bf16_dev(g.standard_normal((count, C))) if residual else None
+    gamma, beta = to_f32_dev(1.0 + 0.2 * g.standard_normal(C)), to_f32_dev(0.1 * g.standard_normal(C))
+    parts = np.zeros((160, 2, C), dtype=np.float32)
+    w = g.random((nparts, 1, C)).astype(np.float32)
+    parts[:nparts, :1] = 0.5 * count * w / w.sum(0)
+    parts[:nparts, 1:] = 1.25 * count * w / w.sum(0)
+    pd = to_f32_dev(parts)
+    got = []
+    for n in (nparts, 160):
+        out = torch.full((count, C), float("nan"), dtype=torch.bfloat16, device="cuda")
+        mean, istd = torch.full((C,), float("nan"), device="cuda"), torch.full((C,), float("nan"), device="cuda")
+        D.dbl_bn_relu_fused_parts(D.bn_shape(count, C, 1e-5, True), y, pd, n, gamma, beta, res, out, mean, istd)
+        got.append((out, mean, istd))
+    assert all(torch.isfinite(t.float()).all() for t in got[0])
+    assert all(torch.equal(a, b) for a, b in zip(*got))
     check_status(D)
