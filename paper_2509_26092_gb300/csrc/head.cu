@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(256) avgpool_kernel(const act_t* __restrict__ 
 // sums that need the same input, share a launch.
 // Bound by fp32 issue: 512 x 1000 x 512 is 7 us of the GPU's fp32 rate.  With 4 x 4 outputs per thread
 // (half the FMAs per shared-memory byte), the partial sums through global memory and a launch of their
-// own, the head of 512 images and 1000 classes took 128.2 us in ten launches; now 75.3 in five.
+// own, the head of 512 images and 1000 classes took 128.2 us in ten launches; now 72.6 in five.
 constexpr int GBM = 64, GBN = 128, GBK = 16;
 constexpr int GLA = GBM + 4, GLB = GBN + 4;  // row pitches of the K-major tiles
 constexpr int kGemmThreads = 128;
@@ -728,11 +728,19 @@ __device__ __forceinline__ int pool_slices(int groups) { return groups >= 1024 ?
 __global__ void __launch_bounds__(1024) avgpool_img_kernel(const act_t* __restrict__ x, float* __restrict__ feat,
                                                            int hw, int C, Dropout dp)
 {
-    extern __shared__ float slice_sum[];  // [S][C]
+    extern __shared__ float slice_sum[];  // [S][C], then the keep bits of the C / 4 dropout blocks
     const int groups = C / 8, S = pool_slices(groups);
+    uint8_t* keep = reinterpret_cast<uint8_t*>(slice_sum + S * C);
     const int g = threadIdx.x % groups, sl = threadIdx.x / groups;
     const int b = blockIdx.x;
+    // the draws first, a block per thread: their long chain of 64-bit products overlaps the other warps' loads
+    if (dp.thr) {
+        const uint64_t st = *dp.step;
+        for (int q = threadIdx.x; q < C / 4; q += blockDim.x)
+            keep[q] = (uint8_t)dropout_keep4(dp.seed, st, (uint64_t)b * (uint64_t)(C / 4) + q, dp.thr);
+    }
     float acc[8] = {};
+#pragma unroll 4
     for (int i = sl; i < hw; i += S) {
         float f[8];
         unpack8(__ldg(reinterpret_cast<const uint4*>(x + ((int64_t)b * hw + i) * C) + g), f);
@@ -742,24 +750,18 @@ __global__ void __launch_bounds__(1024) avgpool_img_kernel(const act_t* __restri
 #pragma unroll
     for (int k = 0; k < 8; ++k) slice_sum[sl * C + 8 * g + k] = acc[k];
     __syncthreads();
-    if (sl != 0) return;
-    for (int q = 1; q < S; ++q)
-#pragma unroll
-        for (int k = 0; k < 8; ++k) acc[k] += slice_sum[q * C + 8 * g + k];
+    // one feature per thread: its slices in order (consecutive threads on consecutive features)
     const float inv = 1.0f / (float)hw;
-    if (dp.thr) {
-        const uint64_t st = *dp.step;
-        const uint64_t q = (uint64_t)b * (uint64_t)(C / 4) + 2 * (uint64_t)g;
-        const unsigned bits = dropout_keep4(dp.seed, st, q, dp.thr) | dropout_keep4(dp.seed, st, q + 1, dp.thr) << 4;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const float m = (bits >> k) & 1 ? dp.scale : 0.f;
-            dp.mult[(int64_t)b * C + 8 * g + k] = m;
-            feat[(int64_t)b * C + 8 * g + k] = acc[k] * inv * m;
+    for (int c = threadIdx.x; c < C; c += blockDim.x) {
+        float t = slice_sum[c];
+        for (int q = 1; q < S; ++q) t += slice_sum[q * C + c];
+        if (dp.thr) {
+            const float m = (keep[c / 4] >> (c % 4)) & 1 ? dp.scale : 0.f;
+            dp.mult[(int64_t)b * C + c] = m;
+            feat[(int64_t)b * C + c] = t * inv * m;
+        } else {
+            feat[(int64_t)b * C + c] = t * inv;
         }
-    } else {
-#pragma unroll
-        for (int k = 0; k < 8; ++k) feat[(int64_t)b * C + 8 * g + k] = acc[k] * inv;
     }
 }
 
@@ -930,7 +932,7 @@ int head_fwd_bwd(int32_t n, int32_t hw, int32_t c, int32_t classes, const void* 
     const bool per_image = groups <= 1024;  // one CTA per image (at most 1024 threads)
     const int S = groups >= 1024 ? 1 : std::min(8, 1024 / groups);
     if (per_image)
-        avgpool_img_kernel<<<n, S * groups, (size_t)S * c * sizeof(float), s>>>(static_cast<const act_t*>(x), feat,
+        avgpool_img_kernel<<<n, S * groups, (size_t)S * c * sizeof(float) + c / 4, s>>>(static_cast<const act_t*>(x), feat,
                                                                                  hw, c, dp);
     else
         avgpool_kernel<<<grid_for((int64_t)n * groups, 256), 256, 0, s>>>(static_cast<const act_t*>(x), feat, n, hw,
