@@ -215,6 +215,145 @@ __global__ void __launch_bounds__(256)
     }
 }
 
+// The same for large tensors (kPoolRowsBytes): a thread owns one channel group g of two neighbouring output columns and walks down `rows` output
+// rows: each input row is normalised once, in five vectors of which the middle one serves both columns,
+// and reduced along the row (its maximum and the first column that has it); an output row combines three
+// such row results, the last of which is the next output row's first.  That is 5 vectors per output
+// instead of the 9 of a window taken by itself.  The row maxima combined last row first with >= leave the same
+// first maximum.  The five vectors come through a ring of kPoolDepth rows in shared memory that the
+// thread fills for itself (cp.async, zeros outside the image): with them in registers, one row ahead, 16 warps
+// per SM waited for memory (245 us at 112 x 112 x 64, batch 512, like a window per thread); now 224, 80 x 80 135 -> 120, 144 x 144, batch 185 157 -> 140.
+constexpr int kPoolDepth = 5;
+// Below this a few long runs of rows leave SMs idle or a last round nearly empty: 64 x 64, batch 64 (34 MB) 15.6 us
+// with a window per thread against 16.0 with the best run, 144 x 144, batch 16 (42 MB) 18.4 against 18.3 to 25.9;
+// 112 x 112, batch 64 (103 MB) 38.9 against 34.2 to 38.1.
+constexpr int64_t kPoolRowsBytes = 96ll << 20;
+constexpr int kPoolThreads = 256;
+
+struct PoolRow {  // per column and channel pair: maximum of a row's three taps, and its tap (0..2 in each half)
+    uint32_t best[2][4], idx[2][4];
+};
+
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool in)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
+}
+
+__global__ void __launch_bounds__(kPoolThreads, 2)
+    bn_relu_maxpool_rows_kernel(const act_t* __restrict__ x, const float* __restrict__ gamma,
+                               const float* __restrict__ beta, const float* __restrict__ mean,
+                               const float* __restrict__ invstd, act_t* __restrict__ y,
+                               uint8_t* __restrict__ arg, int n, int H, int W, int C, int P, int Q, int rows)
+{
+    dbl::dev::grid_dependency_trigger();  // a convolution launched next may start its set-up
+    extern __shared__ uint4 ring[];       // [depth][5][thread]
+    const unsigned groups = (unsigned)C / 8u;
+    const unsigned per_block = blockDim.x / groups;
+    const unsigned g = threadIdx.x % groups;
+    const unsigned cols = ((unsigned)Q + 1u) / 2u, chunks = ((unsigned)P + rows - 1u) / rows;
+    const unsigned items = (unsigned)n * chunks * cols;
+    float2 sc[4], sh[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int c0 = 8 * g + 2 * k;
+        dbl::dev::bn_scale_shift(gamma[c0], beta[c0], mean[c0], invstd[c0], sc[k].x, sh[k].x);
+        dbl::dev::bn_scale_shift(gamma[c0 + 1], beta[c0 + 1], mean[c0 + 1], invstd[c0 + 1], sc[k].y, sh[k].y);
+    }
+    const int64_t row_vecs = (int64_t)W * groups;  // uint4 vectors per input row
+    const uint32_t mine = dbl::dev::smem_u32(ring + threadIdx.x), vec = blockDim.x * 16u;
+    for (unsigned item = blockIdx.x * per_block + threadIdx.x / groups; item < items; item += gridDim.x * per_block) {
+        const int j = (int)(item % cols), ch = (int)((item / cols) % chunks), b = (int)(item / (cols * chunks));
+        const int p0 = ch * rows, p1 = min(P, p0 + rows);
+        const int w0 = 4 * j - 1;  // first of the five input columns
+        const uint4* xv = reinterpret_cast<const uint4*>(x) + (int64_t)b * H * row_vecs + g;
+        bool w_ok[5];
+#pragma unroll
+        for (int s = 0; s < 5; ++s) w_ok[s] = w0 + s >= 0 && w0 + s < W;
+        const int h0 = 2 * p0 - 1, count = 2 * (p1 - p0) + 1;  // input rows h0 .. h0 + count - 1
+        auto fetch = [&](int i) {                               // row h0 + i into its slot; always one group
+            const int h = h0 + i;
+            if (i < count) {
+                const bool ok = h >= 0 && h < H;
+                const uint32_t dst = mine + (uint32_t)(i % kPoolDepth) * 5u * vec;
+#pragma unroll
+                for (int s = 0; s < 5; ++s)
+                    cp_async16(dst + (uint32_t)s * vec, ok && w_ok[s] ? xv + (int64_t)h * row_vecs + (w0 + s) * (int64_t)groups : xv,
+                               ok && w_ok[s]);
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        // taps outside the image take no part: best starts at zero, and >= against it is only asked of
+        // taps inside (every tap is >= 0 after the ReLU, so the last one inside always enters)
+        auto reduce_row = [&](int i, PoolRow& row) {
+            fetch(i + kPoolDepth - 1);
+            asm volatile("cp.async.wait_group %0;" ::"n"(kPoolDepth - 1) : "memory");
+#pragma unroll
+            for (int o = 0; o < 2; ++o)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) row.best[o][k] = row.idx[o][k] = 0u;
+            const uint4* v = ring + threadIdx.x + (i % kPoolDepth) * 5 * blockDim.x;
+#pragma unroll
+            for (int s = 4; s >= 0; --s) {
+                const uint4 t = v[s * blockDim.x];
+                if (!w_ok[s]) continue;
+                const uint32_t w[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const uint32_t a = bn_relu_pair(w[k], sc[k], sh[k]);
+#pragma unroll
+                    for (int o = 0; o < 2; ++o) {
+                        const int tap = s - 2 * o;
+                        if (tap < 0 || tap > 2) continue;
+                        uint32_t ge, m;
+                        asm("set.ge.u32." DBL_ACT_X2 " %0, %1, %2;" : "=r"(ge) : "r"(a), "r"(row.best[o][k]));
+                        asm("max." DBL_ACT_X2 " %0, %1, %2;" : "=r"(m) : "r"(row.best[o][k]), "r"(a));
+                        row.best[o][k] = m;
+                        row.idx[o][k] = (ge & ((uint32_t)tap * 0x10001u)) | (~ge & row.idx[o][k]);
+                    }
+                }
+            }
+        };
+#pragma unroll
+        for (int i = 0; i < kPoolDepth - 1; ++i) fetch(i);
+        PoolRow top;  // row 2p - 1 of the next output row
+        reduce_row(0, top);
+        for (int p = p0; p < p1; ++p) {
+            PoolRow mid, bot;
+            reduce_row(2 * (p - p0) + 1, mid);
+            reduce_row(2 * (p - p0) + 2, bot);
+            const bool top_ok = p > 0, bot_ok = 2 * p + 1 < H;
+#pragma unroll
+            for (int o = 0; o < 2; ++o) {
+                if (2 * j + o >= Q) continue;
+                uint32_t best[4], idx[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    // rows last to first; the middle row is always inside the image
+                    uint32_t m = bot.best[o][k], id = bot.idx[o][k] + 0x60006u, ge;
+                    if (!bot_ok) m = id = 0u;
+                    asm("set.ge.u32." DBL_ACT_X2 " %0, %1, %2;" : "=r"(ge) : "r"(mid.best[o][k]), "r"(m));
+                    asm("max." DBL_ACT_X2 " %0, %1, %2;" : "=r"(m) : "r"(m), "r"(mid.best[o][k]));
+                    id = (ge & (mid.idx[o][k] + 0x30003u)) | (~ge & id);
+                    if (top_ok) {
+                        asm("set.ge.u32." DBL_ACT_X2 " %0, %1, %2;" : "=r"(ge) : "r"(top.best[o][k]), "r"(m));
+                        asm("max." DBL_ACT_X2 " %0, %1, %2;" : "=r"(m) : "r"(m), "r"(top.best[o][k]));
+                        id = (ge & top.idx[o][k]) | (~ge & id);
+                    }
+                    // +0 for a maximum of zero (a -0 lane is negative as a signed 16-bit value)
+                    asm("max.s16x2 %0, %1, %2;" : "=r"(best[k]) : "r"(m), "r"(0u));
+                    idx[k] = id;
+                }
+                const int64_t at = (((int64_t)b * P + p) * Q + 2 * j + o) * C + 8 * g;
+                *reinterpret_cast<uint4*>(y + at) = make_uint4(best[0], best[1], best[2], best[3]);
+                *reinterpret_cast<uint2*>(arg + at) = make_uint2(__byte_perm(idx[0], idx[1], 0x6420),
+                                                                 __byte_perm(idx[2], idx[3], 0x6420));
+            }
+            top = bot;
+        }
+        asm volatile("cp.async.wait_group 0;" ::: "memory");  // the empty groups: counts start anew
+    }
+}
+
 // dst[k] += src[k] where byte k of the argmax word pair equals tap (fp32; a
 // skipped term leaves dst as it is)
 __device__ __forceinline__ void add_if_tap(float (&dst)[8], const float (&src)[8], uint2 a, uint32_t tap)
@@ -856,10 +995,42 @@ int dbl_bn_relu_maxpool_fwd(const dbl_bn_shape* s, int32_t n, int32_t h, int32_t
     int rc = bn_fwd_finalize(s->count, c, s->eps, ch_sum, ch_sumsq, save_mean, save_invstd, st);
     if (rc) return rc;
     // a block size that is a multiple of the channel groups: each thread keeps its group
-    const int groups = c / 8, block = groups * std::max(1, 256 / groups);
-    bn_relu_maxpool_fwd_kernel<<<grid_for((int64_t)n * P * Q, block / groups), block, 0, st>>>(
+    const int groups = c / 8, block = groups * std::max(1, kPoolThreads / groups);
+    if (s->count * c * (int64_t)sizeof(act_t) < kPoolRowsBytes || block > kPoolThreads) {
+        bn_relu_maxpool_fwd_kernel<<<grid_for((int64_t)n * P * Q, block / groups), block, 0, st>>>(
+            static_cast<const act_t*>(x), gamma, beta, save_mean, save_invstd, static_cast<act_t*>(y),
+            argmax, n, h, w, c, P, Q);
+        return launch_check("bn_relu_maxpool_fwd launch");
+    }
+    // output rows per thread: the count of two to eight with the least modelled time, rounds of two CTAs per SM
+    // (between fractional and whole) x (input rows of a run + ~5 of set-up)
+    const int cols = (Q + 1) / 2;
+    int rows = 2;
+    double best = 0.0;
+    for (int r = 2; r <= 8; ++r) {
+        const double ctas = (double)n * ((P + r - 1) / r) * cols * groups / kPoolThreads;
+        const double waves = std::max(1.0, ctas / (2.0 * sm_count()));
+        const double cost = (0.3 * waves + 0.7 * ceil(waves)) * (2 * r + 6);
+        if (r == 2 || cost < best) {
+            best = cost;
+            rows = r;
+        }
+    }
+    const int64_t items = (int64_t)n * ((P + rows - 1) / rows) * cols;
+    const size_t smem = (size_t)kPoolDepth * 5 * block * 16;
+    static bool attr_set[64] = {false};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev >= 0 && dev < 64 && !attr_set[dev]) {
+        if ((rc = cuda_check(cudaFuncSetAttribute(bn_relu_maxpool_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                  kPoolDepth * 5 * kPoolThreads * 16),
+                             "bn_relu_maxpool_fwd: set smem attribute")))
+            return rc;
+        attr_set[dev] = true;
+    }
+    bn_relu_maxpool_rows_kernel<<<grid_for(items, block / groups), block, smem, st>>>(
         static_cast<const act_t*>(x), gamma, beta, save_mean, save_invstd, static_cast<act_t*>(y),
-        argmax, n, h, w, c, P, Q);
+        argmax, n, h, w, c, P, Q, rows);
     return launch_check("bn_relu_maxpool_fwd launch");
 }
 
