@@ -780,7 +780,7 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, CG>::THREADS, 1)
     }
 }
 
-// ----------------------------------------------------------------------------- split-K forward / data gradient
+// ----------------------------------------------------------------------------- split-K on chip
 // The 256-column pair tiles of the forward pass and the data gradient when there are too few of them
 // for the GPU (the layers of a few thousand pixels): a cluster of SK CTA pairs shares one tile, pair j
 // reducing K-blocks j*nkb/SK .. (j+1)*nkb/SK - 1.  When every pair's MMAs are done (cluster barrier;
@@ -793,28 +793,33 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, CG>::THREADS, 1)
 // Why: with one pair per tile a 4x4 or 3x3 map of 512 channels runs 72 K-blocks (36.9 k tensor cycles)
 // on 6 to 36 of 76 pairs.  128-column tiles instead would need 1.5 times the operand bytes per MMA.
 // Channel sums: the CTAs of a row block write disjoint columns of one partial row (2 * m_tiles rows).
-template <int SK>
+// The weight gradient's pair tiles share their K range the same way where that saves slices of fp32 partial
+// sums (p.zdim of them are left for wgrad_reduce_kernel; none when it is 1): 7x7x512,
+// batch 512 91.6 -> 85.7 us and 128 32.1 -> 27.1, 3x3x512, batch 512 26.7 -> 22.0, 12x12 128 -> 256 stride 2,
+// batch 512 25.7 -> 20.8, a 14x14 projection 256 -> 512, batch 128 15.9 -> 13.0 (with the reduce).
+template <int BN, int FAM, int SK>
 struct SplitCfg {
-    using C = Cfg<256, kFamFwd, 2>;
-    static constexpr int W = 256 / SK;              // columns a CTA finishes
+    using C = Cfg<BN, FAM, 2>;
+    static_assert(C::ACC == 1 && BN / SK >= 32, "one accumulator, whole chunks");
+    static constexpr int W = BN / SK;              // columns a CTA finishes
     static constexpr int SLOT = 128 * W * 4;        // one received part: [W / 4][128 rows] float4
     static constexpr int CW = W > 32 ? W / 2 : 32;  // columns an epilogue warp finishes (of W = 32: one warp per quarter)
-    static constexpr int EPI_TILE = 8 * 32 * 33 * 4;
+    static constexpr int EPI_TILE = FAM == kFamFwd ? 8 * 32 * 33 * 4 : 0;  // transposes of the channel sums
     static constexpr int EPI_SUM = 4 * 2 * W * 4;   // channel sums per lane quarter
     static constexpr int SMEM = C::RING + EPI_SUM + 1024;
     static_assert((SK - 1) * SLOT + EPI_TILE <= C::RING, "received parts and transposes fit in the ring");
 };
 
-template <int SK>
-__global__ void __launch_bounds__(Cfg<256, kFamFwd, 2>::THREADS, 1)
+template <int BN, int FAM, int SK>
+__global__ void __launch_bounds__(Cfg<BN, FAM, 2>::THREADS, 1)
     conv_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                        const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2,
                        const ConvParams p)
 {
     dbl::dev::grid_dependency_trigger();  // a convolution launched next may start its set-up
-    using S = SplitCfg<SK>;
+    using S = SplitCfg<BN, FAM, SK>;
     using C = typename S::C;
-    constexpr int BN = 256, STAGES = C::STAGES, W = S::W;
+    constexpr int STAGES = C::STAGES, W = S::W;
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[STAGES], empty_bar[STAGES], accf_bar, drain_bar;
     __shared__ uint32_t tmem_slot;
@@ -827,9 +832,16 @@ __global__ void __launch_bounds__(Cfg<256, kFamFwd, 2>::THREADS, 1)
     const uint32_t leader = (uint32_t)(crank & ~1);  // the CTA of this pair that issues its MMAs
     const int t = blockIdx.x / (2 * SK);
     const TileCoord tc = decode_tile(p, t, gridDim.x);
-    int kb0 = 0, nkb_all = 0;
-    kb_range(p, tc.z, kb0, nkb_all);
-    const int k0 = nkb_all * split / SK, nkb = nkb_all * (split + 1) / SK - k0;
+    int k0 = 0, nkb = 0;  // this pair's K-blocks
+    if constexpr (FAM == kFamWgrad) {
+        k0 = (tc.z * SK + split) * p.kb_per_split;
+        nkb = max(0, min(p.num_kb, k0 + p.kb_per_split) - k0);
+    } else {
+        int first = 0, all = 0;
+        kb_range(p, tc.z, first, all);
+        k0 = all * split / SK;
+        nkb = all * (split + 1) / SK - k0;
+    }
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
@@ -864,10 +876,14 @@ __global__ void __launch_bounds__(Cfg<256, kFamFwd, 2>::THREADS, 1)
     if (warp >= C::EPI && warp < C::MMA_WARP) {
         // ------------------------------------------------------------------ TMA producers
         const int prod = warp - C::EPI;
-        const int64_t m0 = ((int64_t)tc.m_tile * 2 + rank) * 128;
-        const int tn = (int)(m0 / gPQ);
-        const int64_t rem = m0 - (int64_t)tn * gPQ;
-        const int tp = (int)(rem / p.gQ), tq = (int)(rem - (int64_t)tp * p.gQ);
+        int tn = 0, tp = 0, tq = 0;
+        if constexpr (FAM == kFamFwd) {
+            const int64_t m0 = ((int64_t)tc.m_tile * 2 + rank) * 128;
+            tn = (int)(m0 / gPQ);
+            const int64_t rem = m0 - (int64_t)tn * gPQ;
+            tp = (int)(rem / p.gQ);
+            tq = (int)(rem - (int64_t)tp * p.gQ);
+        }
         bool failed = false;
         int last_it = -1;
         for (int k = prod; k < nkb; k += kProducers) {
@@ -879,7 +895,7 @@ __global__ void __launch_bounds__(Cfg<256, kFamFwd, 2>::THREADS, 1)
             }
             uint8_t* sa = sgen + s * C::STAGE_BYTES;
             if (rank == 0) mbar_arrive_expect_tx_elect(&full_bar[s], (uint32_t)(2 * C::STAGE_BYTES));
-            load_kblock<BN, kFamFwd, 2>(p, &tmA, &tmB, &tmA2, &tmB2, sa, sa + C::A_BYTES,
+            load_kblock<BN, FAM, 2>(p, &tmA, &tmB, &tmA2, &tmB2, sa, sa + C::A_BYTES,
                                         mapa_shared(smem_u32(&full_bar[s]), leader), tc, k0 + k, tn, tp, tq, rank);
             last_it = k;
         }
@@ -899,12 +915,13 @@ __global__ void __launch_bounds__(Cfg<256, kFamFwd, 2>::THREADS, 1)
     } else if (warp == C::MMA_WARP) {
         // ------------------------------------------------------------------ MMA issuer (rank 0 of each pair)
         if (rank == 0) {
-            const bool fwd = p.mode == kFwd;
-            const uint32_t idesc = idesc_act(BM * 2, BN, 0u, fwd ? 0u : 1u);
+            // operand layouts as in conv_igemm_kernel
+            const bool wg = FAM == kFamWgrad, fwd = p.mode == kFwd;
+            const uint32_t idesc = idesc_act(BM * 2, BN, wg ? 1u : 0u, fwd ? 0u : 1u);
             const uint16_t both = (uint16_t)(3u << leader);
-            const uint64_t dA = smem_desc(0, 16, 1024, kSwizzle128B);
-            const uint64_t dB = fwd ? smem_desc(0, 16, 1024, kSwizzle128B) : smem_desc(0, 8192, 1024, kSwizzle128B);
-            const int b_step16 = fwd ? 2 : 2048 / 16;
+            const uint64_t dA = smem_desc(0, wg ? 16384 : 16, 1024, kSwizzle128B);
+            const uint64_t dB = smem_desc(0, wg ? 16384 : fwd ? 16 : 8192, 1024, kSwizzle128B);
+            const int a_step16 = wg ? 2048 / 16 : 2, b_step16 = fwd ? 2 : 2048 / 16;
             bool failed = false;
             if (nkb > 0) {
                 const uint32_t ok = mbar_wait_warp(&full_bar[0], 0, &abort_flag);
@@ -922,7 +939,7 @@ __global__ void __launch_bounds__(Cfg<256, kFamFwd, 2>::THREADS, 1)
                             mbar_wait_warp(&full_bar[(k + 1) % STAGES], ((k + 1) / STAGES) & 1, &abort_flag);
                         failed = __any_sync(0xffffffffu, ok == 0u);
                     }
-                    mma_act_elect_cg<2>(tmem, ad0 + (uint64_t)(j * 2), bd0 + (uint64_t)(j * b_step16), idesc,
+                    mma_act_elect_cg<2>(tmem, ad0 + (uint64_t)(j * a_step16), bd0 + (uint64_t)(j * b_step16), idesc,
                                         (k > 0 || j > 0) ? 1u : 0u);
                 }
                 mma_commit_elect_cg<2>(&empty_bar[s], both);
@@ -989,7 +1006,7 @@ __global__ void __launch_bounds__(Cfg<256, kFamFwd, 2>::THREADS, 1)
     if (warp < C::EPI) {
         // ------------------------------------------------------------------ epilogue of this CTA's columns
         float* sums = reinterpret_cast<float*>(sgen + C::RING);
-        const bool want_stats = p.mode == kFwd && p.stats != nullptr;
+        const bool want_stats = FAM == kFamFwd && p.mode == kFwd && p.stats != nullptr;
         const int64_t m = ((int64_t)tc.m_tile * 2 + rank) * 128 + row;
         const bool valid = m < p.M;
         int64_t out_row = m;
@@ -1015,9 +1032,22 @@ __global__ void __launch_bounds__(Cfg<256, kFamFwd, 2>::THREADS, 1)
                         v[4 * k + 2] = __float_as_uint(__uint_as_float(v[4 * k + 2]) + f.z);
                         v[4 * k + 3] = __float_as_uint(__uint_as_float(v[4 * k + 3]) + f.w);
                     }
-                float back[32];
-                store_row_chunk_act(p, v, valid, out_row, tc.n_tile * BN + split * W + half * CW + ch * 32, back);
-                if (want_stats) rs.add(ch, back);
+                const int col0 = tc.n_tile * BN + split * W + half * CW + ch * 32;
+                if constexpr (FAM == kFamWgrad) {
+                    // [slice][k][m]: consecutive lanes hold consecutive m, one 128-byte line per store
+                    float* o = static_cast<float*>(p.out) + ((int64_t)tc.z * p.Ncols + col0) * p.M + m;
+                    if (valid && p.zdim == 1 && p.wg_accumulate) {
+#pragma unroll
+                        for (int k = 0; k < 32; ++k) o[(int64_t)k * p.M] += __uint_as_float(v[k]);
+                    } else if (valid) {
+#pragma unroll
+                        for (int k = 0; k < 32; ++k) o[(int64_t)k * p.M] = __uint_as_float(v[k]);
+                    }
+                } else {
+                    float back[32];
+                    store_row_chunk_act(p, v, valid, out_row, col0, back);
+                    if (want_stats) rs.add(ch, back);
+                }
             }
             if (want_stats) {
                 float* st_tile = reinterpret_cast<float*>(sgen + (SK - 1) * S::SLOT) + warp * 32 * 33;
@@ -2856,6 +2886,34 @@ int fwd_splits(int tiles, int num_kb)
     return best;
 }
 
+// CTA pairs per tile of the implicit-GEMM weight gradient (conv_splitk_kernel), against `splits` slices of one pair
+// each: the least modelled time in SM cycles on a 152-SM GPU.  A K-block takes ~1570 (256 columns) or ~1000
+// (128) cycles, a tile ~8000 of set-up, first loads and epilogue, the exchange of partial sums ~2500 of
+// barriers and 22 bytes per cycle, the reduce of slices ~5000 and 1800 bytes per cycle.
+void wgrad_cluster(Plan& pl, int splits)
+{
+    static const int counts[3] = {2, 4, 8}, resident[3] = {36, 15, 7};
+    ConvParams& p = pl.p;
+    const int tiles = p.m_tiles * p.n_tiles;
+    const double kbc = pl.BN == 256 ? 1570.0 : 1000.0, acc = 128.0 * pl.BN * 4.0;
+    auto reduce = [&](int slices) { return slices > 1 ? 5000.0 + (double)p.M * p.Ncols * 4.0 * slices / 1800.0 : 0.0; };
+    double best = ((tiles * splits + 75) / 76) * (double)((p.num_kb + splits - 1) / splits) * kbc + 8000.0 + acc / 40.0 +
+                  reduce(splits);
+    for (int i = 0; i < 3; ++i) {
+        const int sk = counts[i], slices = resident[i] / tiles;
+        if (slices < 1 || pl.BN / sk < 32) continue;
+        const int kbs = (p.num_kb + slices * sk - 1) / (slices * sk);
+        const int used = (p.num_kb + kbs * sk - 1) / (kbs * sk);  // no slice without a K-block
+        const double cost = kbs * kbc + 10500.0 + acc * (sk - 1) / sk / 22.0 + reduce(used);
+        if (cost < best) {
+            best = cost;
+            pl.sk = sk;
+            p.kb_per_split = kbs;
+            p.zdim = used;
+        }
+    }
+}
+
 int make_plan(const dbl_conv_shape* s, int pass, Plan& pl)
 {
     using dbl::set_error;
@@ -2989,7 +3047,8 @@ int make_plan(const dbl_conv_shape* s, int pass, Plan& pl)
         const int splits = wgrad_splits(p.m_tiles * p.n_tiles, p.num_kb, p.M, s->k, pl.BN, pl.cg);
         p.kb_per_split = (p.num_kb + splits - 1) / splits;
         p.zdim = splits;
-        pl.ws_main = splits > 1 ? (size_t)splits * p.M * s->k * sizeof(float) : 0;
+        if (pl.cg == 2) wgrad_cluster(pl, splits);
+        pl.ws_main = p.zdim > 1 ? (size_t)p.zdim * p.M * s->k * sizeof(float) : 0;
     }
     p.total_tiles = p.m_tiles * p.n_tiles * p.zdim;
     if (!pl.win && pl.BN == 256 && pl.cg == 2 && (pl.mode == kFwd || pl.mode == kDgrad)) {
@@ -3172,7 +3231,7 @@ int launch_cfg(const Plan& pl, const CUtensorMap& a, const CUtensorMap& b, const
     return dbl::launch_check("conv_igemm launch");
 }
 
-template <int SK>
+template <int BN, int FAM, int SK>
 int launch_splitk(const Plan& pl, const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& a2,
                   const CUtensorMap& b2, int grid, cudaStream_t st)
 {
@@ -3180,23 +3239,23 @@ int launch_splitk(const Plan& pl, const CUtensorMap& a, const CUtensorMap& b, co
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev >= 0 && dev < 64 && !attr_set[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(conv_splitk_kernel<SK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             SplitCfg<SK>::SMEM);
+        cudaError_t e = cudaFuncSetAttribute(conv_splitk_kernel<BN, FAM, SK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             SplitCfg<BN, FAM, SK>::SMEM);
         // a cluster of sixteen CTAs is above the portable size of eight
         if (e == cudaSuccess && 2 * SK > 8)
-            e = cudaFuncSetAttribute(conv_splitk_kernel<SK>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            e = cudaFuncSetAttribute(conv_splitk_kernel<BN, FAM, SK>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return dbl::cuda_check(e, "conv: set smem attribute");
         attr_set[dev] = true;
     }
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[2];
     cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(Cfg<256, kFamFwd, 2>::THREADS);
-    cfg.dynamicSmemBytes = SplitCfg<SK>::SMEM;
+    cfg.blockDim = dim3(Cfg<BN, FAM, 2>::THREADS);
+    cfg.dynamicSmemBytes = SplitCfg<BN, FAM, SK>::SMEM;
     cfg.stream = st;
     cfg.attrs = at;
     cfg.numAttrs = conv_attrs(2 * SK, at);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, conv_splitk_kernel<SK>, a, b, a2, b2, pl.p);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, conv_splitk_kernel<BN, FAM, SK>, a, b, a2, b2, pl.p);
     if (e != cudaSuccess) {
         dbl::count_launch();
         return dbl::cuda_check(e, "conv_splitk launch");
@@ -3209,9 +3268,16 @@ int launch(const Plan& pl, const CUtensorMap& a, const CUtensorMap& b, const CUt
            int grid, cudaStream_t st)
 {
     const bool wg = pl.mode == kWgrad || pl.mode == kWgradC8;
-    if (pl.sk == 2) return launch_splitk<2>(pl, a, b, a2, b2, grid, st);
-    if (pl.sk == 4) return launch_splitk<4>(pl, a, b, a2, b2, grid, st);
-    if (pl.sk == 8) return launch_splitk<8>(pl, a, b, a2, b2, grid, st);
+    if (pl.sk > 1 && wg) {
+        if (pl.BN == 256) return pl.sk == 2   ? launch_splitk<256, kFamWgrad, 2>(pl, a, b, a2, b2, grid, st)
+                                 : pl.sk == 4 ? launch_splitk<256, kFamWgrad, 4>(pl, a, b, a2, b2, grid, st)
+                                              : launch_splitk<256, kFamWgrad, 8>(pl, a, b, a2, b2, grid, st);
+        return pl.sk == 2 ? launch_splitk<128, kFamWgrad, 2>(pl, a, b, a2, b2, grid, st)
+                          : launch_splitk<128, kFamWgrad, 4>(pl, a, b, a2, b2, grid, st);
+    }
+    if (pl.sk == 2) return launch_splitk<256, kFamFwd, 2>(pl, a, b, a2, b2, grid, st);
+    if (pl.sk == 4) return launch_splitk<256, kFamFwd, 4>(pl, a, b, a2, b2, grid, st);
+    if (pl.sk == 8) return launch_splitk<256, kFamFwd, 8>(pl, a, b, a2, b2, grid, st);
     if (pl.cg == 2) {
         if (pl.BN == 256) return wg ? launch_cfg<256, kFamWgrad, 2>(pl, a, b, a2, b2, grid, st)
                                     : launch_cfg<256, kFamFwd, 2>(pl, a, b, a2, b2, grid, st);

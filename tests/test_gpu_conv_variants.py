@@ -155,3 +155,27 @@ def test_pixel_pair_conv_matches_oracle(D, n, h, w):
     assert np.all(np.isfinite(host(dx)))
     assert max_norm_rel(host(dx), orc.conv2d_dgrad(dy, wt, x.shape, 1, 1)) <= CONV_TOL
     check_status(D)
+
+
+@pytest.mark.parametrize("n,h,c,k,r,stride", [
+    (33, 14, 64, 128, 3, 2),   # 128 columns, two pairs per tile, seven slices; a last row tile of 64
+    (33, 5, 256, 128, 3, 1),   # 128 columns, four pairs, no slices: written straight into dw
+    (65, 3, 512, 512, 3, 1),   # 256 columns, two pairs of three and two K-blocks
+    (65, 14, 256, 512, 1, 2),  # four pairs, seven slices, pairs without a K-block
+    (17, 14, 128, 256, 3, 2),  # eight pairs
+])
+def test_split_wgrad_matches_oracle(D, n, h, c, k, r, stride):
+    """Weight gradients whose tiles are shared by clusters of CTA pairs."""
+    pad = 1 if r == 3 else 0
+    shape, x, wt, p = _conv_case(D, n, h, c, k, r, stride, pad, n + c)
+    dy = bf16_values(rng(n).standard_normal((n, p, p, k)))
+    ref = orc.conv2d_wgrad(x, dy, wt.shape, stride, pad)
+    wsb = D.dbl_conv_workspace_bytes(shape, D.DBL_PASS_WGRAD)
+    dw = torch.full((k, r, r, c), float("nan"), device="cuda")
+    work, xd, dyd = ws(wsb), to_bf16_dev(x), to_bf16_dev(dy)
+    D.dbl_conv_wgrad(shape, xd, dyd, dw, False, work, wsb)
+    assert np.all(np.isfinite(host(dw)))
+    assert max_norm_rel(host(dw), ref) <= WGRAD_TOL
+    D.dbl_conv_wgrad(shape, xd, dyd, dw, True, work, wsb)
+    assert max_norm_rel(host(dw), 2 * ref) <= WGRAD_TOL
+    check_status(D)
