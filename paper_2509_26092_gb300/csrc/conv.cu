@@ -87,7 +87,7 @@ struct ConvParams {
                               // row-block weight gradient: offset of the dy strip in a stage
     int win_stages;           // row-block weight gradient: x + dy stages
     int win_bpi;              // row-block and filter-row weight gradient: K-blocks per image
-    int win_ni;               // filter-row weight gradient: images per K-block
+    int win_ni;               // filter-row weight gradient: images per K-block; bands: bands per image
     int win_cl;               // filter-row weight gradient: CTAs per cluster, which add their sums on chip
     int test_stall;           // dbl_conv_test_stall_next: block 0 never loads its first K-block
 };
@@ -1929,8 +1929,17 @@ __global__ void __launch_bounds__(kWinThreads, 1)
 // 185 75.5 -> 59.9; 24x24, batch 512 36.3 -> 28.7; 32x32, batch 64 19.2 -> 17.4.
 // Position shifts reach two rows past the dy strip and one past the x strip: those 128-byte rows
 // are the next row's columns -2, -1 and -pw, which are zeros in any strip and are written here once.
+// COL: an R x 1 filter (R = 3 or 4: the stems over their unrolled inputs).  A K-block is a band of
+// `win_Wp` columns of several output rows: without column taps a band needs no neighbouring columns,
+// and a narrow band of many rows reads few x rows twice (R - 1 per block; conv_wgwin_kernel's blocks
+// of one or two whole rows read each x row two to four times from L2).  Accumulator 0 holds taps 0
+// and 1 (x rows one band row apart), accumulator 1 taps 2 and 3, both 128 x 64.  Bound by memory;
+// against conv_wgwin_kernel, with the reduce: 4 taps, 115x112, batch 512 277.7 -> 248.7 us (6.7 TB/s),
+// 83x80 175.7 -> 136.5, 67x64 134.7 -> 92.0, batch 64 23.9 -> 17.3; 147x144, batch 185 218.4 -> 163.4;
+// 3 taps, 32x32, batch 512 36.8 -> 31.6, 24x24 27.5 -> 18.0.
 constexpr int kWgRowMaxStages = 4;
 
+template <bool COL>
 __global__ void __launch_bounds__(kWinThreads, 1)
     conv_wgrow_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmDY,
                       const ConvParams p)
@@ -1961,6 +1970,7 @@ __global__ void __launch_bounds__(kWinThreads, 1)
     }
     // the zero rows behind each strip (8 16-byte words per row), before any MMA reads them
     for (int i = threadIdx.x; i < stages * 24; i += blockDim.x) {
+        if (COL) break;  // no shifts
         const int s = i / 24, w = i % 24;
         uint8_t* dst = sgen + s * stage_bytes + (w < 8 ? xbytes + 16 * w : xalign + ybytes + 16 * (w - 8));
         *reinterpret_cast<uint4*>(dst) = make_uint4(0, 0, 0, 0);
@@ -1994,12 +2004,13 @@ __global__ void __launch_bounds__(kWinThreads, 1)
                 break;
             }
             uint8_t* dst = sgen + s * stage_bytes + (is_x ? 0 : xalign);
-            const int n = kb / bpi, h0 = (kb - n * bpi) * rows;
+            const int n = kb / bpi, rem = kb - n * bpi;
+            const int h0 = (COL ? rem / p.win_ni : rem) * rows, w0 = COL ? rem % p.win_ni * pitch : 0;
             mbar_arrive_expect_tx_elect(&full_bar[s], (uint32_t)(is_x ? xbytes : ybytes));
             if (is_x)
-                tma_load_4d_elect(dst, &tmX, &full_bar[s], 0, -p.win_pw, h0 - p.win_ph, n);
+                tma_load_4d_elect(dst, &tmX, &full_bar[s], 0, w0 - p.win_pw, h0 - p.win_ph, n);
             else
-                tma_load_4d_elect(dst, &tmDY, &full_bar[s], 0, -2, h0, n);
+                tma_load_4d_elect(dst, &tmDY, &full_bar[s], 0, COL ? w0 : -2, h0, n);
             if (++s == stages) {
                 s = 0;
                 phase ^= 1;
@@ -2012,9 +2023,10 @@ __global__ void __launch_bounds__(kWinThreads, 1)
         }
     } else if (warp == 6) {
         // ------------------------------------------------------------------ MMA issuer
-        const uint32_t idesc0 = idesc_act(BM, 192, 1u, 1u), idesc1 = idesc_act(BM, 128, 1u, 1u);
+        constexpr uint32_t kN0 = COL ? 64 : 192, kN1 = COL ? 64 : 128;
+        const uint32_t idesc0 = idesc_act(BM, kN0, 1u, 1u), idesc1 = idesc_act(BM, kN1, 1u, 1u);
         const uint64_t dA0 = smem_desc(0, (uint32_t)(pitch * 128), 1024, kSwizzle128B);
-        const uint64_t dA1 = smem_desc(0, 128, 1024, kSwizzle128B);
+        const uint64_t dA1 = COL ? dA0 : smem_desc(0, 128, 1024, kSwizzle128B);
         const uint64_t dB0 = smem_desc(0, 128, 1024, kSwizzle128B);
         const uint64_t dB1 = smem_desc(0, 256, 1024, kSwizzle128B);
         const uint32_t row2 = (uint32_t)(2 * pitch * 8);  // two rows, in 16-byte units
@@ -2030,7 +2042,7 @@ __global__ void __launch_bounds__(kWinThreads, 1)
             auto step = [&](int j, uint32_t acc) {
                 const uint32_t xj = xa + (uint32_t)(j * 128), yj = ya + (uint32_t)(j * 128);  // 16 rows of 128 bytes
                 mma_act_elect(tmem, dA0 + xj, dB0 + yj, idesc0, acc);
-                mma_act_elect(tmem + 192, dA1 + (xj + row2), dB1 + yj, idesc1, acc);
+                mma_act_elect(tmem + kN0, dA1 + (xj + row2), dB1 + yj, idesc1, acc);
             };
             step(0, kb > kb0 ? 1u : 0u);
 #pragma unroll 4
@@ -2062,8 +2074,10 @@ __global__ void __launch_bounds__(kWinThreads, 1)
         } else {
             tc_fence_after();
 #pragma unroll 1
-            for (int b = 0; b < 5; ++b) {  // 64-column blocks: one tap per half
-                const int tap = b < 3 ? half * 3 + 2 - b : half == 0 ? 6 + (b == 3 ? 2 : 0) : b == 4 ? 7 : -1;
+            for (int b = 0; b < (COL ? 2 : 5); ++b) {  // 64-column blocks: one tap per half
+                const int tap = COL     ? (2 * b + half < p.win_R ? 2 * b + half : -1)
+                                : b < 3 ? half * 3 + 2 - b
+                                        : half == 0 ? 6 + (b == 3 ? 2 : 0) : b == 4 ? 7 : -1;
                 const int m = tap * 64 + c;  // row of dW viewed as [k][(r, s, c)]
 #pragma unroll 1
                 for (int ch = 0; ch < 2; ++ch) {
@@ -2407,6 +2421,7 @@ struct Plan {
     bool res = false;    // window kernel with all weights resident in shared memory
     bool winpair = false;  // conv_winpair_kernel (64 to 64 channels, even rows)
     bool wgrow = false;  // conv_wgrow_kernel (3x3 stride-1 weight gradient, 64 channels)
+    bool wgband = false; // conv_wgrow_kernel<true> (R x 1 weight gradient, 64 channels)
     bool wgtap = false;  // conv_wgtap_kernel (3x3 stride-1 weight gradient, multiples of 128 channels)
     size_t smem = 0;     // window kernel dynamic shared memory
 };
@@ -2770,6 +2785,72 @@ bool wgtap_setup(const dbl_conv_shape* s, Plan& pl)
     return true;
 }
 
+// Band weight-gradient eligibility and geometry (conv_wgrow_kernel<true>): R x 1 filters, R = 3 or 4, at stride 1
+// without padding along W, 64 input and 64 output channels.  The band width and rows minimise the modelled time
+// of the busiest CTA: per K-block the longer of its MMAs (108 cycles per 16 positions) and its loads (40 bytes
+// per cycle), and ~100 cycles of hand-over.
+bool wgband_setup(const dbl_conv_shape* s, Plan& pl)
+{
+    const Geom g = geom(s);
+    if (g.sh != 1 || g.sw != 1 || g.pw != 0 || s->s != 1 || (s->r != 3 && s->r != 4) || s->c != 64 || s->k != 64)
+        return false;
+    const int P = s->h + 2 * g.ph - s->r + 1;
+    if (P <= 0) return false;
+    const int sms = 152;  // a fixed count: the split must not depend on the device
+    double best = 1e300;
+    ConvParams& p = pl.p;
+    for (int bands = 1; bands <= (s->w + 7) / 8; ++bands) {
+        const int bw = (s->w + bands - 1) / bands;
+        if (bw > 256 || (bands > 1 && bw == (s->w + bands - 2) / (bands - 1))) continue;
+        for (int R = 1; R <= 32 && R < P + 16; ++R) {
+            const int xrows = R + s->r - 1;
+            if ((R * bw) % 16 || R * bw > 512) continue;
+            const int xalign = (xrows * bw * 128 + 1023) / 1024 * 1024;
+            const int stage = xalign + (R * bw * 128 + 1023) / 1024 * 1024;
+            const int stages = std::min<int>(kWgRowMaxStages, (int)((kWinSmemMax - 1024) / stage));
+            // with three taps the unused half of accumulator 1 reads one band row past the x strip: into the dy strip
+            if (stages < 2 || (s->r == 3 && xalign + R * bw * 128 < (R + 3) * bw * 128)) continue;
+            const int64_t bpi = (int64_t)bands * ((P + R - 1) / R), blocks = s->n * bpi;
+            if (blocks > INT32_MAX / 4) continue;
+            const double mma = R * bw * 6.75, load = (double)(xrows + R) * bw * 128 / 40.0;
+            const double cost = (double)((blocks + sms - 1) / sms) * (std::max(mma, load) + 100.0);
+            if (cost >= best) continue;
+            best = cost;
+            p.win_Wp = bw;
+            p.win_dyrows = R;
+            p.win_srows = xrows;
+            p.win_tile = R * bw;
+            p.win_margin = xalign;
+            p.win_strip_bytes = stage;
+            p.win_stages = stages;
+            p.win_bpi = (int)bpi;
+            p.win_ni = bands;
+            p.num_kb = (int)blocks;
+            pl.smem = (size_t)stages * stage + 1024;
+        }
+    }
+    if (best == 1e300) return false;
+    pl.win = pl.wgband = true;
+    pl.BN = 64;
+    pl.mode = p.mode = kWgrad;
+    p.win_R = s->r;
+    p.win_S = 1;
+    p.win_ph = g.ph;
+    p.win_pw = 0;
+    p.win_P = P;
+    p.win_Q = s->w;
+    p.M = s->r * 64;
+    p.Ncols = 64;
+    p.m_tiles = p.n_tiles = 1;
+    p.gN = s->n;
+    // one contiguous range of K-blocks per CTA
+    const int splits = grid_size(p.num_kb);
+    p.kb_per_split = (p.num_kb + splits - 1) / splits;
+    p.zdim = (p.num_kb + p.kb_per_split - 1) / p.kb_per_split;
+    pl.ws_main = p.zdim > 1 ? (size_t)p.zdim * p.M * 64 * sizeof(float) : 0;
+    return true;
+}
+
 // Window weight-gradient eligibility and geometry (see conv_wgwin_kernel):
 // stride 1, 64 input and 64 output channels, three or four taps (the stems), padded
 // rows of 10..256 positions.
@@ -2934,7 +3015,7 @@ int make_plan(const dbl_conv_shape* s, int pass, Plan& pl)
         pl.ws_main = (size_t)kMaxGrid * 2 * s->k * sizeof(float);
     } else if (pass == DBL_PASS_DGRAD && s->c % 64 == 0 && (winpair_setup(s, true, pl) || win_setup(s, s->k, s->c, true, pl))) {
         pl.mode = p.mode = kDgrad;
-    } else if (pass == DBL_PASS_WGRAD && (wgrow_setup(s, pl) || wgtap_setup(s, pl) || wgwin_setup(s, pl))) {
+    } else if (pass == DBL_PASS_WGRAD && (wgrow_setup(s, pl) || wgtap_setup(s, pl) || wgband_setup(s, pl) || wgwin_setup(s, pl))) {
         // conv_wgrow_kernel, conv_wgtap_kernel, conv_wgwin_kernel
     } else if (pass == DBL_PASS_FWD) {
         pl.mode = p.mode = c8 ? kFwdC8 : kFwd;
@@ -3711,13 +3792,14 @@ int dbl_conv_wgrad(const dbl_conv_shape* s, const void* x, const void* dy, float
     const bool sliced = pl.p.zdim > 1;
     if (pl.win) {
         // rows (and images) per copy
-        const int xr = pl.wgrow || pl.wgtap ? pl.p.win_srows : 1;
-        const int yr = pl.wgrow ? pl.p.win_dyrows : xr, ni = pl.wgtap ? pl.p.win_ni : 1;
+        const int xr = pl.wgrow || pl.wgband || pl.wgtap ? pl.p.win_srows : 1;
+        const int yr = pl.wgrow || pl.wgband ? pl.p.win_dyrows : xr, ni = pl.wgtap ? pl.p.win_ni : 1;
         if ((rc = enc_win_rows(&ta, x, s->n, s->h, s->w, s->c, pl.p.win_Wp, xr, ni))) return rc;
         if ((rc = enc_win_rows(&tb, dy, s->n, P, Q, s->k, pl.p.win_Wp, yr, ni))) return rc;
         pl.p.out = sliced ? ws : static_cast<void*>(dw);
         pl.p.wg_accumulate = accumulate;
-        if ((rc = pl.wgrow   ? launch_wgwin<conv_wgrow_kernel>(pl, ta, tb, kWinThreads, st)
+        if ((rc = pl.wgrow   ? launch_wgwin<conv_wgrow_kernel<false>>(pl, ta, tb, kWinThreads, st)
+                  : pl.wgband ? launch_wgwin<conv_wgrow_kernel<true>>(pl, ta, tb, kWinThreads, st)
                   : pl.wgtap ? launch_wgwin<conv_wgtap_kernel>(pl, ta, tb, kWgTapThreads, st)
                              : launch_wgwin<conv_wgwin_kernel<2>>(pl, ta, tb, kWinThreads, st)))
             return rc;

@@ -48,6 +48,37 @@ def test_row_block_wgrad_matches_oracle(D, n, h, w, pad):
     check_status(D)
 
 
+@pytest.mark.parametrize("n,h,w,r,ph", [
+    (1, 4, 16, 4, 0),    # one output row, one K-block's width
+    (1, 5, 1, 4, 0),     # the narrowest rows
+    (2, 9, 70, 4, 0),    # a last band past the image
+    (3, 14, 37, 3, 1),   # odd widths, padded rows, the unused half of three taps
+    (1, 40, 23, 3, 0),   # a last block of rows past the image
+    (2, 7, 256, 4, 2),   # the widest rows that one band could hold
+    (1, 4, 300, 3, 1),   # wider than any band
+    (64, 35, 32, 4, 0),  # several K-blocks per CTA
+])
+def test_band_wgrad_matches_oracle(D, n, h, w, r, ph):
+    g = rng(1000 * n + w)
+    x = bf16_values(g.standard_normal((n, h, w, 64)))
+    p = h + 2 * ph - r + 1
+    dy = bf16_values(g.standard_normal((n, p, w, 64)))
+    xp = np.pad(x.astype(np.float64), ((0, 0), (ph, ph), (0, 0), (0, 0)))
+    d2 = dy.astype(np.float64).reshape(-1, 64)
+    ref = np.stack([d2.T @ xp[:, t:t + p].reshape(-1, 64) for t in range(r)], axis=1)[:, :, None]
+    shape = D.conv_shape(n, h, w, 64, 64, r, 1, ph, s=1, stride_w=1, pad_w=0)
+    assert D.dbl_conv_plan(shape, D.DBL_PASS_WGRAD).kernel == D.DBL_KERNEL_WINDOW_WGRAD
+    wsb = D.dbl_conv_workspace_bytes(shape, D.DBL_PASS_WGRAD)
+    dw = torch.full((64, r, 1, 64), float("nan"), device="cuda")
+    work, xd, dyd = ws(wsb), to_bf16_dev(x), to_bf16_dev(dy)
+    D.dbl_conv_wgrad(shape, xd, dyd, dw, False, work, wsb)
+    assert np.all(np.isfinite(host(dw)))
+    assert max_norm_rel(host(dw), ref) <= WGRAD_TOL
+    D.dbl_conv_wgrad(shape, xd, dyd, dw, True, work, wsb)
+    assert max_norm_rel(host(dw), 2 * ref) <= WGRAD_TOL
+    check_status(D)
+
+
 # 16-bit outputs: one rounding of the result, at most 2^-8 of its size (bf16), and the fp32 sums' error
 CONV_TOL = 4e-3
 
