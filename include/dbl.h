@@ -308,6 +308,17 @@ DBL_API int dbl_maxpool_fwd(int32_t n, int32_t h, int32_t w, int32_t c, const vo
 DBL_API int dbl_maxpool_bwd(int32_t n, int32_t h, int32_t w, int32_t c, const void* dy_bf16, const void* dy2_bf16,
                     const uint8_t* argmax, void* dx_bf16, void* stream);
 
+/* Backward of dbl_bn_relu_maxpool_fwd: dbl_maxpool_bwd of dp [+ dp2] into da
+ * [n,h,w,c] (written), then dbl_bn_relu_fused_bwd of da with the mask
+ * recomputed from x (out = NULL): dx [n,h,w,c], dgamma, dbeta.  The pool's
+ * gather and the BatchNorm's channel sums are one pass.  ws: at least
+ * dbl_bn_workspace_bytes(shape). */
+DBL_API int dbl_maxpool_bn_relu_bwd(const dbl_bn_shape* shape, int32_t n, int32_t h, int32_t w, const void* dp_bf16,
+                                    const void* dp2_bf16 /* or NULL */, const uint8_t* argmax, const void* x_bf16,
+                                    const float* gamma, const float* beta, const float* save_mean,
+                                    const float* save_invstd, void* da_bf16, void* dx_bf16, float* dgamma,
+                                    float* dbeta, void* ws, size_t ws_bytes, void* stream);
+
 /* ========================================================================
  * Head forward + backward in one call: global average pooling (the pooling
  * that makes the network resolution-agnostic, Sec. 6), one fully connected

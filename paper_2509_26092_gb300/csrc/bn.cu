@@ -438,6 +438,148 @@ __global__ void __launch_bounds__(kThreads, kReduceBlocksPerSM)
     }
 }
 
+// Max-pool backward and the reduce pass of the BatchNorm + ReLU before the pool, in one: a step takes
+// 2x2 blocks of pixels (i, j) in place of rows, gathers their gradient from the windows (i..i+1, j..j+1)
+// (maxpool_bwd_kernel's taps and order), stores it as da for the apply pass, and sums the stored values
+// masked by y: at most kPoolParts partials, each over blocks in a fixed order, last to first.  Against
+// its own memory traffic (two tensors of the pool's input and a half) at 0.85 of the copy bandwidth; the
+// gather's instructions fill the rest.  Pool pass, reduce, finalize and apply with two gradients -> with this
+// (us): 112x112x64, batch 512 917 -> 740 (with 256 partials in CTAs of 256 threads, two on some SMs, 853;
+// one channel per operation 781; walking runs of rows, the lower windows kept and the next row copied ahead
+// with cp.async, 798), batch 64 125 -> 104; 80x80, batch 512 472 -> 384; 144x144, batch 185 551 -> 447;
+// 64x64, batch 64 44.7 -> 39.1, batch 16 19.2 -> 17.3.
+constexpr int kPoolThreads = 512;
+constexpr int64_t kPoolParts = 152;  // one CTA per SM
+__global__ void __launch_bounds__(kPoolThreads, 1)
+    bn_pool_bwd_reduce_kernel(const act_t* __restrict__ dp, const act_t* __restrict__ dp2,
+                              const uint8_t* __restrict__ arg, const act_t* __restrict__ y, int n, int H, int W,
+                              int C, const float* __restrict__ gamma, const float* __restrict__ beta,
+                              const float* __restrict__ mean, const float* __restrict__ invstd, int nblk,
+                              float* __restrict__ partial, act_t* __restrict__ da)
+{
+    extern __shared__ float4 chan4[];
+    float* chan = reinterpret_cast<float*>(chan4);  // [mean, scale, shift][C]
+    for (int c = threadIdx.x; c < C; c += kPoolThreads) chan[c] = mean[c];
+    stage_relu<kMaskY>(gamma, beta, mean, invstd, 0, C, chan + C);
+    __syncthreads();
+    const int groups = C / 8;
+    const int g = threadIdx.x % groups;
+    const int rstep = kPoolThreads / groups;
+    ReluMask<kMaskY> rm;
+    rm.init(chan + C, C, 8 * g);
+    float mu[8];
+    load8(chan + 8 * g, mu);
+    float2 sc2[4], sh2[4], mu2[4];  // two channels per operation
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        sc2[k] = make_float2(rm.sc[2 * k], rm.sc[2 * k + 1]);
+        sh2[k] = make_float2(rm.sh[2 * k], rm.sh[2 * k + 1]);
+        mu2[k] = make_float2(-mu[2 * k], -mu[2 * k + 1]);
+    }
+    __shared__ float red[kPoolThreads][17];
+    const int P = (H + 1) / 2, Q = (W + 1) / 2;
+    const int total = n * P * Q, cstep = nblk * rstep;
+    const int step_j = cstep % Q, step_i = cstep / Q % P, step_b = cstep / Q / P;
+    const int win_row = Q * groups, px_row = W * groups;
+    for (int blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
+        float2 sg[4] = {}, sgx[4] = {};
+        int r = blk * rstep + threadIdx.x / groups;
+        const int first = max(total - 1 - r, 0);
+        int j = first % Q, i = first / Q % P, b = first / Q / P;
+        for (; r < total; r += cstep) {
+            const bool r1 = i + 1 < P, c1 = j + 1 < Q;              // windows below and to the right
+            const bool h1 = 2 * i + 1 < H, w1 = 2 * j + 1 < W;      // pixels
+            const int o = ((b * P + i) * Q + j) * groups + g;       // window (i, j)
+            const int v = ((b * H + 2 * i) * W + 2 * j) * groups + g;  // pixel (2i, 2j)
+            const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+            uint4 gv[4], gv2[4], yv[4];
+            uint2 av[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const bool ok = (t < 2 || r1) && (t % 2 == 0 || c1);
+                const int ot = o + (t >> 1) * win_row + (t & 1) * groups;
+                gv[t] = ok ? __ldg(reinterpret_cast<const uint4*>(dp) + ot) : zero;
+                gv2[t] = ok && dp2 ? __ldg(reinterpret_cast<const uint4*>(dp2) + ot) : zero;
+                av[t] = ok ? __ldg(reinterpret_cast<const uint2*>(arg) + ot) : make_uint2(~0u, ~0u);
+                yv[t] = (t < 2 || h1) && (t % 2 == 0 || w1)
+                            ? __ldg(reinterpret_cast<const uint4*>(y) + v + (t >> 1) * px_row + (t & 1) * groups)
+                            : zero;
+            }
+            // window t's gradient: dp [+ dp2]
+            auto window = [&](int t, float (&f)[8]) {
+                unpack8(gv[t], f);
+                if (dp2) {
+                    float f2[8];
+                    unpack8(gv2[t], f2);
+#pragma unroll
+                    for (int k = 0; k < 8; k += 2) {
+                        const float2 t2 = dbl::dev::add2(make_float2(f[k], f[k + 1]), make_float2(f2[k], f2[k + 1]));
+                        f[k] = t2.x, f[k + 1] = t2.y;
+                    }
+                }
+            };
+            auto pixel = [&](int t, const float (&acc)[8]) {
+                const uint4 packed = pack8(acc);
+                reinterpret_cast<uint4*>(da)[v + (t >> 1) * px_row + (t & 1) * groups] = packed;
+                float gg[8], yy[8];
+                unpack8(packed, gg);
+                unpack8(yv[t], yy);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const float2 y2 = make_float2(yy[2 * k], yy[2 * k + 1]);
+                    const float2 pre = dbl::dev::fma2(y2, sc2[k], sh2[k]);
+                    const float2 g2 = make_float2(pre.x > 0.f ? gg[2 * k] : 0.f, pre.y > 0.f ? gg[2 * k + 1] : 0.f);
+                    sg[k] = dbl::dev::add2(sg[k], g2);
+                    sgx[k] = dbl::dev::fma2(g2, dbl::dev::add2(y2, mu2[k]), sgx[k]);
+                }
+            };
+            float f[8], acc01[8] = {}, acc10[8] = {}, acc11[8] = {};
+            window(0, f);
+            {
+                float acc00[8] = {};
+                dbl::dev::add_if_tap(acc00, f, av[0], 4);
+                pixel(0, acc00);
+            }
+            dbl::dev::add_if_tap(acc01, f, av[0], 5);
+            dbl::dev::add_if_tap(acc10, f, av[0], 7);
+            dbl::dev::add_if_tap(acc11, f, av[0], 8);
+            window(1, f);
+            dbl::dev::add_if_tap(acc01, f, av[1], 3);
+            dbl::dev::add_if_tap(acc11, f, av[1], 6);
+            if (w1) pixel(1, acc01);
+            window(2, f);
+            dbl::dev::add_if_tap(acc10, f, av[2], 1);
+            dbl::dev::add_if_tap(acc11, f, av[2], 2);
+            if (h1) pixel(2, acc10);
+            window(3, f);
+            dbl::dev::add_if_tap(acc11, f, av[3], 0);
+            if (h1 && w1) pixel(3, acc11);
+            // cstep blocks back
+            j -= step_j;
+            i -= step_i;
+            b -= step_b;
+            if (j < 0) j += Q, --i;
+            if (i < 0) i += P, --b;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            red[threadIdx.x][2 * k] = sg[k].x;
+            red[threadIdx.x][2 * k + 1] = sg[k].y;
+            red[threadIdx.x][8 + 2 * k] = sgx[k].x;
+            red[threadIdx.x][8 + 2 * k + 1] = sgx[k].y;
+        }
+        __syncthreads();
+        float* p = partial + (int64_t)blk * 2 * C;
+        for (int e = threadIdx.x; e < 2 * C; e += kPoolThreads) {  // one sum per thread, blocks in order
+            const int x = e >= C, c = e - x * C;
+            float t = 0.f;
+            for (int q = c / 8; q < rstep * groups; q += groups) t += red[q][8 * x + c % 8];
+            p[e] = x ? t * invstd[c] : t;
+        }
+        __syncthreads();
+    }
+}
+
 // dy = k1*(g - sum(g)/n - xhat*sum(g*xhat)/n), xhat = (y - mean)*invstd, as A*g + B*y + C;
 // inv_n = 1/count, divided on the host.
 __device__ __forceinline__ void bwd_coefficients(double sg, double sgx, double inv_n, float gamma, float invstd,
@@ -721,6 +863,26 @@ int64_t bwd_blocks(int64_t count, int C)
     return b < 1 ? 1 : b > kMaxBwdParts ? kMaxBwdParts : b;
 }
 
+// The passes after the reduce: fixed-order finalize and apply.
+template <int MASK>
+int bwd_finish(const dbl_bn_shape* s, const void* dout, const void* dout2, const void* y, const void* out,
+               const float* gamma, const float* beta, const float* mean, const float* invstd, void* dy, float* dgamma,
+               float* dbeta, float* partial, float* coef, int64_t nblk, cudaStream_t st)
+{
+    using namespace dbl;
+    const int C = s->c;
+    auto bd = [](const void* p) { return static_cast<const act_t*>(p); };
+    bn_bwd_finalize_kernel<<<(C + dbl::dev::kPartialsChannels - 1) / dbl::dev::kPartialsChannels,
+                             dbl::dev::kPartialsThreads, 0, st>>>(partial, (int)nblk, C, 1.0 / (double)s->count, gamma,
+                                                                  mean, invstd, dgamma, dbeta, coef);
+    if (int rc = launch_check("bn_bwd_finalize launch")) return rc;
+    bn_bwd_apply_kernel<MASK><<<bn_grid(s->count * C / 8, kBwdBlocksPerSM), kThreads,
+                                (MASK == kMaskY ? 5 : 3) * C * sizeof(float), st>>>(
+        bd(dout), bd(dout2), bd(out), bd(y), (int)s->count, C, gamma, beta, mean, invstd, coef,
+        static_cast<act_t*>(dy), nullptr);
+    return launch_check("bn_bwd_apply launch");
+}
+
 template <int MASK>
 int bwd_launch_mask(const dbl_bn_shape* s, const void* dout, const void* dout2, const void* y, const void* out,
                     const float* gamma, const float* beta, const float* mean, const float* invstd, void* dy,
@@ -765,21 +927,12 @@ int bwd_launch_mask(const dbl_bn_shape* s, const void* dout, const void* dout2, 
         bn_bwd_reduce_kernel<MASK, false><<<reduce_grid(nblk), kThreads, smem_r, st>>>(
             bd(dout), bd(dout2), bd(out), bd(y), (int)s->count, C, gamma, beta, mean, invstd, (int)nblk, partial,
             nullptr);
-    int rc = launch_check("bn_bwd_reduce launch");
-    if (rc) return rc;
-    bn_bwd_finalize_kernel<<<(C + dbl::dev::kPartialsChannels - 1) / dbl::dev::kPartialsChannels,
-                             dbl::dev::kPartialsThreads, 0, st>>>(partial, (int)nblk, C, 1.0 / (double)s->count,
-                                                                         gamma, mean, invstd, dgamma, dbeta, coef);
-    if ((rc = launch_check("bn_bwd_finalize launch"))) return rc;
+    if (int rc = launch_check("bn_bwd_reduce launch")) return rc;
     if (g_store)
-        bn_bwd_apply_kernel<kMaskNone><<<bn_grid(s->count * C / 8, kBwdBlocksPerSM), kThreads, 3 * C * sizeof(float), st>>>(
-            g_store, nullptr, nullptr, bd(y), (int)s->count, C, gamma, beta, mean, invstd, coef,
-            static_cast<act_t*>(dy), nullptr);
-    else
-        bn_bwd_apply_kernel<MASK><<<bn_grid(s->count * C / 8, kBwdBlocksPerSM), kThreads, (MASK == kMaskY ? 5 : 3) * C * sizeof(float), st>>>(
-            bd(dout), bd(dout2), bd(out), bd(y), (int)s->count, C, gamma, beta, mean, invstd, coef,
-            static_cast<act_t*>(dy), nullptr);
-    return launch_check("bn_bwd_apply launch");
+        return bwd_finish<kMaskNone>(s, g_store, nullptr, y, nullptr, gamma, beta, mean, invstd, dy, dgamma, dbeta,
+                                     partial, coef, nblk, st);
+    return bwd_finish<MASK>(s, dout, dout2, y, out, gamma, beta, mean, invstd, dy, dgamma, dbeta, partial, coef, nblk,
+                            st);
 }
 
 // The three passes of the backward pass (reduce, fixed-order finalize, apply),
@@ -881,6 +1034,45 @@ int dbl_bn_relu_fused_parts(const dbl_bn_shape* s, const void* y, const float* p
         static_cast<act_t*>(out), (int)s->count, s->c, s->relu, apply_reversed(s), gamma, beta,
         save_mean, save_invstd);
     return launch_check("bn_relu_fused_parts launch");
+}
+
+int dbl_maxpool_bn_relu_bwd(const dbl_bn_shape* s, int32_t n, int32_t h, int32_t w, const void* dp, const void* dp2,
+                            const uint8_t* argmax, const void* x, const float* gamma, const float* beta,
+                            const float* save_mean, const float* save_invstd, void* da, void* dx, float* dgamma,
+                            float* dbeta, void* ws, size_t ws_bytes, void* stream)
+{
+    using namespace dbl;
+    int rc = check_shape(s, "maxpool_bn_relu_bwd");
+    if (rc) return rc;
+    if (n <= 0 || h <= 0 || w <= 0 || s->count != (int64_t)n * h * w || !s->relu)
+        return set_error(DBL_ERR_INVALID, "maxpool_bn_relu_bwd: shape must be [n*h*w, c] with relu set");
+    if (!dp || !argmax || !x || !da || !dx || !gamma || !beta || !save_mean || !save_invstd || !dgamma || !dbeta)
+        return set_error(DBL_ERR_INVALID, "maxpool_bn_relu_bwd: null pointer");
+    if (!aligned16(dp) || (dp2 && !aligned16(dp2)) || !aligned16(x) || !aligned16(da) || !aligned16(dx) ||
+        (reinterpret_cast<uintptr_t>(argmax) & 7))
+        return set_error(DBL_ERR_INVALID, "maxpool_bn_relu_bwd: misaligned pointer");
+    const size_t need = dbl_bn_workspace_bytes(s);
+    if (!ws || ws_bytes < need)
+        return set_error(DBL_ERR_WORKSPACE, "maxpool_bn_relu_bwd: workspace %zu < %zu bytes", ws_bytes, need);
+    const int C = s->c;
+    int64_t nblk = bwd_blocks(s->count, C);
+    float* partial = static_cast<float*>(ws);
+    float* coef = partial + nblk * 2 * C;
+    cudaStream_t st = as_stream(stream);
+    // small: the pool pass, then the backward in one launch (above 1024 channels the sums' staging and the
+    // channel constants do not fit in 48 KB of shared memory)
+    if (bwd_cluster(s->count, C, false) || C > 1024) {
+        if ((rc = dbl_maxpool_bwd(n, h, w, C, dp, dp2, argmax, da, stream))) return rc;
+        return bwd_launch(s, da, nullptr, x, nullptr, gamma, beta, save_mean, save_invstd, dx, nullptr, dgamma, dbeta,
+                          partial, coef, nblk, st);
+    }
+    nblk = std::min(nblk, kPoolParts);
+    bn_pool_bwd_reduce_kernel<<<reduce_grid(nblk), kPoolThreads, 3 * C * sizeof(float), st>>>(
+        static_cast<const act_t*>(dp), static_cast<const act_t*>(dp2), argmax, static_cast<const act_t*>(x), n, h, w, C,
+        gamma, beta, save_mean, save_invstd, (int)nblk, partial, static_cast<act_t*>(da));
+    if ((rc = launch_check("bn_pool_bwd_reduce launch"))) return rc;
+    return bwd_finish<kMaskY>(s, da, nullptr, x, nullptr, gamma, beta, save_mean, save_invstd, dx, dgamma, dbeta,
+                              partial, coef, nblk, st);
 }
 
 size_t dbl_bn_workspace_bytes(const dbl_bn_shape* s)

@@ -995,6 +995,17 @@ __host__ __device__ constexpr uint32_t idesc_act(uint32_t M, uint32_t N, uint32_
            | (a_mn << 15) | (b_mn << 16) | ((N >> 3) << 17) | ((M >> 4) << 24);
 }
 
+// Max-pool backward: dst[k] += src[k] where byte k of the argmax word pair equals tap (fp32; a
+// skipped term leaves dst as it is)
+__device__ __forceinline__ void add_if_tap(float (&dst)[8], const float (&src)[8], uint2 a, uint32_t tap)
+{
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const uint32_t byte = ((k < 4 ? a.x : a.y) >> (8 * (k & 3))) & 0xffu;
+        if (byte == tap) dst[k] += src[k];
+    }
+}
+
 }  // namespace dev
 }  // namespace dbl
 

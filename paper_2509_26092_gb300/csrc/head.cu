@@ -354,17 +354,6 @@ __global__ void __launch_bounds__(kPoolThreads, 2)
     }
 }
 
-// dst[k] += src[k] where byte k of the argmax word pair equals tap (fp32; a
-// skipped term leaves dst as it is)
-__device__ __forceinline__ void add_if_tap(float (&dst)[8], const float (&src)[8], uint2 a, uint32_t tap)
-{
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        const uint32_t byte = ((k < 4 ? a.x : a.y) >> (8 * (k & 3))) & 0xffu;
-        if (byte == tap) dst[k] += src[k];
-    }
-}
-
 // Gather form over 2x2 blocks of input pixels: block (i, j) = rows 2i..2i+1,
 // cols 2j..2j+1 is covered by windows (i..i+1, j..j+1); window (p, q) reaches
 // input (h, w) at tap (h - 2p + 1, w - 2q + 1).  So pixel (2i, 2j) takes tap 4
@@ -415,10 +404,10 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
                 for (int k = 0; k < 8; ++k) f[k] += f2[k];
             }
-            add_if_tap(acc00, f, av[0], 4);
-            add_if_tap(acc01, f, av[0], 5);
-            add_if_tap(acc10, f, av[0], 7);
-            add_if_tap(acc11, f, av[0], 8);
+            dbl::dev::add_if_tap(acc00, f, av[0], 4);
+            dbl::dev::add_if_tap(acc01, f, av[0], 5);
+            dbl::dev::add_if_tap(acc10, f, av[0], 7);
+            dbl::dev::add_if_tap(acc11, f, av[0], 8);
             *reinterpret_cast<uint4*>(px) = pack8(acc00);
         }
         {
@@ -429,8 +418,8 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
                 for (int k = 0; k < 8; ++k) f[k] += f2[k];
             }
-            add_if_tap(acc01, f, av[1], 3);
-            add_if_tap(acc11, f, av[1], 6);
+            dbl::dev::add_if_tap(acc01, f, av[1], 3);
+            dbl::dev::add_if_tap(acc11, f, av[1], 6);
             if (w1) *reinterpret_cast<uint4*>(px + C) = pack8(acc01);
         }
         {
@@ -441,8 +430,8 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
                 for (int k = 0; k < 8; ++k) f[k] += f2[k];
             }
-            add_if_tap(acc10, f, av[2], 1);
-            add_if_tap(acc11, f, av[2], 2);
+            dbl::dev::add_if_tap(acc10, f, av[2], 1);
+            dbl::dev::add_if_tap(acc11, f, av[2], 2);
             if (h1) *reinterpret_cast<uint4*>(px + px_row) = pack8(acc10);
         }
         {
@@ -453,7 +442,7 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
                 for (int k = 0; k < 8; ++k) f[k] += f2[k];
             }
-            add_if_tap(acc11, f, av[3], 0);
+            dbl::dev::add_if_tap(acc11, f, av[3], 0);
             if (h1 && w1) *reinterpret_cast<uint4*>(px + px_row + C) = pack8(acc11);
         }
         j += step_j;

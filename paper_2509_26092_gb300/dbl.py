@@ -123,6 +123,8 @@ def lib(p=None):
             "dbl_bn_relu_fused_bwd_noalloc": (ctypes.c_int, [ctypes.POINTER(BnShape)] + [_V] * 13),
             "dbl_maxpool_fwd": (ctypes.c_int, [_I32] * 4 + [_V, _V, _V, _V]),
             "dbl_maxpool_bwd": (ctypes.c_int, [_I32] * 4 + [_V, _V, _V, _V, _V]),
+            "dbl_maxpool_bn_relu_bwd": (ctypes.c_int, [ctypes.POINTER(BnShape), _I32, _I32, _I32] + [_V] * 13
+                                        + [_SZ, _V]),
             "dbl_bn_relu_maxpool_fwd": (ctypes.c_int, [ctypes.POINTER(BnShape), _I32, _I32, _I32] + [_V] * 10),
             "dbl_head_workspace_bytes": (_SZ, [_I32, _I32, _I32]),
             "dbl_head_fwd_bwd": (ctypes.c_int, [_I32] * 4 + [_V] * 8 + [_V, _SZ, _V]),
@@ -317,6 +319,14 @@ def dbl_maxpool_fwd(n, h, w, c, x, y, argmax, stream=None):
 
 def dbl_maxpool_bwd(n, h, w, c, dy, dy2, argmax, dx, stream=None):
     _check(lib().dbl_maxpool_bwd(n, h, w, c, _ptr(dy), _ptr(dy2), _ptr(argmax), _ptr(dx), _stream(stream)))
+
+
+def dbl_maxpool_bn_relu_bwd(shape, n, h, w, dp, dp2, argmax, x, gamma, beta, save_mean, save_invstd, da, dx, dgamma,
+                            dbeta, ws, ws_bytes, stream=None):
+    """dbl_maxpool_bwd into da, then dbl_bn_relu_fused_bwd of da with the mask from x, in one pass fewer."""
+    _check(lib().dbl_maxpool_bn_relu_bwd(ctypes.byref(shape), n, h, w, _ptr(dp), _ptr(dp2), _ptr(argmax), _ptr(x),
+                                         _ptr(gamma), _ptr(beta), _ptr(save_mean), _ptr(save_invstd), _ptr(da),
+                                         _ptr(dx), _ptr(dgamma), _ptr(dbeta), _ptr(ws), ws_bytes, _stream(stream)))
 
 
 def dbl_head_workspace_bytes(n, c, classes):

@@ -521,9 +521,9 @@ class Worker:
                 dout, dout2 = d["din"], d["din2"]
         bns = D.bn_shape(B * self.stem_hw ** 2, st.cout, eps, True)
         if spec.variant == "imagenet":
-            D.dbl_maxpool_bwd(B, self.stem_hw, self.stem_hw, st.cout, dout, dout2, self.pool_arg, self.stem_da, s)
-            D.dbl_bn_relu_fused_bwd(bns, self.stem_da, None, self.stem_y, None, pv("bn1.g"), s_mean, s_istd,
-                                    self.stem_dy, None, gv("bn1.g"), gv("bn1.b"), ws, wsb, s, beta=pv("bn1.b"))
+            D.dbl_maxpool_bn_relu_bwd(bns, B, self.stem_hw, self.stem_hw, dout, dout2, self.pool_arg, self.stem_y,
+                                      pv("bn1.g"), pv("bn1.b"), s_mean, s_istd, self.stem_da, self.stem_dy,
+                                      gv("bn1.g"), gv("bn1.b"), ws, wsb, s)
         else:
             D.dbl_bn_relu_fused_bwd(bns, dout, dout2, self.stem_y, None, pv("bn1.g"), s_mean, s_istd,
                                     self.stem_dy, None, gv("bn1.g"), gv("bn1.b"), ws, wsb, s, beta=pv("bn1.b"))

@@ -43,3 +43,51 @@ def test_large_pool_equals_bn_then_maxpool(D, n, h, w, c):
         got.append((a, arg))
     assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
     check_status(D)
+
+
+@pytest.mark.parametrize("n,h,w,c,two", [
+    (1, 1, 1, 64, False),     # one pixel: the two passes
+    (5, 51, 51, 64, True),    # the smallest general size: odd sides, partials with one block or none
+    (3, 140, 71, 64, True),   # even and odd sides
+    (2, 97, 200, 256, False),  # eight blocks per step
+    (2, 41, 80, 1024, False),  # the most channels
+    (1, 85, 80, 2048, False),  # the two passes
+    (40, 60, 62, 8, True),    # one channel group
+    (33, 112, 112, 64, True),  # several steps per thread
+])
+def test_pool_bn_backward_equals_two_steps(D, n, h, w, c, two):
+    """da bit for bit; dx, dgamma and dbeta up to the order of the channel sums."""
+    g = torch.Generator(device="cuda").manual_seed(n + h)
+    normal = lambda *s: torch.empty(s, device="cuda").normal_(0.1, 1.0, generator=g)
+    p, q = (h - 1) // 2 + 1, (w - 1) // 2 + 1
+    x = normal(n, h, w, c).to(torch.bfloat16)
+    dp, dp2 = normal(n, p, q, c).to(torch.bfloat16), normal(n, p, q, c).to(torch.bfloat16) if two else None
+    gamma, beta = normal(c) + 1.0, normal(c)
+    shape = D.bn_shape(n * h * w, c, 1e-5, True)
+    s1, s2, mean, istd = (torch.empty(c, device="cuda") for _ in range(4))
+    D.dbl_bn_stats(shape, x, s1, s2)
+    pooled = torch.empty((n, p, q, c), dtype=torch.bfloat16, device="cuda")
+    arg = torch.empty((n, p, q, c), dtype=torch.uint8, device="cuda")
+    D.dbl_bn_relu_maxpool_fwd(shape, n, h, w, x, s1, s2, gamma, beta, mean, istd, pooled, arg)
+    wsb = D.dbl_bn_workspace_bytes(shape)
+    got = []
+    for fused in (False, True):
+        work = torch.full((wsb // 4,), float("nan"), device="cuda")
+        da, dx = (torch.full((n, h, w, c), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+        dg, db = (torch.full((c,), float("nan"), device="cuda") for _ in range(2))
+        if fused:
+            D.dbl_maxpool_bn_relu_bwd(shape, n, h, w, dp, dp2, arg, x, gamma, beta, mean, istd, da, dx, dg, db, work, wsb)
+        else:
+            D.dbl_maxpool_bwd(n, h, w, c, dp, dp2, arg, da)
+            D.dbl_bn_relu_fused_bwd(shape, da, None, x, None, gamma, mean, istd, dx, None, dg, db, work, wsb, beta=beta)
+        got.append((da, dx, dg, db))
+    (da0, dx0, dg0, db0), (da1, dx1, dg1, db1) = got
+    assert torch.equal(da0, da1)
+    # fp32 sums of the same terms in two orders: chains of at most 2 * 33 * 112 * 112 / (256 * 32) additions per
+    # thread and 32 more per partial lose at most 2 * (101 + 32) * 2^-24 of the sum of the terms' sizes
+    m = da0.float().abs() * (x.float() - mean).mul(istd).abs().clamp(min=1.0)
+    bound = 2 * 133 * 2.0 ** -24 * m.sum((0, 1, 2)) + 1e-30
+    assert torch.all((dg0 - dg1).abs() <= bound) and torch.all((db0 - db1).abs() <= bound)
+    # their share in dx is far below its rounding: half a unit of bf16 is at most 2^-8 of the value
+    assert torch.all((dx0.float() - dx1.float()).abs() <= 2.0 ** -7 * dx0.float().abs() + 1e-5 * dx0.float().abs().max())
+    check_status(D)
