@@ -2,7 +2,9 @@
 // ResNet-18 (Sec. 5.1.1; the gradients are those of the batch-mean loss of
 // Eq. 1) as implicit GEMMs on the sm_103a tensor cores.
 //
-// One kernel template serves every pass.  A CTA owns a 128 x BN tile of the
+// conv_igemm_kernel serves every pass; conv_splitk_kernel is its form for shapes with fewer tiles than
+// CTA pairs, and the window, pixel-pair, row-block and filter-row kernels further down replace it
+// where a stride-1 pass can read shifted rows of one strip.  A CTA owns a 128 x BN tile of the
 // GEMM result D, accumulated in tensor memory (TMEM) by tcgen05.mma with bf16
 // operands and fp32 accumulation:
 //
@@ -15,10 +17,10 @@
 // im2col-mode tensor maps (the bounding box handles zero padding, stride and
 // the ragged tail of the last tile), the other side with tiled tensor maps,
 // all with 128-byte swizzling (no swizzle for the 8-channel stem input).
-// Warp roles: warp 4 issues TMA loads into a STAGES-deep ring guarded by
-// full/empty mbarriers, warp 5 allocates TMEM and issues the MMAs (one thread),
-// warps 0-3 drain TMEM to global memory (bf16 rows plus BatchNorm channel
-// statistics for fwd, fp32 split-K partials for wgrad).
+// Warp roles: two producer warps issue TMA loads into a ring of stages guarded by
+// full/empty mbarriers, one warp allocates TMEM and issues the MMAs (one thread), and
+// the first four or eight warps drain TMEM to global memory (bf16 rows plus BatchNorm
+// channel statistics for fwd, fp32 split-K partials for wgrad).
 //
 // Stride-2 data gradients are split into the 4 output phases (h mod 2,
 // w mod 2); each phase is a stride-1 correlation with the taps of matching
@@ -1080,18 +1082,18 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, 2>::THREADS, 1)
 // address, so a start at any 128-byte row reads the rows that TMA wrote.  Rows
 // with h >= H or w >= W are computed and not stored (the padding's share of
 // the work: 7% at 56x56, 13% at 28x28).
-// Warp roles: warp 4 loads strips (two buffers), warp 5 loads weights (all
-// nine taps once per CTA when they fit, RES; else a ring of per-tap tiles),
-// warp 6 issues the MMAs, warps 0-3 drain TMEM as in conv_igemm_kernel.
+// Warp roles (WinCfg): a producer of strips (two buffers), a producer of weights (all
+// nine taps once per CTA when they fit, RES; else a ring of per-tap tiles), the MMA
+// issuer, and four or eight warps that drain TMEM as in conv_igemm_kernel.
 constexpr int kWinACC = 2;               // 128-row accumulators per tile
 constexpr int kWinBMT = 128 * kWinACC;   // padded positions per tile
 constexpr int kWinBStages = 4;           // weight-tile ring depth when not resident
-constexpr int kWinThreads = 224;         // conv_wgwin_kernel: 4 epilogue warps, 2 producers, MMA
+constexpr int kWinThreads = 224;         // weight gradients: 4 epilogue warps, 2 producers, MMA
 
 // Warp roles of conv_win_kernel: EPI epilogue warps (0 .. EPI-1), then the strip
-// producer, the weight producer and the MMA issuer.  (Eight epilogue warps, two per
-// TMEM lane quarter, and stores staged in shared memory so that each instruction
-// writes whole lines, both measured slower on the stem than this form.)
+// producer, the weight producer and the MMA issuer.  128-column tiles drain with eight epilogue
+// warps, two per TMEM lane quarter; 64-column ones (the stem) with four: eight there, and stores staged
+// in shared memory so that each instruction writes whole lines, both measured slower.
 template <int BN>
 struct WinCfg {
     static constexpr int B_TILE = BN * 64 * 2;  // one tap x one 64-channel block of weights
@@ -1719,8 +1721,9 @@ __global__ void __launch_bounds__(kWinThreads, 1)
 }
 
 // ----------------------------------------------------------------------------- window weight gradient
-// dW[k][r][s][c] = sum over positions L of dy[L][k] * x_pad[L + r*Wp + s][c] for stride-1
-// layers with 64 input and 64 output channels and at most 10 taps, in the padded position space
+// dW[k][r][s][c] = sum over positions L of dy[L][k] * x_pad[L + r*Wp + s][c] for stride-1 layers with
+// 64 input and 64 output channels and three or four taps over more than one column (2x2, 1x3, 1x4; the
+// other small filters go to conv_wgrow_kernel), in the padded position space
 // of conv_win_kernel: dy is zero at the positions that are not outputs (its strip rows are read
 // with w from 0 to Wp-1 and h from 0 to Hp-1, and the zero fill of TMA covers w >= Q and h >= P).
 // A CTA owns all taps*64 x 64 outputs, as ceil(taps/2) 128 x 64 TMEM accumulators (tap pairs
@@ -2852,8 +2855,8 @@ bool wgband_setup(const dbl_conv_shape* s, Plan& pl)
 }
 
 // Window weight-gradient eligibility and geometry (see conv_wgwin_kernel):
-// stride 1, 64 input and 64 output channels, three or four taps (the stems), padded
-// rows of 10..256 positions.
+// stride 1, 64 input and 64 output channels, three or four taps that wgband_setup does not
+// take, padded rows of 10..256 positions.
 bool wgwin_setup(const dbl_conv_shape* s, Plan& pl)
 {
     const Geom g = geom(s);
@@ -2868,8 +2871,8 @@ bool wgwin_setup(const dbl_conv_shape* s, Plan& pl)
     const int64_t L = (int64_t)s->n * Hp * Wp;
     if (L > INT32_MAX / 4) return false;
     // K-block: two whole padded rows when that is a multiple of 16 positions (no misaligned start), one
-    // when only that fits in 256 (144-wide rows of the 288 px stem, batch 185: with 256 the two stages do
-    // not fit in shared memory and the pass runs as an implicit GEMM, 223 against 209 us), else 256
+    // when only that fits in 256 (at 144-wide rows, batch 185, four taps: with 256 the two stages do not fit
+    // in shared memory and the pass runs as an implicit GEMM, 223 against 209 us), else 256
     const int kb = (Wp >= 64 && 2 * Wp <= kWgWinKB && (2 * Wp) % 16 == 0) ? 2 * Wp
                    : (2 * Wp > kWgWinKB && Wp % 16 == 0)                   ? Wp
                                                                            : kWgWinKB;
