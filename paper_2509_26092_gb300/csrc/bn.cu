@@ -147,10 +147,10 @@ __global__ void __launch_bounds__(dbl::dev::kPartialsThreads) bn_fwd_finalize_pa
                                                                     float* __restrict__ save_mean,
                                                                     float* __restrict__ save_invstd)
 {
-    double ds, dq;
-    const int c = dbl::dev::partials_colsum(part, nparts, C, ds, dq);
+    dbl::dev::ChannelSums sums;
+    const int c = dbl::dev::partials_colsum(part, nparts, C, sums);
     if (c < 0) return;
-    finalize_channel((float)ds, (float)dq, inv_n, eps, save_mean[c], save_invstd[c]);
+    finalize_channel(sums.f32(0), sums.f32(1), inv_n, eps, save_mean[c], save_invstd[c]);
 }
 
 // Thread t of a CTA owns channel group g = t % (C/8) (8 channels, one 16-byte
@@ -220,16 +220,15 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM)
                           float* __restrict__ save_mean, float* __restrict__ save_invstd)
 {
     dbl::dev::grid_dependency_trigger();  // a convolution launched next may start its set-up
-    __shared__ dbl::dev::PairF red[2][kThreads / 32][kFwdSliceC];
     __shared__ __align__(16) float chan[2][kFwdSliceC];  // scale, shift
     const int slices = C / kFwdSliceC, c0 = blockIdx.x % slices * kFwdSliceC;
     const int block = blockIdx.x / slices, blocks = gridDim.x / slices;
-    double ds, dq;
-    dbl::dev::partials_colsum32(part, nparts, C, c0, red, ds, dq);
+    dbl::dev::ChannelSums sums;
+    dbl::dev::partials_colsum32(part, nparts, C, c0, sums);
     if (threadIdx.x < kFwdSliceC) {
         const int c = c0 + threadIdx.x;
         float m, is;
-        finalize_channel((float)ds, (float)dq, inv_n, eps, m, is);
+        finalize_channel(sums.f32(0), sums.f32(1), inv_n, eps, m, is);
         if (block == 0) {
             save_mean[c] = m;
             save_invstd[c] = is;
@@ -600,9 +599,10 @@ __global__ void __launch_bounds__(dbl::dev::kPartialsThreads) bn_bwd_finalize_ke
     const float* __restrict__ mean, const float* __restrict__ invstd, float* __restrict__ dgamma,
     float* __restrict__ dbeta, float* __restrict__ coef)
 {
-    double sg, sgx;
-    const int c = dbl::dev::partials_colsum(partial, nblk, C, sg, sgx);
+    dbl::dev::ChannelSums sums;
+    const int c = dbl::dev::partials_colsum(partial, nblk, C, sums);
     if (c < 0) return;
+    const double sg = sums.f64(0), sgx = sums.f64(1);
     dbeta[c] = (float)sg;
     dgamma[c] = (float)sgx;
     bwd_coefficients(sg, sgx, inv_n, gamma[c], invstd[c], mean[c], coef[c], coef[C + c], coef[2 * C + c]);
@@ -745,11 +745,17 @@ __global__ void __launch_bounds__(kThreads, 2)
         double sums[2];
 #pragma unroll
         for (int st = 0; st < 2; ++st) {
-            dbl::dev::PairF t{0.f, 0.f};
+            dbl::dev::Sum3 t{0.f, 0.f, 0.f};
 #pragma unroll
             for (int r = 0; r < 16; ++r)
-                if (r < CL) t = dbl::dev::pair_add(t, {v[st][r], 0.f});
-            sums[st] = (double)t.hi + (double)t.lo;
+                if (r < CL) t = dbl::dev::sum_add(t, v[st][r]);
+            sums[st] = dbl::dev::sum_f64(t);
+            if (!dbl::dev::sum_held(t)) {  // beyond fp32's range, or not a number
+                sums[st] = 0.0;
+#pragma unroll
+                for (int r = 0; r < 16; ++r)
+                    if (r < CL) sums[st] += (double)v[st][r];
+            }
         }
         if (rank == 0) {
             dbeta[c0 + c] = (float)sums[0];

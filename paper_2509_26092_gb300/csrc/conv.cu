@@ -2338,11 +2338,11 @@ __global__ void __launch_bounds__(kWgTapThreads, 1)
 __global__ void __launch_bounds__(kPartialsThreads) stats_reduce_kernel(const float* __restrict__ part, int nparts, int K,
                                                            float* __restrict__ sum, float* __restrict__ sumsq)
 {
-    double s, q;
-    const int c = partials_colsum(part, nparts, K, s, q);
+    ChannelSums sums;
+    const int c = partials_colsum(part, nparts, K, sums);
     if (c >= 0) {
-        sum[c] = (float)s;
-        sumsq[c] = (float)q;
+        sum[c] = sums.f32(0);
+        sumsq[c] = sums.f32(1);
     }
 }
 

@@ -88,3 +88,42 @@ def test_one_launch_bn_forward_gives_the_same_bits(D, count, C, nparts, residual
     assert all(torch.isfinite(t.float()).all() for t in got[0])
     assert all(torch.equal(a, b) for a, b in zip(*got))
     check_status(D)
+
+
+@pytest.mark.parametrize("nparts", [8, 160])  # one launch, and two
+def test_channel_sums_keep_what_fp64_keeps(D, nparts):
+    """Partial rows whose tree needs all 53 bits of fp64: 1, 2^-25, 2^-52, 0, -1, -2^-25 leave 2^-52 (and the
+    sums of the backward's clusters, added in rank order, the same)."""
+    C, count = 32, 4
+    parts = torch.zeros((nparts, 2, C), device="cuda")
+    parts[:6, 0] = torch.tensor([1.0, 2.0 ** -25, 2.0 ** -52, 0.0, -1.0, -2.0 ** -25], device="cuda")[:, None]
+    parts[0, 1] = count
+    y = torch.zeros((count, C), dtype=torch.bfloat16, device="cuda")
+    out, (mean, istd) = torch.empty_like(y), torch.full((2, C), float("nan"), device="cuda")
+    gamma, beta = torch.ones(C, device="cuda"), torch.zeros(C, device="cuda")
+    D.dbl_bn_relu_fused_parts(D.bn_shape(count, C, 1e-5, True), y, parts, nparts, gamma, beta, None, out, mean, istd)
+    assert torch.equal(mean, torch.full_like(mean, 2.0 ** -54))
+    rows = torch.zeros((16, C), dtype=torch.bfloat16, device="cuda")  # one per CTA of a cluster
+    rows[:5] = torch.tensor([1.0, 2.0 ** -25, 2.0 ** -52, -1.0, -2.0 ** -25], device="cuda")[:, None]
+    shape = D.bn_shape(16, C, 1e-5, False)
+    wsb = D.dbl_bn_workspace_bytes(shape)
+    dg, db = torch.full((2, C), float("nan"), device="cuda")
+    D.dbl_bn_relu_fused_bwd(shape, rows, None, torch.zeros_like(rows), None, gamma, beta, gamma,
+                            torch.empty_like(rows), None, dg, db, ws(wsb), wsb)
+    assert torch.equal(db, torch.full_like(db, 2.0 ** -52))
+    check_status(D)
+
+
+@pytest.mark.parametrize("nparts", [8, 160])
+def test_channel_sums_beyond_fp32_are_infinite(D, nparts):
+    """Finite partials whose sum fp32 cannot hold: the variance is infinite, 1/std zero and the output beta."""
+    C, count = 32, 4
+    parts = torch.zeros((nparts, 2, C), device="cuda")
+    parts[:3, 1] = 3e38
+    y = torch.ones((count, C), dtype=torch.bfloat16, device="cuda")
+    out, (mean, istd) = torch.empty_like(y), torch.full((2, C), float("nan"), device="cuda")
+    gamma, beta = torch.ones(C, device="cuda"), torch.full((C,), 0.5, device="cuda")
+    D.dbl_bn_relu_fused_parts(D.bn_shape(count, C, 1e-5, True), y, parts, nparts, gamma, beta, None, out, mean, istd)
+    assert torch.equal(istd, torch.zeros_like(istd)) and torch.equal(mean, torch.zeros_like(mean))
+    assert torch.equal(out, torch.full_like(out, 0.5))
+    check_status(D)
