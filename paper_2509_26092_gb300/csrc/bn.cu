@@ -109,24 +109,16 @@ __global__ void __launch_bounds__(kThreads) bn_stats_kernel(const act_t* __restr
 // ----------------------------------------------------------------------------- forward apply
 // Batch statistics -> mean and 1/std of a channel (fp64: the variance is E[y^2] - E[y]^2 of sums over up
 // to 10^8 rows).  inv_n = 1/count is divided on the host (the same correctly rounded value; an fp64
-// division on the device is a long chain of the GPU's slow fp64 operations).  1/std: fp32's, and one
-// Newton step in fp64, whose relative error is 3/2 of the square of fp32's (2^-22): 2^-43, which the
-// result's 24 bits do not show.  Variances that fp32 cannot hold as normal numbers take fp64's.
+// division on the device is a long chain of the GPU's slow fp64 operations), and 1/std is one fp64
+// sequence instead of a root and a division.
 __device__ __forceinline__ void finalize_channel(float sum, float sumsq, double inv_n, float eps, float& mean,
                                                  float& invstd)
 {
     const double m = (double)sum * inv_n;
     double var = (double)sumsq * inv_n - m * m;
     if (var < 0.0) var = 0.0;
-    const double v = var + (double)eps;
     mean = (float)m;
-    const float f = (float)v;
-    if (f > 1e-30f && f < 1e30f) {
-        const double r = (double)rsqrtf(f);
-        invstd = (float)(r + 0.5 * r * (1.0 - v * r * r));
-    } else {
-        invstd = (float)rsqrt(v);
-    }
+    invstd = (float)rsqrt(var + (double)eps);
 }
 
 __global__ void bn_fwd_finalize_kernel(double inv_n, int C, float eps, const float* __restrict__ sum,

@@ -1,5 +1,7 @@
 """Edges of the one-launch BatchNorm passes of small tensors: the backward (a cluster of CTAs per 32
 channels) against the fp64 oracle, the forward against the two launches of larger ones."""
+from decimal import Context, Decimal
+
 import numpy as np
 import pytest
 import torch
@@ -126,4 +128,27 @@ def test_channel_sums_beyond_fp32_are_infinite(D, nparts):
     D.dbl_bn_relu_fused_parts(D.bn_shape(count, C, 1e-5, True), y, parts, nparts, gamma, beta, None, out, mean, istd)
     assert torch.equal(istd, torch.zeros_like(istd)) and torch.equal(mean, torch.zeros_like(mean))
     assert torch.equal(out, torch.full_like(out, 0.5))
+    check_status(D)
+
+
+@pytest.mark.parametrize("C", [16, 32])  # two launches, and one
+def test_inverse_std_rounds_like_fp64(D, C):
+    """Sums of squares over three rows (fp32 bit patterns) whose 1/std lies above the middle of two fp32 values
+    by 2^-50 to 2^-47 of it: fp64's 1/sqrt (wrong by at most 2^-52) decides the rounding, less does not."""
+    bits = [1072431535, 1085111321, 1111793036, 1124728303, 1134414601, 1154234959, 1168073971, 1170294655,
+            1174906697, 1180708072]
+    sq = np.resize(np.array(bits, dtype=np.uint32), C).view(np.float32)
+    exact = [Decimal(float(q) * (1.0 / 3) + float(np.float32(1e-5))).sqrt(Context(prec=50)) for q in sq]
+    want = []
+    for e in exact:
+        f = np.float32(1 / float(e))
+        near = [np.nextafter(f, np.float32(0)), f, np.nextafter(f, np.float32(9))]
+        want.append(min(near, key=lambda t: abs(Decimal(float(t)) * e - 1)))
+    parts = torch.zeros((1, 2, C), device="cuda")
+    parts[0, 1] = to_f32_dev(sq)
+    y = torch.zeros((3, C), dtype=torch.bfloat16, device="cuda")
+    mean, istd = torch.full((2, C), float("nan"), device="cuda")
+    D.dbl_bn_relu_fused_parts(D.bn_shape(3, C, 1e-5, True), y, parts, 1, torch.ones(C, device="cuda"),
+                              torch.zeros(C, device="cuda"), None, torch.empty_like(y), mean, istd)
+    assert np.array_equal(istd.cpu().numpy(), np.array(want))
     check_status(D)
