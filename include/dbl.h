@@ -109,12 +109,15 @@ DBL_API int dbl_set_conv_pdl(int32_t mode);
 
 /* Host, for tests of the bounded waits: arms the next implicit-GEMM
  * convolution launch (a pass that dbl_conv_plan reports as
- * DBL_KERNEL_IGEMM) of this process so that its thread block 0 never
- * issues the load of its first K-block.  That block's MMA issuer then waits
+ * DBL_KERNEL_IGEMM), or weight gradient by filter rows
+ * (DBL_KERNEL_WINDOW_WGRAD with 128 tile columns), of this process so that
+ * its thread block 0 never issues the load of its first K-block (by filter
+ * rows: of its x rows).  That block's MMA issuer then waits
  * on a stage that never fills; the wait gives up after its limit (about 2 s),
  * records DBL_ERR_TIMEOUT in the device status (dbl_device_status), and every
  * role of the block winds down through its own bounded waits, letting the
- * copies it issued land before it returns.  The other blocks finish normally;
+ * copies it issued land before it returns.  The other blocks finish normally
+ * (those of its cluster after it);
  * the launch's outputs are not valid.  No fault is raised and the context
  * stays usable.  Applies to one launch, then disarms itself. */
 DBL_API int dbl_conv_test_stall_next(void);

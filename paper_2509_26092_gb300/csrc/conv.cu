@@ -91,7 +91,7 @@ struct ConvParams {
     int win_bpi;              // row-block and filter-row weight gradient: K-blocks per image
     int win_ni;               // filter-row weight gradient: images per K-block; bands: bands per image
     int win_cl;               // filter-row weight gradient: CTAs per cluster, which add their sums on chip
-    int test_stall;           // dbl_conv_test_stall_next: block 0 never loads its first K-block
+    int test_stall;           // dbl_conv_test_stall_next: block 0 never loads (its part of) its first K-block
 };
 
 __device__ __forceinline__ void report_timeout(volatile int* abort)
@@ -889,6 +889,7 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, 2>::THREADS, 1)
         bool failed = false;
         int last_it = -1;
         for (int k = prod; k < nkb; k += kProducers) {
+            if (p.test_stall && blockIdx.x == 0 && k == 0) continue;  // stage 0 never fills (bounded-wait test)
             const int s = k % STAGES;
             const uint32_t ok = mbar_wait_warp(&empty_bar[s], ((k / STAGES) & 1) ^ 1, &abort_flag);
             if (__any_sync(0xffffffffu, ok == 0u)) {
@@ -2194,12 +2195,14 @@ __global__ void __launch_bounds__(kWgTapThreads, 1)
             }
             uint8_t* dst = sgen + (4 * s + (is_x ? 0 : 2)) * strip;
             const int i = kb / p.win_bpi, h0 = (kb - i * p.win_bpi) * p.win_srows, img = i * p.win_ni;
-            mbar_arrive_expect_tx_elect(&full_bar[s], (uint32_t)(2 * loaded));
-            for (int h = 0; h < 2; ++h) {
-                if (is_x)
-                    tma_load_4d_elect(dst + h * strip, &tmX, &full_bar[s], c0 + 64 * h, -p.win_pw, h0 + r - p.win_ph, img);
-                else
-                    tma_load_4d_elect(dst + h * strip, &tmDY, &full_bar[s], n0 + 64 * h, -2, h0, img);
+            if (!(p.test_stall && is_x && blockIdx.x == 0 && it == 0)) {  // stage 0 never fills (bounded-wait test)
+                mbar_arrive_expect_tx_elect(&full_bar[s], (uint32_t)(2 * loaded));
+                for (int h = 0; h < 2; ++h) {
+                    if (is_x)
+                        tma_load_4d_elect(dst + h * strip, &tmX, &full_bar[s], c0 + 64 * h, -p.win_pw, h0 + r - p.win_ph, img);
+                    else
+                        tma_load_4d_elect(dst + h * strip, &tmDY, &full_bar[s], n0 + 64 * h, -2, h0, img);
+                }
             }
             if (++s == stages) {
                 s = 0;
@@ -3258,7 +3261,7 @@ int plan_grid(const Plan& pl)
 // 1.1% slower, because CTAs launched early wait on SMs the other stream's kernels need.  Off by
 // default.
 std::atomic<int> g_conv_pdl_override{-1};  // dbl_set_conv_pdl: -1 = the environment's choice
-std::atomic<int> g_conv_stall_next{0};     // dbl_conv_test_stall_next: arms one implicit-GEMM launch
+std::atomic<int> g_conv_stall_next{0};     // dbl_conv_test_stall_next: arms one launch of a kernel that has the hook
 
 bool conv_pdl()
 {
@@ -3337,7 +3340,9 @@ int launch_splitk(const Plan& pl, const CUtensorMap& a, const CUtensorMap& b, co
     cfg.stream = st;
     cfg.attrs = at;
     cfg.numAttrs = conv_attrs(2 * SK, at);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, conv_splitk_kernel<BN, FAM, SK>, a, b, a2, b2, pl.p);
+    ConvParams prm = pl.p;
+    if (g_conv_stall_next.exchange(0)) prm.test_stall = 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, conv_splitk_kernel<BN, FAM, SK>, a, b, a2, b2, prm);
     if (e != cudaSuccess) {
         dbl::count_launch();
         return dbl::cuda_check(e, "conv_splitk launch");
@@ -3545,7 +3550,9 @@ int launch_wgwin(const Plan& pl, const CUtensorMap& a, const CUtensorMap& b, int
     cfg.stream = st;
     cfg.attrs = at;
     cfg.numAttrs = conv_attrs(pl.wgtap ? pl.p.win_cl : 1, at);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, KERNEL, a, b, pl.p);
+    ConvParams prm = pl.p;
+    if (pl.wgtap && g_conv_stall_next.exchange(0)) prm.test_stall = 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, KERNEL, a, b, prm);
     if (e != cudaSuccess) {
         dbl::count_launch();
         return dbl::cuda_check(e, "conv_wgwin launch");

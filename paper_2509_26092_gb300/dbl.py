@@ -216,8 +216,9 @@ def conv_shape(n, h, w, c, k, r, stride, pad, s=None, stride_w=0, pad_w=0):
 
 
 def dbl_conv_test_stall_next():
-    """Test hook: the next implicit-GEMM convolution launch's block 0 never loads its first
-    K-block, so its bounded MMA wait runs out and the device status reports DBL_ERR_TIMEOUT."""
+    """Test hook: the next implicit-GEMM convolution launch's (or weight gradient by filter rows')
+    block 0 never loads its first K-block, so its bounded MMA wait runs out and the device status
+    reports DBL_ERR_TIMEOUT."""
     _check(lib().dbl_conv_test_stall_next())
 
 
