@@ -2696,7 +2696,7 @@ bool wgrow_setup(const dbl_conv_shape* s, Plan& pl)
     p.m_tiles = p.n_tiles = 1;
     p.gN = s->n;
     // one contiguous range of K-blocks per CTA
-    const int splits = grid_size(p.num_kb);
+    const int splits = std::min(p.num_kb, sms);
     p.kb_per_split = (p.num_kb + splits - 1) / splits;
     p.zdim = (p.num_kb + p.kb_per_split - 1) / p.kb_per_split;
     pl.ws_main = p.zdim > 1 ? (size_t)p.zdim * p.M * 64 * sizeof(float) : 0;
@@ -2848,7 +2848,7 @@ bool wgband_setup(const dbl_conv_shape* s, Plan& pl)
     p.m_tiles = p.n_tiles = 1;
     p.gN = s->n;
     // one contiguous range of K-blocks per CTA
-    const int splits = grid_size(p.num_kb);
+    const int splits = std::min(p.num_kb, sms);
     p.kb_per_split = (p.num_kb + splits - 1) / splits;
     p.zdim = (p.num_kb + p.kb_per_split - 1) / p.kb_per_split;
     pl.ws_main = p.zdim > 1 ? (size_t)p.zdim * p.M * 64 * sizeof(float) : 0;
@@ -3526,7 +3526,8 @@ int launch_win(const Plan& pl, const CUtensorMap& a, const CUtensorMap& b, const
 
 int wgwin_grid(const Plan& pl)
 {
-    return pl.wgtap ? pl.p.m_tiles * pl.p.n_tiles * pl.p.zdim * pl.p.win_cl : grid_size(pl.p.zdim);
+    if (pl.wgtap) return pl.p.m_tiles * pl.p.n_tiles * pl.p.zdim * pl.p.win_cl;
+    return pl.wgrow || pl.wgband ? pl.p.zdim : grid_size(pl.p.zdim);  // one CTA per slice, whatever the device holds
 }
 
 // KERNEL: conv_wgwin_kernel<NACC> or conv_wgrow_kernel (one CTA per split-K range), or

@@ -182,6 +182,17 @@ def test_conv_plans_of_the_resnet18_layers(D):
         D.dbl_conv_plan(D.conv_shape(2, 8, 8, 24, 64, 3, 1, 1), FWD)  # 24 input channels: unsupported
 
 
+@pytest.mark.parametrize("n,h,w,r,s,pad,slices", [(512, 56, 56, 3, 3, 1, 150), (100, 24, 24, 3, 3, 1, 150),
+                                                  (512, 115, 112, 4, 1, 0, 152)])
+def test_row_block_and_band_slices_do_not_depend_on_the_device(D, n, h, w, r, s, pad, slices):
+    """The slices of the 64-channel weight gradients (the order of their sums, and their workspace) are those
+    of a 152-SM GPU on any device, this one without a GPU among them; one CTA each."""
+    i = D.dbl_conv_plan(D.conv_shape(n, h, w, 64, 64, r, 1, pad, s=s, stride_w=1, pad_w=pad if s > 1 else 0),
+                        D.DBL_PASS_WGRAD)
+    assert i.kernel == D.DBL_KERNEL_WINDOW_WGRAD
+    assert (i.zdim, i.grid) == (slices, slices)
+
+
 def test_cta_pairs_can_be_switched_off():
     """DBL_CONV_CTA_PAIRS=0 plans every pass on single CTAs (read once per process)."""
     import subprocess
