@@ -98,7 +98,12 @@ DBL_API int dbl_device_status(int32_t* status);
  * launches the passes with programmatic stream serialization, so that a
  * kernel's set-up overlaps the end of the kernel before it on the stream
  * (faster with one stream of work, slower when another stream competes for
- * the SMs).  Neither changes what is computed.
+ * the SMs); DBL_MAX_CLUSTER=n takes clusters of more than n thread blocks of
+ * these passes and of the BatchNorm backward as not fitting on the device,
+ * where smaller clusters or none are used, as on a device that holds none.
+ * None of them changes what is computed; DBL_CONV_CTA_PAIRS and
+ * DBL_MAX_CLUSTER change the order of fp32 sums (without pairs, or without
+ * their clusters, no tile's reduction is split).
  * ======================================================================== */
 
 /* Host: overrides DBL_CONV_PDL for the convolution launches that follow, in

@@ -793,7 +793,8 @@ __global__ void __launch_bounds__(kThreads, 2)
 
 // CTAs per cluster of the one-launch backward, or 0 for the general path: the channels must come in
 // whole slices, and a CTA's rows (kClusterRows, with g to store kClusterRowsG) stay few enough that its
-// two passes cost less than the two launches saved.
+// two passes cost less than the two launches saved.  (A device that cannot place the cluster takes the general
+// path.)
 constexpr int kClusterRows = 800, kClusterRowsG = 512;
 
 int bwd_cluster(int64_t count, int C, bool with_g)
@@ -893,7 +894,9 @@ int bwd_launch_mask(const dbl_bn_shape* s, const void* dout, const void* dout2, 
     // When the caller wants g (the residual branch's gradient), the reduce pass stores it and the
     // apply pass reads it back instead of re-reading dout, dout2 and out.
     act_t* g_store = static_cast<act_t*>(dresidual);
-    if (const int cl = bwd_cluster(s->count, C, g_store != nullptr)) {
+    const int cl = bwd_cluster(s->count, C, g_store != nullptr);
+    if (cl && (g_store ? cluster_held<bn_bwd_cluster_kernel<MASK, true>>(cl, kThreads, 0)
+                       : cluster_held<bn_bwd_cluster_kernel<MASK, false>>(cl, kThreads, 0))) {
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;

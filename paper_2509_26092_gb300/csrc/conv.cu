@@ -2721,6 +2721,8 @@ bool wgtap_setup(const dbl_conv_shape* s, Plan& pl)
     constexpr int kMaxPos = 208;
     const int groups = 3 * (s->c / 128) * (s->k / 128);
     if (groups > 12) return false;  // see below
+    int max_cl = 1;
+    while (max_cl < 4 && dbl::cluster_held<conv_wgtap_kernel>(max_cl + 1, kWgTapThreads, kWinSmemMax)) ++max_cl;
     const int64_t elems = (int64_t)9 * s->c * s->k;
     double best = 1e300;
     ConvParams& p = pl.p;
@@ -2734,7 +2736,7 @@ bool wgtap_setup(const dbl_conv_shape* s, Plan& pl)
         if (stages < 2) break;
         const int64_t blocks = ni > 1 ? (s->n + ni - 1) / ni : (int64_t)s->n * ((P + R - 1) / R);
         if (blocks > INT32_MAX / 4) continue;
-        for (int cl = 1; cl <= 4; ++cl)
+        for (int cl = 1; cl <= max_cl; ++cl)
             for (int sixth = 6, last = 0; sixth >= 1; --sixth) {  // all the slices that fit, or fewer
                 int slices = std::max(1, resident[cl] / (groups * cl) * sixth / 6);
                 const int64_t kbs = (blocks + slices * cl - 1) / (slices * cl);
@@ -2952,6 +2954,17 @@ bool win_pairs() { return cta_pair_level() != 0; }
 // (3x3x512, batch 128) 26.3 / - / 13.8 / -, 6 of 72 (batch 64) 26.2 / - / 13.2 / 12.1.
 constexpr int kTileCost = 20;
 
+// Whether the device holds clusters of sk CTA pairs of a split kernel.
+template <int BN, int FAM>
+bool split_held(int sk)
+{
+    constexpr int T = Cfg<BN, FAM, 2>::THREADS;
+    if (sk == 2) return dbl::cluster_held<conv_splitk_kernel<BN, FAM, 2>>(4, T, SplitCfg<BN, FAM, 2>::SMEM);
+    if (sk == 4) return dbl::cluster_held<conv_splitk_kernel<BN, FAM, 4>>(8, T, SplitCfg<BN, FAM, 4>::SMEM);
+    if constexpr (BN == 256) return dbl::cluster_held<conv_splitk_kernel<BN, FAM, 8>>(16, T, SplitCfg<BN, FAM, 8>::SMEM);
+    return false;
+}
+
 int fwd_splits(int tiles, int num_kb)
 {
     static const int counts[4] = {1, 2, 4, 8}, resident[4] = {76, 36, 15, 7};
@@ -2960,6 +2973,7 @@ int fwd_splits(int tiles, int num_kb)
     for (int i = 0; i < 4; ++i) {
         const int sk = counts[i];
         if (sk > 1 && (tiles * 2 * sk > kMaxGrid || num_kb < 2 * sk)) continue;
+        if (sk > 1 && !split_held<256, kFamFwd>(sk)) break;
         const int64_t rounds = (tiles + resident[i] - 1) / resident[i];
         const int64_t kb = (num_kb + sk - 1) / sk;
         const int64_t cost = sk == 1 ? rounds * kb + kTileCost : rounds * (kb + kTileCost);
@@ -2987,6 +3001,7 @@ void wgrad_cluster(Plan& pl, int splits)
     for (int i = 0; i < 3; ++i) {
         const int sk = counts[i], slices = resident[i] / tiles;
         if (slices < 1 || pl.BN / sk < 32) continue;
+        if (!(pl.BN == 256 ? split_held<256, kFamWgrad>(sk) : split_held<128, kFamWgrad>(sk))) break;
         const int kbs = (p.num_kb + slices * sk - 1) / (slices * sk);
         const int used = (p.num_kb + kbs * sk - 1) / (kbs * sk);  // no slice without a K-block
         const double cost = kbs * kbc + 10500.0 + acc * (sk - 1) / sk / 22.0 + reduce(used);

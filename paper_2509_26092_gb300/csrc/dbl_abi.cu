@@ -4,6 +4,7 @@
 #include <math.h>
 #include <stdarg.h>
 #include <stdio.h>
+#include <stdlib.h>
 
 #include <atomic>
 #include <mutex>
@@ -38,6 +39,16 @@ int sm_count()
         return 148;  // no device answered: a nominal count, never cached
     }
     if (dev < 64) cached[dev] = n;
+    return n;
+}
+
+int max_cluster()
+{
+    static const int n = [] {
+        const char* e = getenv("DBL_MAX_CLUSTER");
+        const int v = e ? atoi(e) : 0;
+        return v > 0 ? v : 16;
+    }();
     return n;
 }
 

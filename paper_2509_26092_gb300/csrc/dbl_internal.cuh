@@ -9,6 +9,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/dbl.h"
 #include "dbl_act.cuh"
 
@@ -39,6 +41,47 @@ inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s
 
 // Number of SMs of the current device (cached per device).
 int sm_count();
+
+// Largest cluster to launch: DBL_MAX_CLUSTER in the environment (read once per process), or any.
+int max_cluster();
+
+#if defined(__CUDACC__)
+// Whether the current device (or the part of it that this context holds) can place a cluster of `ctas` CTAs of
+// KERNEL: up to eight, the portable size, every whole GPU can, sixteen only one that has so many SMs of a cluster
+// domain free for the context.  Asked once per device, kernel and size; where no device answers, a plan is that
+// of a whole GB300.
+template <auto KERNEL>
+bool cluster_held(int ctas, int threads, size_t smem)
+{
+    static std::atomic<signed char> cached[64][17] = {};
+    int dev = 0, sms = 0;
+    if (ctas > max_cluster()) return false;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return true;
+    }
+    const bool cache = dev >= 0 && dev < 64 && ctas <= 16;
+    if (cache && cached[dev][ctas]) return cached[dev][ctas] > 0;
+    cudaError_t e = cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess && ctas > 8) e = cudaFuncSetAttribute(KERNEL, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = ctas;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, KERNEL, &cfg);
+    if (e != cudaSuccess) (void)cudaGetLastError();
+    const bool held = e == cudaSuccess && n > 0;
+    if (cache) cached[dev][ctas] = held ? 1 : -1;
+    return held;
+}
+#endif
 
 // Tensor-map encoders from the driver, fetched through the runtime's
 // entry-point query so the library does not link libcuda directly.

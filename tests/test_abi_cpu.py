@@ -227,6 +227,31 @@ def test_window_pairs_of_64_columns_only_for_comparison():
     assert got == {"1": 1, "2": 2}
 
 
+def test_clusters_that_the_device_cannot_place_are_not_planned():
+    """DBL_MAX_CLUSTER (read once per process) stands for a device or context that places smaller clusters: the
+    split passes take the next smaller cluster, or none.  Grid: 2 * pairs per tile CTAs of each tile."""
+    import subprocess
+    import sys
+    code = ("from paper_2509_26092_gb300 import build_lib\nbuild_lib.build()\n"
+            "from paper_2509_26092_gb300 import dbl as D\n"
+            "for shp, p in (((1, 3, 3, 512, 512, 3, 1, 1), 0), ((17, 14, 14, 128, 256, 3, 2, 1), 2),\n"
+            "               ((33, 5, 5, 256, 128, 3, 1, 1), 2)):\n"
+            "    i = D.dbl_conv_plan(D.conv_shape(*shp), p)\n"
+            "    print(i.grid // (2 * i.tiles), end=' ')\n"
+            "i = D.dbl_conv_plan(D.conv_shape(512, 28, 28, 128, 128, 3, 1, 1), 2)\n"
+            "print(i.grid // (3 * i.zdim))\n")
+    got = {}
+    for n in ("16", "8", "4", "1"):
+        r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, env=dict(os.environ, DBL_MAX_CLUSTER=n),
+                           capture_output=True, text=True, timeout=300)
+        assert r.returncode == 0, r.stderr[-2000:]
+        got[n] = [int(v) for v in r.stdout.split()]
+    assert got["16"] == [8, 8, 4, 2]
+    assert max(got["8"]) <= 4 and got["8"][0] == 4
+    assert max(got["4"][:3]) <= 2 and got["4"][0] == 2
+    assert got["1"] == [1, 1, 1, 1]
+
+
 def test_conv_pdl_setter_validates_its_mode(D):
     """dbl_set_conv_pdl (host): 1, 0 and -1 are accepted by both libraries, anything else refused."""
     for mode in (1, 0, -1):

@@ -1,5 +1,9 @@
 """Edges of the convolution kernels chosen by shape: row-block weight gradients (3x3 stride 1, 64
 channels) and tiles split over clusters of CTA pairs, against the fp64 oracle."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -210,3 +214,44 @@ def test_split_wgrad_matches_oracle(D, n, h, c, k, r, stride):
     D.dbl_conv_wgrad(shape, xd, dyd, dw, True, work, wsb)
     assert max_norm_rel(host(dw), 2 * ref) <= WGRAD_TOL
     check_status(D)
+
+
+_SMALL_CLUSTERS = r"""
+import sys, torch
+sys.path.insert(0, sys.argv[1])
+from paper_2509_26092_gb300 import dbl as D
+gen = torch.Generator(device="cuda").manual_seed(5)
+normal = lambda *s: torch.randn(s, device="cuda", generator=gen)
+shape = D.conv_shape(1, 3, 3, 512, 512, 3, 1, 1)
+assert D.dbl_conv_plan(shape, 0).grid <= int(sys.argv[3]) * 2
+x, w = normal(1, 3, 3, 512).to(torch.bfloat16), (0.02 * normal(512, 3, 3, 512)).to(torch.bfloat16)
+y, dw = torch.empty_like(x), torch.empty((512, 3, 3, 512), device="cuda")
+D.dbl_conv_fwd(shape, x, w, y)
+work = torch.empty(1 << 24, dtype=torch.uint8, device="cuda")
+D.dbl_conv_wgrad(shape, x, y, dw, False, work, work.numel())
+bn = D.bn_shape(577, 64, 1e-5, False)
+u, v = normal(577, 64).to(torch.bfloat16), normal(577, 64).to(torch.bfloat16)
+one, dg, db, dx = torch.ones(64, device="cuda"), torch.empty(64, device="cuda"), torch.empty(64, device="cuda"), torch.empty_like(u)
+before = D.dbl_kernel_launches()
+D.dbl_bn_relu_fused_bwd(bn, u, None, v, None, one, 0 * one, one, dx, None, dg, db, work, work.numel())
+torch.cuda.synchronize()
+assert D.dbl_device_status() == D.DBL_OK
+torch.save([t.float().cpu() for t in (y, dw, dx, dg, db)] + [D.dbl_kernel_launches() - before], sys.argv[2])
+"""
+
+
+def test_devices_that_place_smaller_clusters_run_the_same_calls(tmp_path):
+    """DBL_MAX_CLUSTER (read once per process) as the answer of such a device: sixteen CTAs, eight, none."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    got = {}
+    for n in (16, 8, 1):
+        path = str(tmp_path / f"{n}.pt")
+        r = subprocess.run([sys.executable, "-c", _SMALL_CLUSTERS, root, path, str(max(n, 2))], capture_output=True,
+                           text=True, timeout=600, env=dict(os.environ, DBL_MAX_CLUSTER=str(n)))
+        assert r.returncode == 0, r.stderr[-2000:]
+        got[n] = torch.load(path)
+    assert [got[n][-1] for n in (16, 8, 1)] == [1, 3, 3]  # the BatchNorm backward's launches
+    for n in (8, 1):
+        for a, b, tol in zip(got[16], got[n], (2.0 ** -7, 2.0 ** -6, 2.0 ** -7, 1e-5, 1e-5)):
+            # 16-bit outputs: a rounding decided otherwise by the order of fp32 sums (y is also dw's operand)
+            assert (a - b).abs().max() <= tol * a.abs().max()
