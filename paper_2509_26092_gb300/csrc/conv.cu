@@ -1723,8 +1723,8 @@ __global__ void __launch_bounds__(kWinThreads, 1)
 
 // ----------------------------------------------------------------------------- window weight gradient
 // dW[k][r][s][c] = sum over positions L of dy[L][k] * x_pad[L + r*Wp + s][c] for stride-1 layers with
-// 64 input and 64 output channels and three or four taps over more than one column (2x2, 1x3, 1x4; the
-// other small filters go to conv_wgrow_kernel), in the padded position space
+// 64 input and 64 output channels and three, four, nine or ten taps (2x2, 1x3, 1x4, 2x5, 5x2; 3x3, 3x1 and 4x1
+// filters go to conv_wgrow_kernel where that can), in the padded position space
 // of conv_win_kernel: dy is zero at the positions that are not outputs (its strip rows are read
 // with w from 0 to Wp-1 and h from 0 to Hp-1, and the zero fill of TMA covers w >= Q and h >= P).
 // A CTA owns all taps*64 x 64 outputs, as ceil(taps/2) 128 x 64 TMEM accumulators (tap pairs
@@ -2858,15 +2858,16 @@ bool wgband_setup(const dbl_conv_shape* s, Plan& pl)
 }
 
 // Window weight-gradient eligibility and geometry (see conv_wgwin_kernel):
-// stride 1, 64 input and 64 output channels, three or four taps that wgband_setup does not
-// take, padded rows of 10..256 positions.
+// stride 1, 64 input and 64 output channels, three, four, nine or ten taps that wgrow_setup and wgband_setup do not
+// take, padded rows of 10..256 positions.  As implicit GEMMs 2x5 and 5x2 filters at 56x56, batch 128 took 56 to 59 us
+// instead of 43 to 44, with five times the rounding error (a K range per CTA pair instead of per CTA).
 bool wgwin_setup(const dbl_conv_shape* s, Plan& pl)
 {
     const Geom g = geom(s);
     if (g.sh != 1 || g.sw != 1) return false;
     if (s->c != 64 || s->k != 64) return false;
     const int ntaps = s->r * s->s;
-    if ((ntaps + 1) / 2 != 2) return false;  // the instantiated accumulator count
+    if ((ntaps + 1) / 2 != 2 && (ntaps + 1) / 2 != 5) return false;  // the instantiated accumulator counts
     const int Wp = s->w + 2 * g.pw, Hp = s->h + 2 * g.ph;
     if (Wp < 10 || Wp > 256) return false;
     const int P = Hp - s->r + 1, Q = Wp - s->s + 1;
@@ -3825,7 +3826,8 @@ int dbl_conv_wgrad(const dbl_conv_shape* s, const void* x, const void* dy, float
         if ((rc = pl.wgrow   ? launch_wgwin<conv_wgrow_kernel<false>>(pl, ta, tb, kWinThreads, st)
                   : pl.wgband ? launch_wgwin<conv_wgrow_kernel<true>>(pl, ta, tb, kWinThreads, st)
                   : pl.wgtap ? launch_wgwin<conv_wgtap_kernel>(pl, ta, tb, kWgTapThreads, st)
-                             : launch_wgwin<conv_wgwin_kernel<2>>(pl, ta, tb, kWinThreads, st)))
+                  : pl.p.win_R * pl.p.win_S > 4 ? launch_wgwin<conv_wgwin_kernel<5>>(pl, ta, tb, kWinThreads, st)
+                                                : launch_wgwin<conv_wgwin_kernel<2>>(pl, ta, tb, kWinThreads, st)))
             return rc;
     } else {
     const bool c8 = pl.mode == kWgradC8;

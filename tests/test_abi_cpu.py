@@ -193,6 +193,13 @@ def test_row_block_and_band_slices_do_not_depend_on_the_device(D, n, h, w, r, s,
     assert (i.zdim, i.grid) == (slices, slices)
 
 
+@pytest.mark.parametrize("r,s", [(2, 5), (5, 2), (2, 2), (1, 3), (1, 4)])
+def test_small_filters_of_64_channels_have_a_window_weight_gradient(D, r, s):
+    for n, h, w in ((128, 56, 56), (64, 24, 24), (1, 8, 37)):
+        i = D.dbl_conv_plan(D.conv_shape(n, h, w, 64, 64, r, 1, 0, s=s), D.DBL_PASS_WGRAD)
+        assert i.kernel == D.DBL_KERNEL_WINDOW_WGRAD
+
+
 def test_cta_pairs_can_be_switched_off():
     """DBL_CONV_CTA_PAIRS=0 plans every pass on single CTAs (read once per process)."""
     import subprocess

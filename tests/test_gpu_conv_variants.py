@@ -83,6 +83,31 @@ def test_band_wgrad_matches_oracle(D, n, h, w, r, ph):
     check_status(D)
 
 
+@pytest.mark.parametrize("n,h,w,r,k", [
+    (3, 14, 37, 2, 5),   # ten taps
+    (2, 9, 20, 5, 2),
+    (40, 24, 24, 5, 2),  # several K-blocks per CTA
+    (1, 4, 13, 1, 3),    # three taps: the unused half of the last pair
+    (2, 5, 10, 2, 2),    # the narrowest rows
+])
+def test_window_wgrad_of_other_filters_matches_oracle(D, n, h, w, r, k):
+    g = rng(10 * n + w)
+    x = bf16_values(g.standard_normal((n, h, w, 64)))
+    p, q = h - r + 1, w - k + 1
+    dy = bf16_values(g.standard_normal((n, p, q, 64)))
+    d2 = dy.reshape(-1, 64)
+    ref = np.stack([np.stack([d2.T @ x[:, a:a + p, b:b + q].reshape(-1, 64) for b in range(k)], axis=1)
+                    for a in range(r)], axis=1)
+    shape = D.conv_shape(n, h, w, 64, 64, r, 1, 0, s=k)
+    assert D.dbl_conv_plan(shape, D.DBL_PASS_WGRAD).kernel == D.DBL_KERNEL_WINDOW_WGRAD
+    wsb = D.dbl_conv_workspace_bytes(shape, D.DBL_PASS_WGRAD)
+    dw = torch.full((64, r, k, 64), float("nan"), device="cuda")
+    D.dbl_conv_wgrad(shape, to_bf16_dev(x), to_bf16_dev(dy), dw, False, ws(wsb), wsb)
+    assert np.all(np.isfinite(host(dw)))
+    assert max_norm_rel(host(dw), ref) <= WGRAD_TOL
+    check_status(D)
+
+
 # 16-bit outputs: one rounding of the result, at most 2^-8 of its size (bf16), and the fp32 sums' error
 CONV_TOL = 4e-3
 
