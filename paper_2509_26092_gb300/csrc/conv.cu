@@ -2874,12 +2874,9 @@ bool wgwin_setup(const dbl_conv_shape* s, Plan& pl)
     if (P <= 0 || Q <= 0) return false;
     const int64_t L = (int64_t)s->n * Hp * Wp;
     if (L > INT32_MAX / 4) return false;
-    // K-block: two whole padded rows when that is a multiple of 16 positions (no misaligned start), one
-    // when only that fits in 256 (at 144-wide rows, batch 185, four taps: with 256 the two stages do not fit
-    // in shared memory and the pass runs as an implicit GEMM, 223 against 209 us), else 256
-    const int kb = (Wp >= 64 && 2 * Wp <= kWgWinKB && (2 * Wp) % 16 == 0) ? 2 * Wp
-                   : (2 * Wp > kWgWinKB && Wp % 16 == 0)                   ? Wp
-                                                                           : kWgWinKB;
+    // K-block: two whole padded rows when that is a multiple of 16 positions (no misaligned start), else 256
+    // (one row of 129 to 256 positions instead: 1x3 and 1x4 at 145x144, batch 32 40.1 -> 42.9 and 40.5 -> 43.5 us)
+    const int kb = (Wp >= 64 && 2 * Wp <= kWgWinKB && (2 * Wp) % 16 == 0) ? 2 * Wp : kWgWinKB;
     const int start = kb % Wp == 0 ? 0 : Wp - 1;
     auto off = [&](int t) { return (t / s->s) * Wp + t % s->s; };
     const int last = (ntaps % 2) ? off(ntaps - 1) + 1 : off(ntaps - 1);  // the unused half of an odd last pair

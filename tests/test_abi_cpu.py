@@ -200,6 +200,12 @@ def test_small_filters_of_64_channels_have_a_window_weight_gradient(D, r, s):
         assert i.kernel == D.DBL_KERNEL_WINDOW_WGRAD
 
 
+def test_window_weight_gradient_of_wide_rows_has_blocks_of_256_positions(D):
+    """1x4 over rows of 144: two stages of three x rows and three dy rows of 128-byte positions, and alignment."""
+    i = D.dbl_conv_plan(D.conv_shape(32, 145, 144, 64, 64, 1, 1, 0, s=4), D.DBL_PASS_WGRAD)
+    assert i.kernel == D.DBL_KERNEL_WINDOW_WGRAD and i.smem_bytes == 2 * 6 * 144 * 128 + 1024
+
+
 def test_cta_pairs_can_be_switched_off():
     """DBL_CONV_CTA_PAIRS=0 plans every pass on single CTAs (read once per process)."""
     import subprocess
