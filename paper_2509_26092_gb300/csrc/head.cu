@@ -9,6 +9,7 @@
 #include <float.h>
 
 #include <algorithm>
+#include <utility>
 
 #include "dbl_internal.cuh"
 
@@ -567,8 +568,9 @@ __global__ void __launch_bounds__(256) avgpool_kernel(const act_t* __restrict__ 
 // next tile is fetched into registers while the current one is multiplied), 8 x 8 outputs per thread,
 // two per instruction (fma.rn.f32x2).  The reduction is cut into chunks of kchunk, each a sequential
 // fmaf over its k; the chunks of a tile are the CTAs of a cluster (along z), which add their partial
-// sums in chunk order through distributed shared memory.  Two products, and the loss and bias-gradient
-// sums that need the same input, share a launch.
+// sums in chunk order through distributed shared memory.  Long reductions of few tiles take several clusters per
+// tile (groups), whose sums a second launch adds in order.  Two products, and the loss and bias-gradient
+// sums that need the same input, share a launch where that suits both (gemm_plan).
 // Bound by fp32 issue: 512 x 1000 x 512 is 7 us of the GPU's fp32 rate.  With 4 x 4 outputs per thread
 // (half the FMAs per shared-memory byte), the partial sums through global memory and a launch of their
 // own, the head of 512 images and 1000 classes took 128.2 us in ten launches; now 72.6 in five.
@@ -580,9 +582,9 @@ constexpr int kGemmMaxChunks = 8;  // a cluster
 
 struct GemmJob {
     const float *A, *B, *bias;
-    float* out;
-    int64_t sam, sak, sbn, sbk, ldo;
-    int M, N, K, kchunk, tiles;
+    float* out;  // of several groups: their sums [groups][M][N], gstride apart
+    int64_t sam, sak, sbn, sbk, ldo, gstride;
+    int M, N, K, kchunk, tiles, clusters;  // clusters: tiles x groups
     int vec;  // bits: A, B and out may be accessed 16 bytes at a time
 };
 
@@ -688,17 +690,22 @@ __global__ void __launch_bounds__(kGemmThreads, 4) head_gemm_kernel(const __grid
     static_assert(2 * GBK * (GLA + GLB) <= GBM * GBN, "K tiles");
     const int nz = gridDim.z, z = blockIdx.z;  // the cluster: one CTA per chunk
     int tile = blockIdx.x;
-    if (tile >= j0.tiles + j1.tiles) {
-        const int b = (tile - j0.tiles - j1.tiles) * nz + z;
+    if (tile >= j0.clusters + j1.clusters) {
+        const int b = (tile - j0.clusters - j1.clusters) * nz + z;
         if (b <= (hs.J + kHeadRedCols - 1) / kHeadRedCols) head_sums(hs, b, sm);
         return;
     }
-    const GemmJob& j = tile < j0.tiles ? j0 : j1;
-    if (tile >= j0.tiles) tile -= j0.tiles;
+    const GemmJob& j = tile < j0.clusters ? j0 : j1;
+    if (tile >= j0.clusters) tile -= j0.clusters;
+    int group = 0;
+    if (tile >= j.tiles) {
+        group = tile / j.tiles;
+        tile -= group * j.tiles;
+    }
     const int tn = (j.N + GBN - 1) / GBN;
     const int m0 = tile / tn * GBM, n0 = tile % tn * GBN;
     const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;  // rows 4ty.., 32 + 4ty..; columns 4tx.., 64 + 4tx..
-    const int kb = z * j.kchunk, ke = min(j.K, kb + j.kchunk);
+    const int kb = (group * nz + z) * j.kchunk, ke = min(j.K, kb + j.kchunk);
     float2 acc[8][4];
 #pragma unroll
     for (int r = 0; r < 8; ++r)
@@ -764,7 +771,7 @@ __global__ void __launch_bounds__(kGemmThreads, 4) head_gemm_kernel(const __grid
         const float o[4] = {s.x + bias[0], s.y + bias[1], s.z + bias[2], s.w + bias[3]};
         const int m = m0 + r;
         if (m < j.M) {
-            float* d = j.out + (int64_t)m * j.ldo + n;
+            float* d = j.out + group * j.gstride + (int64_t)m * j.ldo + n;
             if ((j.vec & 4) && n + 3 < j.N) {
                 *reinterpret_cast<float4*>(d) = make_float4(o[0], o[1], o[2], o[3]);
             } else {
@@ -777,32 +784,159 @@ __global__ void __launch_bounds__(kGemmThreads, 4) head_gemm_kernel(const __grid
     cluster_sync_all();  // no CTA leaves while another may still read its partial sums
 }
 
+// out[m, n] = the groups' sums part[g][M][N] in order (+ bias[n]).
+struct GroupSums {
+    const float *part, *bias;
+    float* out;
+    int64_t ldo;
+    int M, N, groups;  // groups = 0: nothing
+};
+
+__global__ void __launch_bounds__(256) head_group_reduce_kernel(const __grid_constant__ GroupSums s0,
+                                                                const __grid_constant__ GroupSums s1)
+{
+    for (int x = 0; x < 2; ++x) {
+        const GroupSums& s = x ? s1 : s0;
+        if (!s.groups) continue;
+        const int64_t total = (int64_t)s.M * s.N;
+        for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+            float v = s.part[i];
+#pragma unroll 8
+            for (int g = 1; g < s.groups; ++g) v += s.part[g * total + i];
+            const int m = (int)(i / s.N), n = (int)(i % s.N);
+            s.out[(int64_t)m * s.ldo + n] = v + (s.bias ? s.bias[n] : 0.f);
+        }
+    }
+}
+
 GemmJob gemm_job(const float* A, int64_t sam, int64_t sak, const float* B, int64_t sbn, int64_t sbk, const float* bias,
                  float* out, int64_t ldo, int M, int N, int K)
 {
-    GemmJob j{A, B, bias, out, sam, sak, sbn, sbk, ldo, M, N, K, 0, 0, 0};
-    j.tiles = ((M + GBM - 1) / GBM) * ((N + GBN - 1) / GBN);
+    GemmJob j{A, B, bias, out, sam, sak, sbn, sbk, ldo, 0, M, N, K, 0, 0, 0, 0};
     auto vec = [](const float* p, int64_t ld) { return dbl::aligned16(p) && ld % 4 == 0; };
     j.vec = (vec(A, sak == 1 ? sam : sak) ? 1 : 0) | (vec(B, sbk == 1 ? sbn : sbk) ? 2 : 0) | (vec(out, ldo) ? 4 : 0);
     return j;
 }
 
-// One or two products (j1 may have no tiles) and the sums of hs.  The number of K chunks is a function of the
-// shapes only: the most, of 1, 2, 4 and 8, that leaves the longer reduction two K tiles per chunk and
-// the grid within the CTAs that are resident at one time.
-int head_gemm(GemmJob j0, GemmJob j1, const HeadSums& hs, cudaStream_t s, const char* what)
+// A product as the plan sees it.
+struct GemmShape {
+    int M, N, K;
+    int tiles() const { return ((M + GBM - 1) / GBM) * ((N + GBN - 1) / GBN); }
+    // The longest chunk of a product whose result stays fp32: a sum of K terms in few long chains loses more
+    // than one in many short ones.  Up to 96 terms cost no more than 64; beyond that enough chunks for about 304
+    // tiles of 64 x 64, at least 64 terms each (n images, 10 classes, error of dW against 64 bits with chunks of K / 8
+    // and with these: n 1024 9.0e-8 and 6.6e-8, 2048 1.8e-7 and 6.8e-8, 8192 1.3e-6 and 1.0e-7).
+    int limit() const
+    {
+        const int t = ((M + 63) / 64) * ((N + 63) / 64);
+        const int z = std::min(std::max((304 + t - 1) / t, 1), std::max(1, (K + 63) / 64));
+        return std::max(96, ((K + z - 1) / z + GBK - 1) / GBK * GBK);
+    }
+};
+
+// How a launch cuts its products' reductions: nz chunks per cluster, groups clusters per tile.
+struct GemmPlan {
+    int nz, groups[2], kchunk[2];
+    double us;  // modelled time
+};
+
+// One or two products in a launch.  nz: the most, of 1, 2, 4 and 8, that leaves the longest reduction two K tiles
+// per chunk and the grid within the CTAs that are resident at one time.  groups: what the limits ask for, or
+// more, for chunks of four K tiles as far as all CTAs are resident, where the model sees a tenth less time.  The model (us):
+// 4 for the launch; 1.15 for each K tile of the longest chunk (its loads' latency), or the fp32 rate, 0.54 for each of
+// an SM's K tiles; 3 and 3.8 per 1000 CTAs for the exchange; 3 for adding groups.  A function of the shapes only.
+GemmPlan gemm_plan(const GemmShape* j, const int* limit, int count)
 {
-    const int K = std::max(j0.K, j1.tiles ? j1.K : 0), tiles = j0.tiles + j1.tiles;
+    constexpr int kSMs = kGemmMaxCTAs / 4;
+    auto cut = [&](int nz, bool more) {
+        GemmPlan p{nz, {1, 1}, {GBK, GBK}, 0.0};
+        int tiles = 0, ctas = 0, chain = 0;
+        double work = 0.0;
+        bool reduce = false;
+        for (int i = 0; i < count; ++i) tiles += j[i].tiles();
+        for (int i = 0; i < count; ++i) {
+            const int K = j[i].K;
+            int g = (K + nz * limit[i] - 1) / (nz * limit[i]);
+            if (more) g = std::max(g, std::min((K + nz * 4 * GBK - 1) / (nz * 4 * GBK), kGemmMaxCTAs / (tiles * nz)));
+            p.kchunk[i] = ((K + nz * g - 1) / (nz * g) + GBK - 1) / GBK * GBK;
+            p.groups[i] = (K + nz * p.kchunk[i] - 1) / (nz * p.kchunk[i]);  // none without terms
+            ctas += j[i].tiles() * p.groups[i] * nz;
+            chain = std::max(chain, p.kchunk[i] / GBK);
+            work += (double)j[i].tiles() * ((K + GBK - 1) / GBK);
+            reduce = reduce || p.groups[i] > 1;
+        }
+        p.us = 4.0 + std::max(1.15 * chain, 0.54 / kSMs * work) + (nz > 1 ? 3.0 + 0.0038 * ctas : 0.0) + (reduce ? 3.0 : 0.0);
+        return std::make_pair(p, ctas);
+    };
+    int kmax = 0;
+    for (int i = 0; i < count; ++i) kmax = std::max(kmax, j[i].K);
     int nz = 1;
-    while (nz < kGemmMaxChunks && tiles * nz * 2 <= kGemmMaxCTAs && K >= 2 * nz * 2 * GBK) nz *= 2;
-    for (GemmJob* j : {&j0, &j1}) j->kchunk = ((j->K + nz - 1) / nz + GBK - 1) / GBK * GBK;
+    while (nz < kGemmMaxChunks && kmax >= 2 * nz * 2 * GBK && cut(2 * nz, false).second <= kGemmMaxCTAs) nz *= 2;
+    const GemmPlan least = cut(nz, false).first, more = cut(nz, true).first;
+    return more.us < 0.9 * least.us ? more : least;
+}
+
+// The head's three products.
+struct HeadPlan {
+    GemmPlan logits, both, dx, dw;
+    bool joint;        // df and dW in one launch (both), or one each
+    size_t part;       // floats of the groups' sums
+};
+
+HeadPlan head_plan(int n, int c, int classes)
+{
+    const GemmShape f{n, classes, c}, b[2] = {{n, c, classes}, {classes, c, n}};
+    // df is rounded to 16 bits
+    const int lf = f.limit(), lb[2] = {std::max(256, b[0].limit()), b[1].limit()};
+    HeadPlan p;
+    p.logits = gemm_plan(&f, &lf, 1);
+    p.both = gemm_plan(b, lb, 2);
+    p.dx = gemm_plan(&b[0], &lb[0], 1);
+    p.dw = gemm_plan(&b[1], &lb[1], 1);
+    // Apart, a product of many tiles and few terms does not keep the other from its clusters, at a launch more. The
+    // whole head in one launch and so (us): one image of 512 features and 10,000 classes 744 and 70, of 2048 features
+    // and 1000 classes 75 and 46, 8192 images of 512 features and 10 classes 735 and 207, 2048 82 and 61.
+    // (Where the model sees less than a third between them, one launch measured faster.)
+    p.joint = p.both.us <= 1.3 * (p.dx.us + p.dw.us);
+    auto part = [](const GemmShape& j, int groups) { return groups > 1 ? (size_t)groups * j.M * j.N : 0; };
+    const size_t pb = p.joint ? part(b[0], p.both.groups[0]) + part(b[1], p.both.groups[1])
+                              : std::max(part(b[0], p.dx.groups[0]), part(b[1], p.dw.groups[0]));
+    p.part = std::max(part(f, p.logits.groups[0]), pb);
+    return p;
+}
+
+// One or two products (j1 without tiles: none) as plan cuts them, and the sums of hs.
+int head_gemm(GemmJob j0, GemmJob j1, const GemmPlan& plan, float* part, const HeadSums& hs, cudaStream_t s,
+              const char* what)
+{
+    GemmJob* job[2] = {&j0, &j1};
+    GroupSums groups[2] = {};
+    int64_t items = 0;
+    for (int i = 0; i < 2; ++i) {
+        GemmJob& j = *job[i];
+        if (j.M == 0) continue;
+        j.tiles = GemmShape{j.M, j.N, j.K}.tiles();
+        j.clusters = j.tiles * plan.groups[i];
+        j.kchunk = plan.kchunk[i];
+        if (plan.groups[i] > 1) {
+            groups[i] = {part, j.bias, j.out, j.ldo, j.M, j.N, plan.groups[i]};
+            j.gstride = (int64_t)j.M * j.N;
+            items = std::max(items, j.gstride);
+            j.bias = nullptr;
+            j.out = part;
+            j.ldo = j.N;
+            j.vec = (j.vec & 3) | (dbl::aligned16(part) && j.N % 4 == 0 ? 4 : 0);
+            part += plan.groups[i] * j.gstride;
+        }
+    }
+    const int nz = plan.nz;
     const int sums = hs.J ? 1 + (hs.J + kHeadRedCols - 1) / kHeadRedCols : 0;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = nz;
-    cfg.gridDim = dim3(tiles + (sums + nz - 1) / nz, 1, nz);
+    cfg.gridDim = dim3(j0.clusters + j1.clusters + (sums + nz - 1) / nz, 1, nz);
     cfg.blockDim = dim3(kGemmThreads);
     cfg.stream = s;
     cfg.attrs = at;
@@ -812,6 +946,9 @@ int head_gemm(GemmJob j0, GemmJob j1, const HeadSums& hs, cudaStream_t s, const 
         dbl::count_launch();
         return dbl::cuda_check(e, what);
     }
+    int rc = dbl::launch_check(what);
+    if (rc || !items) return rc;
+    head_group_reduce_kernel<<<grid_for(items, 256), 256, 0, s>>>(groups[0], groups[1]);
     return dbl::launch_check(what);
 }
 
@@ -1056,9 +1193,9 @@ int dbl_maxpool_bwd(int32_t n, int32_t h, int32_t w, int32_t c, const void* dy, 
 size_t dbl_head_workspace_bytes(int32_t n, int32_t c, int32_t classes)
 {
     if (n <= 0 || c <= 0 || classes <= 0) return 0;
-    // feat, df and the dropout multipliers [n,c], logits/dlogits [n,classes], row_loss [n]
+    // feat, df and the dropout multipliers [n,c], logits/dlogits [n,classes], row_loss [n], then the groups' sums
     const size_t f = (size_t)n * c * 3 + (size_t)n * classes + (size_t)n;
-    return (f * sizeof(float) + 16 + 255) / 256 * 256;  // 16: alignment of the caller's pointer
+    return (((f + 3) / 4 * 4 + head_plan(n, c, classes).part) * sizeof(float) + 16 + 255) / 256 * 256;  // 16: alignment of the caller's pointer
 }
 
 }  // extern "C"
@@ -1088,6 +1225,8 @@ int head_fwd_bwd(int32_t n, int32_t hw, int32_t c, int32_t classes, const void* 
     float* mult = df + (size_t)n * c;
     float* logits = mult + (size_t)n * c;
     float* row_loss = logits + (size_t)n * classes;
+    float* part = feat + ((size_t)n * c * 3 + (size_t)n * classes + (size_t)n + 3) / 4 * 4;
+    const HeadPlan plan = head_plan(n, c, classes);
     Dropout dp{0u, 1.f, seed, step, mult};
     if (drop_rate > 0.f) {
         dp.thr = (uint32_t)floor((double)drop_rate * 4294967296.0);
@@ -1106,16 +1245,21 @@ int head_fwd_bwd(int32_t n, int32_t hw, int32_t c, int32_t classes, const void* 
                                                                            c, dp);
     if ((rc = launch_check("avgpool launch"))) return rc;
     // logits = feat * W^T + b
-    if ((rc = head_gemm(gemm_job(feat, c, 1, fc_w, c, 1, fc_b, logits, classes, n, classes, c), GemmJob{}, HeadSums{}, s,
-                        "fc fwd launch")))
+    if ((rc = head_gemm(gemm_job(feat, c, 1, fc_w, c, 1, fc_b, logits, classes, n, classes, c), GemmJob{}, plan.logits,
+                        part, HeadSums{}, s, "fc fwd launch")))
         return rc;
     softmax_ce_kernel<<<n, kSoftmaxThreads, 0, s>>>(logits, labels, n, classes, row_loss, loss_scale);
     if ((rc = launch_check("softmax_ce launch"))) return rc;
     // df[n, c] = sum_j dl[n, j] W[j, c]; dW[j, c] = sum_n dl[n, j] feat[n, c]; the loss and db
-    if ((rc = head_gemm(gemm_job(logits, classes, 1, fc_w, 1, c, nullptr, df, c, n, c, classes),
-                        gemm_job(logits, 1, classes, feat, 1, c, nullptr, dfc_w, c, classes, c, n),
-                        HeadSums{row_loss, logits, loss, dfc_b, n, classes}, s, "fc bwd launch")))
-        return rc;
+    const GemmJob jx = gemm_job(logits, classes, 1, fc_w, 1, c, nullptr, df, c, n, c, classes);
+    const GemmJob jw = gemm_job(logits, 1, classes, feat, 1, c, nullptr, dfc_w, c, classes, c, n);
+    const HeadSums sums{row_loss, logits, loss, dfc_b, n, classes};
+    if (plan.joint) {
+        if ((rc = head_gemm(jx, jw, plan.both, part, sums, s, "fc bwd launch"))) return rc;
+    } else {
+        if ((rc = head_gemm(jx, GemmJob{}, plan.dx, part, HeadSums{}, s, "fc dX launch"))) return rc;
+        if ((rc = head_gemm(jw, GemmJob{}, plan.dw, part, sums, s, "fc dW launch"))) return rc;
+    }
     // with dropout, the pool's backward also advances the step counter (the next call draws a fresh mask)
     uint64_t* adv = dp.thr ? step : nullptr;
     if (per_image)
