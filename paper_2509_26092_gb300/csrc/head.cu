@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-// The same for large tensors (kPoolRowsBytes): a thread owns one channel group g of two neighbouring output columns and walks down `rows` output
+// The same for large tensors (pool_by_rows): a thread owns one channel group g of two neighbouring output columns and walks down `rows` output
 // rows: each input row is normalised once, in five vectors of which the middle one serves both columns,
 // and reduced along the row (its maximum and the first column that has it); an output row combines three
 // such row results, the last of which is the next output row's first.  That is 5 vectors per output
@@ -229,6 +229,17 @@ constexpr int kPoolDepth = 5;
 // with a window per thread against 16.0 with the best run, 144 x 144, batch 16 (42 MB) 18.4 against 18.3 to 25.9;
 // 112 x 112, batch 64 (103 MB) 38.9 against 34.2 to 38.1.
 constexpr int64_t kPoolRowsBytes = 96ll << 20;
+// With few channels the five columns of a thread's pair are a short run of bytes, and a warp's lie in many lines
+// (window per thread and rows, us): 112 x 112, 103 MB: 8 channels 36.8 and 51.3, 16 37.2 and 45.8, 32 36.6 and 39.1; 206 MB: 8 66.7
+// and 87.9, 16 66.8 and 76.8, while rows take 65.2 with 32 and 61.7 with 64.  Runs in maps of few rows leave a
+// part of their last run empty: 20 x 20, 105 MB, 64 channels 37.2 and 39.7, 256 39.7 and 41.9; 28 x 28 rows 34.0 and 35.9.
+constexpr int kPoolRowsMinP = 14;
+
+bool pool_by_rows(int64_t count, int C, int P)
+{
+    const int64_t bytes = count * C * (int64_t)sizeof(act_t);
+    return C >= 32 && P >= kPoolRowsMinP && bytes >= (C >= 64 ? 1 : 2) * kPoolRowsBytes;
+}
 constexpr int kPoolThreads = 256;
 
 struct PoolRow {  // per column and channel pair: maximum of a row's three taps, and its tap (0..2 in each half)
@@ -1129,7 +1140,7 @@ int dbl_bn_relu_maxpool_fwd(const dbl_bn_shape* s, int32_t n, int32_t h, int32_t
     if (rc) return rc;
     // a block size that is a multiple of the channel groups: each thread keeps its group
     const int groups = c / 8, block = groups * std::max(1, kPoolThreads / groups);
-    if (s->count * c * (int64_t)sizeof(act_t) < kPoolRowsBytes || block > kPoolThreads) {
+    if (!pool_by_rows(s->count, c, P) || block > kPoolThreads) {
         bn_relu_maxpool_fwd_kernel<<<grid_for((int64_t)n * P * Q, block / groups), block, 0, st>>>(
             static_cast<const act_t*>(x), gamma, beta, save_mean, save_invstd, static_cast<act_t*>(y),
             argmax, n, h, w, c, P, Q);

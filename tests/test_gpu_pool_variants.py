@@ -18,6 +18,8 @@ def D():
     (300, 145, 150, 8),   # one channel group
     (11, 142, 141, 256),  # eight pixel pairs per CTA
     (3, 513, 515, 64),    # few, large images
+    (161, 141, 142, 32),  # 64 pixel pairs per CTA
+    (2700, 27, 27, 64),   # the fewest output rows
 ])
 def test_large_pool_equals_bn_then_maxpool(D, n, h, w, c):
     g = torch.Generator(device="cuda").manual_seed(n)
