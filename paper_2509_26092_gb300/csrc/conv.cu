@@ -803,6 +803,11 @@ template <int BN, int FAM, int SK>
 struct SplitCfg {
     using C = Cfg<BN, FAM, 2>;
     static_assert(C::ACC == 1 && BN / SK >= 32, "one accumulator, whole chunks");
+    // The weight gradient's K ranges are longer than the slices they replace, and the tensor core's sums lose with
+    // their length (it rounds towards zero): each half of the range has an accumulator of its own, added in
+    // fp32.  4x4x256, batch 256: error of dw against 64 bits 8.4e-7 with one, 4.0e-7 with two, 13.8 us both.
+    static constexpr int ACCS = FAM == kFamWgrad ? 2 : 1;
+    static constexpr uint32_t TMEM_COLS = ACCS * BN;
     static constexpr int W = BN / SK;              // columns a CTA finishes
     static constexpr int SLOT = 128 * W * 4;        // one received part: [W / 4][128 rows] float4
     static constexpr int CW = W > 32 ? W / 2 : 32;  // columns an epilogue warp finishes (of W = 32: one warp per quarter)
@@ -864,7 +869,7 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, 2>::THREADS, 1)
         }
     }
     if (warp == C::MMA_WARP) {
-        tmem_alloc_cg<2>(&tmem_slot, BN);
+        tmem_alloc_cg<2>(&tmem_slot, S::TMEM_COLS);
         tmem_relinquish_cg<2>();
     }
     tc_fence_before();
@@ -874,6 +879,7 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, 2>::THREADS, 1)
     grid_dependency_wait();  // the set-up above may overlap the previous kernel; memory only after it
     const uint32_t tmem = tmem_slot;
     const int64_t gPQ = (int64_t)p.gP * p.gQ;
+    const int nkb_first = S::ACCS == 2 ? (nkb + 1) / 2 : nkb;  // K-blocks of the first accumulator
 
     if (warp >= C::EPI && warp < C::MMA_WARP) {
         // ------------------------------------------------------------------ TMA producers
@@ -935,6 +941,8 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, 2>::THREADS, 1)
                 const int s = k % STAGES;
                 const uint32_t sa = sbase + s * C::STAGE_BYTES, sb = sa + C::A_BYTES;
                 const uint64_t ad0 = dA | (uint64_t)((sa >> 4) & 0x3FFFu), bd0 = dB | (uint64_t)((sb >> 4) & 0x3FFFu);
+                const uint32_t d = tmem + (k >= nkb_first ? (uint32_t)BN : 0u);
+                const bool held = k != 0 && k != nkb_first;  // the accumulator holds a K-block already
 #pragma unroll
                 for (int j = 0; j < C::KSTEPS; ++j) {
                     if (j == C::KSTEPS - 1 && k + 1 < nkb) {  // the next stage's wait while MMAs are queued
@@ -942,8 +950,8 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, 2>::THREADS, 1)
                             mbar_wait_warp(&full_bar[(k + 1) % STAGES], ((k + 1) / STAGES) & 1, &abort_flag);
                         failed = __any_sync(0xffffffffu, ok == 0u);
                     }
-                    mma_act_elect_cg<2>(tmem, ad0 + (uint64_t)(j * a_step16), bd0 + (uint64_t)(j * b_step16), idesc,
-                                        (k > 0 || j > 0) ? 1u : 0u);
+                    mma_act_elect_cg<2>(d, ad0 + (uint64_t)(j * a_step16), bd0 + (uint64_t)(j * b_step16), idesc,
+                                        (held || j > 0) ? 1u : 0u);
                 }
                 mma_commit_elect_cg<2>(&empty_bar[s], both);
             }
@@ -965,6 +973,19 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, 2>::THREADS, 1)
     const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16);
     constexpr int CW = S::CW, NCH = CW / 32;
     const bool finishes = warp < C::EPI && half * CW < W;
+    auto load_acc = [&](uint32_t col, uint32_t(&v)[32]) {  // 32 columns of the accumulator, or of both
+        tmem_ld_32x32b_x32(taddr + col, v);
+        if (S::ACCS == 2 && nkb > nkb_first) {
+            uint32_t u[32];
+            tmem_ld_32x32b_x32(taddr + BN + col, u);
+            tmem_ld_wait_regs(v);
+            tmem_ld_wait_regs(u);
+#pragma unroll
+            for (int k = 0; k < 32; ++k) v[k] = __float_as_uint(__uint_as_float(v[k]) + __uint_as_float(u[k]));
+        } else {
+            tmem_ld_wait_regs(v);
+        }
+    };
     uint32_t own[NCH][32];  // this warp's part of the CTA's own columns
     if (warp < C::EPI) {
         // the other pairs' chunks of 32 columns, the two warps of a quarter taking alternate ones
@@ -976,8 +997,7 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, 2>::THREADS, 1)
             const uint32_t dst = mapa_shared(sbase, (uint32_t)(2 * to + rank)) + (uint32_t)(slot * S::SLOT + row * 16);
             uint32_t v[32];
             if (nkb > 0) {
-                tmem_ld_32x32b_x32(taddr + (uint32_t)(to * W + ch * 32), v);
-                tmem_ld_wait_regs(v);
+                load_acc((uint32_t)(to * W + ch * 32), v);
             } else {
 #pragma unroll
                 for (int k = 0; k < 32; ++k) v[k] = 0u;
@@ -990,8 +1010,7 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, 2>::THREADS, 1)
 #pragma unroll
         for (int ch = 0; ch < NCH; ++ch) {
             if (nkb > 0 && finishes) {
-                tmem_ld_32x32b_x32(taddr + (uint32_t)(split * W + half * CW + ch * 32), own[ch]);
-                tmem_ld_wait_regs(own[ch]);
+                load_acc((uint32_t)(split * W + half * CW + ch * 32), own[ch]);
             } else {
 #pragma unroll
                 for (int k = 0; k < 32; ++k) own[ch][k] = 0u;
@@ -1003,7 +1022,7 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, 2>::THREADS, 1)
     cluster_sync_all();  // the parts have arrived, and every accumulator has been read
     if (warp == C::MMA_WARP) {
         tc_fence_after();
-        tmem_dealloc_cg<2>(tmem, BN);
+        tmem_dealloc_cg<2>(tmem, S::TMEM_COLS);
     }
 
     if (warp < C::EPI) {
@@ -2724,6 +2743,12 @@ bool wgtap_setup(const dbl_conv_shape* s, Plan& pl)
     int max_cl = 1;
     while (max_cl < 4 && dbl::cluster_held<conv_wgtap_kernel>(max_cl + 1, kWgTapThreads, kWinSmemMax)) ++max_cl;
     const int64_t elems = (int64_t)9 * s->c * s->k;
+    // outputs a CTA adds up: no more than the implicit GEMM (the tensor core's sums lose with their length)
+    const int BN = choose_bn(s->k), cg = 2;
+    const int64_t pix = (int64_t)s->n * P * (Wp - 2), igemm_kb = (pix + 127) / 128;
+    if (igemm_kb > INT32_MAX / 2) return false;
+    const int igemm_splits = wgrad_splits((9 * s->c + cg * BM - 1) / (cg * BM) * (s->k / BN), (int)igemm_kb, 9 * s->c, s->k, BN, cg);
+    const int64_t longest = (igemm_kb + igemm_splits - 1) / igemm_splits * 128;
     double best = 1e300;
     ConvParams& p = pl.p;
     for (int u = 1; u <= kMaxPos; ++u) {  // u rows of an image, then u - P + 1 images
@@ -2744,6 +2769,7 @@ bool wgtap_setup(const dbl_conv_shape* s, Plan& pl)
                 if (slices == last) continue;
                 last = slices;
                 const int sp = slices * cl;
+                if (kbs * ni * R * (Wp - 2) > longest) continue;
                 if (cl > 1 && (size_t)stages * 4 * strip < (size_t)(cl - 1) * (12 / cl) * 16384) break;
                 const int rounds = (groups * sp + resident[cl] - 1) / resident[cl];
                 const double cost = rounds * (kbs * (ksteps * 192.0 + 150.0) + 4000.0 + 3000.0 / cl +
@@ -3001,6 +3027,7 @@ void wgrad_cluster(Plan& pl, int splits)
         if (slices < 1 || pl.BN / sk < 32) continue;
         if (!(pl.BN == 256 ? split_held<256, kFamWgrad>(sk) : split_held<128, kFamWgrad>(sk))) break;
         const int kbs = (p.num_kb + slices * sk - 1) / (slices * sk);
+        if ((kbs + 1) / 2 > (p.num_kb + splits - 1) / splits) continue;  // an accumulator's K-blocks: no more than a slice's
         const int used = (p.num_kb + kbs * sk - 1) / (kbs * sk);  // no slice without a K-block
         const double cost = kbs * kbc + 10500.0 + acc * (sk - 1) / sk / 22.0 + reduce(used);
         if (cost < best) {

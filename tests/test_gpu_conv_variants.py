@@ -280,3 +280,33 @@ def test_devices_that_place_smaller_clusters_run_the_same_calls(tmp_path):
         for a, b, tol in zip(got[16], got[n], (2.0 ** -7, 2.0 ** -6, 2.0 ** -7, 1e-5, 1e-5)):
             # 16-bit outputs: a rounding decided otherwise by the order of fp32 sums (y is also dw's operand)
             assert (a - b).abs().max() <= tol * a.abs().max()
+
+
+@pytest.mark.parametrize("n,h,c,k,stride,steps", [
+    (256, 4, 256, 256, 1, 32),   # four pairs per tile, eight K-blocks each
+    (64, 8, 256, 256, 1, 32),
+    (37, 32, 128, 256, 2, 40),   # eight pairs
+    (128, 7, 256, 128, 1, 56),   # 128 columns
+])
+def test_split_wgrad_sums_no_longer_chains_than_slices(D, n, h, c, k, stride, steps):
+    """The tensor core rounds its sums towards zero: a chain of K-steps of 16 positions loses with its length.
+    Random terms leave partial sums of sqrt(i / L) of the result after step i of L, each cut by half a unit of 2^-23
+    on average: L / 3 * 2^-24 for all, a quarter more for the fp32 additions.  steps: L of the slices that run
+    without clusters."""
+    shape = D.conv_shape(n, h, h, c, k, 3, stride, 1)
+    info = D.dbl_conv_plan(shape, D.DBL_PASS_WGRAD)
+    assert info.kernel == D.DBL_KERNEL_IGEMM and info.grid > 2 * info.tiles  # tiles split over pairs
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    p = (h - 1) // stride + 1
+    x = torch.randn((n, h, h, c), device="cuda", generator=gen).to(torch.bfloat16)
+    dy = torch.randn((n, p, p, k), device="cuda", generator=gen).to(torch.bfloat16)
+    wsb = D.dbl_conv_workspace_bytes(shape, D.DBL_PASS_WGRAD)
+    dw = torch.full((k, 3, 3, c), float("nan"), device="cuda")
+    D.dbl_conv_wgrad(shape, x, dy, dw, False, ws(wsb), wsb)
+    xp = torch.nn.functional.pad(x.double(), (0, 0, 1, 1, 1, 1))
+    d2 = dy.double().reshape(-1, k)
+    ref = torch.stack([torch.stack([d2.T @ xp[:, a:a + stride * p:stride, b:b + stride * p:stride].reshape(-1, c)
+                                    for b in range(3)], 1) for a in range(3)], 1)
+    err = float((dw.double() - ref).norm() / ref.norm())
+    assert err <= 1.25 * steps / 3 * 2.0 ** -24
+    check_status(D)
