@@ -561,11 +561,14 @@ __global__ void __launch_bounds__(kPoolThreads, 1)
         }
         __syncthreads();
         float* p = partial + (int64_t)blk * 2 * C;
-        for (int e = threadIdx.x; e < 2 * C; e += kPoolThreads) {  // one sum per thread, blocks in order
+        for (int e = threadIdx.x; e < 2 * C; e += kPoolThreads) {  // one sum per thread, of four of every fourth row
             const int x = e >= C, c = e - x * C;
-            float t = 0.f;
-            for (int q = c / 8; q < rstep * groups; q += groups) t += red[q][8 * x + c % 8];
-            p[e] = x ? t * invstd[c] : t;
+            float t[4] = {};
+            for (int q = 0; q < rstep; q += 4)  // rstep: a power of two, 4 or more (at most 1024 channels)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) t[k] += red[(q + k) * groups + c / 8][8 * x + c % 8];
+            const float u = (t[0] + t[1]) + (t[2] + t[3]);
+            p[e] = x ? u * invstd[c] : u;
         }
         __syncthreads();
     }
