@@ -127,7 +127,9 @@ struct Cfg {
     // (the last tile's epilogue is not hidden behind MMAs; with four warps it takes 750 cycles per 32
     // columns with channel sums): forward at 10x10x256, batch 128 20.4 -> 18.5 us, 7x7x512, batch 128
     // 30.1 -> 28.2, its data gradient 27.5 -> 27.2; a 14x14 1x1 projection 256 -> 512 11.5 -> 9.8
-    static constexpr int EPI = BN > 64 ? 8 : 4;
+    // (weight gradients keep four, whose CTAs start sooner: 4x4 maps of 256 channels, one image 8.2 us with eight and
+    // 7.6 with four, 3x3 128 -> 256, batch 16 8.9 and 8.3)
+    static constexpr int EPI = BN > 64 && FAM == kFamFwd ? 8 : 4;
     static constexpr int CW = BN * 4 / EPI;                    // columns one epilogue warp drains
     static constexpr int EPI_TILE = BN > 64 ? 0 : 4 * 32 * 33 * 4;  // per-warp 32x32 transpose scratch (RowStats)
     static constexpr int EPI_SUM = 4 * 2 * kMaxNcols * 4;      // channel sums per lane quarter (fwd)
@@ -808,6 +810,7 @@ struct SplitCfg {
     // fp32.  4x4x256, batch 256: error of dw against 64 bits 8.4e-7 with one, 4.0e-7 with two, 13.8 us both.
     static constexpr int ACCS = FAM == kFamWgrad ? 2 : 1;
     static constexpr uint32_t TMEM_COLS = ACCS * BN;
+    static constexpr int EPI = 8, MMA_WARP = EPI + kProducers, THREADS = 32 * (MMA_WARP + 1);
     static constexpr int W = BN / SK;              // columns a CTA finishes
     static constexpr int SLOT = 128 * W * 4;        // one received part: [W / 4][128 rows] float4
     static constexpr int CW = W > 32 ? W / 2 : 32;  // columns an epilogue warp finishes (of W = 32: one warp per quarter)
@@ -818,7 +821,7 @@ struct SplitCfg {
 };
 
 template <int BN, int FAM, int SK>
-__global__ void __launch_bounds__(Cfg<BN, FAM, 2>::THREADS, 1)
+__global__ void __launch_bounds__(SplitCfg<BN, FAM, SK>::THREADS, 1)
     conv_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                        const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2,
                        const ConvParams p)
@@ -860,7 +863,7 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, 2>::THREADS, 1)
         abort_flag = 0;
         fence_mbar_init();
     }
-    if (warp >= C::EPI && warp < C::MMA_WARP && lane == 0) {
+    if (warp >= S::EPI && warp < S::MMA_WARP && lane == 0) {
         tma_prefetch_desc(&tmA);
         tma_prefetch_desc(&tmB);
         if (p.proj_kb) {
@@ -868,7 +871,7 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, 2>::THREADS, 1)
             tma_prefetch_desc(&tmB2);
         }
     }
-    if (warp == C::MMA_WARP) {
+    if (warp == S::MMA_WARP) {
         tmem_alloc_cg<2>(&tmem_slot, S::TMEM_COLS);
         tmem_relinquish_cg<2>();
     }
@@ -881,9 +884,9 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, 2>::THREADS, 1)
     const int64_t gPQ = (int64_t)p.gP * p.gQ;
     const int nkb_first = S::ACCS == 2 ? (nkb + 1) / 2 : nkb;  // K-blocks of the first accumulator
 
-    if (warp >= C::EPI && warp < C::MMA_WARP) {
+    if (warp >= S::EPI && warp < S::MMA_WARP) {
         // ------------------------------------------------------------------ TMA producers
-        const int prod = warp - C::EPI;
+        const int prod = warp - S::EPI;
         int tn = 0, tp = 0, tq = 0;
         if constexpr (FAM == kFamFwd) {
             const int64_t m0 = ((int64_t)tc.m_tile * 2 + rank) * 128;
@@ -921,7 +924,7 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, 2>::THREADS, 1)
                 }
             }
         }
-    } else if (warp == C::MMA_WARP) {
+    } else if (warp == S::MMA_WARP) {
         // ------------------------------------------------------------------ MMA issuer (rank 0 of each pair)
         if (rank == 0) {
             // operand layouts as in conv_igemm_kernel
@@ -972,7 +975,7 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, 2>::THREADS, 1)
     const int row = quarter * 32 + lane;             // row within the 128-row accumulator
     const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16);
     constexpr int CW = S::CW, NCH = CW / 32;
-    const bool finishes = warp < C::EPI && half * CW < W;
+    const bool finishes = warp < S::EPI && half * CW < W;
     auto load_acc = [&](uint32_t col, uint32_t(&v)[32]) {  // 32 columns of the accumulator, or of both
         tmem_ld_32x32b_x32(taddr + col, v);
         if (S::ACCS == 2 && nkb > nkb_first) {
@@ -987,7 +990,7 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, 2>::THREADS, 1)
         }
     };
     uint32_t own[NCH][32];  // this warp's part of the CTA's own columns
-    if (warp < C::EPI) {
+    if (warp < S::EPI) {
         // the other pairs' chunks of 32 columns, the two warps of a quarter taking alternate ones
 #pragma unroll 1
         for (int e = half; e < (SK - 1) * (W / 32); e += 2) {
@@ -1020,12 +1023,12 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, 2>::THREADS, 1)
     }
     __syncwarp();
     cluster_sync_all();  // the parts have arrived, and every accumulator has been read
-    if (warp == C::MMA_WARP) {
+    if (warp == S::MMA_WARP) {
         tc_fence_after();
         tmem_dealloc_cg<2>(tmem, S::TMEM_COLS);
     }
 
-    if (warp < C::EPI) {
+    if (warp < S::EPI) {
         // ------------------------------------------------------------------ epilogue of this CTA's columns
         float* sums = reinterpret_cast<float*>(sgen + C::RING);
         const bool want_stats = FAM == kFamFwd && p.mode == kFwd && p.stats != nullptr;
@@ -2982,7 +2985,7 @@ constexpr int kTileCost = 20;
 template <int BN, int FAM>
 bool split_held(int sk)
 {
-    constexpr int T = Cfg<BN, FAM, 2>::THREADS;
+    constexpr int T = SplitCfg<BN, FAM, 2>::THREADS;
     if (sk == 2) return dbl::cluster_held<conv_splitk_kernel<BN, FAM, 2>>(4, T, SplitCfg<BN, FAM, 2>::SMEM);
     if (sk == 4) return dbl::cluster_held<conv_splitk_kernel<BN, FAM, 4>>(8, T, SplitCfg<BN, FAM, 4>::SMEM);
     if constexpr (BN == 256) return dbl::cluster_held<conv_splitk_kernel<BN, FAM, 8>>(16, T, SplitCfg<BN, FAM, 8>::SMEM);
@@ -3375,7 +3378,7 @@ int launch_splitk(const Plan& pl, const CUtensorMap& a, const CUtensorMap& b, co
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[2];
     cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(Cfg<BN, FAM, 2>::THREADS);
+    cfg.blockDim = dim3(SplitCfg<BN, FAM, SK>::THREADS);
     cfg.dynamicSmemBytes = SplitCfg<BN, FAM, SK>::SMEM;
     cfg.stream = st;
     cfg.attrs = at;
