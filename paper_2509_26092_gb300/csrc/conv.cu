@@ -128,7 +128,7 @@ struct Cfg {
     // columns with channel sums): forward at 10x10x256, batch 128 20.4 -> 18.5 us, 7x7x512, batch 128
     // 30.1 -> 28.2, its data gradient 27.5 -> 27.2; a 14x14 1x1 projection 256 -> 512 11.5 -> 9.8
     // (weight gradients keep four, whose CTAs start sooner: 4x4 maps of 256 channels, one image 8.2 us with eight and
-    // 7.6 with four, 3x3 128 -> 256, batch 16 8.9 and 8.3)
+    // 7.7 with four, 3x3 maps 128 -> 256, batch 16 8.8 and 8.4)
     static constexpr int EPI = BN > 64 && FAM == kFamFwd ? 8 : 4;
     static constexpr int CW = BN * 4 / EPI;                    // columns one epilogue warp drains
     static constexpr int EPI_TILE = BN > 64 ? 0 : 4 * 32 * 33 * 4;  // per-warp 32x32 transpose scratch (RowStats)

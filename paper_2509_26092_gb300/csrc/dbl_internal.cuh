@@ -54,14 +54,14 @@ template <auto KERNEL>
 bool cluster_held(int ctas, int threads, size_t smem)
 {
     static std::atomic<signed char> cached[64][17] = {};
-    int dev = 0, sms = 0;
     if (ctas > max_cluster()) return false;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    int dev = 0, sms = 0;
+    const bool current = cudaGetDevice(&dev) == cudaSuccess, cache = current && dev >= 0 && dev < 64 && ctas <= 16;
+    if (cache && cached[dev][ctas]) return cached[dev][ctas] > 0;
+    if (!current || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
         (void)cudaGetLastError();
         return true;
     }
-    const bool cache = dev >= 0 && dev < 64 && ctas <= 16;
-    if (cache && cached[dev][ctas]) return cached[dev][ctas] > 0;
     cudaError_t e = cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess && ctas > 8) e = cudaFuncSetAttribute(KERNEL, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     cudaLaunchConfig_t cfg = {};
