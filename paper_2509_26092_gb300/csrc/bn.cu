@@ -139,10 +139,10 @@ __global__ void __launch_bounds__(dbl::dev::kPartialsThreads) bn_fwd_finalize_pa
                                                                     float* __restrict__ save_mean,
                                                                     float* __restrict__ save_invstd)
 {
-    dbl::dev::ChannelSums sums;
-    const int c = dbl::dev::partials_colsum(part, nparts, C, sums);
+    float sum, sumsq;
+    const int c = dbl::dev::partials_colsum(part, nparts, C, sum, sumsq);
     if (c < 0) return;
-    finalize_channel(sums.f32(0), sums.f32(1), inv_n, eps, save_mean[c], save_invstd[c]);
+    finalize_channel(sum, sumsq, inv_n, eps, save_mean[c], save_invstd[c]);
 }
 
 // Thread t of a CTA owns channel group g = t % (C/8) (8 channels, one 16-byte
@@ -215,12 +215,12 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM)
     __shared__ __align__(16) float chan[2][kFwdSliceC];  // scale, shift
     const int slices = C / kFwdSliceC, c0 = blockIdx.x % slices * kFwdSliceC;
     const int block = blockIdx.x / slices, blocks = gridDim.x / slices;
-    dbl::dev::ChannelSums sums;
-    dbl::dev::partials_colsum32(part, nparts, C, c0, sums);
+    float sum, sumsq;
+    dbl::dev::partials_colsum32(part, nparts, C, c0, sum, sumsq);
     if (threadIdx.x < kFwdSliceC) {
         const int c = c0 + threadIdx.x;
         float m, is;
-        finalize_channel(sums.f32(0), sums.f32(1), inv_n, eps, m, is);
+        finalize_channel(sum, sumsq, inv_n, eps, m, is);
         if (block == 0) {
             save_mean[c] = m;
             save_invstd[c] = is;
@@ -594,10 +594,9 @@ __global__ void __launch_bounds__(dbl::dev::kPartialsThreads) bn_bwd_finalize_ke
     const float* __restrict__ mean, const float* __restrict__ invstd, float* __restrict__ dgamma,
     float* __restrict__ dbeta, float* __restrict__ coef)
 {
-    dbl::dev::ChannelSums sums;
-    const int c = dbl::dev::partials_colsum(partial, nblk, C, sums);
+    double sg, sgx;
+    const int c = dbl::dev::partials_colsum(partial, nblk, C, sg, sgx);
     if (c < 0) return;
-    const double sg = sums.f64(0), sgx = sums.f64(1);
     dbeta[c] = (float)sg;
     dgamma[c] = (float)sgx;
     bwd_coefficients(sg, sgx, inv_n, gamma[c], invstd[c], mean[c], coef[c], coef[C + c], coef[2 * C + c]);
@@ -676,6 +675,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     dbl::dev::grid_dependency_trigger();  // a convolution launched next may start its set-up
     __shared__ float red[kThreads / 32][2][kSliceC];
     __shared__ float tot[2][kSliceC];   // this CTA's sums, read by the whole cluster
+    __shared__ double all[2][kSliceC];  // the cluster's
     __shared__ __align__(16) float coef[3][kSliceC];
     const int rank = (int)dbl::dev::cluster_ctarank(), slice = blockIdx.x / CL;
     const int c0 = slice * kSliceC, vl = threadIdx.x % kSliceVec, g = c0 / 8 + vl, groups = C / 8;
@@ -728,30 +728,29 @@ __global__ void __launch_bounds__(kThreads, 2)
     }
     __syncwarp();
     dbl::dev::cluster_sync_all();
-    if (threadIdx.x < kSliceC) {
-        const int c = threadIdx.x;
-        float v[2][16];
+    if (threadIdx.x < 2 * kSliceC) {  // one sum per thread
+        const int st = threadIdx.x / kSliceC, c = threadIdx.x % kSliceC;
+        float v[16];
 #pragma unroll
         for (int r = 0; r < 16; ++r)
+            v[r] = r < CL ? dbl::dev::ld_cluster_f32(dbl::dev::mapa_shared(dbl::dev::smem_u32(&tot[st][c]), r)) : 0.f;
+        dbl::dev::Sum3 t{0.f, 0.f, 0.f};
 #pragma unroll
-            for (int st = 0; st < 2; ++st)
-                v[st][r] = r < CL ? dbl::dev::ld_cluster_f32(dbl::dev::mapa_shared(dbl::dev::smem_u32(&tot[st][c]), r))
-                                  : 0.f;
-        double sums[2];
-#pragma unroll
-        for (int st = 0; st < 2; ++st) {
-            dbl::dev::Sum3 t{0.f, 0.f, 0.f};
+        for (int r = 0; r < 16; ++r)
+            if (r < CL) t = dbl::dev::sum_add(t, v[r]);
+        double sum = dbl::dev::sum_f64(t);
+        if (!dbl::dev::sum_held(t)) {  // beyond fp32's range, or not a number
+            sum = 0.0;
 #pragma unroll
             for (int r = 0; r < 16; ++r)
-                if (r < CL) t = dbl::dev::sum_add(t, v[st][r]);
-            sums[st] = dbl::dev::sum_f64(t);
-            if (!dbl::dev::sum_held(t)) {  // beyond fp32's range, or not a number
-                sums[st] = 0.0;
-#pragma unroll
-                for (int r = 0; r < 16; ++r)
-                    if (r < CL) sums[st] += (double)v[st][r];
-            }
+                if (r < CL) sum += (double)v[r];
         }
+        all[st][c] = sum;
+    }
+    __syncthreads();
+    if (threadIdx.x < kSliceC) {
+        const int c = threadIdx.x;
+        const double sums[2] = {all[0][c], all[1][c]};
         if (rank == 0) {
             dbeta[c0 + c] = (float)sums[0];
             dgamma[c0 + c] = (float)sums[1];

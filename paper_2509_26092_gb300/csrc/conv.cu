@@ -2363,11 +2363,11 @@ __global__ void __launch_bounds__(kWgTapThreads, 1)
 __global__ void __launch_bounds__(kPartialsThreads) stats_reduce_kernel(const float* __restrict__ part, int nparts, int K,
                                                            float* __restrict__ sum, float* __restrict__ sumsq)
 {
-    ChannelSums sums;
-    const int c = partials_colsum(part, nparts, K, sums);
+    float s, q;
+    const int c = partials_colsum(part, nparts, K, s, q);
     if (c >= 0) {
-        sum[c] = sums.f32(0);
-        sumsq[c] = sums.f32(1);
+        sum[c] = s;
+        sumsq[c] = q;
     }
 }
 

@@ -332,8 +332,8 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
 // An unevaluated sum a + b + c of three fp32 values, for sums that fp64 would hold, at the rate of fp32 (this
 // GPU runs an fp64 instruction of a warp in about 16 cycles): additions are exact but for c, whose rounding
 // is below 2^-68 of the terms' sizes, where an fp64 addition rounds at 2^-53 of its result.  The same trees in
-// fp64: forward BatchNorm of 2048 rows of 256 channels, 32 partials, 8.3 us against 4.3; 576 rows of 512
-// channels, 152 partials, 6.5 against 5.9.
+// fp64: forward BatchNorm of 2048 rows of 256 channels, 32 partials, 8.3 us against 4.2; 576 rows of 512
+// channels, 152 partials, 6.5 against 5.8.
 struct Sum3 {
     float a, b, c;
 };
@@ -398,15 +398,9 @@ __device__ __forceinline__ float sum_f32(Sum3 x)
 // Whether fp32 held the sum.
 __device__ __forceinline__ bool sum_held(Sum3 x) { return isfinite(x.a + (x.b + x.c)); }
 
-// A channel's two sums: as Sum3, or in fp64 where those are beyond fp32's range or not a number.
-struct ChannelSums {
-    Sum3 s[2];
-    double wide[2];
-    bool held;
-
-    __device__ __forceinline__ double f64(int x) const { return held ? sum_f64(s[x]) : wide[x]; }
-    __device__ __forceinline__ float f32(int x) const { return held ? sum_f32(s[x]) : (float)wide[x]; }
-};
+// A sum as fp32 (rounded once) or fp64.
+__device__ __forceinline__ void sum_to(Sum3 x, float& r) { r = sum_f32(x); }
+__device__ __forceinline__ void sum_to(Sum3 x, double& r) { r = sum_f64(x); }
 
 // Eight sums in pairs, neighbours first.
 template <class T, class F>
@@ -443,11 +437,12 @@ constexpr int kPartialsThreads = 256;
 constexpr int kPartialsChannels = 8;
 static_assert(kPartialsThreads == 32 * kPartialsChannels, "32 streams of 8 channels");
 
-// The tree over the 32 streams' sums of a block's eight channels; threads t < 8 get channel t's.
+// The tree over the 32 streams' sums of a block's eight channels; threads t < 16 get sum t / 8 of channel t % 8.
 template <class T>
-__device__ __forceinline__ void partials_tree(float s, float sc, float q, float qc,
-                                              T (&red)[2][kPartialsThreads / 32][kPartialsChannels], T (&d)[2])
+__device__ __forceinline__ T partials_tree(float s, float sc, float q, float qc,
+                                           T (&red)[2][kPartialsThreads / 32][kPartialsChannels])
 {
+    T d[2];
     sum_from(s, sc, d[0]);
     sum_from(q, qc, d[1]);
     // stream bits 0 and 1 are lane bits 3 and 4
@@ -461,14 +456,15 @@ __device__ __forceinline__ void partials_tree(float s, float sc, float q, float 
         red[1][w][cl] = d[1];
     }
     __syncthreads();
-    if (threadIdx.x < kPartialsChannels) {
-        // stream bits 2, 3 and 4 are warp bits 0, 1 and 2
-        d[0] = sum_tree8<T>([&](int i) { return red[0][i][cl]; });
-        d[1] = sum_tree8<T>([&](int i) { return red[1][i][cl]; });
-    }
+    // stream bits 2, 3 and 4 are warp bits 0, 1 and 2
+    if (threadIdx.x < 2 * kPartialsChannels)
+        d[0] = sum_tree8<T>([&](int i) { return red[threadIdx.x / kPartialsChannels][i][cl]; });
+    return d[0];
 }
 
-__device__ __forceinline__ int partials_colsum(const float* __restrict__ part, int nparts, int K, ChannelSums& sums)
+// R: float or double.
+template <class R>
+__device__ __forceinline__ int partials_colsum(const float* __restrict__ part, int nparts, int K, R& sum0, R& sum1)
 {
     __shared__ Sum3 red[2][kPartialsThreads / 32][kPartialsChannels];
     __shared__ double wide[2][kPartialsThreads / 32][kPartialsChannels];
@@ -493,16 +489,26 @@ __device__ __forceinline__ int partials_colsum(const float* __restrict__ part, i
                 }
         }
     }
-    partials_tree(s, sc, q, qc, red, sums.s);
-    sums.held = threadIdx.x >= kPartialsChannels || (sum_held(sums.s[0]) && sum_held(sums.s[1]));
-    if (__syncthreads_or(!sums.held)) partials_tree(s, sc, q, qc, wide, sums.wide);
+    const bool sums = threadIdx.x < 2 * kPartialsChannels;
+    const Sum3 d = partials_tree(s, sc, q, qc, red);
+    const bool held = !sums || sum_held(d);
+    double w = 0.0;
+    if (__syncthreads_or(!held)) w = partials_tree(s, sc, q, qc, wide);
+    sum0 = sum1 = R(0);
+    if (sums) {
+        if (held)
+            sum_to(d, sum0);
+        else
+            sum0 = (R)w;
+        sum1 = __shfl_down_sync((1u << 2 * kPartialsChannels) - 1u, sum0, kPartialsChannels);
+    }
     return (threadIdx.x < kPartialsChannels && c < K) ? c : -1;
 }
 
-// The tree of partials_colsum32, from its four streams per warp and channel.
+// The tree of partials_colsum32, from its four streams per warp and channel: threads t < 64 get sum t / 32 of
+// channel t % 32.
 template <class T>
-__device__ __forceinline__ void partials_tree32(const float (&s)[2][4], const float (&sc)[2][4], T (&red)[2][8][32],
-                                                T (&d)[2])
+__device__ __forceinline__ T partials_tree32(const float (&s)[2][4], const float (&sc)[2][4], T (&red)[2][8][32])
 {
     const int cl = threadIdx.x % 32, w = threadIdx.x / 32;
 #pragma unroll
@@ -513,19 +519,20 @@ __device__ __forceinline__ void partials_tree32(const float (&s)[2][4], const fl
         red[x][w][cl] = sum_add(sum_add(a[0], a[1]), sum_add(a[2], a[3]));
     }
     __syncthreads();
-    if (threadIdx.x < 32)
-#pragma unroll
-        for (int x = 0; x < 2; ++x) d[x] = sum_tree8<T>([&](int i) { return red[x][i][cl]; });
+    T d{};
+    if (threadIdx.x < 64) d = sum_tree8<T>([&](int i) { return red[w][i][cl]; });
+    return d;
 }
 
 // The same sums, bit for bit, of 32 channels from c0 by a block of 256 threads (K a multiple of 32): thread t
 // takes channel t % 32 and the four streams 4*(t/32) .., whose tree it walks itself; the warps' trees
-// are the upper stream bits.  Threads t < 32 get the sums of channel c0 + t.
+// are the upper stream bits.  Threads t < 32 get the sums of channel c0 + t, rounded to fp32.
 __device__ __forceinline__ void partials_colsum32(const float* __restrict__ part, int nparts, int K, int c0,
-                                                  ChannelSums& sums)
+                                                  float& sum0, float& sum1)
 {
     __shared__ Sum3 red[2][8][32];
     __shared__ double wide[2][8][32];
+    __shared__ float out[2][32];
     const int cl = threadIdx.x % 32, w = threadIdx.x / 32;
     const float* p = part + c0 + cl;
     const int64_t ld = 2 * (int64_t)K;
@@ -539,9 +546,16 @@ __device__ __forceinline__ void partials_colsum32(const float* __restrict__ part
             kahan_add(s[1][u], sc[1][u], __ldg(p + t * ld + K));
         }
     }
-    partials_tree32(s, sc, red, sums.s);
-    sums.held = threadIdx.x >= 32 || (sum_held(sums.s[0]) && sum_held(sums.s[1]));
-    if (__syncthreads_or(!sums.held)) partials_tree32(s, sc, wide, sums.wide);
+    const Sum3 d = partials_tree32(s, sc, red);
+    const bool held = threadIdx.x >= 64 || sum_held(d);
+    if (threadIdx.x < 64) out[w][cl] = sum_f32(d);
+    if (__syncthreads_or(!held)) {
+        const double v = partials_tree32(s, sc, wide);
+        if (!held) out[w][cl] = (float)v;
+        __syncthreads();
+    }
+    sum0 = out[0][cl];
+    sum1 = out[1][cl];
 }
 
 // ---------------------------------------------------------------------------- TMA
