@@ -120,17 +120,21 @@ def _conv_case(D, n, h, c, k, r, stride, pad, seed):
     return D.conv_shape(n, h, h, c, k, r, stride, pad), x, wt, p
 
 
-@pytest.mark.parametrize("n,h,c,k,r,stride,pad", [
-    (1, 3, 512, 512, 3, 1, 1),     # 9 rows in a 256-row tile: eight pairs per tile
-    (29, 3, 512, 512, 3, 1, 1),    # 261 rows: a second tile with five rows, all of rank 1's beyond the batch
-    (100, 3, 512, 512, 3, 1, 1),   # 8 tiles: four pairs per tile
-    (65, 8, 256, 512, 3, 2, 1),    # ragged batch, two column tiles
-    (500, 3, 512, 512, 3, 1, 1),   # 36 tiles: two pairs per tile
-    (32, 6, 256, 256, 1, 2, 0),    # a short reduction (4 K-blocks): not split
+@pytest.mark.parametrize("n,h,c,k,r,stride,pad,pairs,dgrad_pairs", [
+    (1, 3, 512, 512, 3, 1, 1, 8, 8),     # 9 rows in a 256-row tile: eight pairs per tile
+    (29, 3, 512, 512, 3, 1, 1, 8, 8),    # 261 rows: a second tile with five rows, all of rank 1's beyond the batch
+    (100, 3, 512, 512, 3, 1, 1, 4, 4),   # 8 tiles: four pairs per tile
+    (65, 8, 256, 512, 3, 2, 1, 4, 2),    # ragged batch, two column tiles
+    (500, 3, 512, 512, 3, 1, 1, 2, 2),   # 36 tiles: two pairs per tile
+    (32, 6, 256, 256, 1, 2, 0, 2, 2),    # a short reduction: two K-blocks a pair
+    (32, 6, 128, 256, 1, 2, 0, 1, None),  # two K-blocks: not split
 ])
-def test_split_conv_matches_oracle(D, n, h, c, k, r, stride, pad):
+def test_split_conv_matches_oracle(D, n, h, c, k, r, stride, pad, pairs, dgrad_pairs):
     """Forward (with its channel sums) and data gradient of layers with few 256-column tiles."""
     shape, x, wt, p = _conv_case(D, n, h, c, k, r, stride, pad, n + h)
+    for pss, want in ((D.DBL_PASS_FWD, pairs), (D.DBL_PASS_DGRAD, dgrad_pairs)):
+        info = D.dbl_conv_plan(shape, pss)
+        assert want is None or (info.kernel == D.DBL_KERNEL_IGEMM and info.grid == 2 * want * info.tiles)
     xd, wd = to_bf16_dev(x), to_bf16_dev(wt)
     y = torch.full((n, p, p, k), float("nan"), dtype=torch.bfloat16, device="cuda")
     s1, s2 = torch.empty(k, device="cuda"), torch.empty(k, device="cuda")
@@ -171,7 +175,8 @@ def test_filter_row_wgrad_matches_oracle(D, n, h, w, c, k, pad):
     at += [tuple(int(g.integers(0, m)) for m in (k, 3, 3, c)) for _ in range(20)]
     ref = np.array([orc.conv2d_wgrad_at(x, dy, (k, 3, 3, c), 1, pad, *i) for i in at])
     shape = D.conv_shape(n, h, w, c, k, 3, 1, pad)
-    assert D.dbl_conv_plan(shape, D.DBL_PASS_WGRAD).kernel == D.DBL_KERNEL_WINDOW_WGRAD
+    info = D.dbl_conv_plan(shape, D.DBL_PASS_WGRAD)
+    assert info.kernel == D.DBL_KERNEL_WINDOW_WGRAD and info.tile_cols == 128
     wsb = D.dbl_conv_workspace_bytes(shape, D.DBL_PASS_WGRAD)
     dw = torch.full((k, 3, 3, c), float("nan"), device="cuda")
     work, xd, dyd = ws(wsb), to_bf16_dev(x), to_bf16_dev(dy)
@@ -217,17 +222,19 @@ def test_pixel_pair_conv_matches_oracle(D, n, h, w):
     check_status(D)
 
 
-@pytest.mark.parametrize("n,h,c,k,r,stride", [
-    (33, 14, 64, 128, 3, 2),   # 128 columns, two pairs per tile, seven slices; a last row tile of 64
-    (33, 5, 256, 128, 3, 1),   # 128 columns, four pairs, no slices: written straight into dw
-    (65, 3, 512, 512, 3, 1),   # 256 columns, two pairs of three and two K-blocks
-    (65, 14, 256, 512, 1, 2),  # four pairs, seven slices, pairs without a K-block
-    (17, 14, 128, 256, 3, 2),  # eight pairs
+@pytest.mark.parametrize("n,h,c,k,r,stride,pairs,slices", [
+    (33, 14, 64, 128, 3, 2, 2, 7),   # 128 columns, two pairs per tile, seven slices; a last row tile of 64
+    (33, 5, 256, 128, 3, 1, 4, 1),   # 128 columns, four pairs, no slices: written straight into dw
+    (65, 3, 512, 512, 3, 1, 2, 1),   # 256 columns, two pairs of three and two K-blocks
+    (65, 14, 256, 512, 1, 2, 4, 7),  # four pairs, seven slices, pairs without a K-block
+    (17, 14, 128, 256, 3, 2, 8, 1),  # eight pairs
 ])
-def test_split_wgrad_matches_oracle(D, n, h, c, k, r, stride):
+def test_split_wgrad_matches_oracle(D, n, h, c, k, r, stride, pairs, slices):
     """Weight gradients whose tiles are shared by clusters of CTA pairs."""
     pad = 1 if r == 3 else 0
     shape, x, wt, p = _conv_case(D, n, h, c, k, r, stride, pad, n + c)
+    info = D.dbl_conv_plan(shape, D.DBL_PASS_WGRAD)
+    assert info.kernel == D.DBL_KERNEL_IGEMM and info.zdim == slices and info.grid == 2 * pairs * info.tiles
     dy = bf16_values(rng(n).standard_normal((n, p, p, k)))
     ref = orc.conv2d_wgrad(x, dy, wt.shape, stride, pad)
     wsb = D.dbl_conv_workspace_bytes(shape, D.DBL_PASS_WGRAD)
