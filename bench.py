@@ -700,7 +700,7 @@ def run_ours(args, cfg):
                          "CUDA-graph replays; traffic = ncu DRAM bytes of the same launches, null if the kernel "
                          "changed since the capture)",
                 "kernel": "conv_igemm_kernel, conv_splitk_kernel, conv_win_kernel, conv_winpair_kernel, "
-                          "conv_wgrow_kernel, conv_wgtap_kernel, conv_wgwin_kernel with their channel-sum and "
+                          "conv_wgrow_kernel, conv_wgtap_kernel with their channel-sum and "
                           f"split-K reduce kernels (fwd/dgrad/wgrad, every layer of both workers at {top['res']} px)",
                 "peak_source": src}
     with D.precision(args.precision):

@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM)
 // Finalize and apply in one launch, for small tensors whose convolution left few partials: every CTA takes 32
 // channels (64 bytes of a row) and a run of the rows, and adds up its channels' partials for itself with the
 // finalize's own tree (the same bits).  The partials come from L2 once per CTA, 256 bytes each, against a
-// launch that reads them once.  576 rows of 512 channels, 32 partials: 5.8 -> 4.0 us.
+// launch that reads them once.  576 rows of 512 channels, 32 partials: 5.2 -> 3.6 us.
 constexpr int kFwdSliceC = 32, kFwdSliceRows = kThreads * 8 / kFwdSliceC;
 
 __global__ void __launch_bounds__(kThreads, kBlocksPerSM)
@@ -657,8 +657,8 @@ __global__ void __launch_bounds__(kThreads, kBwdBlocksPerSM)
 // memory, in rank order, and each forms the three coefficients of the apply pass for itself.  Bound
 // by latency: three launches of the general path cost about 3 us each before they move a byte.
 // General path -> here, bwd without / with a second gradient and g stored (us): 576 rows of 512 channels
-// 11.4 -> 6.2 / 11.0 -> 6.5; 4608 of 512 14.7 -> 12.6 / 15.6 -> 16.3 (stays); 4608 of 256 12.4 -> 8.7 /
-// 12.7 -> 11.5; 12,800 of 256 16.2 -> 15.5 / 17.8 -> 20.9 (stays); 16,384 of 128 12.9 -> 14.0 (stays).
+// 11.1 -> 5.4 / 10.8 -> 5.8; 4608 of 512 13.2 -> 9.8 / 12.8 -> 11.2 (stays); 4608 of 256 11.4 -> 7.8 /
+// 11.1 -> 8.8; 12,800 of 256 13.6 -> 12.5 / 13.5 -> 14.0 (stays); 16,384 of 128 11.2 -> 11.6 (stays).
 constexpr int kSliceC = 32;                    // channels of a slice: 64 bytes of a row
 constexpr int kSliceVec = kSliceC / 8;         // 16-byte vectors of a slice row
 constexpr int kSliceRows = kThreads / kSliceVec;  // rows a CTA covers in one step
@@ -823,10 +823,10 @@ int reduce_grid(int64_t nblk)
     return (int)((nblk + per_cta - 1) / per_cta);
 }
 
-// Forward in one launch (bn_apply_parts_kernel)?  Above 8 MB whole rows stream better than 64-byte slices, and
-// above ~100 partials every CTA's own sum costs what the second launch does (us, two launches -> one):
-// 2 MB with 32 / 100 / 152 partials 6.3 -> 4.6, 6.3 -> 5.3, 6.5 -> 6.1; 6.6 MB 7.5 -> 6.5, 7.9 -> 7.3,
-// 7.8 -> 8.0; 12.8 MB with 32 8.9 -> 9.2.
+// Forward in one launch (bn_apply_parts_kernel)?  Whole rows stream better than 64-byte slices, and above ~100
+// partials every CTA's own sum costs what the second launch does (us, two launches -> one): 2 MB with 32 /
+// 100 / 152 partials 5.9 -> 4.4, 6.1 -> 5.2, 6.1 -> 6.0; 6.6 MB 6.6 -> 5.6, 6.8 -> 6.4, 6.9 -> 7.1; 12.8 MB with 32
+// 7.8 -> 7.0, with 152 8.0 -> 8.5.  The line lies where one launch is still the better one with most partials.
 bool fwd_one_launch(int64_t count, int C, int nparts)
 {
     return C % kFwdSliceC == 0 && nparts <= 104 && count * C * (int64_t)sizeof(act_t) <= (int64_t)8 << 20;

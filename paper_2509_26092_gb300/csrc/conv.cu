@@ -2146,6 +2146,9 @@ __global__ void __launch_bounds__(kWinThreads, 1)
 // Two N = 192 MMAs per 16 positions (192 tensor cycles) read 16 x 512 bytes that TMA loaded once, 43
 // bytes per cycle, where the implicit GEMM loads x once per tap (96 bytes per cycle at 128 columns).
 // The positions of a block are rounded up to 16: the rows behind the strips are zeros written once.
+// Zeros of dy meet the x of their positions, as in conv_wgwin_kernel and conv_wgrow_kernel: an infinite x at a row's
+// end (or in rows past a last block) makes the taps that do not read it NaN as well; the taps that do are not finite
+// in any form.
 // Every CTA ends with 196 KB of partial sums.  A cluster of CL CTAs (win_cl; the same outputs, CL
 // consecutive K ranges) adds them before they leave the SMs: when all MMAs of the cluster are done, each
 // CTA sends the 32-column chunks it does not own into the strip buffers of their owner (distributed
