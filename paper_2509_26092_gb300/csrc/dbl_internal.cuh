@@ -78,7 +78,7 @@ bool cluster_held(int ctas, int threads, size_t smem)
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, KERNEL, &cfg);
     if (e != cudaSuccess) (void)cudaGetLastError();
     const bool held = e == cudaSuccess && n > 0;
-    if (cache) cached[dev][ctas] = held ? 1 : -1;
+    if (cache && (e == cudaSuccess || e == cudaErrorInvalidClusterSize)) cached[dev][ctas] = held ? 1 : -1;  // its answer
     return held;
 }
 #endif
