@@ -584,7 +584,7 @@ __global__ void __launch_bounds__(256) avgpool_kernel(const act_t* __restrict__ 
 // sums that need the same input, share a launch where that suits both (gemm_plan).
 // Bound by fp32 issue: 512 x 1000 x 512 is 7 us of the GPU's fp32 rate.  With 4 x 4 outputs per thread
 // (half the FMAs per shared-memory byte), the partial sums through global memory and a launch of their
-// own, the head of 512 images and 1000 classes took 128.2 us in ten launches; now 74 in five.
+// own, the head of 512 images and 1000 classes took 128.2 us in ten launches; now 73 in five.
 constexpr int GBM = 64, GBN = 128, GBK = 16;
 constexpr int GLA = GBM + 4, GLB = GBN + 4;  // row pitches of the K-major tiles
 constexpr int kGemmThreads = 128;
