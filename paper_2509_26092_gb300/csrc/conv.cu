@@ -2382,12 +2382,14 @@ __global__ void __launch_bounds__(kPartialsThreads) stats_reduce_kernel(const fl
 // rounds bounds it: four loads a round and a remainder one by one were seven rounds of 152 slices' 19 per
 // thread, eight with the remainder together three; weight gradient and reduce 28x28x128, batch 512 79.1 -> 78.1 us,
 // 16x16x128, batch 64 16.4 -> 15.9, a 14x14 projection 256 -> 512, batch 128 12.8 -> 12.2; the same bits.
+// Few slices (LANES = 1) keep four loads a round, as half of eight would be empty: 16x16, 256 -> 512 stride 2, batch 64
+// 16.9 -> 16.6 us.
 template <int LANES>
 __global__ void __launch_bounds__(256) wgrad_reduce_kernel(const float* __restrict__ part, int slices, int64_t n,
                                                            float* __restrict__ dw, int accumulate)
 {
     dbl::dev::grid_dependency_trigger();  // a convolution launched next may start its set-up
-    constexpr int U = 8;
+    constexpr int U = LANES == 1 ? 4 : 8;
     const int j = threadIdx.x % LANES;
     const int64_t n4 = n >> 2;
     const int64_t groups = blockDim.x / LANES;
