@@ -2751,7 +2751,7 @@ bool wgtap_setup(const dbl_conv_shape* s, Plan& pl)
     int max_cl = 1;
     while (max_cl < 4 && dbl::cluster_held<conv_wgtap_kernel>(max_cl + 1, kWgTapThreads, kWinSmemMax)) ++max_cl;
     const int64_t elems = (int64_t)9 * s->c * s->k;
-    // outputs a CTA adds up: no more than the implicit GEMM (the tensor core's sums lose with their length)
+    // positions a CTA adds up: no more than the implicit GEMM (the tensor core's sums lose with their steps)
     const int BN = choose_bn(s->k), cg = 2;
     const int64_t pix = (int64_t)s->n * P * (Wp - 2), igemm_kb = (pix + 127) / 128;
     if (igemm_kb > INT32_MAX / 2) return false;
@@ -2770,16 +2770,17 @@ bool wgtap_setup(const dbl_conv_shape* s, Plan& pl)
         const int64_t blocks = ni > 1 ? (s->n + ni - 1) / ni : (int64_t)s->n * ((P + R - 1) / R);
         if (blocks > INT32_MAX / 4) continue;
         for (int cl = 1; cl <= max_cl; ++cl)
-            for (int sixth = 6, last = 0; sixth >= 1; --sixth) {  // all the slices that fit, or fewer
+            for (int sixth = 18, last = 0; sixth >= 1; --sixth) {  // three rounds of the slices that fit, or fewer
                 int slices = std::max(1, resident[cl] / (groups * cl) * sixth / 6);
                 const int64_t kbs = (blocks + slices * cl - 1) / (slices * cl);
                 slices = (int)((blocks + cl * kbs - 1) / (cl * kbs));  // no cluster without a K-block
                 if (slices == last) continue;
                 last = slices;
                 const int sp = slices * cl;
-                if (kbs * ni * R * (Wp - 2) > longest) continue;
+                if (kbs * ksteps * 16 > longest) continue;
                 if (cl > 1 && (size_t)stages * 4 * strip < (size_t)(cl - 1) * (12 / cl) * 16384) break;
                 const int rounds = (groups * sp + resident[cl] - 1) / resident[cl];
+                if (rounds > 1 && ksteps < 11) continue;  // see below
                 const double cost = rounds * (kbs * (ksteps * 192.0 + 150.0) + 4000.0 + 3000.0 / cl +
                                               (cl > 1 ? 2000.0 + kExchange * (cl - 1) / cl : 0.0)) +
                                     (slices > 1 ? kReduce + kReduceSlice * elems * slices : 0.0);
@@ -2806,7 +2807,9 @@ bool wgtap_setup(const dbl_conv_shape* s, Plan& pl)
     // the better one where the padding of a block's positions costs more than a fifth of them (10x10x256,
     // batch 128 21.4 -> 23.6), where a CTA's K range is shorter than ~22,000 tensor cycles (12x12x128, batch
     // 128 16.7 -> 18.0) and for 512 x 512 channels, whose 48 tiles leave three ranges (7x7, batch 512, three
-    // slices without clusters 91.6 -> 94.6).
+    // slices without clusters 91.6 -> 94.6).  Large maps of 256 channels run in up to three rounds, whose ranges are
+    // as short as the implicit GEMM's: 48x48, batch 219 418 -> 364 and error of dw against 64 bits 2.3e-5 -> 1.7e-5
+    // (one round 334 and 5.2e-5); short K-blocks lose there (16x16, batch 2330, 144 positions 485 -> 532).
     const double used = (double)s->n * P * (Wp - 2) / ((double)p.num_kb * p.win_tile);
     if (used < 0.8 || (double)p.kb_per_split * p.win_tile * 12 < 22000.0) return false;
     pl.win = pl.wgtap = true;
