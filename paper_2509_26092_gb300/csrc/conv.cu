@@ -141,6 +141,7 @@ struct Cfg {
     static_assert(STAGES >= 2, "ring too shallow");
     static_assert(TMEM_COLS <= 512, "TMEM holds 512 columns");
     static_assert(SMEM <= 232448 - 1024, "shared memory per CTA");
+    static_assert(CG == 1 || SMEM >= 117 * 1024, "a cluster kernel's CTA has its SM to itself (kClusterSmem)");
 };
 
 struct TileCoord {
@@ -2542,6 +2543,12 @@ int grid_size(int total_tiles)
 // static barriers and 1 KB of alignment slack).
 constexpr size_t kWinSmemMax = 232448 - 2048;
 
+// Least dynamic shared memory of a cluster kernel: more than half of an SM's 228 KB with the block's own 1 KB, so
+// that no SM holds two of their CTAs. Each takes TMEM for itself, and with two of different clusters on an SM each
+// cluster could hold the columns that the other's CTA waits for, before a cluster barrier that none would pass.
+constexpr size_t kClusterSmem = 117 * 1024;
+static_assert(2 * (kClusterSmem + 1024) > 228 * 1024, "one CTA per SM");
+
 // Positions per tile of the window kernels: 256 (any start), or, for rows of at
 // least 64 positions, the whole rows that fit in 256 (row-aligned starts need no
 // strip row for a misaligned start).
@@ -2576,7 +2583,7 @@ bool winpair_setup(const dbl_conv_shape* s, bool dgrad, Plan& pl)
     pl.win = pl.winpair = pl.res = true;
     pl.BN = 64;
     pl.cg = cg;
-    pl.smem = smem;
+    pl.smem = cg == 2 ? std::max(smem, kClusterSmem) : smem;
     p.win_margin = 128 % pitch;
     p.win_R = p.win_S = 3;
     p.win_ph = p.win_pw = 1;
@@ -2648,7 +2655,7 @@ bool win_setup(const dbl_conv_shape* s, int red_c, int out_c, bool dgrad, Plan& 
     pl.res = res;
     pl.BN = BN;
     pl.cg = cg;
-    pl.smem = smem;
+    pl.smem = cg == 2 ? std::max(smem, kClusterSmem) : smem;
     p.win_margin = margin;
     p.win_R = s->r;
     p.win_S = s->s;
@@ -2812,6 +2819,7 @@ bool wgtap_setup(const dbl_conv_shape* s, Plan& pl)
     // (one round 334 and 5.2e-5); short K-blocks lose there (16x16, batch 2330, 144 positions 485 -> 532).
     const double used = (double)s->n * P * (Wp - 2) / ((double)p.num_kb * p.win_tile);
     if (used < 0.8 || (double)p.kb_per_split * p.win_tile * 12 < 22000.0) return false;
+    if (p.win_cl > 1) pl.smem = std::max(pl.smem, kClusterSmem);
     pl.win = pl.wgtap = true;
     pl.BN = 128;
     pl.mode = p.mode = kWgrad;

@@ -240,6 +240,21 @@ def test_window_pairs_of_64_columns_only_for_comparison():
     assert got == {"1": 1, "2": 2}
 
 
+@pytest.mark.parametrize("shape,pad_w,pass_", [
+    ((1, 51, 10, 128, 128, 1, 1, 1), 3, 0),      # window pairs at their narrowest
+    ((4000, 3, 39, 128, 128, 3, 1, 2), 2, 2),    # filter rows, short K-blocks
+    ((512, 28, 28, 128, 128, 3, 1, 1), 1, 0),
+    ((512, 28, 28, 128, 128, 3, 1, 1), 1, 2),
+])
+def test_cluster_ctas_do_not_share_an_sm(D, shape, pad_w, pass_):
+    """Two CTAs of cluster kernels, 1 KB of shared memory for each block besides, exceed an SM's 228 KB: sharing one,
+    two clusters could wait for each other's tensor memory."""
+    n, h, w, c, k, r, st, pad = shape
+    i = D.dbl_conv_plan(D.conv_shape(n, h, w, c, k, r, st, pad, s=r, stride_w=1, pad_w=pad_w), pass_)
+    assert i.ctas_per_mma == 2 or i.grid > 3 * i.zdim  # pairs; filter rows in clusters
+    assert 2 * (i.smem_bytes + 1024) > 228 * 1024
+
+
 def test_clusters_that_the_device_cannot_place_are_not_planned():
     """DBL_MAX_CLUSTER (read once per process) stands for a device or context that places smaller clusters: the
     split passes take the next smaller cluster, or none.  Grid: 2 * pairs per tile CTAs of each tile."""
