@@ -450,7 +450,6 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, CG>::THREADS, 1)
                       const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2,
                       const ConvParams p)
 {
-    dbl::dev::grid_dependency_trigger();  // a convolution launched next may start its set-up
     using C = Cfg<BN, FAM, CG>;
     constexpr int STAGES = C::STAGES;
     extern __shared__ uint8_t smem_raw[];
@@ -498,6 +497,7 @@ __global__ void __launch_bounds__(Cfg<BN, FAM, CG>::THREADS, 1)
     __syncthreads();
     if constexpr (CG == 2) cluster_sync_all();  // both CTAs' barriers initialised, TMEM allocated
     tc_fence_after();
+    grid_dependency_trigger();  // a convolution launched next may start its set-up: this CTA has its TMEM
     grid_dependency_wait();  // the set-up above may overlap the previous kernel; memory only after it
     const uint32_t tmem = tmem_slot;
     const int64_t gPQ = (int64_t)p.gP * p.gQ;
@@ -827,7 +827,6 @@ __global__ void __launch_bounds__(SplitCfg<BN, FAM, SK>::THREADS, 1)
                        const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2,
                        const ConvParams p)
 {
-    dbl::dev::grid_dependency_trigger();  // a convolution launched next may start its set-up
     using S = SplitCfg<BN, FAM, SK>;
     using C = typename S::C;
     constexpr int STAGES = C::STAGES, W = S::W;
@@ -880,6 +879,7 @@ __global__ void __launch_bounds__(SplitCfg<BN, FAM, SK>::THREADS, 1)
     __syncthreads();
     cluster_sync_all();  // every CTA's barriers initialised, TMEM allocated
     tc_fence_after();
+    grid_dependency_trigger();  // a convolution launched next may start its set-up: this CTA has its TMEM
     grid_dependency_wait();  // the set-up above may overlap the previous kernel; memory only after it
     const uint32_t tmem = tmem_slot;
     const int64_t gPQ = (int64_t)p.gP * p.gQ;
@@ -1165,7 +1165,6 @@ __global__ void __launch_bounds__(WinCfg<BN>::THREADS, 1)
     conv_win_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const ConvParams p)
 {
-    dbl::dev::grid_dependency_trigger();  // a convolution launched next may start its set-up
     using C = WinCfg<BN>;
     static_assert(CG == 1 || BN == 128 || !DG, "data-gradient pairs split the weights in 64-column halves");
     constexpr int BT = C::B_TILE / CG;  // this CTA's bytes of one tap x 64-channel block of weights
@@ -1223,6 +1222,7 @@ __global__ void __launch_bounds__(WinCfg<BN>::THREADS, 1)
     __syncthreads();
     if constexpr (CG == 2) cluster_sync_all();  // both CTAs' barriers initialised, TMEM allocated
     tc_fence_after();
+    grid_dependency_trigger();  // a convolution launched next may start its set-up: this CTA has its TMEM
     grid_dependency_wait();  // the set-up above may overlap the previous kernel; memory only after it
     const uint32_t tmem = tmem_slot;
     const int Wp = p.win_Wp;
@@ -1513,7 +1513,6 @@ __global__ void __launch_bounds__(kWinThreads, 1)
     conv_winpair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                         const __grid_constant__ CUtensorMap tmB32, const ConvParams p)
 {
-    dbl::dev::grid_dependency_trigger();  // a convolution launched next may start its set-up
     static_assert(CG == 1 || !DG, "a 32-column half of an MN-major operand has no layout");
     constexpr int BT = 64 * 64 * 2;  // one tap of weights
     // Resident weights.  CG = 1: tap (r, s) at slot 3r + 2 - s.  CG = 2, per filter row r: this rank's tap of
@@ -1563,6 +1562,7 @@ __global__ void __launch_bounds__(kWinThreads, 1)
     __syncthreads();
     if constexpr (CG == 2) cluster_sync_all();  // both CTAs' barriers initialised, TMEM allocated
     tc_fence_after();
+    grid_dependency_trigger();  // a convolution launched next may start its set-up: this CTA has its TMEM
     grid_dependency_wait();  // the set-up above may overlap the previous kernel; memory only after it
     const uint32_t tmem = tmem_slot;
 
@@ -1765,7 +1765,6 @@ __global__ void __launch_bounds__(kWinThreads, 1)
     conv_wgwin_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmDY,
                       const ConvParams p)
 {
-    dbl::dev::grid_dependency_trigger();  // a convolution launched next may start its set-up
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[2], empty_bar[2], accf_bar, acce_bar, drain_bar;
     __shared__ uint32_t tmem_slot;
@@ -1798,6 +1797,7 @@ __global__ void __launch_bounds__(kWinThreads, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    grid_dependency_trigger();  // a convolution launched next may start its set-up: this CTA has its TMEM
     grid_dependency_wait();  // the set-up above may overlap the previous kernel; memory only after it
     const uint32_t tmem = tmem_slot;
 
@@ -1971,7 +1971,6 @@ __global__ void __launch_bounds__(kWinThreads, 1)
     conv_wgrow_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmDY,
                       const ConvParams p)
 {
-    dbl::dev::grid_dependency_trigger();  // a convolution launched next may start its set-up
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[kWgRowMaxStages], empty_bar[kWgRowMaxStages], accf_bar, drain_bar;
     __shared__ uint32_t tmem_slot;
@@ -2011,6 +2010,7 @@ __global__ void __launch_bounds__(kWinThreads, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    grid_dependency_trigger();  // a convolution launched next may start its set-up: this CTA has its TMEM
     grid_dependency_wait();  // the set-up above may overlap the previous kernel; memory only after it
     const uint32_t tmem = tmem_slot;
     // this CTA's K-blocks (grid = slices: at least one K-block each)
@@ -2161,7 +2161,6 @@ __global__ void __launch_bounds__(kWgTapThreads, 1)
     conv_wgtap_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmDY,
                       const ConvParams p)
 {
-    dbl::dev::grid_dependency_trigger();  // a convolution launched next may start its set-up
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[kWgTapMaxStages], empty_bar[kWgTapMaxStages], accf_bar, drain_bar;
     __shared__ uint32_t tmem_slot;
@@ -2197,6 +2196,7 @@ __global__ void __launch_bounds__(kWgTapThreads, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    grid_dependency_trigger();  // a convolution launched next may start its set-up: this CTA has its TMEM
     grid_dependency_wait();  // the set-up above may overlap the previous kernel; memory only after it
     const uint32_t tmem = tmem_slot;
     // this CTA's outputs and K-blocks (possibly none): the clusters of one slice are adjacent

@@ -1111,7 +1111,8 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo_bytes
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Lets the next kernel on the stream (if launched with programmatic stream serialization) be
 // scheduled once every CTA of this one has issued this or exited; it still waits for this
-// kernel's completion before touching memory.
+// kernel's completion before touching memory.  Kernels that take TMEM issue it once they have it: the next
+// kernel's CTA on the same SM could otherwise take the columns first and keep them while it waits for this one.
 __device__ __forceinline__ void grid_dependency_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Instruction descriptor, kind::f16 with A and B both in the storage format (bf16, or f16 in the
